@@ -100,7 +100,26 @@ SoftmaxPlan plan_softmax(int R, int B, int Hq, int Hkv, int D, int page_size, in
   memset(&pl, 0, sizeof pl);
   const int G = Hq / Hkv, M = B * G;
   const long prefix_max = (long)max_pages * page_size;
-  if (bf16 && softmax_tc_supported(B, Hq, Hkv, D, page_size)) {
+  if (bf16 && softmax_pair_supported(B, Hq, Hkv, D, page_size)) {
+    // two-SM kernel, for every shape with a second row tile to share the keys
+    // with (at M <= 128 the second CTA would have no rows): 256 query rows per
+    // pair of CTAs, one pair per two SMs.  One SM per row tile takes 1.023 ms
+    // where this takes 0.763 (128 requests, B = 64, G = 8) and 0.150 against
+    // 0.128 (64 requests, B = 32, G = 8).  Splits as below, over 128-key tiles.
+    pl.kernel = 2;
+    pl.rows_per_cta = 128;
+    const long items = (long)R * Hkv * ((M + 255) / 256), pairs = num_sms / 2;
+    const long tiles = (prefix_max + 127) / 128;
+    long ns = 1;
+    if (items > 0 && items < pairs) ns = (2L * pairs + items - 1) / items;
+    const long cap = tiles / 8 > 1 ? tiles / 8 : 1;
+    if (ns > cap) ns = cap;
+    if (ns > 64) ns = 64;  // the merge keeps 128 x n_split weights in shared memory
+    const long tps = ns > 0 ? (tiles + ns - 1) / ns : 1;
+    pl.split_len = (int)((tps > 0 ? tps : 1) * 128);
+    pl.n_split = tiles > 0 ? (int)((tiles + tps - 1) / tps) : 1;
+    if (pl.n_split < 1) pl.n_split = 1;
+  } else if (bf16 && softmax_tc_supported(B, Hq, Hkv, D, page_size)) {
     // tensor-core kernel: 128 query rows per CTA, one CTA per SM, work units
     // started longest first.  Split the prefix only when the batch has fewer
     // work items than SMs (then aim at two CTAs per SM), and keep at least 16
@@ -139,16 +158,18 @@ SoftmaxPlan plan_softmax(int R, int B, int Hq, int Hkv, int D, int page_size, in
     pl.ws_o_bytes = (rows * D * sizeof(float) + 255) / 256 * 256;
     pl.ws_lse_bytes = (rows * sizeof(float) + 255) / 256 * 256;
   }
-  // tensor-core kernel: the work units in longest-first order, and per row
+  // tensor-core kernels: the work units in longest-first order, and per row
   // tile a count of finished splits (the last one merges the partials)
-  if (pl.kernel == 1) {
+  if (pl.kernel != 0) {
     // order [R*n_split], n_valid [1], bad-request mask [ceil(R/32)]
     pl.ws_order_bytes =
         (((size_t)R * pl.n_split + 1 + (size_t)(R + 31) / 32) * sizeof(int32_t) + 255) / 256 * 256;
-    // one CTA per work item when the prefix is split, else one per SM (at most
-    // one per work item) walking the items
-    const long n_items = (long)((M + 127) / 128) * Hkv * R * pl.n_split;
-    pl.num_ctas = (int)(pl.n_split > 1 ? n_items : (n_items < num_sms ? n_items : num_sms));
+    // one CTA (or pair) per work item when the prefix is split, else one per SM
+    // (at most one per work item) walking the items
+    const long group = pl.kernel == 2 ? 2 : 1;
+    const long n_items = (M + 128 * group - 1) / (128 * group) * Hkv * R * pl.n_split;
+    const long groups = num_sms / group;
+    pl.num_ctas = (int)(group * (pl.n_split > 1 || n_items < groups ? n_items : groups));
     if (pl.n_split > 1)
       pl.ws_count_bytes =
           ((size_t)R * Hkv * ((M + 127) / 128) * sizeof(int32_t) + 255) / 256 * 256;
@@ -159,6 +180,7 @@ SoftmaxPlan plan_softmax(int R, int B, int Hq, int Hkv, int D, int page_size, in
 
 cudaError_t launch_softmax(const SoftmaxParams& p, const SoftmaxPlan& plan, bool bf16,
                            cudaStream_t stream) {
+  if (plan.kernel == 2) return launch_softmax_pair(p, plan, stream);
   if (plan.kernel == 1) return launch_softmax_tc(p, plan, stream);
   return launch_softmax_simt(p, plan, bf16, stream);
 }

@@ -61,11 +61,11 @@ struct SoftmaxParams {
 // Work decomposition of the softmax call; identical for the workspace query
 // and the launch.
 struct SoftmaxPlan {
-  int kernel;  // 0 = CUDA-core kernel, 1 = tensor-core kernel
+  int kernel;  // 0 = CUDA-core kernel, 1 = tensor-core kernel, 2 = two-SM tensor-core kernel
   int rows_per_cta;
   int n_split;
   int split_len;
-  int num_ctas;  // tensor-core kernel: CTAs launched
+  int num_ctas;  // tensor-core kernels: CTAs launched
   size_t ws_o_bytes, ws_lse_bytes, ws_order_bytes, ws_count_bytes;
   size_t workspace_bytes;
 };
@@ -140,6 +140,9 @@ cudaError_t launch_softmax_tc(const SoftmaxParams& p, const SoftmaxPlan& plan,
                               cudaStream_t stream);
 cudaError_t launch_softmax_combine(const SoftmaxParams& p, bool bf16, cudaStream_t stream);
 bool softmax_tc_supported(int B, int Hq, int Hkv, int D, int page_size);
+cudaError_t launch_softmax_pair(const SoftmaxParams& p, const SoftmaxPlan& plan,
+                                cudaStream_t stream);
+bool softmax_pair_supported(int B, int Hq, int Hkv, int D, int page_size);
 cudaError_t launch_append_kv(const SoftmaxParams& p, const int32_t* append_len, void* k_pool,
                              void* v_pool, int elem_bytes, cudaStream_t stream);
 cudaError_t launch_debug_wait_timeout(int32_t* status, uint64_t limit_ns, cudaStream_t stream);

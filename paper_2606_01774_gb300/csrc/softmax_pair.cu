@@ -1,0 +1,856 @@
+// Block-query softmax attention over a paged KV prefix with two-SM tensor-core
+// products (tcgen05, cta_group::2): bf16, head dim 128 or 256, more than 128
+// query rows (block positions x grouped query heads) per kv head.
+//
+// A work item is (request r, kv head, pair of 128-row tiles, prefix split), run
+// by a cluster of two CTAs on the two SMs of a TPC.  Each CTA owns one row
+// tile: its Q rows, its S and O accumulators in its own tensor memory, its
+// softmax rows, its outputs.  The K and V tiles are shared: an M = 256 product
+// takes half of its B operand from each CTA's shared memory, so each CTA loads
+// keys 64*rank .. +63 of a 128-key K tile and value columns (D/2)*rank .. of
+// the V tile.  What this is for: with one SM per row tile (softmax_tc.cu) each
+// SM moves every K and V byte in by TMA and out as an MMA operand, and those
+// two streams through its shared memory and the rings' bytes in flight set the
+// tile rate, not the tensor pipe; the pair halves both per product.
+//
+// Measured (GB300, start against this kernel): 128 requests, blocks of 64,
+// prefixes of 1024..16384, D = 256: 1.023 -> 0.763 ms per call back to back
+// (1.54 PFLOP/s, at the power cap; 0.65 ms, 1.81 PFLOP/s, in short bursts);
+// 64 requests, blocks of 32, prefixes of 512..8192: 0.150 -> 0.128 ms.  Bound
+// by the tensor pipe (1.26 us per 128-key tile of a pair, 0.99 us at the clock's
+// peak rate) and, for the smaller call, by HBM.
+
+// Tensor memory: O [0, D), then two S buffers of 128 columns, each overwritten
+// in place by its bf16 probabilities P.  Q sits in shared memory (128-byte
+// swizzle, loaded by TMA, once per item) so that S tiles can be 128 keys
+// wide: the softmax of a tile then has two products (S of the tile after
+// next, P.V of the one before) to hide behind, and half the hand-offs of
+// 64-key tiles.  The rest of shared memory is one ring of K and V half tiles in
+// the order the products consume them (K_0, K_1, V_0, K_2, V_1, ...).
+//
+// Warp roles (256 threads per CTA):
+//   warps 0, 6 K and V producers: page ids a window ahead in registers, one TMA box
+//              per page and 64-column chunk, completing on the leader's barriers.
+//   warp 1     tensor-memory owner; in the leader (rank 0) one thread issues the
+//              products of the pair and commits to both CTAs' barriers.
+//   warps 2-5  softmax, one query row per thread, as in softmax_tc.cu.
+//   warp 7     loads Q, and zeroes the up to 15 V rows between the prefix end and the next
+//              multiple of 16 (a P.V step), which hold stale cache rows.
+// Barriers the leader's MMA thread waits on live in the leader and are
+// arrived at by both CTAs; barriers its commits complete exist in both CTAs
+// (multicast commit).  Every wait is bounded (2 s); a timeout sets
+// FLARE_DEV_WAIT_TIMEOUT, ends the CTA's roles (the peer's waits then run out
+// too) and nothing more is written.  The two cluster barriers and the paired
+// tensor-memory allocation are reached by every thread on every path.
+#include "common.cuh"
+#include "kernels.h"
+#include "softmax_common.cuh"
+#include "tc.cuh"
+
+namespace flare {
+
+namespace {
+
+constexpr int kPairKeys = 128;     // keys per tile
+constexpr int kPairThreads = 256;
+constexpr float kPairRescale = 8.0f;  // log2 units
+
+struct PairMaps {
+  CUtensorMap q;      // (D, Hq, B, R)          box (64, G, 128/G, 1)
+  CUtensorMap kblk;   // (D, Hkv, B, R)         box (64, 1, 32, 1)
+  CUtensorMap vblk;   // (D, Hkv, B, R)         box (64, 1, 64, 1)
+  // (64, p, D/64, Hkv, num_pages): a page-head as 64-column chunks.  Pages of 64 or
+  // 128 tokens: box (64, 64, chunks of a slot, 1, 1); smaller: box (64, p, 1, 1, 1)
+  CUtensorMap kpool;
+  CUtensorMap vpool;
+};
+
+template <int D>
+struct PairCfg {
+  // 64-column chunks of a CTA's K half tile (64 keys, all columns) and V half tile
+  // (128 keys, half the columns): a slot holds [chunk][64 rows][128 B] for K and
+  // [64-key half][chunk][64 rows][128 B] for V
+  static constexpr int kKChunks = D / 64;
+  static constexpr int kVChunks = D / 128;
+  static constexpr int kSlotBytes = D * 128;
+  static constexpr int kQBytes = kRowsM * D * 2;
+  static constexpr int kSlots = (225 * 1024 - kQBytes) / kSlotBytes;
+  static constexpr int kSmem = kQBytes + kSlots * kSlotBytes;
+  static constexpr int kSCol = D;
+  static constexpr int kTmemCols = 512;
+};
+
+struct PairShared {
+  uint64_t full[16];     // leader: a slot's loads of both CTAs have landed (2 arrivals)
+  uint64_t empty[16];    // both: the products reading a slot are done
+  uint64_t vr_full[16];  // both: a ragged V slot has landed here, to be fixed
+  uint64_t s_full[2];    // both: S tile ready
+  uint64_t p_full[2];    // leader: P tile of both row tiles ready (8 warps)
+  uint64_t pv_done[2];   // both
+  uint64_t q_full;       // leader: Q of both row tiles (2 arrivals)
+  uint64_t q_empty;      // both: the item's S products are done
+  uint64_t o_final;      // both: the item's last P.V is done
+  uint64_t o_free;       // leader: O read out by both CTAs (8 warps)
+  uint32_t tmem_base;
+  int abort_flag;
+  int last_split;
+};
+
+// ------------------------------------------------------------------ cluster PTX
+
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+
+// One lane of a converged warp, always the same one.  The products and copies are
+// issued under this branch: the compiler then knows that a single thread is
+// active and takes their descriptors from uniform registers.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t pred;
+  asm volatile(
+      "{\n"
+      " .reg .pred p;\n"
+      " elect.sync _|p, 0xffffffff;\n"
+      " selp.b32 %0, 1, 0, p;\n"
+      "}\n"
+      : "=r"(pred));
+  return pred != 0;
+}
+
+__device__ __forceinline__ uint32_t map_rank(uint32_t saddr, uint32_t rank) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(saddr), "r"(rank));
+  return a;
+}
+
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// Arrivals on a barrier given by its cluster address (either CTA's).  At the
+// default scope, like every wait of this kernel: what the arrivals publish
+// is tensor memory (ordered by the tcgen05 fences) and shared memory read by
+// the async proxy (ordered by its proxy fence), and an explicit cluster
+// scope costs about 0.5 us per operation (2.07 against 1.03 ms per
+// multistep_batch128 call).
+__device__ __forceinline__ void arrive_at(uint32_t caddr) {
+  asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(caddr)
+               : "memory");
+}
+__device__ __forceinline__ void expect_at(uint32_t caddr, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cluster.b64 _, [%0], %1;" ::"r"(
+                   caddr),
+               "r"(bytes)
+               : "memory");
+}
+
+__device__ __forceinline__ bool pair_warp_wait(uint64_t* bar, uint32_t parity, const int* abort) {
+  return __all_sync(0xffffffffu, tc::mbar_wait(bar, parity, abort));
+}
+
+// TMA into this CTA's shared memory, completing on a barrier of either CTA of the pair
+__device__ __forceinline__ void tma2_load_5d(uint32_t dst, const CUtensorMap* map, uint32_t bar,
+                                             int c0, int c1, int c2, int c3, int c4) {
+  asm volatile(
+      "cp.async.bulk.tensor.5d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes"
+      " [%0], [%1, {%3, %4, %5, %6, %7}], [%2];" ::"r"(dst),
+      "l"(map), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4)
+      : "memory");
+}
+
+__device__ __forceinline__ void tma2_load_4d(uint32_t dst, const CUtensorMap* map, uint32_t bar,
+                                             int c0, int c1, int c2, int c3) {
+  asm volatile(
+      "cp.async.bulk.tensor.4d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes"
+      " [%0], [%1, {%3, %4, %5, %6}], [%2];" ::"r"(dst),
+      "l"(map), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
+      : "memory");
+}
+
+__device__ __forceinline__ void mma2_ss(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc,
+                                        uint32_t accumulate) {
+  asm volatile(
+      "{\n"
+      " .reg .pred p;\n"
+      " setp.ne.b32 p, %4, 0;\n"
+      " tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n"
+      "}\n" ::"r"(d),
+      "l"(a), "l"(b), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+
+__device__ __forceinline__ void mma2_ts(uint32_t d, uint32_t a, uint64_t b, uint32_t idesc,
+                                        uint32_t accumulate) {
+  asm volatile(
+      "{\n"
+      " .reg .pred p;\n"
+      " setp.ne.b32 p, %4, 0;\n"
+      " tcgen05.mma.cta_group::2.kind::f16 [%0], [%1], %2, %3, p;\n"
+      "}\n" ::"r"(d),
+      "r"(a), "l"(b), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+
+// One arrival on `bar` in both CTAs once the products issued so far are done.
+__device__ __forceinline__ void commit2(uint64_t* bar) {
+  asm volatile(
+      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64"
+      " [%0], %1;" ::"r"(tc::smem_u32(bar)),
+      "h"((uint16_t)3)
+      : "memory");
+}
+
+// ------------------------------------------------------------------ work items
+
+struct PairWork {
+  int r, kvh, mpair, split, item, P;
+  int tok_lo, n_pref, n_tiles;  // first prefix token, prefix tiles, all tiles
+  int tok_hi;                   // prefix tokens of this split end here
+  bool block;                   // the last tile holds the block's own keys
+};
+
+// Item `idx`: (row-tile pair, kv head) fastest, then the valid work units
+// (request, prefix split) in longest-first order.
+__device__ __forceinline__ PairWork pair_work(const SoftmaxParams& p, int n_mp, int idx) {
+  PairWork w;
+  w.mpair = idx % n_mp;
+  w.kvh = (idx / n_mp) % p.Hkv;
+  const int unit = p.order[idx / (n_mp * p.Hkv)];
+  w.r = unit / p.n_split;
+  w.split = unit % p.n_split;
+  w.item = w.r * p.Hkv + w.kvh;
+  w.P = p.prefix_len[w.r];
+  w.tok_lo = min(w.P, w.split * p.split_len);
+  w.tok_hi = min(w.P, w.tok_lo + p.split_len);
+  w.n_pref = (w.tok_hi - w.tok_lo + kPairKeys - 1) / kPairKeys;
+  w.block = w.split == p.n_split - 1;
+  w.n_tiles = w.n_pref + (w.block ? 1 : 0);
+  return w;
+}
+
+// Keys of tile j that exist (a P.V takes ceil(valid / 16) steps).
+__device__ __forceinline__ int tile_valid(const SoftmaxParams& p, const PairWork& w, int j) {
+  return j >= w.n_pref ? p.B : min(kPairKeys, w.tok_hi - (w.tok_lo + j * kPairKeys));
+}
+
+__device__ __forceinline__ bool pair_aborted(const PairShared& sh) {
+  return *reinterpret_cast<const volatile int*>(&sh.abort_flag) != 0;
+}
+
+__device__ __forceinline__ void pair_abort(PairShared& sh, int32_t* status) {
+  if (!sh.abort_flag) {
+    sh.abort_flag = 1;
+    flag(status, FLARE_DEV_WAIT_TIMEOUT);
+  }
+}
+
+// Online softmax of one query row over one tile of NC keys: reads the row's
+// raw scores from tensor memory, moves the running max, writes P as bf16 pairs
+// over them.  FULL: no mask (a whole prefix tile); else keys c >= lim are
+// hidden.  `rescale(corr)` multiplies O by corr (warp-uniform decision).
+template <int NC, bool FULL, typename F>
+__device__ __forceinline__ bool softmax_row(uint32_t sbuf, int lim, float scale_log2, bool first,
+                                            float& m_run, float& l_run, F&& rescale) {
+  uint32_t sr[NC];
+#pragma unroll
+  for (int c = 0; c < NC; c += 16)
+    tc::tmem_ld16(sbuf + c, *reinterpret_cast<uint32_t(*)[16]>(&sr[c]));
+  tc::tmem_ld_wait();
+  float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+  for (int c = 0; c < NC; ++c)
+    if (FULL || c < lim) mx[c & 3] = fmaxf(mx[c & 3], __uint_as_float(sr[c]));
+  const float mt = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
+  const float m_new = fmaxf(m_run, mt * scale_log2);
+  const bool need = first || (m_new > m_run + kPairRescale);
+  const bool warp_rescale = __any_sync(0xffffffffu, need);
+  float m_use = m_run;
+  if (warp_rescale) m_use = (first || m_new > m_run) ? m_new : m_run;
+  const float corr = first ? 0.f : tc::ex2(m_run - m_use);
+  const uint64_t neg_m = f2_dup(-m_use), sc = f2_dup(scale_log2);
+  uint64_t sum[2] = {0, 0};  // fp32 pairs of zero
+#pragma unroll
+  for (int c0 = 0; c0 < NC; c0 += 32) {
+    uint32_t pk[16];
+#pragma unroll
+    for (int e = 0; e < 16; ++e) {
+      const int c = c0 + 2 * e;
+      const uint64_t z =
+          f2_fma(f2(__uint_as_float(sr[c]), __uint_as_float(sr[c + 1])), sc, neg_m);
+      float z0, z1;
+      f2_split(z, z0, z1);
+      float p0 = tc::ex2(z0), p1 = tc::ex2(z1);
+      if (!FULL) {
+        p0 = c < lim ? p0 : 0.f;
+        p1 = c + 1 < lim ? p1 : 0.f;
+      }
+      sum[e & 1] = f2_add(sum[e & 1], f2(p0, p1));
+      __nv_bfloat162 h2 = __floats2bfloat162_rn(p0, p1);
+      pk[e] = *reinterpret_cast<uint32_t*>(&h2);
+    }
+    tc::tmem_st16(sbuf + c0 / 2, pk);
+  }
+  float s0, s1;
+  f2_split(f2_add(sum[0], sum[1]), s0, s1);
+  const float s = s0 + s1;
+  l_run = first ? s : l_run * corr + s;
+  m_run = m_use;
+  return (warp_rescale && !first) ? rescale(corr) : true;
+}
+
+}  // namespace
+
+template <int D>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
+    softmax_pair_kernel(const __grid_constant__ PairMaps maps, SoftmaxParams p) {
+  using C = PairCfg<D>;
+  extern __shared__ uint8_t smem_raw[];
+  __shared__ PairShared sh;
+  uint8_t* base = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  uint8_t* Qs = base;
+  uint8_t* ring = base + C::kQBytes;
+
+  const int M = p.B * p.G;
+  const int n_mt = (M + kRowsM - 1) / kRowsM;
+  const int n_mp = (n_mt + 1) / 2;
+  const int n_items = n_mp * p.Hkv * *p.n_valid;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const uint32_t rank = cluster_rank();
+  const bool split_mode = p.n_split > 1;
+  const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
+  // k-th work item of this pair, or -1 (the same answer in both CTAs)
+  auto item_of = [&](int k) -> int {
+    if (split_mode) return (k == 0 && pair < n_items) ? pair : -1;
+    const int idx = k * n_pairs + ((k & 1) ? n_pairs - 1 - pair : pair);
+    return idx < n_items ? idx : -1;
+  };
+  const int idx0 = item_of(0);
+  if (idx0 < 0) return;
+  if (split_mode) {
+    const PairWork w = pair_work(p, n_mp, idx0);
+    if (w.n_tiles == 0) {  // empty split: mark its partial as empty for the merge
+      const int mtile = 2 * w.mpair + (int)rank;
+      if (mtile >= n_mt) return;
+      const size_t ws_row0 = ((size_t)w.item * p.n_split + w.split) * M;
+      for (int i = tid; i < kRowsM; i += blockDim.x) {
+        const int m = mtile * kRowsM + i;
+        if (m < M) p.ws_lse[ws_row0 + m] = -INFINITY;
+      }
+      finish_split<D>(p, w.item, w.r, w.kvh, mtile, n_mt, &sh.last_split,
+                      reinterpret_cast<float*>(base));
+      return;
+    }
+  }
+
+  if (tid == 0) {
+    sh.abort_flag = 0;
+    sh.last_split = 0;
+    for (int s = 0; s < C::kSlots; ++s) {
+      tc::mbar_init(&sh.full[s], 2);
+      tc::mbar_init(&sh.empty[s], 1);
+      tc::mbar_init(&sh.vr_full[s], 1);
+    }
+    for (int b = 0; b < 2; ++b) {
+      tc::mbar_init(&sh.s_full[b], 1);
+      tc::mbar_init(&sh.p_full[b], 8);
+      tc::mbar_init(&sh.pv_done[b], 1);
+    }
+    tc::mbar_init(&sh.q_full, 2);
+    tc::mbar_init(&sh.q_empty, 1);
+    tc::mbar_init(&sh.o_final, 1);
+    tc::mbar_init(&sh.o_free, 8);
+    tc::fence_mbar_init();
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     tc::smem_u32(&sh.tmem_base)),
+                 "r"((uint32_t)C::kTmemCols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+  }
+  tc::fence_before_sync();
+  __syncthreads();
+  cluster_sync();  // both CTAs' barriers initialised before any arrival from the peer
+  tc::fence_after_sync();
+  const uint32_t tmem = sh.tmem_base;  // all 512 columns: the same base in both CTAs
+  const uint32_t tmem_o = tmem;
+  const uint32_t tmem_s = tmem + C::kSCol;
+  const uint32_t ring_u = tc::smem_u32(ring);
+
+  if (warp == 0 || warp == 6) {
+    // ------------------------------------------------------------ K, V producers
+    // warp 0 loads the K tiles and warp 6 the V tiles; both walk the ring in the
+    // order the products run (K_0, K_1, V_0, ..., K_{n-1}, V_{n-2}, V_{n-1}), each
+    // passing over the other's slots.  One issuing warp was the bound: about
+    // 0.6 us per slot against 0.25 us of tensor work (1.24 ms per
+    // multistep_batch128 call).
+    const bool is_v = warp == 6;
+    const CUtensorMap* pool_map = is_v ? &maps.vpool : &maps.kpool;
+    const CUtensorMap* blk_map = is_v ? &maps.vblk : &maps.kblk;
+    if (lane == 0) {
+      tc::prefetch_tmap(pool_map);
+      tc::prefetch_tmap(blk_map);
+    }
+    const int pshift = 31 - __clz(p.page_size);  // page sizes are powers of two
+    const int bshift = min(pshift, 6);           // log2 of a box's rows
+    const uint32_t full0 = map_rank(tc::smem_u32(&sh.full[0]), 0);  // the leader's barriers
+    const uint32_t vr0 = tc::smem_u32(&sh.vr_full[0]);
+    bool ok = true;
+    int st = 0;
+    uint32_t ph = 0;
+    auto pass = [&]() {
+      if (++st == C::kSlots) st = 0, ph ^= 1u;
+    };
+    auto acquire = [&]() { return pair_warp_wait(&sh.empty[st], ph ^ 1u, &sh.abort_flag); };
+    for (int k = 0; ok && !pair_aborted(sh); ++k) {
+      const int idx = item_of(k);
+      if (idx < 0) break;
+      const PairWork w = pair_work(p, n_mp, idx);
+      // page ids of the window [pbase, pbase + 64): two per lane, in cur and nxt
+      const int n_pages = (w.tok_hi + p.page_size - 1) >> pshift;
+      const int32_t* table = p.page_table + (size_t)w.r * p.max_pages;
+      int pbase = w.tok_lo >> pshift;
+      auto fetch = [&](int first) { return first + lane < n_pages ? table[first + lane] : 0; };
+      int cur = fetch(pbase), nxt = fetch(pbase + 32);
+      // keys [tok, tok + rows) of the prefix (at most 64) to dst: n_chunks chunks of
+      // 64 rows, from chunk ch
+      auto load_keys = [&](uint32_t dst, uint32_t bar, int tok, int rows, int ch, int n_chunks) {
+        const int nb = (rows + (1 << bshift) - 1) >> bshift;
+        for (int bx = 0; bx < nb; ++bx) {
+          const int t = tok + (bx << bshift);
+          const int o = (t >> pshift) - pbase;
+          const int pa = __shfl_sync(0xffffffffu, cur, o & 31);
+          const int pb = __shfl_sync(0xffffffffu, nxt, o & 31);
+          const int page = o < 32 ? pa : pb;
+          if (elect_one()) {
+            const int row = t & (p.page_size - 1);
+            if (bshift == 6) {
+              tma2_load_5d(dst, pool_map, bar, 0, row, ch, w.kvh, page);
+            } else {
+              for (int c = 0; c < n_chunks; ++c)
+                tma2_load_5d(dst + c * 8192 + ((uint32_t)bx << (bshift + 7)), pool_map, bar, 0, row,
+                             ch + c, w.kvh, page);
+            }
+          }
+          __syncwarp();
+        }
+      };
+      auto bytes_of = [&](int rows, int n_chunks) {
+        return (uint32_t)(((rows + (1 << bshift) - 1) >> bshift) * n_chunks) << (bshift + 7);
+      };
+      auto load_k = [&](int j) -> bool {
+        if (!acquire()) return false;
+        const uint32_t dst = ring_u + st * C::kSlotBytes, bar = full0 + st * 8;
+        if (j >= w.n_pref) {
+          if (elect_one()) {
+            expect_at(bar, C::kKChunks * 32 * 128);
+            for (int c = 0; c < C::kKChunks; ++c)
+              tma2_load_4d(dst + c * 8192, blk_map, bar, c * 64, w.kvh, (int)rank * 32, w.r);
+          }
+          __syncwarp();
+        } else {
+          const int tok = w.tok_lo + j * kPairKeys + (int)rank * 64;
+          const int rows = min(64, max(0, w.tok_hi - tok));
+          if (elect_one()) expect_at(bar, bytes_of(rows, C::kKChunks));
+          __syncwarp();
+          load_keys(dst, bar, tok, rows, 0, C::kKChunks);
+        }
+        return true;
+      };
+      auto load_v = [&](int j) -> bool {
+        if (!acquire()) return false;
+        const uint32_t dst = ring_u + st * C::kSlotBytes, bar = full0 + st * 8;
+        const int ch = (int)rank * C::kVChunks;
+        if (j >= w.n_pref) {
+          if (elect_one()) {
+            expect_at(bar, C::kVChunks * 64 * 128);
+            for (int c = 0; c < C::kVChunks; ++c)
+              tma2_load_4d(dst + c * 8192, blk_map, bar, (ch + c) * 64, w.kvh, 0, w.r);
+          }
+          __syncwarp();
+        } else {
+          const int tok = w.tok_lo + j * kPairKeys;
+          const int keys = min(kPairKeys, w.tok_hi - tok);
+          const int r0 = min(keys, 64), r1 = keys - r0;
+          // a tile the prefix ends in, off a 16-key step: it lands on this CTA's own
+          // barrier and the fixer arrives at the leader's once its rows are zero
+          const uint32_t to = (keys & 15) ? vr0 + st * 8 : bar;
+          if (elect_one()) expect_at(to, bytes_of(r0, C::kVChunks) + bytes_of(r1, C::kVChunks));
+          __syncwarp();
+          load_keys(dst, to, tok, r0, ch, C::kVChunks);
+          if (r1 > 0) load_keys(dst + C::kVChunks * 8192, to, tok + 64, r1, ch, C::kVChunks);
+        }
+        return true;
+      };
+      for (int j = 0; ok && j <= w.n_tiles; ++j) {
+        // the window follows the V tile (j - 1), the earlier of the two
+        if (j >= 1 && j <= w.n_pref &&
+            ((w.tok_lo + (j - 1) * kPairKeys) >> pshift) - pbase >= 32) {
+          pbase += 32;
+          cur = nxt;
+          nxt = fetch(pbase + 32);
+        }
+        if (j < w.n_tiles) {
+          if (!is_v) ok = load_k(j);
+          pass();
+        }
+        if (ok && j >= 1) {
+          if (is_v) ok = load_v(j - 1);
+          pass();
+        }
+      }
+    }
+    // every slot released: no commit of the leader is on its way to a barrier here
+    for (int s = 0; ok && s < C::kSlots; ++s) {
+      ok = acquire();
+      pass();
+    }
+    if (!ok && lane == 0) pair_abort(sh, p.dev_status);
+  } else if (warp == 1) {
+    // ------------------------------------------------------------ MMA issuer
+    // The whole warp walks the tiles and waits; one elected lane issues.
+    if (rank == 0) {
+      const uint32_t id_s128 = tc::idesc_bf16(2 * kRowsM, 128, false, false);
+      const uint32_t id_s64 = tc::idesc_bf16(2 * kRowsM, 64, false, false);
+      const uint32_t id_o = tc::idesc_bf16(2 * kRowsM, D, false, true);
+      const uint64_t qdesc = tc::sdesc_sw128(tc::smem_u32(Qs), 16, 1024);
+      const uint64_t kdesc0 = tc::sdesc_sw128(ring_u, 16, 1024);
+      const uint64_t vdesc0 = tc::sdesc_sw128(ring_u, 8192, 1024);
+      bool ok = true;
+      int g = 0;  // running tile count
+      int st = 0;
+      uint32_t ph = 0;
+      auto pass = [&]() {
+        if (++st == C::kSlots) st = 0, ph ^= 1u;
+      };
+      for (int k = 0; ok && !pair_aborted(sh); ++k) {
+        const int idx = item_of(k);
+        if (idx < 0) break;
+        const PairWork w = pair_work(p, n_mp, idx);
+        if (!pair_warp_wait(&sh.q_full, (uint32_t)k & 1u, &sh.abort_flag)) {
+          ok = false;
+          break;
+        }
+        // S_j = Q K_j^T (the block tile: 64 keys)
+        auto issue_s = [&](int j) -> bool {
+          const int sb = (g + j) & 1;
+          const uint32_t id_s = j >= w.n_pref ? id_s64 : id_s128;
+          if (!pair_warp_wait(&sh.full[st], ph, &sh.abort_flag)) return false;
+          tc::fence_after_sync();
+          if (elect_one()) {
+            const uint64_t kd = kdesc0 + (uint64_t)((st * C::kSlotBytes) >> 4);
+#pragma unroll
+            for (int kk = 0; kk < D / 16; ++kk) {
+              const int c = kk >> 2, off = (kk & 3) * 32;
+              mma2_ss(tmem_s + sb * 128, qdesc + (uint64_t)((c * 16384 + off) >> 4),
+                      kd + (uint64_t)((c * 8192 + off) >> 4), id_s, kk > 0 ? 1u : 0u);
+            }
+            commit2(&sh.s_full[sb]);
+            commit2(&sh.empty[st]);
+            if (j == w.n_tiles - 1) commit2(&sh.q_empty);
+          }
+          __syncwarp();
+          pass();
+          return true;
+        };
+        // O (+)= P_j V_j over the steps of 16 keys that hold one
+        auto issue_pv = [&](int j) -> bool {
+          const int gg = g + j, pb = gg & 1;
+          if (!pair_warp_wait(&sh.full[st], ph, &sh.abort_flag)) return false;
+          // the first P.V of an item overwrites O: the previous item's must be out
+          if (j == 0 && k > 0 &&
+              !pair_warp_wait(&sh.o_free, (uint32_t)(k - 1) & 1u, &sh.abort_flag))
+            return false;
+          if (!pair_warp_wait(&sh.p_full[pb], (uint32_t)(gg >> 1) & 1u, &sh.abort_flag))
+            return false;
+          tc::fence_after_sync();
+          if (elect_one()) {
+            const uint64_t vd = vdesc0 + (uint64_t)((st * C::kSlotBytes) >> 4);
+            const uint32_t pt = tmem_s + pb * 128;
+            auto step = [&](int kk) {
+              mma2_ts(tmem_o, pt + kk * 8,
+                      vd + (uint64_t)(((kk >> 2) * (C::kVChunks * 8192) + (kk & 3) * 2048) >> 4),
+                      id_o, (j > 0 || kk > 0) ? 1u : 0u);
+            };
+            const int steps = (tile_valid(p, w, j) + 15) >> 4;
+            if (steps == 8) {
+#pragma unroll
+              for (int kk = 0; kk < 8; ++kk) step(kk);
+            } else {
+#pragma unroll 1
+              for (int kk = 0; kk < steps; ++kk) step(kk);
+            }
+            commit2(&sh.pv_done[pb]);
+            commit2(&sh.empty[st]);
+          }
+          __syncwarp();
+          pass();
+          return true;
+        };
+        for (int j = 0; ok && j <= w.n_tiles; ++j) {
+          if (j < w.n_tiles) ok = issue_s(j);
+          if (ok && j >= 1) ok = issue_pv(j - 1);
+        }
+        g += w.n_tiles;
+      }
+      if (!ok && lane == 0) pair_abort(sh, p.dev_status);
+    }
+    __syncwarp();
+  } else if (warp == 7) {
+    // ------------------------------------------------------------ Q loads, V fixer
+    if (lane == 0) tc::prefetch_tmap(&maps.q);
+    const uint32_t q_full_c = map_rank(tc::smem_u32(&sh.q_full), 0);
+    bool ok = true;
+    int cnt = 0;               // running slot count at the item's start
+    uint32_t par = 0u;         // per slot: parity of its next ragged phase
+    for (int k = 0; ok && !pair_aborted(sh); ++k) {
+      // the previous item's S products, the last readers of its Q, are done
+      if (k > 0 && !pair_warp_wait(&sh.q_empty, (uint32_t)(k - 1) & 1u, &sh.abort_flag)) {
+        ok = false;
+        break;
+      }
+      const int idx = item_of(k);
+      if (idx < 0) break;
+      const PairWork w = pair_work(p, n_mp, idx);
+      if (lane == 0) {
+        expect_at(q_full_c, C::kQBytes);
+        // rows past the block (t >= B) read as zero
+        const int t0 = (2 * w.mpair + (int)rank) * (kRowsM / p.G);
+        for (int c = 0; c < D / 64; ++c)
+          tma2_load_4d(tc::smem_u32(Qs) + c * 16384, &maps.q, q_full_c, c * 64, w.kvh * p.G, t0,
+                       w.r);
+      }
+      const int keys = w.n_pref > 0 ? tile_valid(p, w, w.n_pref - 1) : 0;
+      if (keys & 15) {
+        // ring position of V_j: 2j + 2, the item's last V: 2n - 1
+        const int j = w.n_pref - 1;
+        const int st = (cnt + (j < w.n_tiles - 1 ? 2 * j + 2 : 2 * w.n_tiles - 1)) % C::kSlots;
+        if (!pair_warp_wait(&sh.vr_full[st], (par >> st) & 1u, &sh.abort_flag)) {
+          ok = false;
+          break;
+        }
+        par ^= 1u << st;
+        uint8_t* dst = ring + st * C::kSlotBytes + (keys >> 6) * (C::kVChunks * 8192) +
+                       (keys & 63) * 128;
+        const int n16 = (16 - (keys & 15)) * 8;  // 16-byte pieces per 64-column chunk
+#pragma unroll
+        for (int c = 0; c < C::kVChunks; ++c)
+          for (int e = lane; e < n16; e += 32)
+            *reinterpret_cast<uint4*>(dst + c * 8192 + e * 16) = make_uint4(0u, 0u, 0u, 0u);
+        tc::fence_async_smem();
+        __syncwarp();
+        if (lane == 0) arrive_at(map_rank(tc::smem_u32(&sh.full[st]), 0));
+      }
+      cnt = (cnt + 2 * w.n_tiles) % C::kSlots;
+    }
+    if (!ok && lane == 0) pair_abort(sh, p.dev_status);
+  } else {
+    // ------------------------------------------------------------ softmax warps
+    const int quarter = warp & 3;
+    const int row = quarter * 32 + lane;
+    const uint32_t lane_off = (uint32_t)(quarter * 32) << 16;
+    const uint32_t o_free_c = map_rank(tc::smem_u32(&sh.o_free), 0);
+    const uint32_t p_full_c = map_rank(tc::smem_u32(&sh.p_full[0]), 0);
+    bool ok = true;
+    int g = 0;  // running tile count
+    for (int k = 0; ok && !pair_aborted(sh); ++k) {
+      const int idx = item_of(k);
+      if (idx < 0) break;
+      const PairWork w = pair_work(p, n_mp, idx);
+      const int m = (2 * w.mpair + (int)rank) * kRowsM + row;
+      const int trow = m / p.G;
+      const bool causal_row =
+          p.row_type ? (trow < p.B && p.row_type[(size_t)w.r * p.row_type_stride + trow] == 0)
+                     : p.causal != 0;
+      float m_run = -INFINITY, l_run = 0.f;
+      for (int j = 0; j < w.n_tiles; ++j) {
+        const int gg = g + j, sb = gg & 1;
+        if (!pair_warp_wait(&sh.s_full[sb], (uint32_t)(gg >> 1) & 1u, &sh.abort_flag)) {
+          ok = false;
+          break;
+        }
+        tc::fence_after_sync();
+        const uint32_t sbuf = tmem_s + lane_off + sb * 128;
+        // multiplies O by corr once the P.V of the previous tile is done
+        auto rescale = [&](float corr) -> bool {
+          if (!pair_warp_wait(&sh.pv_done[sb ^ 1], (uint32_t)((gg - 1) >> 1) & 1u, &sh.abort_flag))
+            return false;
+          tc::fence_after_sync();
+#pragma unroll 1
+          for (int c = 0; c < D; c += 16) {
+            uint32_t o[16];
+            tc::tmem_ld16(tmem_o + lane_off + c, o);
+            tc::tmem_ld_wait();
+#pragma unroll
+            for (int i = 0; i < 16; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * corr);
+            tc::tmem_st16(tmem_o + lane_off + c, o);
+          }
+          return true;
+        };
+        const int valid = tile_valid(p, w, j);
+        if (j < w.n_pref && valid == kPairKeys) {
+          ok = softmax_row<128, true>(sbuf, 128, p.scale_log2, j == 0, m_run, l_run, rescale);
+        } else if (j < w.n_pref) {
+          ok = softmax_row<128, false>(sbuf, valid, p.scale_log2, j == 0, m_run, l_run, rescale);
+        } else {
+          const int lim = causal_row ? min(valid, trow + 1) : valid;
+          ok = softmax_row<64, false>(sbuf, lim, p.scale_log2, j == 0, m_run, l_run, rescale);
+        }
+        if (!ok) break;
+        tc::tmem_st_wait();
+        tc::fence_before_sync();
+        __syncwarp();
+        if (lane == 0) arrive_at(p_full_c + sb * 8);
+      }
+      if (!ok) break;
+      g += w.n_tiles;
+      // epilogue: O / l (or the split partial) and the log-sum-exp
+      if (!pair_warp_wait(&sh.pv_done[(g - 1) & 1], (uint32_t)((g - 1) >> 1) & 1u,
+                          &sh.abort_flag)) {
+        ok = false;
+        break;
+      }
+      tc::fence_after_sync();
+      const bool write = m < M;
+      const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
+      const int gq = m % p.G;
+      const size_t orow = (((size_t)w.r * p.B + trow) * p.Hq + w.kvh * p.G + gq);
+      const size_t ws_row = ((size_t)w.item * p.n_split + w.split) * M + m;
+#pragma unroll 1
+      for (int c = 0; c < D; c += 32) {
+        uint32_t o[32];
+        tc::tmem_ld16(tmem_o + lane_off + c, *reinterpret_cast<uint32_t(*)[16]>(&o[0]));
+        tc::tmem_ld16(tmem_o + lane_off + c + 16, *reinterpret_cast<uint32_t(*)[16]>(&o[16]));
+        tc::tmem_ld_wait();
+        if (!write) continue;
+        if (!split_mode) {
+          uint4* dst = reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(p.out) + orow * D + c);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            uint32_t pk[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              __nv_bfloat162 h2 = __floats2bfloat162_rn(__uint_as_float(o[8 * i + 2 * e]) * inv,
+                                                        __uint_as_float(o[8 * i + 2 * e + 1]) * inv);
+              pk[e] = *reinterpret_cast<uint32_t*>(&h2);
+            }
+            dst[i] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+          }
+        } else {
+          float4* dst = reinterpret_cast<float4*>(p.ws_o + ws_row * D + c);
+#pragma unroll
+          for (int i = 0; i < 8; ++i)
+            dst[i] = make_float4(__uint_as_float(o[4 * i]) * inv, __uint_as_float(o[4 * i + 1]) * inv,
+                                 __uint_as_float(o[4 * i + 2]) * inv,
+                                 __uint_as_float(o[4 * i + 3]) * inv);
+        }
+      }
+      tc::fence_before_sync();
+      __syncwarp();
+      if (lane == 0) arrive_at(o_free_c);
+      if (write) {
+        const float lse = l_run > 0.f ? (m_run + __log2f(l_run)) * 0.6931471805599453f : -INFINITY;
+        if (!split_mode) {
+          if (p.lse) p.lse[orow] = lse;
+        } else {
+          p.ws_lse[ws_row] = lse;
+        }
+      }
+    }
+    // the other buffer's last P.V commit has arrived too
+    if (ok && g >= 2)
+      ok = pair_warp_wait(&sh.pv_done[g & 1], (uint32_t)((g - 2) >> 1) & 1u, &sh.abort_flag);
+    if (!ok && lane == 0) pair_abort(sh, p.dev_status);
+  }
+  __syncwarp();
+  if (pair_aborted(sh)) {  // copies and products in flight land within microseconds
+    const uint64_t t0 = tc::globaltimer_ns();
+    while (tc::globaltimer_ns() - t0 < 1000000ull) __nanosleep(1000);
+  }
+  tc::fence_before_sync();
+  __syncthreads();
+  cluster_sync();  // neither CTA goes while the other can still reach its shared memory
+  if (warp == 1) {
+    tc::fence_after_sync();
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem),
+                 "r"((uint32_t)C::kTmemCols)
+                 : "memory");
+  }
+  // a CTA that gave up wrote no partial: its row tile is never merged
+  if (split_mode && !pair_aborted(sh)) {  // shared memory is free: merge weights go there
+    const PairWork w = pair_work(p, n_mp, idx0);
+    const int mtile = 2 * w.mpair + (int)rank;
+    if (mtile < n_mt)
+      finish_split<D>(p, w.item, w.r, w.kvh, mtile, n_mt, &sh.last_split,
+                      reinterpret_cast<float*>(base));
+  }
+}
+
+// ------------------------------------------------------------------ host side
+
+namespace {
+
+template <int D>
+cudaError_t launch_pair_d(const SoftmaxParams& p, const SoftmaxPlan& plan, cudaStream_t stream) {
+  using C = PairCfg<D>;
+  PairMaps maps;
+  const uint64_t e = 2;
+  {
+    const uint64_t dims[4] = {(uint64_t)D, (uint64_t)p.Hq, (uint64_t)p.B, (uint64_t)p.R};
+    const uint64_t str[3] = {D * e, (uint64_t)p.Hq * D * e, (uint64_t)p.B * p.Hq * D * e};
+    const uint32_t box[4] = {64, (uint32_t)p.G, (uint32_t)(kRowsM / p.G), 1};
+    if (!encode_map(&maps.q, p.q, 4, dims, str, box)) return cudaErrorInvalidValue;
+  }
+  {
+    const uint64_t dims[4] = {(uint64_t)D, (uint64_t)p.Hkv, (uint64_t)p.B, (uint64_t)p.R};
+    const uint64_t str[3] = {D * e, (uint64_t)p.Hkv * D * e, (uint64_t)p.B * p.Hkv * D * e};
+    const uint32_t kbox[4] = {64, 1, 32, 1}, vbox[4] = {64, 1, 64, 1};
+    if (!encode_map(&maps.kblk, p.k_blk, 4, dims, str, kbox) ||
+        !encode_map(&maps.vblk, p.v_blk, 4, dims, str, vbox))
+      return cudaErrorInvalidValue;
+  }
+  {
+    const int npages = p.num_pages > 0 ? p.num_pages : 1;
+    const uint64_t row = D * e, head = (uint64_t)p.page_size * row;
+    const uint64_t dims[5] = {64, (uint64_t)p.page_size, (uint64_t)D / 64, (uint64_t)p.Hkv,
+                              (uint64_t)npages};
+    const uint64_t str[4] = {row, 128, head, (uint64_t)p.Hkv * head};
+    const bool whole = p.page_size >= 64;  // a 64-key half tile lies in one page
+    const uint32_t rows = whole ? 64 : (uint32_t)p.page_size;
+    const uint32_t kbox[5] = {64, rows, whole ? (uint32_t)C::kKChunks : 1u, 1, 1};
+    const uint32_t vbox[5] = {64, rows, whole ? (uint32_t)C::kVChunks : 1u, 1, 1};
+    // an empty pool is never read (every prefix is empty); point the map at the block tensor
+    const void* kp = p.num_pages > 0 ? p.k_pool : p.k_blk;
+    const void* vp = p.num_pages > 0 ? p.v_pool : p.v_blk;
+    if (!encode_map(&maps.kpool, kp, 5, dims, str, kbox) ||
+        !encode_map(&maps.vpool, vp, 5, dims, str, vbox))
+      return cudaErrorInvalidValue;
+  }
+  const int smem = C::kSmem + 1024;
+  cudaError_t err = cudaFuncSetAttribute(softmax_pair_kernel<D>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (err != cudaSuccess) return err;
+  if (plan.num_ctas <= 0) return cudaErrorInvalidValue;
+  err = launch_softmax_order(p, stream);
+  if (err != cudaSuccess) return err;
+  softmax_pair_kernel<D><<<(unsigned)plan.num_ctas, kPairThreads, smem, stream>>>(maps, p);
+  note_launches(1);
+  return cudaGetLastError();
+}
+
+}  // namespace
+
+bool softmax_pair_supported(int B, int Hq, int Hkv, int D, int page_size) {
+  return (D == 128 || D == 256) && B * (Hq / Hkv) > kRowsM &&
+         softmax_tc_supported(B, Hq, Hkv, D, page_size);
+}
+
+cudaError_t launch_softmax_pair(const SoftmaxParams& p, const SoftmaxPlan& plan,
+                                cudaStream_t stream) {
+  return p.D == 128 ? launch_pair_d<128>(p, plan, stream) : launch_pair_d<256>(p, plan, stream);
+}
+
+}  // namespace flare

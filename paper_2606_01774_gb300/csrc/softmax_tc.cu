@@ -47,6 +47,7 @@
 
 #include "common.cuh"
 #include "kernels.h"
+#include "softmax_common.cuh"
 #include "tc.cuh"
 
 namespace flare {
@@ -54,7 +55,6 @@ namespace flare {
 namespace {
 
 constexpr int kTileN = 64;     // keys per tile
-constexpr int kRowsM = 128;    // query rows per work item (TMEM lanes)
 constexpr int kSoftmaxThreads = 128;  // warps 2-5, one per TMEM lane quarter
 constexpr int kVWarp = 6;             // V producer
 constexpr int kFixWarp = 7;           // zeroes the V rows past a prefix end
@@ -173,93 +173,6 @@ __device__ __forceinline__ TcWork tc_work(const SoftmaxParams& p, int n_mt, int 
 }
 
 }  // namespace
-
-// Merge of the split partials of one row tile (rows mtile*128 ..) of one
-// (request, kv head): out = sum_s w_s o_s with w_s = exp(lse_s - lse) and
-// lse = log sum_s exp(lse_s) (the splits' partial outputs are already
-// normalised by their own row sums).  The weights go to shared memory first
-// (one thread per row); then every thread combines 8 (row, 4-column) pieces at
-// a time with all their loads in flight.  All threads of the CTA call this;
-// `wts` holds 128 * n_split floats.
-template <int D>
-__device__ void merge_splits(const SoftmaxParams& p, int item, int r, int kvh, int mtile,
-                             float* wts) {
-  const int M = p.B * p.G;
-  const int ns = p.n_split;
-  const int m0 = mtile * kRowsM;
-  const int rows = min(kRowsM, M - m0);
-  const size_t base = (size_t)item * ns * M + m0;  // row i of split s at base + s * M + i
-  for (int i = threadIdx.x; i < rows; i += blockDim.x) {
-    float mx = -INFINITY;
-    for (int s = 0; s < ns; ++s) mx = fmaxf(mx, p.ws_lse[base + (size_t)s * M + i]);
-    float den = 0.f;
-    for (int s = 0; s < ns; ++s) {
-      const float l = p.ws_lse[base + (size_t)s * M + i];
-      const float e = l == -INFINITY ? 0.f : expf(l - mx);
-      wts[i * ns + s] = e;
-      den += e;
-    }
-    const float inv = 1.f / den;
-    for (int s = 0; s < ns; ++s) wts[i * ns + s] *= inv;
-    const int m = m0 + i, t = m / p.G, g = m % p.G;
-    if (p.lse) p.lse[((size_t)r * p.B + t) * p.Hq + kvh * p.G + g] = mx + logf(den);
-  }
-  __syncthreads();
-  constexpr int kC = D / 4;  // 4-column pieces per row
-  constexpr int kBatch = 8;
-  const int n_items = rows * kC;
-  for (int i0 = threadIdx.x; i0 < n_items; i0 += kBatch * blockDim.x) {
-    float4 acc[kBatch];
-#pragma unroll
-    for (int k = 0; k < kBatch; ++k) acc[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int s = 0; s < ns; ++s) {
-      float4 o[kBatch];
-#pragma unroll
-      for (int k = 0; k < kBatch; ++k) {
-        const int it = i0 + k * blockDim.x;
-        o[k] = it < n_items ? *reinterpret_cast<const float4*>(
-                                  p.ws_o + (base + (size_t)s * M + it / kC) * D + (it % kC) * 4)
-                            : make_float4(0.f, 0.f, 0.f, 0.f);
-      }
-#pragma unroll
-      for (int k = 0; k < kBatch; ++k) {
-        const int it = i0 + k * blockDim.x;
-        const float w = it < n_items ? wts[(it / kC) * ns + s] : 0.f;
-        acc[k].x = fmaf(w, o[k].x, acc[k].x);
-        acc[k].y = fmaf(w, o[k].y, acc[k].y);
-        acc[k].z = fmaf(w, o[k].z, acc[k].z);
-        acc[k].w = fmaf(w, o[k].w, acc[k].w);
-      }
-    }
-#pragma unroll
-    for (int k = 0; k < kBatch; ++k) {
-      const int it = i0 + k * blockDim.x;
-      if (it >= n_items) continue;
-      const int m = m0 + it / kC, t = m / p.G, g = m % p.G;
-      const size_t orow = ((size_t)r * p.B + t) * p.Hq + kvh * p.G + g;
-      __nv_bfloat162 lo = __floats2bfloat162_rn(acc[k].x, acc[k].y);
-      __nv_bfloat162 hi = __floats2bfloat162_rn(acc[k].z, acc[k].w);
-      *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(p.out) + orow * D + (it % kC) * 4) =
-          make_uint2(*reinterpret_cast<uint32_t*>(&lo), *reinterpret_cast<uint32_t*>(&hi));
-    }
-  }
-}
-
-// Publishes this CTA's split partial and, if it is the last split of its row
-// tile to finish, merges them all (all threads of the CTA call this).
-template <int D>
-__device__ void finish_split(const SoftmaxParams& p, int item, int r, int kvh, int mtile,
-                             int n_mt, int* last_flag, float* wts) {
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0)
-    *last_flag = atomicAdd(&p.counters[(size_t)item * n_mt + mtile], 1) == p.n_split - 1;
-  __syncthreads();
-  if (*last_flag) {
-    __threadfence();
-    merge_splits<D>(p, item, r, kvh, mtile, wts);
-  }
-}
 
 // Validation and longest-first order of the work units u = (request r, prefix
 // split), on one CTA:
@@ -895,19 +808,30 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
   return fn;
 }
 
-bool encode4(CUtensorMap* m, const void* ptr, const uint64_t dims[4], const uint64_t strides[3],
-             const uint32_t box[4]) {
+}  // namespace
+
+bool encode_map(CUtensorMap* m, const void* ptr, int rank, const uint64_t* dims,
+                const uint64_t* strides, const uint32_t* box) {
   auto fn = encode_fn();
   if (!fn) return false;
-  cuuint64_t gd[4] = {dims[0], dims[1], dims[2], dims[3]};
-  cuuint64_t gs[3] = {strides[0], strides[1], strides[2]};
-  cuuint32_t bx[4] = {box[0], box[1], box[2], box[3]};
-  cuuint32_t es[4] = {1, 1, 1, 1};
-  return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(ptr), gd, gs, bx, es,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+  cuuint64_t gd[5], gs[4];
+  cuuint32_t bx[5], es[5];
+  for (int i = 0; i < rank; ++i) gd[i] = dims[i], bx[i] = box[i], es[i] = 1;
+  for (int i = 0; i + 1 < rank; ++i) gs[i] = strides[i];
+  return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (cuuint32_t)rank, const_cast<void*>(ptr), gd, gs,
+            bx, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) ==
          CUDA_SUCCESS;
 }
+
+cudaError_t launch_softmax_order(const SoftmaxParams& p, cudaStream_t stream) {
+  if (!p.order || !p.n_valid || !p.bad_mask) return cudaErrorInvalidValue;
+  softmax_order_kernel<<<1, kOrderThreads, 0, stream>>>(p);
+  note_launches(1);
+  return cudaGetLastError();
+}
+
+namespace {
 
 template <int D>
 cudaError_t launch_tc_d(const SoftmaxParams& p, const SoftmaxPlan& plan, cudaStream_t stream) {
@@ -918,8 +842,8 @@ cudaError_t launch_tc_d(const SoftmaxParams& p, const SoftmaxPlan& plan, cudaStr
     const uint64_t dims[4] = {(uint64_t)D, (uint64_t)p.Hkv, (uint64_t)p.B, (uint64_t)p.R};
     const uint64_t str[3] = {D * e, (uint64_t)p.Hkv * D * e, (uint64_t)p.B * p.Hkv * D * e};
     const uint32_t box[4] = {64, 1, (uint32_t)kTileN, 1};
-    if (!encode4(&maps.kblk, p.k_blk, dims, str, box) ||
-        !encode4(&maps.vblk, p.v_blk, dims, str, box))
+    if (!encode_map(&maps.kblk, p.k_blk, 4, dims, str, box) ||
+        !encode_map(&maps.vblk, p.v_blk, 4, dims, str, box))
       return cudaErrorInvalidValue;
   }
   {
@@ -932,17 +856,15 @@ cudaError_t launch_tc_d(const SoftmaxParams& p, const SoftmaxPlan& plan, cudaStr
     // an empty pool is never read (every prefix is empty); point the map at the block tensor
     const void* kp = p.num_pages > 0 ? p.k_pool : p.k_blk;
     const void* vp = p.num_pages > 0 ? p.v_pool : p.v_blk;
-    if (!encode4(&maps.kpool, kp, dims, str, box) || !encode4(&maps.vpool, vp, dims, str, box))
+    if (!encode_map(&maps.kpool, kp, 4, dims, str, box) || !encode_map(&maps.vpool, vp, 4, dims, str, box))
       return cudaErrorInvalidValue;
   }
   const int smem = C::kSmem + 1024;
   cudaError_t err = cudaFuncSetAttribute(softmax_tc_kernel<D>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (err != cudaSuccess) return err;
-  if (!p.order || !p.n_valid || !p.bad_mask || plan.num_ctas <= 0) return cudaErrorInvalidValue;
-  softmax_order_kernel<<<1, kOrderThreads, 0, stream>>>(p);
-  note_launches(1);
-  err = cudaGetLastError();
+  if (plan.num_ctas <= 0) return cudaErrorInvalidValue;
+  err = launch_softmax_order(p, stream);
   if (err != cudaSuccess) return err;
   softmax_tc_kernel<D><<<(unsigned)plan.num_ctas, kThreadsTC, smem, stream>>>(maps, p);
   note_launches(1);

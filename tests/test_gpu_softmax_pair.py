@@ -1,0 +1,65 @@
+"""GPU parity of the two-SM softmax kernel (more than 128 query rows per kv head,
+head dim 128 or 256) where its tiles can go wrong: prefixes that end on each side
+of a 16-key step, a 64-key half and a 128-key tile, odd row-tile counts, page
+sizes on each side of a half tile, split prefixes and row types."""
+import numpy as np
+import pytest
+import torch
+
+from gpu_helpers import OUT_MAX_ABS, assert_out_close, gen, oracle_softmax, run_softmax
+from paper_2606_01774_gb300 import workloads
+
+pytestmark = pytest.mark.gpu
+LARGE = workloads.WORKLOADS["serving_batch64"]  # 16 query / 2 kv heads, D = 256
+SMALL = workloads.WORKLOADS["small_model_batch256"]  # 16 / 4, D = 128
+# bf16 probabilities and outputs: each output is within a few bf16 roundings
+# (2^-9 relative) of values below 4, the bound of the other softmax tests
+LSE_ABS = 2e-3
+
+# (base, requests, block, prefix lengths, page size): the lengths are given to the
+# requests in turn
+EDGES = [0, 1, 15, 16, 17, 48, 63, 64, 65, 79, 80, 113, 127, 128, 129, 144, 191, 193, 256, 300]
+CASES = {
+    "d256_edges": (LARGE, len(EDGES), 32, EDGES, 64),
+    "d256_edges_page16": (LARGE, len(EDGES), 17, EDGES, 16),
+    "d256_edges_page128": (LARGE, len(EDGES), 33, EDGES, 128),
+    "d256_three_row_tiles": (LARGE, 90, 48, [1, 200, 127, 64, 255], 32),
+    "d128_edges": (SMALL, len(EDGES), 64, EDGES, 64),
+    "d128_edges_page16": (SMALL, 2 * len(EDGES), 40, EDGES, 16),
+    "d256_split": (LARGE, 1, 64, [4097], 64),
+    "d256_split_ragged": (LARGE, 3, 32, [5000, 1100, 2303], 16),
+    "d128_split": (SMALL, 1, 48, [2500], 128),
+}
+
+
+def _workload(base, requests, block, lens, page):
+    spec = base.replace(num_requests=requests, block_len=block, page_size=page,
+                        prefix_lo=max(lens), prefix_hi=max(lens), seed=91)
+    w = gen(spec)
+    P = torch.tensor([lens[r % len(lens)] for r in range(requests)], dtype=torch.int32)
+    w.prefix_len = P.cuda()
+    # rows of the last page past each prefix end, and every page past it, hold NaN
+    for r, n in enumerate(P.tolist()):
+        for i in range(w.page_table.shape[1]):
+            page_id = int(w.page_table[r, i])
+            lo = min(max(n - i * page, 0), page)
+            if page_id >= 0 and lo < page:
+                w.k_pool[page_id, :, lo:] = float("nan")
+                w.v_pool[page_id, :, lo:] = float("nan")
+    return w
+
+
+@pytest.mark.parametrize("mode", [0, 1, 3])
+@pytest.mark.parametrize("name", list(CASES))
+def test_pair_matches_oracle(name, mode):
+    w = _workload(*CASES[name])
+    spec = w.spec
+    rows = None
+    if mode == 3:
+        held = torch.arange(spec.num_requests) % spec.block_len
+        rows = (torch.arange(spec.block_len)[None] > held[:, None]).to(torch.uint8).cuda()
+    out, lse = run_softmax(w, 0, mode, row_type=rows)
+    ref, ref_lse = oracle_softmax(w, 0, mode=mode, row_type=rows)
+    err, _ = assert_out_close(out, ref, "bf16", name)
+    assert err <= OUT_MAX_ABS
+    assert np.abs(lse.double().cpu().numpy() - ref_lse).max() < LSE_ABS
