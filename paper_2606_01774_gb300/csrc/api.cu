@@ -94,6 +94,24 @@ namespace flare {
 static std::atomic<uint64_t> g_launches{0};
 void note_launches(int n) { g_launches.fetch_add((uint64_t)n, std::memory_order_relaxed); }
 
+// Prefix splits of a tensor-core call with `items` (request, kv head, row tile
+// group) items on `workers` CTAs or pairs, for prefixes of up to `tiles` tiles.
+// Half the workers or fewer have an item: one wave, as many splits as there
+// are workers, of at least `few` tiles each (256 keys; one request of 4096 tokens
+// takes 16 splits where it took 4 of 1024 keys, merged by one CTA per row tile:
+// the step around it 66.5 -> 46.6 us).  More items than that, but fewer than
+// workers: about two splits per worker, of at least `many` tiles (1024 keys), so
+// that a partial second wave is short.  Otherwise none.
+static int tc_splits(long items, long workers, long tiles, long few, long many) {
+  if (items <= 0 || items >= workers || tiles <= 0) return 1;
+  const bool one_wave = 2 * items <= workers;
+  long ns = one_wave ? workers / items : (2 * workers + items - 1) / items;
+  const long cap = tiles / (one_wave ? few : many);
+  if (ns > cap) ns = cap;
+  if (ns > 64) ns = 64;  // the merge holds two weights per lane
+  return ns > 1 ? (int)ns : 1;
+}
+
 SoftmaxPlan plan_softmax(int R, int B, int Hq, int Hkv, int D, int page_size, int max_pages,
                          bool bf16, int num_sms) {
   SoftmaxPlan pl;
@@ -108,35 +126,14 @@ SoftmaxPlan plan_softmax(int R, int B, int Hq, int Hkv, int D, int page_size, in
     // 0.128 (64 requests, B = 32, G = 8).  Splits as below, over 128-key tiles.
     pl.kernel = 2;
     pl.rows_per_cta = 128;
-    const long items = (long)R * Hkv * ((M + 255) / 256), pairs = num_sms / 2;
-    const long tiles = (prefix_max + 127) / 128;
-    long ns = 1;
-    if (items > 0 && items < pairs) ns = (2L * pairs + items - 1) / items;
-    const long cap = tiles / 8 > 1 ? tiles / 8 : 1;
-    if (ns > cap) ns = cap;
-    if (ns > 64) ns = 64;  // the merge keeps 128 x n_split weights in shared memory
-    const long tps = ns > 0 ? (tiles + ns - 1) / ns : 1;
-    pl.split_len = (int)((tps > 0 ? tps : 1) * 128);
-    pl.n_split = tiles > 0 ? (int)((tiles + tps - 1) / tps) : 1;
-    if (pl.n_split < 1) pl.n_split = 1;
+    pl.n_split = tc_splits((long)R * Hkv * ((M + 255) / 256), num_sms / 2, (prefix_max + 127) / 128,
+                           2, 8);
   } else if (bf16 && softmax_tc_supported(B, Hq, Hkv, D, page_size)) {
-    // tensor-core kernel: 128 query rows per CTA, one CTA per SM, work units
-    // started longest first.  Split the prefix only when the batch has fewer
-    // work items than SMs (then aim at two CTAs per SM), and keep at least 16
-    // tiles (1024 keys) per split so partials stay small.
+    // tensor-core kernel: 128 query rows per CTA, one CTA per SM
     pl.kernel = 1;
     pl.rows_per_cta = 128;
-    const long items = (long)R * Hkv * ((M + 127) / 128);
-    const long tiles = (prefix_max + 63) / 64;
-    long ns = 1;
-    if (items > 0 && items < num_sms) ns = (2L * num_sms + items - 1) / items;
-    const long cap = tiles / 16 > 1 ? tiles / 16 : 1;
-    if (ns > cap) ns = cap;
-    if (ns > 64) ns = 64;  // the merge keeps 128 x n_split weights in shared memory
-    const long tps = ns > 0 ? (tiles + ns - 1) / ns : 1;
-    pl.split_len = (int)((tps > 0 ? tps : 1) * 64);
-    pl.n_split = tiles > 0 ? (int)((tiles + tps - 1) / tps) : 1;
-    if (pl.n_split < 1) pl.n_split = 1;
+    pl.n_split = tc_splits((long)R * Hkv * ((M + 127) / 128), num_sms, (prefix_max + 63) / 64, 4,
+                           16);
   } else {
     pl.kernel = 0;
     pl.rows_per_cta = 16;
@@ -158,23 +155,19 @@ SoftmaxPlan plan_softmax(int R, int B, int Hq, int Hkv, int D, int page_size, in
     pl.ws_o_bytes = (rows * D * sizeof(float) + 255) / 256 * 256;
     pl.ws_lse_bytes = (rows * sizeof(float) + 255) / 256 * 256;
   }
-  // tensor-core kernels: the work units in longest-first order, and per row
-  // tile a count of finished splits (the last one merges the partials)
+  // tensor-core kernels: the requests longest first, unless the attention
+  // kernel orders them itself
   if (pl.kernel != 0) {
-    // order [R*n_split], n_valid [1], bad-request mask [ceil(R/32)]
-    pl.ws_order_bytes =
-        (((size_t)R * pl.n_split + 1 + (size_t)(R + 31) / 32) * sizeof(int32_t) + 255) / 256 * 256;
+    if (pl.n_split == 1 && R > kOrderOnChip)  // order [R], n_valid [1]
+      pl.ws_order_bytes = (((size_t)R + 1) * sizeof(int32_t) + 255) / 256 * 256;
     // one CTA (or pair) per work item when the prefix is split, else one per SM
     // (at most one per work item) walking the items
     const long group = pl.kernel == 2 ? 2 : 1;
     const long n_items = (M + 128 * group - 1) / (128 * group) * Hkv * R * pl.n_split;
     const long groups = num_sms / group;
     pl.num_ctas = (int)(group * (pl.n_split > 1 || n_items < groups ? n_items : groups));
-    if (pl.n_split > 1)
-      pl.ws_count_bytes =
-          ((size_t)R * Hkv * ((M + 127) / 128) * sizeof(int32_t) + 255) / 256 * 256;
   }
-  pl.workspace_bytes = pl.ws_o_bytes + pl.ws_lse_bytes + pl.ws_order_bytes + pl.ws_count_bytes;
+  pl.workspace_bytes = pl.ws_o_bytes + pl.ws_lse_bytes + pl.ws_order_bytes;
   return pl;
 }
 
@@ -507,12 +500,8 @@ flare_status flare_block_softmax_attn(const flare_softmax_desc* d, const void* q
     }
     if (plan.ws_order_bytes) {
       p.order = reinterpret_cast<int32_t*>(ws + plan.ws_o_bytes + plan.ws_lse_bytes);
-      p.n_valid = p.order + (size_t)p.R * plan.n_split;
-      p.bad_mask = reinterpret_cast<uint32_t*>(p.n_valid + 1);
+      p.n_valid = p.order + p.R;
     }
-    if (plan.ws_count_bytes)
-      p.counters = reinterpret_cast<int32_t*>(ws + plan.ws_o_bytes + plan.ws_lse_bytes +
-                                              plan.ws_order_bytes);
   }
   p.dev_status = dev_status;
   const cudaError_t e = launch_softmax(p, plan, d->act_dtype == FLARE_DT_BF16,

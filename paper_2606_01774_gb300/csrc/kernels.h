@@ -50,13 +50,14 @@ struct SoftmaxParams {
   float* lse;                 // [R,B,Hq] or nullptr
   float* ws_o;                // split partial outputs [R*Hkv][n_split][B*G][D]
   float* ws_lse;              // split partial lse     [R*Hkv][n_split][B*G]
-  int n_split, split_len;
-  int32_t* order;             // [R*n_split] valid work units (r, split), longest first
-  int32_t* n_valid;           // number of valid work units in `order`
-  uint32_t* bad_mask;         // [ceil(R/32)] requests with a bad prefix length or page id
-  int32_t* counters;          // [R*Hkv*ceil(B*G/128)] finished splits per row tile (n_split > 1)
+  int n_split, split_len;     // split_len: CUDA-core kernel only
+  int32_t* order;             // [R] valid requests, longest first (R > kOrderOnChip), else nullptr
+  int32_t* n_valid;           // their number
   int32_t* dev_status;
 };
+
+// Batches up to this size are ordered by the attention kernel itself.
+constexpr int kOrderOnChip = 512;
 
 // Work decomposition of the softmax call; identical for the workspace query
 // and the launch.
@@ -66,7 +67,7 @@ struct SoftmaxPlan {
   int n_split;
   int split_len;
   int num_ctas;  // tensor-core kernels: CTAs launched
-  size_t ws_o_bytes, ws_lse_bytes, ws_order_bytes, ws_count_bytes;
+  size_t ws_o_bytes, ws_lse_bytes, ws_order_bytes;
   size_t workspace_bytes;
 };
 

@@ -1,5 +1,5 @@
-// Shared by the tensor-core softmax kernels: tensor maps, the pre-pass and the
-// merge of split prefixes.
+// Shared by the tensor-core softmax kernels: tensor maps, the order of the work
+// units, the page check and the combination of split prefixes.
 #pragma once
 
 #include <cuda.h>
@@ -14,94 +14,86 @@ constexpr int kRowsM = 128;  // query rows per row tile (tensor-memory lanes)
 // bf16 tensor map of `rank` dimensions with the 128-byte swizzle.
 bool encode_map(CUtensorMap* m, const void* ptr, int rank, const uint64_t* dims,
                 const uint64_t* strides, const uint32_t* box);
-// Validates the requests and orders the work units (one CTA).
+// Orders the requests of a batch too large for order_on_chip (one CTA).
 cudaError_t launch_softmax_order(const SoftmaxParams& p, cudaStream_t stream);
+// Combines the split partials in the workspace into the outputs.
+cudaError_t launch_softmax_merge(const SoftmaxParams& p, cudaStream_t stream);
 
-// Merge of the split partials of one row tile (rows mtile*128 ..) of one
-// (request, kv head): out = sum_s w_s o_s with w_s = exp(lse_s - lse) and
-// lse = log sum_s exp(lse_s) (the splits' partial outputs are already
-// normalised by their own row sums).  The weights go to shared memory first
-// (one thread per row); then every thread combines 8 (row, 4-column) pieces at
-// a time with all their loads in flight.  All threads of the CTA call this;
-// `wts` holds 128 * n_split floats.
-template <int D>
-__device__ void merge_splits(const SoftmaxParams& p, int item, int r, int kvh, int mtile,
-                             float* wts) {
-  const int M = p.B * p.G;
-  const int ns = p.n_split;
-  const int m0 = mtile * kRowsM;
-  const int rows = min(kRowsM, M - m0);
-  const size_t base = (size_t)item * ns * M + m0;  // row i of split s at base + s * M + i
-  for (int i = threadIdx.x; i < rows; i += blockDim.x) {
-    float mx = -INFINITY;
-    for (int s = 0; s < ns; ++s) mx = fmaxf(mx, p.ws_lse[base + (size_t)s * M + i]);
-    float den = 0.f;
-    for (int s = 0; s < ns; ++s) {
-      const float l = p.ws_lse[base + (size_t)s * M + i];
-      const float e = l == -INFINITY ? 0.f : expf(l - mx);
-      wts[i * ns + s] = e;
-      den += e;
-    }
-    const float inv = 1.f / den;
-    for (int s = 0; s < ns; ++s) wts[i * ns + s] *= inv;
-    const int m = m0 + i, t = m / p.G, g = m % p.G;
-    if (p.lse) p.lse[((size_t)r * p.B + t) * p.Hq + kvh * p.G + g] = mx + logf(den);
-  }
-  __syncthreads();
-  constexpr int kC = D / 4;  // 4-column pieces per row
-  constexpr int kBatch = 8;
-  const int n_items = rows * kC;
-  for (int i0 = threadIdx.x; i0 < n_items; i0 += kBatch * blockDim.x) {
-    float4 acc[kBatch];
-#pragma unroll
-    for (int k = 0; k < kBatch; ++k) acc[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int s = 0; s < ns; ++s) {
-      float4 o[kBatch];
-#pragma unroll
-      for (int k = 0; k < kBatch; ++k) {
-        const int it = i0 + k * blockDim.x;
-        o[k] = it < n_items ? *reinterpret_cast<const float4*>(
-                                  p.ws_o + (base + (size_t)s * M + it / kC) * D + (it % kC) * 4)
-                            : make_float4(0.f, 0.f, 0.f, 0.f);
-      }
-#pragma unroll
-      for (int k = 0; k < kBatch; ++k) {
-        const int it = i0 + k * blockDim.x;
-        const float w = it < n_items ? wts[(it / kC) * ns + s] : 0.f;
-        acc[k].x = fmaf(w, o[k].x, acc[k].x);
-        acc[k].y = fmaf(w, o[k].y, acc[k].y);
-        acc[k].z = fmaf(w, o[k].z, acc[k].z);
-        acc[k].w = fmaf(w, o[k].w, acc[k].w);
-      }
-    }
-#pragma unroll
-    for (int k = 0; k < kBatch; ++k) {
-      const int it = i0 + k * blockDim.x;
-      if (it >= n_items) continue;
-      const int m = m0 + it / kC, t = m / p.G, g = m % p.G;
-      const size_t orow = ((size_t)r * p.B + t) * p.Hq + kvh * p.G + g;
-      __nv_bfloat162 lo = __floats2bfloat162_rn(acc[k].x, acc[k].y);
-      __nv_bfloat162 hi = __floats2bfloat162_rn(acc[k].z, acc[k].w);
-      *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(p.out) + orow * D + (it % kC) * 4) =
-          make_uint2(*reinterpret_cast<uint32_t*>(&lo), *reinterpret_cast<uint32_t*>(&hi));
-    }
-  }
+__device__ __forceinline__ bool prefix_ok(const SoftmaxParams& p, int P) {
+  return P >= 0 && P <= (long long)p.max_pages * p.page_size;
 }
 
-// Publishes this CTA's split partial and, if it is the last split of its row
-// tile to finish, merges them all (all threads of the CTA call this).
-template <int D>
-__device__ void finish_split(const SoftmaxParams& p, int item, int r, int kvh, int mtile,
-                             int n_mt, int* last_flag, float* wts) {
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0)
-    *last_flag = atomicAdd(&p.counters[(size_t)item * n_mt + mtile], 1) == p.n_split - 1;
-  __syncthreads();
-  if (*last_flag) {
-    __threadfence();
-    merge_splits<D>(p, item, r, kvh, mtile, wts);
+// Keys of one prefix split of a request with P prefix tokens: an equal share of
+// its own prefix, in whole tiles of `tile` keys.
+__device__ __forceinline__ int split_keys(const SoftmaxParams& p, int P, int tile) {
+  return ((P + p.n_split - 1) / p.n_split + tile - 1) / tile * tile;
+}
+
+// Longest-first order of the requests, computed by every CTA for itself from the
+// R <= kOrderOnChip prefix lengths: rank = number of requests with more tiles (or as many
+// and a lower index).  Requests with a bad prefix length are left out (and
+// flagged by CTA 0).  Returns the number of valid requests.  `keys` holds
+// kOrderOnChip ints, 16-byte aligned; all threads of the CTA call this (it ends with a
+// __syncthreads).
+//
+// A pre-pass kernel on one CTA did this and the page check before: 8 us of a
+// 128 us call (64 requests; now 118 us), 17 us for 128 requests of up to 256
+// pages.  Above kOrderOnChip the comparisons, which grow with R^2, would take
+// longer than the pre-pass, which then still serves.
+__device__ __forceinline__ int order_on_chip(const SoftmaxParams& p, int tile, int* keys,
+                                             uint16_t* order) {
+  int n_bad = 0;
+  const int R4 = (p.R + 3) & ~3;
+  for (int r = threadIdx.x; r < R4; r += blockDim.x) {
+    int key = -1;
+    if (r < p.R) {
+      const int P = p.prefix_len[r];
+      if (prefix_ok(p, P)) {
+        key = (((P + tile - 1) / tile) << 9) | (kOrderOnChip - 1 - r);
+      } else {
+        ++n_bad;
+        if (blockIdx.x == 0) flag(p.dev_status, FLARE_DEV_BAD_PREFIX_LEN);
+      }
+    }
+    keys[r] = key;
   }
+  int bad = 0;
+  if (__syncthreads_or(n_bad))  // rare: count them
+    for (int r = 0; r < p.R; ++r) bad += keys[r] < 0;
+  for (int r = threadIdx.x; r < p.R; r += blockDim.x) {
+    const int key = keys[r];
+    int rank = 0;
+    for (int i = 0; i < R4; i += 4) {
+      const int4 k = *reinterpret_cast<const int4*>(keys + i);
+      rank += (k.x > key) + (k.y > key) + (k.z > key) + (k.w > key);
+    }
+    if (key >= 0) order[rank] = (uint16_t)r;
+  }
+  __syncthreads();
+  return p.R - bad;
+}
+
+// The check of a request's page ids against [0, num_pages), by each softmax warp
+// for the items it works on.  The first 32 ids are loaded when the item starts
+// and looked at when it ends; further ones (rest) while the second S product
+// runs, so the loads' latency stays off the items' chain.
+__device__ __forceinline__ int first_page(const SoftmaxParams& p, int r, int P) {
+  const int i = threadIdx.x & 31;
+  return i * p.page_size < P ? p.page_table[(size_t)r * p.max_pages + i] : -1;
+}
+__device__ __forceinline__ bool rest_bad(const SoftmaxParams& p, int r, int P) {
+  const int n = (P + p.page_size - 1) / p.page_size;
+  const int32_t* table = p.page_table + (size_t)r * p.max_pages;
+  bool bad = false;
+#pragma unroll 4
+  for (int i = 32 + (threadIdx.x & 31); i < n; i += 32)
+    bad |= (unsigned)table[i] >= (unsigned)p.num_pages;
+  return bad;
+}
+// called by a converged warp
+__device__ __forceinline__ bool bad_pages(const SoftmaxParams& p, int first, int P, bool rest) {
+  const bool used = (threadIdx.x & 31) * p.page_size < P;
+  return __any_sync(0xffffffffu, rest || (used && (unsigned)first >= (unsigned)p.num_pages));
 }
 
 }  // namespace flare

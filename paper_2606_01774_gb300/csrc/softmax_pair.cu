@@ -93,7 +93,7 @@ struct PairShared {
   uint64_t o_free;       // leader: O read out by both CTAs (8 warps)
   uint32_t tmem_base;
   int abort_flag;
-  int last_split;
+  uint16_t order[kOrderOnChip];  // unsplit: the requests, longest first
 };
 
 // ------------------------------------------------------------------ cluster PTX
@@ -212,19 +212,29 @@ struct PairWork {
   bool block;                   // the last tile holds the block's own keys
 };
 
-// Item `idx`: (row-tile pair, kv head) fastest, then the valid work units
-// (request, prefix split) in longest-first order.
-__device__ __forceinline__ PairWork pair_work(const SoftmaxParams& p, int n_mp, int idx) {
+// Item `idx`: (row-tile pair, kv head) fastest, then the prefix splits of each
+// request (split) or the valid requests longest first (unsplit).
+__device__ __forceinline__ PairWork pair_work(const SoftmaxParams& p, const uint16_t* order,
+                                              int n_mp, int idx) {
   PairWork w;
   w.mpair = idx % n_mp;
   w.kvh = (idx / n_mp) % p.Hkv;
-  const int unit = p.order[idx / (n_mp * p.Hkv)];
-  w.r = unit / p.n_split;
-  w.split = unit % p.n_split;
+  const int unit = idx / (n_mp * p.Hkv);
+  if (p.n_split > 1) {
+    w.r = unit / p.n_split;
+    w.split = unit % p.n_split;
+    w.P = p.prefix_len[w.r];
+    const int len = split_keys(p, w.P, kPairKeys);
+    w.tok_lo = min(w.P, w.split * len);
+    w.tok_hi = min(w.P, w.tok_lo + len);
+  } else {
+    w.r = p.order ? p.order[unit] : order[unit];
+    w.split = 0;
+    w.P = p.prefix_len[w.r];
+    w.tok_lo = 0;
+    w.tok_hi = w.P;
+  }
   w.item = w.r * p.Hkv + w.kvh;
-  w.P = p.prefix_len[w.r];
-  w.tok_lo = min(w.P, w.split * p.split_len);
-  w.tok_hi = min(w.P, w.tok_lo + p.split_len);
   w.n_pref = (w.tok_hi - w.tok_lo + kPairKeys - 1) / kPairKeys;
   w.block = w.split == p.n_split - 1;
   w.n_tiles = w.n_pref + (w.block ? 1 : 0);
@@ -316,10 +326,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
   const int M = p.B * p.G;
   const int n_mt = (M + kRowsM - 1) / kRowsM;
   const int n_mp = (n_mt + 1) / 2;
-  const int n_items = n_mp * p.Hkv * *p.n_valid;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t rank = cluster_rank();
   const bool split_mode = p.n_split > 1;
+  const int units = split_mode ? p.R * p.n_split
+                    : p.order  ? *p.n_valid
+                               : order_on_chip(p, kPairKeys, reinterpret_cast<int*>(base), sh.order);
+  const int n_items = n_mp * p.Hkv * units;
   const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
   // k-th work item of this pair, or -1 (the same answer in both CTAs)
   auto item_of = [&](int k) -> int {
@@ -330,24 +343,24 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
   const int idx0 = item_of(0);
   if (idx0 < 0) return;
   if (split_mode) {
-    const PairWork w = pair_work(p, n_mp, idx0);
+    const PairWork w = pair_work(p, sh.order, n_mp, idx0);
+    if (!prefix_ok(p, w.P)) {
+      if (tid == 0) flag(p.dev_status, FLARE_DEV_BAD_PREFIX_LEN);
+      return;
+    }
     if (w.n_tiles == 0) {  // empty split: mark its partial as empty for the merge
       const int mtile = 2 * w.mpair + (int)rank;
-      if (mtile >= n_mt) return;
       const size_t ws_row0 = ((size_t)w.item * p.n_split + w.split) * M;
       for (int i = tid; i < kRowsM; i += blockDim.x) {
         const int m = mtile * kRowsM + i;
         if (m < M) p.ws_lse[ws_row0 + m] = -INFINITY;
       }
-      finish_split<D>(p, w.item, w.r, w.kvh, mtile, n_mt, &sh.last_split,
-                      reinterpret_cast<float*>(base));
       return;
     }
   }
 
   if (tid == 0) {
     sh.abort_flag = 0;
-    sh.last_split = 0;
     for (int s = 0; s < C::kSlots; ++s) {
       tc::mbar_init(&sh.full[s], 2);
       tc::mbar_init(&sh.empty[s], 1);
@@ -371,6 +384,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
   }
+  tc::fence_async_smem();  // the order's keys lay in Q's shared memory
   tc::fence_before_sync();
   __syncthreads();
   cluster_sync();  // both CTAs' barriers initialised before any arrival from the peer
@@ -408,7 +422,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
     for (int k = 0; ok && !pair_aborted(sh); ++k) {
       const int idx = item_of(k);
       if (idx < 0) break;
-      const PairWork w = pair_work(p, n_mp, idx);
+      const PairWork w = pair_work(p, sh.order, n_mp, idx);
       // page ids of the window [pbase, pbase + 64): two per lane, in cur and nxt
       const int n_pages = (w.tok_hi + p.page_size - 1) >> pshift;
       const int32_t* table = p.page_table + (size_t)w.r * p.max_pages;
@@ -424,7 +438,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
           const int o = (t >> pshift) - pbase;
           const int pa = __shfl_sync(0xffffffffu, cur, o & 31);
           const int pb = __shfl_sync(0xffffffffu, nxt, o & 31);
-          const int page = o < 32 ? pa : pb;
+          const int id = o < 32 ? pa : pb;
+          const int page = id < p.num_pages ? id : -1;  // out of range reads as zero
           if (elect_one()) {
             const int row = t & (p.page_size - 1);
             if (bshift == 6) {
@@ -529,7 +544,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
       for (int k = 0; ok && !pair_aborted(sh); ++k) {
         const int idx = item_of(k);
         if (idx < 0) break;
-        const PairWork w = pair_work(p, n_mp, idx);
+        const PairWork w = pair_work(p, sh.order, n_mp, idx);
         if (!pair_warp_wait(&sh.q_full, (uint32_t)k & 1u, &sh.abort_flag)) {
           ok = false;
           break;
@@ -614,7 +629,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
       }
       const int idx = item_of(k);
       if (idx < 0) break;
-      const PairWork w = pair_work(p, n_mp, idx);
+      const PairWork w = pair_work(p, sh.order, n_mp, idx);
       if (lane == 0) {
         expect_at(q_full_c, C::kQBytes);
         // rows past the block (t >= B) read as zero
@@ -659,13 +674,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
     for (int k = 0; ok && !pair_aborted(sh); ++k) {
       const int idx = item_of(k);
       if (idx < 0) break;
-      const PairWork w = pair_work(p, n_mp, idx);
+      const PairWork w = pair_work(p, sh.order, n_mp, idx);
       const int m = (2 * w.mpair + (int)rank) * kRowsM + row;
       const int trow = m / p.G;
       const bool causal_row =
           p.row_type ? (trow < p.B && p.row_type[(size_t)w.r * p.row_type_stride + trow] == 0)
                      : p.causal != 0;
       float m_run = -INFINITY, l_run = 0.f;
+      const int page0 = first_page(p, w.r, w.P);
+      bool rest = false;
       for (int j = 0; j < w.n_tiles; ++j) {
         const int gg = g + j, sb = gg & 1;
         if (!pair_warp_wait(&sh.s_full[sb], (uint32_t)(gg >> 1) & 1u, &sh.abort_flag)) {
@@ -704,8 +721,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
         tc::fence_before_sync();
         __syncwarp();
         if (lane == 0) arrive_at(p_full_c + sb * 8);
+        if (j == 0) rest = rest_bad(p, w.r, w.P);
       }
       if (!ok) break;
+      // every item of a request looks at all its pages
+      const bool bad = bad_pages(p, page0, w.P, rest);
+      if (bad && lane == 0) flag(p.dev_status, FLARE_DEV_BAD_PAGE);
       g += w.n_tiles;
       // epilogue: O / l (or the split partial) and the log-sum-exp
       if (!pair_warp_wait(&sh.pv_done[(g - 1) & 1], (uint32_t)((g - 1) >> 1) & 1u,
@@ -714,7 +735,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
         break;
       }
       tc::fence_after_sync();
-      const bool write = m < M;
+      const bool write = m < M && !bad;
       const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
       const int gq = m % p.G;
       const size_t orow = (((size_t)w.r * p.B + trow) * p.Hq + w.kvh * p.G + gq);
@@ -779,14 +800,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
                  "r"((uint32_t)C::kTmemCols)
                  : "memory");
   }
-  // a CTA that gave up wrote no partial: its row tile is never merged
-  if (split_mode && !pair_aborted(sh)) {  // shared memory is free: merge weights go there
-    const PairWork w = pair_work(p, n_mp, idx0);
-    const int mtile = 2 * w.mpair + (int)rank;
-    if (mtile < n_mt)
-      finish_split<D>(p, w.item, w.r, w.kvh, mtile, n_mt, &sh.last_split,
-                      reinterpret_cast<float*>(base));
-  }
 }
 
 // ------------------------------------------------------------------ host side
@@ -834,11 +847,12 @@ cudaError_t launch_pair_d(const SoftmaxParams& p, const SoftmaxPlan& plan, cudaS
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (err != cudaSuccess) return err;
   if (plan.num_ctas <= 0) return cudaErrorInvalidValue;
-  err = launch_softmax_order(p, stream);
+  if (p.order) err = launch_softmax_order(p, stream);
   if (err != cudaSuccess) return err;
   softmax_pair_kernel<D><<<(unsigned)plan.num_ctas, kPairThreads, smem, stream>>>(maps, p);
   note_launches(1);
-  return cudaGetLastError();
+  err = cudaGetLastError();
+  return err == cudaSuccess && p.n_split > 1 ? launch_softmax_merge(p, stream) : err;
 }
 
 }  // namespace

@@ -11,12 +11,13 @@
 // every prefix token; the mask only touches the ragged prefix end and the
 // block tile (bidirectional, or token-causal for the state-update pass).
 //
-// A one-CTA pre-pass validates every request (prefix length, page ids), drops
-// bad ones from the work list and orders the work units longest first.  When
-// prefixes are not split, one CTA per SM walks its share of the items (snake
-// order over the CTAs), so setup happens once per CTA and the next item's
-// loads and S products overlap the current item's epilogue; when they are,
-// one CTA runs each item and the last split of a row tile merges the partials.
+// Requests with a bad prefix length are left out; bad page ids read as zero keys
+// and keep the request's outputs from being written.  When prefixes are not
+// split, the requests are taken longest first and one CTA per SM walks its share
+// of the items (snake order over the CTAs), so setup happens once per CTA and
+// the next item's loads and S products overlap the current item's epilogue;
+// when they are, one CTA runs each item and a second kernel combines the
+// partials.
 //
 // Tensor memory holds Q (bf16 pairs, loaded per item), the O accumulator and the
 // S buffers (three for D <= 128, two for D = 256); each S buffer is
@@ -93,8 +94,8 @@ struct TcShared {
   uint64_t v_fix[8];  // per V slot: a partial prefix tile's V rows past the prefix end are zeroed
   uint32_t tmem_base;
   int abort_flag;
-  int last_split;     // this CTA merges the split partials of its row tile
   int v_issued;       // V tiles whose loads the V producer has issued (running count)
+  uint16_t order[kOrderOnChip];  // unsplit: the requests, longest first
 };
 
 // All lanes of the warp wait; the outcome is made warp-uniform so that the
@@ -149,21 +150,31 @@ struct TcWork {
   int j0, n_pref_here, n_tiles, j_part;
 };
 
-// Work item `idx` of the flat list: (row tile, kv head) fastest, then the
-// valid work units (request, prefix split) in longest-first order.
-__device__ __forceinline__ TcWork tc_work(const SoftmaxParams& p, int n_mt, int idx) {
+// Work item `idx` of the flat list: (row tile, kv head) fastest, then the prefix
+// splits of each request (split) or the valid requests longest first (unsplit).
+__device__ __forceinline__ TcWork tc_work(const SoftmaxParams& p, const uint16_t* order, int n_mt,
+                                          int idx) {
   TcWork w;
   w.mtile = idx % n_mt;
   w.kvh = (idx / n_mt) % p.Hkv;
-  const int unit = p.order[idx / (n_mt * p.Hkv)];
-  w.r = unit / p.n_split;
-  w.split = unit % p.n_split;
+  const int unit = idx / (n_mt * p.Hkv);
+  if (p.n_split > 1) {
+    w.r = unit / p.n_split;
+    w.split = unit % p.n_split;
+  } else {
+    w.r = p.order ? p.order[unit] : order[unit];
+    w.split = 0;
+  }
   w.item = w.r * p.Hkv + w.kvh;
   w.P = p.prefix_len[w.r];
   const int n_pref = (w.P + kTileN - 1) / kTileN;
-  const int tps = p.split_len / kTileN;
-  w.j0 = w.split * tps;
-  const int j1 = min(n_pref, w.j0 + tps);
+  w.j0 = 0;
+  int j1 = n_pref;
+  if (p.n_split > 1) {
+    const int tps = split_keys(p, w.P, kTileN) / kTileN;
+    w.j0 = w.split * tps;
+    j1 = min(n_pref, w.j0 + tps);
+  }
   w.n_pref_here = max(0, j1 - w.j0);
   w.n_tiles = w.n_pref_here + (w.split == p.n_split - 1 ? 1 : 0);
   // the last prefix tile when the prefix ends inside it (its V rows past the
@@ -174,16 +185,11 @@ __device__ __forceinline__ TcWork tc_work(const SoftmaxParams& p, int n_mt, int 
 
 }  // namespace
 
-// Validation and longest-first order of the work units u = (request r, prefix
-// split), on one CTA:
-//  - a request whose prefix length is out of range or whose prefix uses a page
-//    id outside [0, num_pages) is flagged in the status word and left out of
-//    the order (its outputs stay untouched);
-//  - the other units are counting-sorted by their tile count (keys capped at
-//    4095 tiles), longest first; *n_valid receives their number.
-// Units with equal counts come in any order; each unit writes its own
-// outputs, so the results do not depend on it.  Also zeroes the split-merge
-// counters.
+// Longest-first order of the requests of a large batch, on one CTA: those whose
+// prefix length is in range are counting-sorted by their tile count (keys
+// capped at 4095 tiles); *n_valid receives their number.  A bad prefix length is
+// flagged in the status word.  Requests with equal counts come in any order;
+// each writes its own outputs, so the results do not depend on it.
 constexpr int kOrderThreads = 1024;
 constexpr int kOrderKeys = 4 * kOrderThreads;
 
@@ -191,74 +197,25 @@ __global__ void __launch_bounds__(kOrderThreads) softmax_order_kernel(SoftmaxPar
   __shared__ int start[kOrderKeys];
   __shared__ int wsum[kOrderThreads / 32];
   __shared__ int n_valid;
-  const int U = p.R * p.n_split;
-  const int tps = p.split_len / kTileN;
   const int t = threadIdx.x;
-  const int nw = (p.R + 31) / 32;
-  const long long prefix_cap = (long long)p.max_pages * p.page_size;
   for (int i = t; i < kOrderKeys; i += kOrderThreads) start[i] = 0;
-  for (int i = t; i < nw; i += kOrderThreads) p.bad_mask[i] = 0u;
-  if (p.counters) {
-    const int n_cnt = p.R * p.Hkv * ((p.B * p.G + kRowsM - 1) / kRowsM);
-    for (int i = t; i < n_cnt; i += kOrderThreads) p.counters[i] = 0;
-  }
   if (t == 0) n_valid = 0;
   __syncthreads();
-  for (int r = t; r < p.R; r += kOrderThreads) {
+  auto key_of = [&](int r) -> int {
     const int P = p.prefix_len[r];
-    if (P < 0 || P > prefix_cap) {
-      atomicOr(&p.bad_mask[r >> 5], 1u << (r & 31));
-      flag(p.dev_status, FLARE_DEV_BAD_PREFIX_LEN);
-    }
-  }
-  // page ids in use: eight table entries per thread in flight at a time
-  const long long n_entries = (long long)p.R * p.max_pages;
-  constexpr int kIn = 8;
-  for (long long i0 = t; i0 < n_entries; i0 += (long long)kIn * kOrderThreads) {
-    int id[kIn], rr[kIn];
-    bool used[kIn];
-#pragma unroll
-    for (int u = 0; u < kIn; ++u) {
-      const long long i = i0 + (long long)u * kOrderThreads;
-      used[u] = false;
-      rr[u] = 0;
-      id[u] = 0;
-      if (i < n_entries) {
-        const int r = (int)(i / p.max_pages);
-        const int pg = (int)(i - (long long)r * p.max_pages);
-        const int P = p.prefix_len[r];
-        used[u] = P >= 0 && P <= prefix_cap && (long long)pg * p.page_size < P;
-        rr[u] = r;
-        id[u] = p.page_table[i];
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < kIn; ++u) {
-      if (used[u] && (id[u] < 0 || id[u] >= p.num_pages)) {
-        atomicOr(&p.bad_mask[rr[u] >> 5], 1u << (rr[u] & 31));
-        flag(p.dev_status, FLARE_DEV_BAD_PAGE);
-      }
-    }
-  }
-  __syncthreads();
-  auto key_of = [&](int u) -> int {
-    const int r = u / p.n_split, split = u % p.n_split;
-    if (p.bad_mask[r >> 5] & (1u << (r & 31))) return -1;
-    const int P = p.prefix_len[r];
-    const int n_pref = (P + kTileN - 1) / kTileN;
-    const int j0 = split * tps;
-    const int here = max(0, min(n_pref, j0 + tps) - j0);
-    return min(here + (split == p.n_split - 1 ? 1 : 0), kOrderKeys - 1);
+    return prefix_ok(p, P) ? min((P + kTileN - 1) / kTileN, kOrderKeys - 1) : -1;
   };
-  for (int u = t; u < U; u += kOrderThreads) {
-    const int k = key_of(u);
+  for (int r = t; r < p.R; r += kOrderThreads) {
+    const int k = key_of(r);
     if (k >= 0) {
       atomicAdd(&start[k], 1);
       atomicAdd(&n_valid, 1);
+    } else {
+      flag(p.dev_status, FLARE_DEV_BAD_PREFIX_LEN);
     }
   }
   __syncthreads();
-  // start[k] = number of valid units with a larger key; thread t owns the
+  // start[k] = number of valid requests with a larger key; thread t owns the
   // keys at descending positions 4t .. 4t+3
   int v[4], sum = 0;
 #pragma unroll
@@ -292,11 +249,64 @@ __global__ void __launch_bounds__(kOrderThreads) softmax_order_kernel(SoftmaxPar
     run += v[e];
   }
   __syncthreads();
-  for (int u = t; u < U; u += kOrderThreads) {
-    const int k = key_of(u);
-    if (k >= 0) p.order[atomicAdd(&start[k], 1)] = u;
+  for (int r = t; r < p.R; r += kOrderThreads) {
+    const int k = key_of(r);
+    if (k >= 0) p.order[atomicAdd(&start[k], 1)] = r;
   }
   if (t == 0) *p.n_valid = n_valid;
+}
+
+// Combines the split partials: out = sum_s w_s o_s with w_s = exp(lse_s - lse)
+// and lse = log sum_s exp(lse_s) (the partial outputs are already normalised by
+// their own row sums; an empty split has lse = -inf).  One warp per query row.
+// A launch of its own, over the whole chip: one CTA, the last of a row tile's
+// splits to finish, read every partial of its 128 rows before, which kept the
+// number of splits down.
+constexpr int kMergeWarps = 8;
+
+template <int D>
+__global__ void __launch_bounds__(32 * kMergeWarps) softmax_merge_kernel(SoftmaxParams p) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int M = p.B * p.G;
+  const long long row = (long long)blockIdx.x * kMergeWarps + warp;
+  if (row >= (long long)p.R * p.Hkv * M) return;
+  const int item = (int)(row / M), m = (int)(row % M);
+  const int r = item / p.Hkv, kvh = item % p.Hkv;
+  const size_t base = (size_t)item * p.n_split * M + m;  // split s at base + s * M
+  const int ns = p.n_split;  // at most 64: two per lane
+  const float l0 = lane < ns ? p.ws_lse[base + (size_t)lane * M] : -INFINITY;
+  const float l1 = lane + 32 < ns ? p.ws_lse[base + (size_t)(lane + 32) * M] : -INFINITY;
+  const int P = p.prefix_len[r];
+  if (!prefix_ok(p, P) || bad_pages(p, first_page(p, r, P), P, rest_bad(p, r, P)))
+    return;  // flagged by the attention kernel
+  const float mx = warp_max(fmaxf(l0, l1));
+  float w0 = l0 == -INFINITY ? 0.f : expf(l0 - mx);
+  float w1 = l1 == -INFINITY ? 0.f : expf(l1 - mx);
+  const float den = warp_sum(w0 + w1);
+  const float inv = 1.f / den;
+  w0 *= inv;
+  w1 *= inv;
+  constexpr int kC = D / 64;  // 2-column pieces of a lane
+  float2 acc[kC];
+#pragma unroll
+  for (int c = 0; c < kC; ++c) acc[c] = make_float2(0.f, 0.f);
+#pragma unroll 4
+  for (int s = 0; s < ns; ++s) {
+    const float w = __shfl_sync(0xffffffffu, s < 32 ? w0 : w1, s & 31);
+    if (w == 0.f) continue;  // an empty split's partial is never written
+    const float2* o = reinterpret_cast<const float2*>(p.ws_o + (base + (size_t)s * M) * D);
+#pragma unroll
+    for (int c = 0; c < kC; ++c) {
+      const float2 v = o[c * 32 + lane];
+      acc[c].x = fmaf(w, v.x, acc[c].x);
+      acc[c].y = fmaf(w, v.y, acc[c].y);
+    }
+  }
+  const size_t orow = ((size_t)r * p.B + m / p.G) * p.Hq + kvh * p.G + m % p.G;
+  __nv_bfloat162* out = reinterpret_cast<__nv_bfloat162*>(static_cast<__nv_bfloat16*>(p.out) + orow * D);
+#pragma unroll
+  for (int c = 0; c < kC; ++c) out[c * 32 + lane] = __floats2bfloat162_rn(acc[c].x, acc[c].y);
+  if (p.lse && lane == 0) p.lse[orow] = mx + logf(den);
 }
 
 // The attention kernel.  Unsplit prefixes (n_split == 1): one CTA per SM walks
@@ -304,7 +314,7 @@ __global__ void __launch_bounds__(kOrderThreads) softmax_order_kernel(SoftmaxPar
 // k*G + G - 1, in reverse on odd rounds), so that tensor memory, barriers and
 // tensor maps are set up once and the next item's loads and S products
 // overlap the current item's epilogue.  Split prefixes: one CTA per work item,
-// and the last split of a row tile to finish merges the partials.
+// the partials combined by softmax_merge_kernel.
 template <int D>
 __global__ void __launch_bounds__(kThreadsTC, 1)
     softmax_tc_kernel(const __grid_constant__ TcMaps maps, SoftmaxParams p) {
@@ -318,9 +328,12 @@ __global__ void __launch_bounds__(kThreadsTC, 1)
 
   const int M = p.B * p.G;
   const int n_mt = (M + kRowsM - 1) / kRowsM;
-  const int n_items = n_mt * p.Hkv * *p.n_valid;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const bool split_mode = p.n_split > 1;
+  const int units = split_mode ? p.R * p.n_split
+                    : p.order  ? *p.n_valid
+                               : order_on_chip(p, kTileN, reinterpret_cast<int*>(Ks), sh.order);
+  const int n_items = n_mt * p.Hkv * units;
   // k-th work item of this CTA, or -1
   auto item_of = [&](int k) -> int {
     const int G = gridDim.x, b = blockIdx.x;
@@ -331,22 +344,23 @@ __global__ void __launch_bounds__(kThreadsTC, 1)
   const int idx0 = item_of(0);
   if (idx0 < 0) return;
   if (split_mode) {
-    const TcWork w = tc_work(p, n_mt, idx0);
+    const TcWork w = tc_work(p, sh.order, n_mt, idx0);
+    if (!prefix_ok(p, w.P)) {
+      if (tid == 0) flag(p.dev_status, FLARE_DEV_BAD_PREFIX_LEN);
+      return;
+    }
     if (w.n_tiles == 0) {  // empty split: mark its partial as empty for the merge
       const size_t ws_row0 = ((size_t)w.item * p.n_split + w.split) * M;
       for (int i = tid; i < kRowsM; i += blockDim.x) {
         const int m = w.mtile * kRowsM + i;
         if (m < M) p.ws_lse[ws_row0 + m] = -INFINITY;
       }
-      finish_split<D>(p, w.item, w.r, w.kvh, w.mtile, n_mt, &sh.last_split,
-                      reinterpret_cast<float*>(Ks));
       return;
     }
   }
 
   if (tid == 0) {
     sh.abort_flag = 0;
-    sh.last_split = 0;
     sh.v_issued = 0;
     for (int s = 0; s < C::kKStages; ++s) {
       tc::mbar_init(&sh.k_full[s], 1);
@@ -368,6 +382,7 @@ __global__ void __launch_bounds__(kThreadsTC, 1)
     tc::fence_mbar_init();
   }
   if (warp == 1) tc::tmem_alloc(&sh.tmem_base, C::kTmemCols);
+  tc::fence_async_smem();  // the order's keys lay in the K ring
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
@@ -395,7 +410,7 @@ __global__ void __launch_bounds__(kThreadsTC, 1)
       for (int k = 0; ok && !aborted(sh); ++k) {
         const int idx = item_of(k);
         if (idx < 0) break;
-        const TcWork w = tc_work(p, n_mt, idx);
+        const TcWork w = tc_work(p, sh.order, n_mt, idx);
         for (int j = 0; j < w.n_tiles; ++j, ++g) {
           const int st = g % ns;
           const uint32_t ph = (uint32_t)(g / ns) & 1u;
@@ -419,7 +434,8 @@ __global__ void __launch_bounds__(kThreadsTC, 1)
           tc::mbar_expect_tx(full, (uint32_t)(C::kChunks * nbox * box_rows * 128));
           for (int bx = 0; bx < nbox; ++bx) {
             const int tok = tok0 + bx * box_rows;
-            const int page = p.page_table[(size_t)w.r * p.max_pages + tok / p.page_size];
+            const int id = p.page_table[(size_t)w.r * p.max_pages + tok / p.page_size];
+            const int page = id < p.num_pages ? id : -1;  // out of range reads as zero
             const int row0 = tok % p.page_size;
             for (int c = 0; c < C::kChunks; ++c)
               tc::tma_load_4d(dst + c * (kTileN * 128) + bx * box_rows * 128, pool_map, full,
@@ -442,7 +458,7 @@ __global__ void __launch_bounds__(kThreadsTC, 1)
     for (int k = 0; ok && !aborted(sh); ++k) {
       const int idx = item_of(k);
       if (idx < 0) break;
-      const TcWork w = tc_work(p, n_mt, idx);
+      const TcWork w = tc_work(p, sh.order, n_mt, idx);
       if (w.j_part >= 0) {
         const int gg = g + w.j_part;
         const int st = gg % C::kVStages;
@@ -496,7 +512,7 @@ __global__ void __launch_bounds__(kThreadsTC, 1)
       for (int k = 0; ok && !aborted(sh); ++k) {
         const int idx = item_of(k);
         if (idx < 0) break;
-        const TcWork w = tc_work(p, n_mt, idx);
+        const TcWork w = tc_work(p, sh.order, n_mt, idx);
         if (!tc::mbar_wait(&sh.q_ready, (uint32_t)k & 1u, &sh.abort_flag)) {
           ok = false;
           break;
@@ -616,7 +632,7 @@ __global__ void __launch_bounds__(kThreadsTC, 1)
     bool ok = true;
     int g = 0;  // running tile count
     int idx = idx0;
-    TcWork w = tc_work(p, n_mt, idx);
+    TcWork w = tc_work(p, sh.order, n_mt, idx);
     load_q(w);
     for (int k = 0; idx >= 0; ++k) {
       const int m = w.mtile * kRowsM + row;
@@ -627,6 +643,8 @@ __global__ void __launch_bounds__(kThreadsTC, 1)
           p.row_type ? (trow < p.B && p.row_type[(size_t)w.r * p.row_type_stride + trow] == 0)
                      : p.causal != 0;
       float m_run = -INFINITY, l_run = 0.f;
+      const int page0 = first_page(p, w.r, w.P);
+      bool rest = false;
       for (int j = 0; j < w.n_tiles; ++j) {
         const int gg = g + j;
         const int sb = gg % kSB;
@@ -713,7 +731,11 @@ __global__ void __launch_bounds__(kThreadsTC, 1)
         tmem_st_wait();
         tc::fence_before_sync();
         tc::mbar_arrive(&sh.p_full[sb]);
+        if (j == 0) rest = rest_bad(p, w.r, w.P);
       }
+      // every item of a request looks at all its pages
+      const bool bad = bad_pages(p, page0, w.P, rest);
+      if (bad && lane == 0) flag(p.dev_status, FLARE_DEV_BAD_PAGE);
       g += w.n_tiles;
       if (ok && aborted(sh)) ok = false;
       // the next item's Q can go into tensor memory now: every S product of
@@ -721,7 +743,7 @@ __global__ void __launch_bounds__(kThreadsTC, 1)
       const int idx_next = ok ? item_of(k + 1) : -1;
       TcWork wn = w;
       if (idx_next >= 0) {
-        wn = tc_work(p, n_mt, idx_next);
+        wn = tc_work(p, sh.order, n_mt, idx_next);
         load_q(wn);
       }
       // epilogue: O / l (or the split partial) and the log-sum-exp
@@ -731,7 +753,7 @@ __global__ void __launch_bounds__(kThreadsTC, 1)
         break;
       }
       tc::fence_after_sync();
-      const bool write = m < M;
+      const bool write = m < M && !bad;
       const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
       const int gq = m % p.G;
       const size_t orow = (((size_t)w.r * p.B + trow) * p.Hq + w.kvh * p.G + gq);
@@ -783,12 +805,6 @@ __global__ void __launch_bounds__(kThreadsTC, 1)
     tc::fence_after_sync();
     tc::tmem_dealloc(tmem, C::kTmemCols);
   }
-  // a CTA that gave up wrote no partial: its row tile is never merged
-  if (split_mode && !aborted(sh)) {  // the K/V rings are free: merge weights go there
-    const TcWork w = tc_work(p, n_mt, idx0);
-    finish_split<D>(p, w.item, w.r, w.kvh, w.mtile, n_mt, &sh.last_split,
-                    reinterpret_cast<float*>(Ks));
-  }
 }
 
 // ------------------------------------------------------------------ host side
@@ -825,8 +841,20 @@ bool encode_map(CUtensorMap* m, const void* ptr, int rank, const uint64_t* dims,
 }
 
 cudaError_t launch_softmax_order(const SoftmaxParams& p, cudaStream_t stream) {
-  if (!p.order || !p.n_valid || !p.bad_mask) return cudaErrorInvalidValue;
+  if (!p.order || !p.n_valid) return cudaErrorInvalidValue;
   softmax_order_kernel<<<1, kOrderThreads, 0, stream>>>(p);
+  note_launches(1);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_softmax_merge(const SoftmaxParams& p, cudaStream_t stream) {
+  const long long rows = (long long)p.R * p.Hkv * p.B * p.G;
+  const unsigned grid = (unsigned)((rows + kMergeWarps - 1) / kMergeWarps);
+  switch (p.D) {
+    case 64: softmax_merge_kernel<64><<<grid, 32 * kMergeWarps, 0, stream>>>(p); break;
+    case 128: softmax_merge_kernel<128><<<grid, 32 * kMergeWarps, 0, stream>>>(p); break;
+    default: softmax_merge_kernel<256><<<grid, 32 * kMergeWarps, 0, stream>>>(p); break;
+  }
   note_launches(1);
   return cudaGetLastError();
 }
@@ -864,11 +892,12 @@ cudaError_t launch_tc_d(const SoftmaxParams& p, const SoftmaxPlan& plan, cudaStr
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (err != cudaSuccess) return err;
   if (plan.num_ctas <= 0) return cudaErrorInvalidValue;
-  err = launch_softmax_order(p, stream);
+  if (p.order) err = launch_softmax_order(p, stream);
   if (err != cudaSuccess) return err;
   softmax_tc_kernel<D><<<(unsigned)plan.num_ctas, kThreadsTC, smem, stream>>>(maps, p);
   note_launches(1);
-  return cudaGetLastError();
+  err = cudaGetLastError();
+  return err == cudaSuccess && p.n_split > 1 ? launch_softmax_merge(p, stream) : err;
 }
 
 }  // namespace
