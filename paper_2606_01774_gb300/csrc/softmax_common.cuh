@@ -6,6 +6,7 @@
 
 #include "common.cuh"
 #include "kernels.h"
+#include "tc.cuh"
 
 namespace flare {
 
@@ -27,6 +28,27 @@ __device__ __forceinline__ bool prefix_ok(const SoftmaxParams& p, int P) {
 // its own prefix, in whole tiles of `tile` keys.
 __device__ __forceinline__ int split_keys(const SoftmaxParams& p, int P, int tile) {
   return ((P + p.n_split - 1) / p.n_split + tile - 1) / tile * tile;
+}
+
+// 16 columns of an output row, o * inv as bf16.  Each lane of a warp writes a
+// row of its own, so a store instruction touches 32 lines whatever its width: whole
+// 32-byte sectors (where the array starts on one) halve the instructions and the
+// sector writes.
+__device__ __forceinline__ void store_bf16x16(__nv_bfloat16* dst, const uint32_t (&o)[16],
+                                              float inv, bool sector) {
+  uint32_t pk[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    __nv_bfloat162 h2 = __floats2bfloat162_rn(__uint_as_float(o[2 * i]) * inv,
+                                              __uint_as_float(o[2 * i + 1]) * inv);
+    pk[i] = *reinterpret_cast<uint32_t*>(&h2);
+  }
+  if (sector) {
+    tc::store32(dst, pk);
+  } else {
+    reinterpret_cast<uint4*>(dst)[0] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+    reinterpret_cast<uint4*>(dst)[1] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+  }
 }
 
 // Longest-first order of the requests, computed by every CTA for itself from the

@@ -104,21 +104,6 @@ __device__ __forceinline__ uint32_t cluster_rank() {
   return r;
 }
 
-// One lane of a converged warp, always the same one.  The products and copies are
-// issued under this branch: the compiler then knows that a single thread is
-// active and takes their descriptors from uniform registers.
-__device__ __forceinline__ bool elect_one() {
-  uint32_t pred;
-  asm volatile(
-      "{\n"
-      " .reg .pred p;\n"
-      " elect.sync _|p, 0xffffffff;\n"
-      " selp.b32 %0, 1, 0, p;\n"
-      "}\n"
-      : "=r"(pred));
-  return pred != 0;
-}
-
 __device__ __forceinline__ uint32_t map_rank(uint32_t saddr, uint32_t rank) {
   uint32_t a;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(saddr), "r"(rank));
@@ -214,27 +199,35 @@ struct PairWork {
 
 // Item `idx`: (row-tile pair, kv head) fastest, then the prefix splits of each
 // request (split) or the valid requests longest first (unsplit).
-__device__ __forceinline__ PairWork pair_work(const SoftmaxParams& p, const uint16_t* order,
-                                              int n_mp, int idx) {
+// In two parts: pair_fetch, one item ahead, has the prefix length's load in flight;
+// pair_plan looks at it.
+__device__ __forceinline__ PairWork pair_fetch(const SoftmaxParams& p, const uint16_t* order,
+                                               int n_mp, int idx) {
   PairWork w;
+  if (idx < 0) idx = 0;
   w.mpair = idx % n_mp;
   w.kvh = (idx / n_mp) % p.Hkv;
   const int unit = idx / (n_mp * p.Hkv);
+  w.split = 0;
   if (p.n_split > 1) {
     w.r = unit / p.n_split;
     w.split = unit % p.n_split;
-    w.P = p.prefix_len[w.r];
+  } else {
+    w.r = p.order ? p.order[unit] : order[unit];
+  }
+  w.item = w.r * p.Hkv + w.kvh;
+  w.P = p.prefix_len[w.r];
+  return w;
+}
+
+__device__ __forceinline__ PairWork pair_plan(const SoftmaxParams& p, PairWork w) {
+  w.tok_lo = 0;
+  w.tok_hi = w.P;
+  if (p.n_split > 1) {
     const int len = split_keys(p, w.P, kPairKeys);
     w.tok_lo = min(w.P, w.split * len);
     w.tok_hi = min(w.P, w.tok_lo + len);
-  } else {
-    w.r = p.order ? p.order[unit] : order[unit];
-    w.split = 0;
-    w.P = p.prefix_len[w.r];
-    w.tok_lo = 0;
-    w.tok_hi = w.P;
   }
-  w.item = w.r * p.Hkv + w.kvh;
   w.n_pref = (w.tok_hi - w.tok_lo + kPairKeys - 1) / kPairKeys;
   w.block = w.split == p.n_split - 1;
   w.n_tiles = w.n_pref + (w.block ? 1 : 0);
@@ -343,7 +336,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
   const int idx0 = item_of(0);
   if (idx0 < 0) return;
   if (split_mode) {
-    const PairWork w = pair_work(p, sh.order, n_mp, idx0);
+    const PairWork w = pair_plan(p, pair_fetch(p, sh.order, n_mp, idx0));
     if (!prefix_ok(p, w.P)) {
       if (tid == 0) flag(p.dev_status, FLARE_DEV_BAD_PREFIX_LEN);
       return;
@@ -419,10 +412,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
       if (++st == C::kSlots) st = 0, ph ^= 1u;
     };
     auto acquire = [&]() { return pair_warp_wait(&sh.empty[st], ph ^ 1u, &sh.abort_flag); };
+    int idx = idx0;
+    PairWork next = pair_fetch(p, sh.order, n_mp, idx);
     for (int k = 0; ok && !pair_aborted(sh); ++k) {
-      const int idx = item_of(k);
       if (idx < 0) break;
-      const PairWork w = pair_work(p, sh.order, n_mp, idx);
+      const PairWork w = pair_plan(p, next);
+      idx = item_of(k + 1);
+      next = pair_fetch(p, sh.order, n_mp, idx);
       // page ids of the window [pbase, pbase + 64): two per lane, in cur and nxt
       const int n_pages = (w.tok_hi + p.page_size - 1) >> pshift;
       const int32_t* table = p.page_table + (size_t)w.r * p.max_pages;
@@ -440,7 +436,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
           const int pb = __shfl_sync(0xffffffffu, nxt, o & 31);
           const int id = o < 32 ? pa : pb;
           const int page = id < p.num_pages ? id : -1;  // out of range reads as zero
-          if (elect_one()) {
+          if (tc::elect_one()) {
             const int row = t & (p.page_size - 1);
             if (bshift == 6) {
               tma2_load_5d(dst, pool_map, bar, 0, row, ch, w.kvh, page);
@@ -460,7 +456,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
         if (!acquire()) return false;
         const uint32_t dst = ring_u + st * C::kSlotBytes, bar = full0 + st * 8;
         if (j >= w.n_pref) {
-          if (elect_one()) {
+          if (tc::elect_one()) {
             expect_at(bar, C::kKChunks * 32 * 128);
             for (int c = 0; c < C::kKChunks; ++c)
               tma2_load_4d(dst + c * 8192, blk_map, bar, c * 64, w.kvh, (int)rank * 32, w.r);
@@ -469,7 +465,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
         } else {
           const int tok = w.tok_lo + j * kPairKeys + (int)rank * 64;
           const int rows = min(64, max(0, w.tok_hi - tok));
-          if (elect_one()) expect_at(bar, bytes_of(rows, C::kKChunks));
+          if (tc::elect_one()) expect_at(bar, bytes_of(rows, C::kKChunks));
           __syncwarp();
           load_keys(dst, bar, tok, rows, 0, C::kKChunks);
         }
@@ -480,7 +476,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
         const uint32_t dst = ring_u + st * C::kSlotBytes, bar = full0 + st * 8;
         const int ch = (int)rank * C::kVChunks;
         if (j >= w.n_pref) {
-          if (elect_one()) {
+          if (tc::elect_one()) {
             expect_at(bar, C::kVChunks * 64 * 128);
             for (int c = 0; c < C::kVChunks; ++c)
               tma2_load_4d(dst + c * 8192, blk_map, bar, (ch + c) * 64, w.kvh, 0, w.r);
@@ -493,7 +489,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
           // a tile the prefix ends in, off a 16-key step: it lands on this CTA's own
           // barrier and the fixer arrives at the leader's once its rows are zero
           const uint32_t to = (keys & 15) ? vr0 + st * 8 : bar;
-          if (elect_one()) expect_at(to, bytes_of(r0, C::kVChunks) + bytes_of(r1, C::kVChunks));
+          if (tc::elect_one()) expect_at(to, bytes_of(r0, C::kVChunks) + bytes_of(r1, C::kVChunks));
           __syncwarp();
           load_keys(dst, to, tok, r0, ch, C::kVChunks);
           if (r1 > 0) load_keys(dst + C::kVChunks * 8192, to, tok + 64, r1, ch, C::kVChunks);
@@ -541,10 +537,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
       auto pass = [&]() {
         if (++st == C::kSlots) st = 0, ph ^= 1u;
       };
+      int idx = idx0;
+      PairWork next = pair_fetch(p, sh.order, n_mp, idx);
       for (int k = 0; ok && !pair_aborted(sh); ++k) {
-        const int idx = item_of(k);
         if (idx < 0) break;
-        const PairWork w = pair_work(p, sh.order, n_mp, idx);
+        const PairWork w = pair_plan(p, next);
+        idx = item_of(k + 1);
+        next = pair_fetch(p, sh.order, n_mp, idx);
         if (!pair_warp_wait(&sh.q_full, (uint32_t)k & 1u, &sh.abort_flag)) {
           ok = false;
           break;
@@ -555,7 +554,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
           const uint32_t id_s = j >= w.n_pref ? id_s64 : id_s128;
           if (!pair_warp_wait(&sh.full[st], ph, &sh.abort_flag)) return false;
           tc::fence_after_sync();
-          if (elect_one()) {
+          if (tc::elect_one()) {
             const uint64_t kd = kdesc0 + (uint64_t)((st * C::kSlotBytes) >> 4);
 #pragma unroll
             for (int kk = 0; kk < D / 16; ++kk) {
@@ -582,7 +581,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
           if (!pair_warp_wait(&sh.p_full[pb], (uint32_t)(gg >> 1) & 1u, &sh.abort_flag))
             return false;
           tc::fence_after_sync();
-          if (elect_one()) {
+          if (tc::elect_one()) {
             const uint64_t vd = vdesc0 + (uint64_t)((st * C::kSlotBytes) >> 4);
             const uint32_t pt = tmem_s + pb * 128;
             auto step = [&](int kk) {
@@ -621,15 +620,18 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
     bool ok = true;
     int cnt = 0;               // running slot count at the item's start
     uint32_t par = 0u;         // per slot: parity of its next ragged phase
+    int idx = idx0;
+    PairWork next = pair_fetch(p, sh.order, n_mp, idx);
     for (int k = 0; ok && !pair_aborted(sh); ++k) {
       // the previous item's S products, the last readers of its Q, are done
       if (k > 0 && !pair_warp_wait(&sh.q_empty, (uint32_t)(k - 1) & 1u, &sh.abort_flag)) {
         ok = false;
         break;
       }
-      const int idx = item_of(k);
       if (idx < 0) break;
-      const PairWork w = pair_work(p, sh.order, n_mp, idx);
+      const PairWork w = pair_plan(p, next);
+      idx = item_of(k + 1);
+      next = pair_fetch(p, sh.order, n_mp, idx);
       if (lane == 0) {
         expect_at(q_full_c, C::kQBytes);
         // rows past the block (t >= B) read as zero
@@ -669,12 +671,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
     const uint32_t lane_off = (uint32_t)(quarter * 32) << 16;
     const uint32_t o_free_c = map_rank(tc::smem_u32(&sh.o_free), 0);
     const uint32_t p_full_c = map_rank(tc::smem_u32(&sh.p_full[0]), 0);
+    const bool sector = ((uintptr_t)p.out & 31) == 0;  // rows start on 32-byte sectors
     bool ok = true;
     int g = 0;  // running tile count
+    int idx = idx0;
+    PairWork next = pair_fetch(p, sh.order, n_mp, idx);
     for (int k = 0; ok && !pair_aborted(sh); ++k) {
-      const int idx = item_of(k);
       if (idx < 0) break;
-      const PairWork w = pair_work(p, sh.order, n_mp, idx);
+      const PairWork w = pair_plan(p, next);
+      idx = item_of(k + 1);
+      next = pair_fetch(p, sh.order, n_mp, idx);
       const int m = (2 * w.mpair + (int)rank) * kRowsM + row;
       const int trow = m / p.G;
       const bool causal_row =
@@ -748,25 +754,18 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
         tc::tmem_ld_wait();
         if (!write) continue;
         if (!split_mode) {
-          uint4* dst = reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(p.out) + orow * D + c);
+          __nv_bfloat16* dst = static_cast<__nv_bfloat16*>(p.out) + orow * D + c;
+          store_bf16x16(dst, *reinterpret_cast<const uint32_t(*)[16]>(&o[0]), inv, sector);
+          store_bf16x16(dst + 16, *reinterpret_cast<const uint32_t(*)[16]>(&o[16]), inv, sector);
+        } else {
+          float* dst = p.ws_o + ws_row * D + c;
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
-            uint32_t pk[4];
+            uint32_t v[8];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              __nv_bfloat162 h2 = __floats2bfloat162_rn(__uint_as_float(o[8 * i + 2 * e]) * inv,
-                                                        __uint_as_float(o[8 * i + 2 * e + 1]) * inv);
-              pk[e] = *reinterpret_cast<uint32_t*>(&h2);
-            }
-            dst[i] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+            for (int e = 0; e < 8; ++e) v[e] = __float_as_uint(__uint_as_float(o[8 * i + e]) * inv);
+            tc::store32(dst + 8 * i, v);
           }
-        } else {
-          float4* dst = reinterpret_cast<float4*>(p.ws_o + ws_row * D + c);
-#pragma unroll
-          for (int i = 0; i < 8; ++i)
-            dst[i] = make_float4(__uint_as_float(o[4 * i]) * inv, __uint_as_float(o[4 * i + 1]) * inv,
-                                 __uint_as_float(o[4 * i + 2]) * inv,
-                                 __uint_as_float(o[4 * i + 3]) * inv);
         }
       }
       tc::fence_before_sync();

@@ -65,7 +65,9 @@ constexpr float kRescaleThreshold = 8.0f;  // log2 units
 struct TcMaps {
   CUtensorMap kblk;   // (D, Hkv, B, R)          box (64, 1, 64, 1)
   CUtensorMap vblk;
-  CUtensorMap kpool;  // (D, p, Hkv, num_pages)  box (64, min(p,64), 1, 1)
+  // (64, p, D/64, Hkv, num_pages): a page-head as 64-column chunks.  Pages of 64 or
+  // 128 tokens: box (64, 64, D/64, 1, 1), a whole tile; smaller: (64, p, 1, 1, 1)
+  CUtensorMap kpool;
   CUtensorMap vpool;
 };
 
@@ -152,21 +154,28 @@ struct TcWork {
 
 // Work item `idx` of the flat list: (row tile, kv head) fastest, then the prefix
 // splits of each request (split) or the valid requests longest first (unsplit).
-__device__ __forceinline__ TcWork tc_work(const SoftmaxParams& p, const uint16_t* order, int n_mt,
-                                          int idx) {
+// In two parts: tc_fetch, one item ahead, has the prefix length's load in flight;
+// tc_plan looks at it.
+__device__ __forceinline__ TcWork tc_fetch(const SoftmaxParams& p, const uint16_t* order, int n_mt,
+                                           int idx) {
   TcWork w;
+  if (idx < 0) idx = 0;
   w.mtile = idx % n_mt;
   w.kvh = (idx / n_mt) % p.Hkv;
   const int unit = idx / (n_mt * p.Hkv);
+  w.split = 0;
   if (p.n_split > 1) {
     w.r = unit / p.n_split;
     w.split = unit % p.n_split;
   } else {
     w.r = p.order ? p.order[unit] : order[unit];
-    w.split = 0;
   }
   w.item = w.r * p.Hkv + w.kvh;
   w.P = p.prefix_len[w.r];
+  return w;
+}
+
+__device__ __forceinline__ TcWork tc_plan(const SoftmaxParams& p, TcWork w) {
   const int n_pref = (w.P + kTileN - 1) / kTileN;
   w.j0 = 0;
   int j1 = n_pref;
@@ -344,7 +353,7 @@ __global__ void __launch_bounds__(kThreadsTC, 1)
   const int idx0 = item_of(0);
   if (idx0 < 0) return;
   if (split_mode) {
-    const TcWork w = tc_work(p, sh.order, n_mt, idx0);
+    const TcWork w = tc_plan(p, tc_fetch(p, sh.order, n_mt, idx0));
     if (!prefix_ok(p, w.P)) {
       if (tid == 0) flag(p.dev_status, FLARE_DEV_BAD_PREFIX_LEN);
       return;
@@ -396,56 +405,86 @@ __global__ void __launch_bounds__(kThreadsTC, 1)
     // warp 0 streams the K tiles and warp kVWarp the V tiles of every work
     // item of this CTA, each into its own ring (slot = running tile count mod
     // ring depth), so neither waits behind the other's slot.
+    // The page ids of a window ahead sit in registers; one lane issues.
+    const int kv = warp == 0 ? 0 : 1;
+    const CUtensorMap* pool_map = kv ? &maps.vpool : &maps.kpool;
+    const CUtensorMap* blk_map = kv ? &maps.vblk : &maps.kblk;
     if (lane == 0) {
-      const int kv = warp == 0 ? 0 : 1;
-      const CUtensorMap* pool_map = kv ? &maps.vpool : &maps.kpool;
-      const CUtensorMap* blk_map = kv ? &maps.vblk : &maps.kblk;
       tc::prefetch_tmap(pool_map);
       tc::prefetch_tmap(blk_map);
-      const int box_rows = p.page_size < kTileN ? p.page_size : kTileN;
-      const int ns = kv ? C::kVStages : C::kKStages;
-      uint8_t* ring = kv ? Vs : Ks;
-      bool ok = true;
-      int g = 0;  // running tile count
-      for (int k = 0; ok && !aborted(sh); ++k) {
-        const int idx = item_of(k);
-        if (idx < 0) break;
-        const TcWork w = tc_work(p, sh.order, n_mt, idx);
-        for (int j = 0; j < w.n_tiles; ++j, ++g) {
-          const int st = g % ns;
-          const uint32_t ph = (uint32_t)(g / ns) & 1u;
-          uint64_t* empty = kv ? &sh.v_empty[st] : &sh.k_empty[st];
-          uint64_t* full = kv ? &sh.v_full[st] : &sh.k_full[st];
-          uint8_t* dst = ring + st * C::kKVBytes;
-          if (!tc::mbar_wait(empty, ph ^ 1u, &sh.abort_flag)) {
-            ok = false;
-            break;
-          }
-          if (j >= w.n_pref_here) {  // the block's own keys / values
+    }
+    const int pshift = 31 - __clz(p.page_size);  // page sizes are powers of two
+    const int bshift = min(pshift, 6);           // log2 of a box's rows
+    const int ns = kv ? C::kVStages : C::kKStages;
+    uint8_t* ring = kv ? Vs : Ks;
+    bool ok = true;
+    int g = 0;  // running tile count
+    int st = 0;
+    uint32_t ph = 0;
+    int idx = idx0;
+    TcWork next = tc_fetch(p, sh.order, n_mt, idx);
+    for (int k = 0; ok && idx >= 0 && !aborted(sh); ++k) {
+      const TcWork w = tc_plan(p, next);
+      idx = item_of(k + 1);
+      next = tc_fetch(p, sh.order, n_mt, idx);
+      // page ids of the window [pbase, pbase + 64): two per lane, in cur and nxt
+      const int n_pages = (w.P + p.page_size - 1) >> pshift;
+      const int32_t* table = p.page_table + (size_t)w.r * p.max_pages;
+      auto fetch = [&](int first) { return first + lane < n_pages ? table[first + lane] : 0; };
+      int pbase = (w.j0 * kTileN) >> pshift;
+      int cur = fetch(pbase), nxt = fetch(pbase + 32);
+      for (int j = 0; j < w.n_tiles; ++j, ++g) {
+        uint64_t* empty = kv ? &sh.v_empty[st] : &sh.k_empty[st];
+        uint64_t* full = kv ? &sh.v_full[st] : &sh.k_full[st];
+        uint8_t* dst = ring + st * C::kKVBytes;
+        if (!warp_wait(empty, ph ^ 1u, &sh.abort_flag)) {
+          ok = false;
+          break;
+        }
+        if (++st == ns) st = 0, ph ^= 1u;
+        if (j >= w.n_pref_here) {  // the block's own keys / values
+          if (tc::elect_one()) {
             tc::mbar_expect_tx(full, C::kKVBytes);
             for (int c = 0; c < C::kChunks; ++c)
               tc::tma_load_4d(dst + c * (kTileN * 128), blk_map, full, c * 64, w.kvh, 0, w.r);
-            if (kv) *reinterpret_cast<volatile int*>(&sh.v_issued) = g + 1;
-            continue;
           }
+        } else {
           const int tok0 = (w.j0 + j) * kTileN;
-          const int valid = min(kTileN, w.P - tok0);
-          const int nbox = (valid + box_rows - 1) / box_rows;
-          tc::mbar_expect_tx(full, (uint32_t)(C::kChunks * nbox * box_rows * 128));
-          for (int bx = 0; bx < nbox; ++bx) {
-            const int tok = tok0 + bx * box_rows;
-            const int id = p.page_table[(size_t)w.r * p.max_pages + tok / p.page_size];
-            const int page = id < p.num_pages ? id : -1;  // out of range reads as zero
-            const int row0 = tok % p.page_size;
-            for (int c = 0; c < C::kChunks; ++c)
-              tc::tma_load_4d(dst + c * (kTileN * 128) + bx * box_rows * 128, pool_map, full,
-                              c * 64, row0, w.kvh, page);
+          if ((tok0 >> pshift) - pbase >= 32) {
+            pbase += 32;
+            cur = nxt;
+            nxt = fetch(pbase + 32);
           }
-          if (kv) *reinterpret_cast<volatile int*>(&sh.v_issued) = g + 1;
+          const int valid = min(kTileN, w.P - tok0);
+          const int nbox = (valid + (1 << bshift) - 1) >> bshift;
+          if (tc::elect_one())
+            tc::mbar_expect_tx(full, (uint32_t)(C::kChunks * nbox) << (bshift + 7));
+          __syncwarp();
+          for (int bx = 0; bx < nbox; ++bx) {
+            const int tok = tok0 + (bx << bshift);
+            const int o = (tok >> pshift) - pbase;
+            const int pa = __shfl_sync(0xffffffffu, cur, o & 31);
+            const int pb = __shfl_sync(0xffffffffu, nxt, o & 31);
+            const int id = o < 32 ? pa : pb;
+            const int page = id < p.num_pages ? id : -1;  // out of range reads as zero
+            if (tc::elect_one()) {
+              const int row0 = tok & (p.page_size - 1);
+              if (bshift == 6) {
+                tc::tma_load_5d(dst, pool_map, full, 0, row0, 0, w.kvh, page);
+              } else {
+                for (int c = 0; c < C::kChunks; ++c)
+                  tc::tma_load_5d(dst + c * (kTileN * 128) + ((uint32_t)bx << (bshift + 7)),
+                                  pool_map, full, 0, row0, c, w.kvh, page);
+              }
+            }
+            __syncwarp();
+          }
         }
+        __syncwarp();
+        if (kv && lane == 0) *reinterpret_cast<volatile int*>(&sh.v_issued) = g + 1;
       }
-      if (!ok) set_abort(sh, p.dev_status);
     }
+    if (!ok && lane == 0) set_abort(sh, p.dev_status);
   } else if (warp == kFixWarp) {
     // ------------------------------------------------------------ V fixer
     // The last prefix tile of an item ends inside the tile: its V rows past the
@@ -455,10 +494,12 @@ __global__ void __launch_bounds__(kThreadsTC, 1)
     // A warp of its own, so the V producer never stops to wait for a load.
     bool ok = true;
     int g = 0;  // running tile count
-    for (int k = 0; ok && !aborted(sh); ++k) {
-      const int idx = item_of(k);
-      if (idx < 0) break;
-      const TcWork w = tc_work(p, sh.order, n_mt, idx);
+    int idx = idx0;
+    TcWork next = tc_fetch(p, sh.order, n_mt, idx);
+    for (int k = 0; ok && idx >= 0 && !aborted(sh); ++k) {
+      const TcWork w = tc_plan(p, next);
+      idx = item_of(k + 1);
+      next = tc_fetch(p, sh.order, n_mt, idx);
       if (w.j_part >= 0) {
         const int gg = g + w.j_part;
         const int st = gg % C::kVStages;
@@ -499,64 +540,69 @@ __global__ void __launch_bounds__(kThreadsTC, 1)
     if (!ok && lane == 0) set_abort(sh, p.dev_status);
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
-    // One thread waits and issues; operand descriptors advance by adding the
-    // byte offset (>> 4) to the start-address field of a base descriptor.
-    if (lane == 0) {
-      const uint32_t id_s = tc::idesc_bf16(kRowsM, kTileN, false, false);
-      const uint32_t id_o = tc::idesc_bf16(kRowsM, D, false, true);
-      const uint64_t kdesc0 = tc::sdesc_sw128(tc::smem_u32(Ks), 16, 1024);
-      const uint64_t vdesc0 = tc::sdesc_sw128(tc::smem_u32(Vs), kTileN * 128, 1024);
-      bool ok = true;
-      int g = 0;              // running tile count
-      uint32_t fix_par = 0u;  // per V slot: parity of its next zeroed-partial-tile phase
-      for (int k = 0; ok && !aborted(sh); ++k) {
-        const int idx = item_of(k);
-        if (idx < 0) break;
-        const TcWork w = tc_work(p, sh.order, n_mt, idx);
-        if (!tc::mbar_wait(&sh.q_ready, (uint32_t)k & 1u, &sh.abort_flag)) {
-          ok = false;
-          break;
+    // The whole warp walks the tiles and waits; one elected lane issues (under a
+    // plain lane branch each product took about 60 cycles to issue and the issuing
+    // thread, not memory, set the tile rate: 0.85 us per tile of small_model_batch256,
+    // now 0.75, which is 6.6 TB/s over the chip; the call 141 -> 134 us).  Operand descriptors advance by
+    // adding the byte offset (>> 4) to the start-address field of a base descriptor.
+    const uint32_t id_s = tc::idesc_bf16(kRowsM, kTileN, false, false);
+    const uint32_t id_o = tc::idesc_bf16(kRowsM, D, false, true);
+    const uint64_t kdesc0 = tc::sdesc_sw128(tc::smem_u32(Ks), 16, 1024);
+    const uint64_t vdesc0 = tc::sdesc_sw128(tc::smem_u32(Vs), kTileN * 128, 1024);
+    bool ok = true;
+    int g = 0;              // running tile count
+    int kst = 0, vst = 0;   // K and V slots
+    uint32_t kph = 0, vph = 0;
+    uint32_t fix_par = 0u;  // per V slot: parity of its next zeroed-partial-tile phase
+    int idx = idx0;
+    TcWork next = tc_fetch(p, sh.order, n_mt, idx);
+    for (int k = 0; ok && idx >= 0 && !aborted(sh); ++k) {
+      const TcWork w = tc_plan(p, next);
+      idx = item_of(k + 1);
+      next = tc_fetch(p, sh.order, n_mt, idx);
+      if (!warp_wait(&sh.q_ready, (uint32_t)k & 1u, &sh.abort_flag)) {
+        ok = false;
+        break;
+      }
+      auto issue_pv = [&](int j) -> bool {
+        const int gg = g + j;
+        const int pb = gg % kSB;
+        // a slot's partial tiles are in order: the next one can only be
+        // loaded once the P.V issued after this wait has freed the slot
+        bool ready;
+        if (j == w.j_part) {
+          ready = warp_wait(&sh.v_fix[vst], (fix_par >> vst) & 1u, &sh.abort_flag);
+          fix_par ^= 1u << vst;
+        } else {
+          ready = warp_wait(&sh.v_full[vst], vph, &sh.abort_flag);
         }
-        auto issue_pv = [&](int j) -> bool {
-          const int gg = g + j;
-          const int st = gg % C::kVStages;
-          const int pb = gg % kSB;
-          if (!tc::mbar_wait(&sh.p_full[pb], (uint32_t)(gg / kSB) & 1u, &sh.abort_flag))
-            return false;
-          // the first P.V of an item overwrites O: the previous item's O must be out
-          if (j == 0 && k > 0 &&
-              !tc::mbar_wait(&sh.o_free, (uint32_t)(k - 1) & 1u, &sh.abort_flag))
-            return false;
-          // a slot's partial tiles are in order: the next one can only be
-          // loaded once the P.V issued after this wait has freed the slot
-          bool ready;
-          if (j == w.j_part) {
-            ready = tc::mbar_wait(&sh.v_fix[st], (fix_par >> st) & 1u, &sh.abort_flag);
-            fix_par ^= 1u << st;
-          } else {
-            ready = tc::mbar_wait(&sh.v_full[st], (uint32_t)(gg / C::kVStages) & 1u,
-                                  &sh.abort_flag);
-          }
-          if (!ready) return false;
-          tc::fence_after_sync();
-          const uint64_t vd = vdesc0 + (uint64_t)((st * C::kKVBytes) >> 4);
+        if (!ready) return false;
+        // the first P.V of an item overwrites O: the previous item's O must be out
+        if (j == 0 && k > 0 && !warp_wait(&sh.o_free, (uint32_t)(k - 1) & 1u, &sh.abort_flag))
+          return false;
+        if (!warp_wait(&sh.p_full[pb], (uint32_t)(gg / kSB) & 1u, &sh.abort_flag)) return false;
+        tc::fence_after_sync();
+        if (tc::elect_one()) {
+          const uint64_t vd = vdesc0 + (uint64_t)((vst * C::kKVBytes) >> 4);
 #pragma unroll
           for (int kk = 0; kk < kTileN / 16; ++kk)
             mma_bf16_ts(tmem_o, tmem_s + pb * kTileN + kk * 8, vd + (uint64_t)(kk * (2048 >> 4)),
                         id_o, (j > 0 || kk > 0) ? 1u : 0u);
           tc::mma_commit(&sh.pv_done[pb]);
-          tc::mma_commit(&sh.v_empty[st]);
-          return true;
-        };
-        // S_j = Q K_j^T into S buffer (g + j) % kSB (Q from tensor memory)
-        auto issue_s = [&](int j) -> bool {
-          const int gg = g + j;
-          const int st = gg % C::kKStages;
-          const int sb = gg % kSB;
-          if (!tc::mbar_wait(&sh.k_full[st], (uint32_t)(gg / C::kKStages) & 1u, &sh.abort_flag))
-            return false;
-          tc::fence_after_sync();
-          const uint64_t kd = kdesc0 + (uint64_t)((st * C::kKVBytes) >> 4);
+          tc::mma_commit(&sh.v_empty[vst]);
+          if (j == w.n_tiles - 1) tc::mma_commit(&sh.o_final);
+        }
+        __syncwarp();
+        if (++vst == C::kVStages) vst = 0, vph ^= 1u;
+        return true;
+      };
+      // S_j = Q K_j^T into S buffer (g + j) % kSB (Q from tensor memory)
+      auto issue_s = [&](int j) -> bool {
+        const int sb = (g + j) % kSB;
+        if (!warp_wait(&sh.k_full[kst], kph, &sh.abort_flag)) return false;
+        tc::fence_after_sync();
+        if (tc::elect_one()) {
+          const uint64_t kd = kdesc0 + (uint64_t)((kst * C::kKVBytes) >> 4);
 #pragma unroll
           for (int kk = 0; kk < D / 16; ++kk) {
             const int c = kk >> 2, off = (kk & 3) * 32;
@@ -564,31 +610,32 @@ __global__ void __launch_bounds__(kThreadsTC, 1)
                         kd + (uint64_t)((c * (kTileN * 128) + off) >> 4), id_s, kk > 0 ? 1u : 0u);
           }
           tc::mma_commit(&sh.s_full[sb]);
-          tc::mma_commit(&sh.k_empty[st]);
-          return true;
-        };
-        // Three S buffers: issue order S0, S1, S2, PV0, S3, PV1, ...: S_{j+2}
-        // is queued before the P.V of tile j waits on its probabilities and
-        // reuses the buffer of tile j-1, whose P.V was issued (and, in issue
-        // order, executes) before it.  Two buffers: S0, S1, PV0, S2, PV1, ...:
-        // S_{j+2} reuses the buffer of tile j, so it follows P_j V_j.  The
-        // running tile count carries the buffers across work items.
-        const int n = w.n_tiles;
-        for (int j = 0; j < 2 && j < n && ok; ++j) ok = issue_s(j);
-        for (int j = 0; j < n && ok; ++j) {
-          if (kSB == 3) {
-            if (j + 2 < n) ok = issue_s(j + 2);
-            if (ok) ok = issue_pv(j);
-          } else {
-            ok = issue_pv(j);
-            if (ok && j + 2 < n) ok = issue_s(j + 2);
-          }
+          tc::mma_commit(&sh.k_empty[kst]);
         }
-        if (ok) tc::mma_commit(&sh.o_final);
-        g += n;
+        __syncwarp();
+        if (++kst == C::kKStages) kst = 0, kph ^= 1u;
+        return true;
+      };
+      // Three S buffers: issue order S0, S1, S2, PV0, S3, PV1, ...: S_{j+2}
+      // is queued before the P.V of tile j waits on its probabilities and
+      // reuses the buffer of tile j-1, whose P.V was issued (and, in issue
+      // order, executes) before it.  Two buffers: S0, S1, PV0, S2, PV1, ...:
+      // S_{j+2} reuses the buffer of tile j, so it follows P_j V_j.  The
+      // running tile count carries the buffers across work items.
+      const int n = w.n_tiles;
+      for (int j = 0; j < 2 && j < n && ok; ++j) ok = issue_s(j);
+      for (int j = 0; j < n && ok; ++j) {
+        if (kSB == 3) {
+          if (j + 2 < n) ok = issue_s(j + 2);
+          if (ok) ok = issue_pv(j);
+        } else {
+          ok = issue_pv(j);
+          if (ok && j + 2 < n) ok = issue_s(j + 2);
+        }
       }
-      if (!ok) set_abort(sh, p.dev_status);
+      g += n;
     }
+    if (!ok && lane == 0) set_abort(sh, p.dev_status);
     __syncwarp();
   } else {
     // ------------------------------------------------------------ softmax warps
@@ -632,9 +679,12 @@ __global__ void __launch_bounds__(kThreadsTC, 1)
     bool ok = true;
     int g = 0;  // running tile count
     int idx = idx0;
-    TcWork w = tc_work(p, sh.order, n_mt, idx);
+    TcWork w = tc_plan(p, tc_fetch(p, sh.order, n_mt, idx));
     load_q(w);
+    const bool sector = ((uintptr_t)p.out & 31) == 0;  // rows start on 32-byte sectors
     for (int k = 0; idx >= 0; ++k) {
+      const int idx_ahead = item_of(k + 1);
+      const TcWork ahead = tc_fetch(p, sh.order, n_mt, idx_ahead);
       const int m = w.mtile * kRowsM + row;
       const int trow = m / p.G;
       // token-causal block row: the state-update pass, or an anchor / verify
@@ -740,10 +790,10 @@ __global__ void __launch_bounds__(kThreadsTC, 1)
       if (ok && aborted(sh)) ok = false;
       // the next item's Q can go into tensor memory now: every S product of
       // this item has completed
-      const int idx_next = ok ? item_of(k + 1) : -1;
+      const int idx_next = ok ? idx_ahead : -1;
       TcWork wn = w;
       if (idx_next >= 0) {
-        wn = tc_work(p, sh.order, n_mt, idx_next);
+        wn = tc_plan(p, ahead);
         load_q(wn);
       }
       // epilogue: O / l (or the split partial) and the log-sum-exp
@@ -765,23 +815,16 @@ __global__ void __launch_bounds__(kThreadsTC, 1)
         tc::tmem_ld_wait();
         if (!write) continue;
         if (!split_mode) {
-          uint32_t pkd[8];
-#pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            __nv_bfloat162 h2 = __floats2bfloat162_rn(__uint_as_float(o[2 * i]) * inv,
-                                                      __uint_as_float(o[2 * i + 1]) * inv);
-            pkd[i] = *reinterpret_cast<uint32_t*>(&h2);
-          }
-          uint4* dst = reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(p.out) + orow * D + c);
-          dst[0] = make_uint4(pkd[0], pkd[1], pkd[2], pkd[3]);
-          dst[1] = make_uint4(pkd[4], pkd[5], pkd[6], pkd[7]);
+          store_bf16x16(static_cast<__nv_bfloat16*>(p.out) + orow * D + c, o, inv, sector);
         } else {
-          float4* dst = reinterpret_cast<float4*>(p.ws_o + ws_row * D + c);
+          float* dst = p.ws_o + ws_row * D + c;
 #pragma unroll
-          for (int i = 0; i < 4; ++i)
-            dst[i] = make_float4(__uint_as_float(o[4 * i]) * inv, __uint_as_float(o[4 * i + 1]) * inv,
-                                 __uint_as_float(o[4 * i + 2]) * inv,
-                                 __uint_as_float(o[4 * i + 3]) * inv);
+          for (int i = 0; i < 2; ++i) {
+            uint32_t v[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) v[e] = __float_as_uint(__uint_as_float(o[8 * i + e]) * inv);
+            tc::store32(dst + 8 * i, v);
+          }
         }
       }
       if (write) {
@@ -876,15 +919,18 @@ cudaError_t launch_tc_d(const SoftmaxParams& p, const SoftmaxPlan& plan, cudaStr
   }
   {
     const int npages = p.num_pages > 0 ? p.num_pages : 1;
-    const uint64_t dims[4] = {(uint64_t)D, (uint64_t)p.page_size, (uint64_t)p.Hkv,
+    const uint64_t row = D * e, head = (uint64_t)p.page_size * row;
+    const uint64_t dims[5] = {64, (uint64_t)p.page_size, (uint64_t)D / 64, (uint64_t)p.Hkv,
                               (uint64_t)npages};
-    const uint64_t str[3] = {D * e, (uint64_t)p.page_size * D * e,
-                             (uint64_t)p.Hkv * p.page_size * D * e};
-    const uint32_t box[4] = {64, (uint32_t)(p.page_size < kTileN ? p.page_size : kTileN), 1, 1};
+    const uint64_t str[4] = {row, 128, head, (uint64_t)p.Hkv * head};
+    const bool whole = p.page_size >= kTileN;  // a tile lies in one page
+    const uint32_t box[5] = {64, whole ? (uint32_t)kTileN : (uint32_t)p.page_size,
+                             whole ? (uint32_t)C::kChunks : 1u, 1, 1};
     // an empty pool is never read (every prefix is empty); point the map at the block tensor
     const void* kp = p.num_pages > 0 ? p.k_pool : p.k_blk;
     const void* vp = p.num_pages > 0 ? p.v_pool : p.v_blk;
-    if (!encode_map(&maps.kpool, kp, 4, dims, str, box) || !encode_map(&maps.vpool, vp, 4, dims, str, box))
+    if (!encode_map(&maps.kpool, kp, 5, dims, str, box) ||
+        !encode_map(&maps.vpool, vp, 5, dims, str, box))
       return cudaErrorInvalidValue;
   }
   const int smem = C::kSmem + 1024;

@@ -63,3 +63,25 @@ def test_pair_matches_oracle(name, mode):
     err, _ = assert_out_close(out, ref, "bf16", name)
     assert err <= OUT_MAX_ABS
     assert np.abs(lse.double().cpu().numpy() - ref_lse).max() < LSE_ABS
+
+
+@pytest.mark.parametrize("base,block", [(LARGE, 32), (SMALL, 16)])
+def test_outputs_off_a_32_byte_sector(base, block):
+    """An output array that starts on a 16-byte boundary only is stored in 16-byte
+    pieces instead of whole sectors: the same bits."""
+    from gpu_helpers import softmax_desc
+    from paper_2606_01774_gb300 import flare
+
+    w = gen(base.replace(num_requests=160, block_len=block, prefix_lo=1, prefix_hi=200, seed=93))
+    aligned, _ = run_softmax(w)
+    sb, desc = w.softmax[0], softmax_desc(w.spec, w)
+    n = sb.q.numel()
+    out = torch.zeros(n + 16, dtype=sb.q.dtype, device="cuda")[8:8 + n].view_as(sb.q)
+    assert aligned.data_ptr() % 32 == 0 and out.data_ptr() % 32 == 16
+    nb = flare.flare_softmax_workspace_size(desc)
+    ws = torch.empty(max(nb, 1), dtype=torch.uint8, device="cuda")
+    st = torch.zeros(1, dtype=torch.int32, device="cuda")
+    flare.check(flare.flare_block_softmax_attn(desc, sb.q, sb.k_blk, sb.v_blk, w.k_pool, w.v_pool,
+                                               w.page_table, w.prefix_len, out, None, ws, nb, st))
+    assert flare.flare_read_status(st) == (flare.FLARE_OK, 0)
+    assert torch.equal(out.view(torch.int16), aligned.view(torch.int16))
