@@ -31,6 +31,11 @@
 // first K-1 verify tokens are streamed out as S^(0..K-1), the state after
 // token K is written to the pool, and the draft rows read the block-end state
 // once the loop is done.
+//
+// And it is the denoise pass of fp32 activations: every token is stepped, no state
+// is written, and all rows read the block-end state.  That pass had a kernel with
+// the state in shared memory and four CTA barriers per token; its latency for one
+// request (2 heads, d = 64, B = 8) was 18 us, here 4 us.
 #include "common.cuh"
 #include "kernels.h"
 
@@ -79,11 +84,13 @@ __device__ __forceinline__ void stage_rows(float* dst, const T* src, size_t stri
 
 }  // namespace
 
-// MODE 0: commit; 1: commit with token-causal outputs; 2: AR-Trust verify round.
+// MODE 0: commit; 1: commit with token-causal outputs; 2: AR-Trust verify round;
+// 3: denoise pass (block-end readout, the pool is only read).
 template <typename T, int DK, int DV, int MODE>
 __global__ void __launch_bounds__(2 * DV, 2) gdr_commit_kernel(GdrParams p) {
   constexpr bool CAUSAL = MODE != 0;  // queries staged, readouts written
   constexpr bool VERIFY = MODE == 2;
+  constexpr bool DENOISE = MODE == 3;
   constexpr int kThreads = 2 * DV;   // DV / 16 warps
   constexpr int kR = DK / 8;         // state rows per thread
   extern __shared__ float smc[];
@@ -104,7 +111,9 @@ __global__ void __launch_bounds__(2 * DV, 2) gdr_commit_kernel(GdrParams p) {
     return;
   }
   int n, K = 0;
-  if constexpr (VERIFY) {
+  if constexpr (DENOISE) {
+    n = K = -1;  // no state written, every row read after the loop
+  } else if constexpr (VERIFY) {
     K = p.verify_len[r];
     if (K < 0 || K > p.max_verify || K > B - 1) {
       if (threadIdx.x == 0) flag(p.dev_status, FLARE_DEV_BAD_VERIFY_LEN);
@@ -167,7 +176,13 @@ __global__ void __launch_bounds__(2 * DV, 2) gdr_commit_kernel(GdrParams p) {
     constexpr float kMinLog = -27.725887222397812f;  // ln 2^-40
     const bool fold = __any_sync(0xffffffffu, (lane < steps && g0 < kMinLog) ||
                                                   (lane + 32 < steps && g1 < kMinLog));
-    if (!fold) {
+    if constexpr (DENOISE) {
+      // the decay folded in at every token, S <- alpha_t S + k_t delta_t: the lazy form's
+      // Gam_t = exp(gamma_t) carries the rounding of a sum as large as 27 (outputs of
+      // B = 32 were 4.7e-7 off, 8e-8 in this form)
+      tok_s[lane] = make_float4(a0, b0, 0.f, 1.f);
+      tok_s[lane + 32] = make_float4(a1, b1, 0.f, 1.f);
+    } else if (!fold) {
       const float e0 = expf(g0), e1 = expf(g1);
       tok_s[lane] = make_float4(e0, b0, expf(-g0), e0);
       tok_s[lane + 32] = make_float4(e1, b1, expf(-g1), e1);
@@ -218,7 +233,8 @@ __global__ void __launch_bounds__(2 * DV, 2) gdr_commit_kernel(GdrParams p) {
       o.w += __shfl_xor_sync(0xffffffffu, o.w, sh);
     }
     if (rg == 0) {
-      T* out = static_cast<T*>(p.out_causal) + (((size_t)r * B + t) * p.Hv + j) * DV + c0;
+      T* out = static_cast<T*>(DENOISE ? p.out_blockend : p.out_causal) +
+               (((size_t)r * B + t) * p.Hv + j) * DV + c0;
       const float sc = p.scale * g;
       out[0] = from_f32<T>(sc * o.x);
       out[1] = from_f32<T>(sc * o.y);
@@ -311,10 +327,10 @@ __global__ void __launch_bounds__(2 * DV, 2) gdr_commit_kernel(GdrParams p) {
         *reinterpret_cast<ulonglong2*>(Sg + (size_t)m * DV) =
             make_ulonglong2(f2_mul(g2, s[m][0]), f2_mul(g2, s[m][1]));
     }
-    if (CAUSAL && (!VERIFY || t <= K)) readout(t, gam);
+    if (CAUSAL && (MODE == 1 || t <= K)) readout(t, gam);
   }
-  if constexpr (VERIFY) {
-    // padding and draft rows read the block-end state
+  if constexpr (VERIFY || DENOISE) {
+    // padding and draft rows (denoise pass: all rows) read the block-end state
 #pragma unroll 1
     for (int t = K + 1; t < B; ++t) readout(t, gam);
   }
@@ -354,6 +370,11 @@ cudaError_t launch_gdr_commit(const GdrParams& p, bool bf16, cudaStream_t stream
     return causal ? launch_commit_c<__nv_bfloat16, 1>(p, stream)
                   : launch_commit_c<__nv_bfloat16, 0>(p, stream);
   return causal ? launch_commit_c<float, 1>(p, stream) : launch_commit_c<float, 0>(p, stream);
+}
+
+cudaError_t launch_gdr_denoise_f32(const GdrParams& p, cudaStream_t stream) {
+  if (p.R == 0) return cudaSuccess;
+  return launch_commit_c<float, 3>(p, stream);
 }
 
 cudaError_t launch_gdr_verify(const GdrParams& p, bool bf16, cudaStream_t stream) {

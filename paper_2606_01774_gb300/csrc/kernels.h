@@ -71,7 +71,6 @@ struct SoftmaxPlan {
   size_t workspace_bytes;
 };
 
-size_t gdr_recurrent_smem_bytes(int dk, int dv, int threads);
 bool gdr_denoise_tc_supported(int B, int dk, int dv);
 bool gdr_denoise_persist_supported(int B, int dk, int dv);
 cudaError_t launch_gdr_denoise_persist(const GdrParams& p, cudaStream_t stream);
@@ -129,7 +128,7 @@ cudaError_t launch_two_stream_fwd(const TwoStreamParams& p, bool bf16, cudaStrea
 bool two_stream_chunk_supported(int B, int dk, int dv);
 cudaError_t launch_two_stream_chunk(const TwoStreamParams& p, cudaStream_t stream);
 cudaError_t launch_gdr_denoise_tc(const GdrParams& p, cudaStream_t stream);
-cudaError_t launch_gdr_recurrent(const GdrParams& p, bool bf16, cudaStream_t stream);
+cudaError_t launch_gdr_denoise_f32(const GdrParams& p, cudaStream_t stream);
 
 SoftmaxPlan plan_softmax(int R, int B, int Hq, int Hkv, int D, int page_size, int max_pages,
                          bool bf16, int num_sms);
