@@ -19,29 +19,65 @@ constexpr int kRows = 16;     // query rows per CTA (4 per warp)
 constexpr int kTile = 32;     // keys per smem tile (one per lane)
 constexpr int kThreads = 128;
 
+// 16 bytes of a row as fp32
 template <typename T>
-__device__ __forceinline__ const T* key_row(const SoftmaxParams& p, const T* pool, const T* blk,
-                                            int r, int kvh, int P, int idx) {
-  if (idx < P) {
-    const int page = p.page_table[(size_t)r * p.max_pages + idx / p.page_size];
-    return pool + (((size_t)page * p.Hkv + kvh) * p.page_size + idx % p.page_size) * p.D;
+__device__ __forceinline__ void widen(const uint4& v, float* f) {
+  if constexpr (sizeof(T) == 2) {
+    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      f[2 * e] = __uint_as_float(w[e] << 16);
+      f[2 * e + 1] = __uint_as_float(w[e] & 0xffff0000u);
+    }
+  } else {
+    f[0] = __uint_as_float(v.x), f[1] = __uint_as_float(v.y);
+    f[2] = __uint_as_float(v.z), f[3] = __uint_as_float(v.w);
   }
-  return blk + (((size_t)r * p.B + (idx - P)) * p.Hkv + kvh) * p.D;
 }
 }  // namespace
 
+// Latency-bound (a few CTAs of one request): the tile's key rows are located
+// once per row, all of a tile's 16-byte loads are in flight together and a tile
+// ahead of its use, and each key and value read from shared memory serves the
+// warp's four rows.  (Element by element, with the page looked up for each,
+// one request of 2 heads, D = 64, 40 keys took 22 us.)
 template <typename T, int D>
 __global__ void __launch_bounds__(kThreads) softmax_simt_kernel(SoftmaxParams p) {
-  extern __shared__ float sm[];
+  constexpr int kVec = 16 / sizeof(T);         // elements of a 16-byte load
+  constexpr int kLoads = kTile * (D / kVec) / kThreads;  // per thread and array
+  constexpr int kKs = D + 4;                   // key row stride: 16-byte reads of 8 rows tile the banks
+  extern __shared__ __align__(16) float sm[];
   float* Qs = sm;                     // [kRows][D]
-  float* Ks = Qs + kRows * D;         // [kTile][D+1]
-  float* Vs = Ks + kTile * (D + 1);   // [kTile][D]
+  float* Ks = Qs + kRows * D;         // [kTile][kKs]
+  float* Vs = Ks + kTile * kKs;       // [kTile][D]
+  __shared__ long long off_s[2][kTile];  // element offset of a key row: >= 0 in the pools,
+                                         // -1 - offset in the block, kNone past the split
+  constexpr long long kNone = -(1ll << 62);
 
   const int split = blockIdx.x, item = blockIdx.y, mt = blockIdx.z;
   const int r = item / p.Hkv, kvh = item % p.Hkv;
   const int M = p.B * p.G;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int P = p.prefix_len[r];
+
+  const T* q = static_cast<const T*>(p.q);
+  const T* kpool = static_cast<const T*>(p.k_pool);
+  const T* vpool = static_cast<const T*>(p.v_pool);
+  const T* kblk = static_cast<const T*>(p.k_blk);
+  const T* vblk = static_cast<const T*>(p.v_blk);
+
+  for (int e = tid * kVec; e < kRows * D; e += kThreads * kVec) {
+    const int i = e / D, d = e % D, m = mt * kRows + i;
+    uint4 x = make_uint4(0u, 0u, 0u, 0u);
+    if (m < M) {
+      const int t = m / p.G, g = m % p.G;
+      x = *reinterpret_cast<const uint4*>(q + (((size_t)r * p.B + t) * p.Hq + kvh * p.G + g) * D + d);
+    }
+    float f[kVec];
+    widen<T>(x, f);
+#pragma unroll
+    for (int v = 0; v < kVec; ++v) Qs[e + v] = f[v] * p.scale_log2;
+  }
   const int bad = check_request_pages(p.page_table, P, r, p.max_pages, p.page_size, p.num_pages);
   if (bad) {
     if (tid == 0) flag(p.dev_status, bad);
@@ -51,21 +87,36 @@ __global__ void __launch_bounds__(kThreads) softmax_simt_kernel(SoftmaxParams p)
   const int kv_lo = split * p.split_len;
   const int kv_hi = min(total, kv_lo + p.split_len);
 
-  const T* q = static_cast<const T*>(p.q);
-  const T* kpool = static_cast<const T*>(p.k_pool);
-  const T* vpool = static_cast<const T*>(p.v_pool);
-  const T* kblk = static_cast<const T*>(p.k_blk);
-  const T* vblk = static_cast<const T*>(p.v_blk);
-
-  for (int e = tid; e < kRows * D; e += kThreads) {
-    const int i = e / D, d = e % D, m = mt * kRows + i;
-    float x = 0.f;
-    if (m < M) {
-      const int t = m / p.G, g = m % p.G;
-      x = to_f32(q[(((size_t)r * p.B + t) * p.Hq + kvh * p.G + g) * D + d]) * p.scale_log2;
+  // the rows of tile `lo` into off_s[b] (the first warp)
+  auto locate = [&](int lo, int b) {
+    if (warp != 0) return;
+    const int idx = lo + lane;
+    long long off = kNone;
+    if (idx < min(P, kv_hi)) {
+      const int page = p.page_table[(size_t)r * p.max_pages + idx / p.page_size];
+      off = (((long long)page * p.Hkv + kvh) * p.page_size + idx % p.page_size) * D;
+    } else if (idx < kv_hi) {
+      off = -1 - (((long long)r * p.B + (idx - P)) * p.Hkv + kvh) * D;
     }
-    Qs[e] = x;
-  }
+    off_s[b][lane] = off;
+  };
+  uint4 kr[kLoads], vr[kLoads];  // the tile ahead
+  auto load = [&](int b) {
+#pragma unroll
+    for (int u = 0; u < kLoads; ++u) {
+      const int e = tid + u * kThreads;
+      const int jj = e / (D / kVec), d = (e % (D / kVec)) * kVec;
+      const long long off = off_s[b][jj];
+      kr[u] = vr[u] = make_uint4(0u, 0u, 0u, 0u);
+      if (off >= 0) {
+        kr[u] = *reinterpret_cast<const uint4*>(kpool + off + d);
+        vr[u] = *reinterpret_cast<const uint4*>(vpool + off + d);
+      } else if (off != kNone) {
+        kr[u] = *reinterpret_cast<const uint4*>(kblk - 1 - off + d);
+        vr[u] = *reinterpret_cast<const uint4*>(vblk - 1 - off + d);
+      }
+    }
+  };
 
   constexpr int NC = D / 32;
   float acc[4][NC];
@@ -78,51 +129,74 @@ __global__ void __launch_bounds__(kThreads) softmax_simt_kernel(SoftmaxParams p)
     for (int x = 0; x < NC; ++x) acc[w][x] = 0.f;
   }
 
-  for (int lo = kv_lo; lo < kv_hi; lo += kTile) {
-    __syncthreads();
-    for (int e = tid; e < kTile * D; e += kThreads) {
-      const int jj = e / D, d = e % D, idx = lo + jj;
-      float kx = 0.f, vx = 0.f;
-      if (idx < kv_hi) {
-        kx = to_f32(key_row<T>(p, kpool, kblk, r, kvh, P, idx)[d]);
-        vx = to_f32(key_row<T>(p, vpool, vblk, r, kvh, P, idx)[d]);
-      }
-      Ks[jj * (D + 1) + d] = kx;
-      Vs[jj * D + d] = vx;
+  locate(kv_lo, 0);
+  __syncthreads();
+  load(0);
+  locate(kv_lo + kTile, 1);
+  int b = 1;
+  for (int lo = kv_lo; lo < kv_hi; lo += kTile, b ^= 1) {
+    __syncthreads();  // the previous tile read; off_s[b] written
+#pragma unroll
+    for (int u = 0; u < kLoads; ++u) {
+      const int e = tid + u * kThreads;
+      const int jj = e / (D / kVec), d = (e % (D / kVec)) * kVec;
+      widen<T>(kr[u], Ks + jj * kKs + d);
+      widen<T>(vr[u], Vs + jj * D + d);
     }
     __syncthreads();
+    if (lo + kTile < kv_hi) {
+      load(b);
+      locate(lo + 2 * kTile, b ^ 1);
+    }
+    // scores: lane = key, the warp's four rows
+    float s[4] = {0.f, 0.f, 0.f, 0.f};
+    const float4* k4 = reinterpret_cast<const float4*>(Ks + lane * kKs);
+    const float4* q4 = reinterpret_cast<const float4*>(Qs + warp * 4 * D);
+#pragma unroll 8
+    for (int d = 0; d < D / 4; ++d) {
+      const float4 k = k4[d];
+#pragma unroll
+      for (int w = 0; w < 4; ++w) {
+        const float4 x = q4[w * (D / 4) + d];
+        s[w] = fmaf(x.x, k.x, s[w]);
+        s[w] = fmaf(x.y, k.y, s[w]);
+        s[w] = fmaf(x.z, k.z, s[w]);
+        s[w] = fmaf(x.w, k.w, s[w]);
+      }
+    }
     const int idx = lo + lane;
+    float pj[4];
 #pragma unroll
     for (int w = 0; w < 4; ++w) {
-      const int i = warp * 4 + w, m = mt * kRows + i;
+      const int m = mt * kRows + warp * 4 + w;
+      pj[w] = 0.f;
       if (m >= M) continue;  // warp-uniform
       const int trow = m / p.G;
       const bool causal_row =
           p.row_type ? p.row_type[(size_t)r * p.row_type_stride + trow] == 0 : p.causal != 0;
       const bool vis = idx < kv_hi && (!causal_row || idx < P || idx - P <= trow);
-      float s = -INFINITY;
-      if (vis) {
-        float a = 0.f;
-#pragma unroll 8
-        for (int d = 0; d < D; ++d) a = fmaf(Qs[i * D + d], Ks[lane * (D + 1) + d], a);
-        s = a;
-      }
-      const float mx = warp_max(s);
-      const float mnew = fmaxf(mrow[w], mx);
+      const float mnew = fmaxf(mrow[w], warp_max(vis ? s[w] : -INFINITY));
       if (mnew == -INFINITY) continue;  // nothing visible yet for this row
-      const float pj = vis ? exp2f(s - mnew) : 0.f;
+      pj[w] = vis ? exp2f(s[w] - mnew) : 0.f;
       const float corr = exp2f(mrow[w] - mnew);
-      lrow[w] = lrow[w] * corr + warp_sum(pj);
+      lrow[w] = lrow[w] * corr + warp_sum(pj[w]);
 #pragma unroll
       for (int x = 0; x < NC; ++x) acc[w][x] *= corr;
-      for (int jj = 0; jj < kTile; ++jj) {
-        const float pb = __shfl_sync(0xffffffffu, pj, jj);
-        if (pb != 0.f) {
+      mrow[w] = mnew;
+    }
+#pragma unroll 4
+    for (int jj = 0; jj < kTile; ++jj) {
+      float v[NC];
 #pragma unroll
-          for (int x = 0; x < NC; ++x) acc[w][x] = fmaf(pb, Vs[jj * D + lane + 32 * x], acc[w][x]);
+      for (int x = 0; x < NC; ++x) v[x] = Vs[jj * D + lane + 32 * x];
+#pragma unroll
+      for (int w = 0; w < 4; ++w) {
+        const float pb = __shfl_sync(0xffffffffu, pj[w], jj);
+        if (pb != 0.f) {  // a hidden value row may hold anything
+#pragma unroll
+          for (int x = 0; x < NC; ++x) acc[w][x] = fmaf(pb, v[x], acc[w][x]);
         }
       }
-      mrow[w] = mnew;
     }
   }
 
@@ -204,7 +278,7 @@ __global__ void gather_prefix_kernel(SoftmaxParams p, int r, T* k_out, T* v_out)
 namespace {
 template <typename T, int D>
 cudaError_t launch_simt_d(const SoftmaxParams& p, const SoftmaxPlan& plan, cudaStream_t stream) {
-  const size_t smem = sizeof(float) * ((size_t)kRows * D + (size_t)kTile * (D + 1) + kTile * D);
+  const size_t smem = sizeof(float) * ((size_t)kRows * D + (size_t)kTile * (D + 4) + kTile * D);
   cudaError_t e = cudaFuncSetAttribute(softmax_simt_kernel<T, D>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
