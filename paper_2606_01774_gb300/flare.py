@@ -131,17 +131,26 @@ def declared_functions():
 
 
 def _p(t):
-    if t is None:
-        return None
-    return ctypes.c_void_p(t.data_ptr())
+    """Data pointer of a tensor (or None): an int, which the c_void_p argument types take."""
+    return None if t is None else t.data_ptr()
+
+
+_raw_stream = None
 
 
 def _stream(stream):
-    if stream is None:
+    """cudaStream_t of `stream`; None is torch's current stream of the
+    current device (read without building a Stream object: 2.8 us of a 9.5 us call)."""
+    if stream is not None:
+        return ctypes.c_void_p(getattr(stream, "cuda_stream", stream))
+    global _raw_stream
+    if _raw_stream is None:
         import torch
 
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(getattr(stream, "cuda_stream", stream))
+        torch.cuda.init()
+        _raw_stream = (torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice)
+    raw, device = _raw_stream
+    return raw(device())
 
 
 def flare_launch_count() -> int:
