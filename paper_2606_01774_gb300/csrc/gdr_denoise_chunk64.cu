@@ -11,7 +11,8 @@
 //   X       = diag(beta) (V - diag(Gam) K S0),   delta = (I + A)^{-1} X
 //   out[l]  = s (Gam_{B-1} S0^T q_l + sum_i exp(gamma_{B-1} - gamma_i) (q_l . k_i) delta_i)
 //
-// Value column c on tensor-memory lane c; thread c owns column c.  Per item:
+// Value column c on tensor-memory lane c; threads c and c + 128 (two warp
+// groups) own column c, each half of its rows or tokens.  Per item:
 //   MMA 1  G   = [K; Q] K^T       M=128 (K rows on lanes 0..63, Q rows on 64..127), N=64, K=128
 //          W^T = S0^T [K; Q]^T    M=128 (c), N=128, K=128   (A: S0^T bf16, tensor memory)
 //   T      = (I + A)^{-1}          fp32, 16 x 16 blocks: the diagonal ones by forward
@@ -25,8 +26,11 @@
 // vanish there and T is the identity.
 //
 // Persistent CTAs, two per SM (113 KiB of shared memory, 256 tensor-memory
-// columns and 128 threads each), so that each SM holds two items' latency
-// chains.  The state arrives in two 32 KiB halves into two buffers: the first
+// columns and 256 threads each), so that each SM holds two items' latency
+// chains.  Two groups instead of one, the products issued by an elected lane of
+// a converged warp, and waits that read no timer before their first retry took
+// multistep_batch128's call from 154 to 141 us (floor 70 us, HBM; 128 registers a
+// thread).  The state arrives in two 32 KiB halves into two buffers: the first
 // half's buffer takes the next item's first half as soon as it has been read,
 // a whole item ahead; the second half's buffer then holds A^T and T, and takes
 // the next item's second half once T is formed.  The key/query buffer holds
@@ -48,7 +52,7 @@ namespace flare {
 
 namespace {
 
-constexpr int kD6Threads = 128;
+constexpr int kD6Threads = 256;
 constexpr int kD6D = 128;  // d_k = d_v
 using namespace chunk64;   // kCkC = 64 and the chunk-system helpers
 
@@ -108,7 +112,7 @@ __device__ __forceinline__ int d6_next(const GdrParams& p, int it, int total, in
 __global__ void __launch_bounds__(kD6Threads, 2)
     gdr_denoise_chunk64_kernel(const __grid_constant__ D6Maps maps, GdrParams p) {
   using C = D6Cfg;
-  constexpr int kIssuer = 32;  // one thread of warp 1 issues every copy and MMA
+  constexpr int kIssuer = 32;  // warp 1 issues every copy and MMA
   // no static shared memory, so that the dynamic window starts 1024-byte
   // aligned (the 128-byte swizzled operands need it): checked below
   extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -124,6 +128,7 @@ __global__ void __launch_bounds__(kD6Threads, 2)
   uint8_t* Vs = base + C::oV;
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int col = tid & 127, grp = tid >> 7;
   const int total = p.R * p.Hv;
   const int B = p.B;
 
@@ -153,7 +158,7 @@ __global__ void __launch_bounds__(kD6Threads, 2)
   const uint32_t tmS = tmem;        // S0^T bf16 (64 columns); X^T high | low; delta^T (32)
   const uint32_t tmW = tmem + 64;   // W^T: [K | Q] parts, 2 x 64 columns; delta^T fp32 over K
   const uint32_t tmG = tmem + 192;  // G (rows on lanes), 64 columns; then O2^T
-  const uint32_t lane_off = (uint32_t)(warp * 32) << 16;
+  const uint32_t lane_off = (uint32_t)((warp & 3) * 32) << 16;
 
   auto issue_s0 = [&](int item, int s, int h) {  // rows 64 h .. 64 h + 63 of the state
     const float* src = p.state_pool + ((size_t)s * p.Hv + item % p.Hv) * kD6D * kD6D +
@@ -255,19 +260,17 @@ __global__ void __launch_bounds__(kD6Threads, 2)
       cs = cand_slot(cand);
     }
 
-    // S0^T into tensor memory as bf16 pairs, the state's two halves from
-    // their two buffers
-#pragma unroll 1
-    for (int h = 0; h < 2; ++h) {
-      bad |= !tc::mbar_wait(h ? &sh.bar_s0b : &sh.bar_s0a, ph, &sh.abort_flag);
-      const float* S0h = h ? S0b : S0a;
+    // S0^T into tensor memory as bf16 pairs, a half of the state per group
+    {
+      bad |= !tc::mbar_wait(grp ? &sh.bar_s0b : &sh.bar_s0a, ph, &sh.abort_flag);
+      const float* S0h = grp ? S0b : S0a;
 #pragma unroll 1
       for (int i0 = 0; i0 < 64; i0 += 32) {
         uint32_t w[16];
 #pragma unroll
         for (int e = 0; e < 16; ++e)
-          w[e] = ck_pack(S0h[(i0 + 2 * e) * kD6D + tid], S0h[(i0 + 2 * e + 1) * kD6D + tid]);
-        tc::tmem_st16(tmS + lane_off + (64 * h + i0) / 2, w);
+          w[e] = ck_pack(S0h[(i0 + 2 * e) * kD6D + col], S0h[(i0 + 2 * e + 1) * kD6D + col]);
+        tc::tmem_st16(tmS + lane_off + (64 * grp + i0) / 2, w);
       }
     }
     if (tid == kIssuer) s0a_out = s0b_out = false;
@@ -279,83 +282,80 @@ __global__ void __launch_bounds__(kD6Threads, 2)
       s0a_out = true;
       s0a_par = ph ^ 1u;
     }
-    if (tid == kIssuer) {
+    if (warp == kIssuer / 32) {  // converged; one elected lane issues
       bad |= !tc::mbar_wait(&sh.bar_kq, ph, &sh.abort_flag);
       kq_out = false;
-      tc::fence_after_sync();
-      // the Gram first, committed on its own: the tables are built from it
-      // while the state products run
-#pragma unroll
-      for (int kk = 0; kk < kD6D / 16; ++kk) {
-        const uint64_t kd = tc::sdesc_sw128(
-            tc::smem_u32(KQ + (kk >> 2) * (128 * 128) + (kk & 3) * 32), 16, 1024);
-        tc::mma_bf16_ss(tmG, kd, kd, idG, kk > 0);  // G = [K; Q] K^T
-      }
-      tc::mma_commit(&sh.bar_g);
-#pragma unroll
-      for (int kk = 0; kk < kD6D / 16; ++kk) {
-        const uint64_t kd = tc::sdesc_sw128(
-            tc::smem_u32(KQ + (kk >> 2) * (128 * 128) + (kk & 3) * 32), 16, 1024);
-        tc::mma_bf16_ts(tmW, tmS + kk * 8, kd, idW, kk > 0);  // W^T = S0^T [K; Q]^T
-      }
-      tc::mma_commit(&sh.bar_mma);
       mma_out = true;
+      __syncwarp();
+      tc::fence_after_sync();
+      if (tc::elect_one()) {
+        // the Gram first, committed on its own: the tables are built from it
+        // while the state products run
+#pragma unroll
+        for (int kk = 0; kk < kD6D / 16; ++kk) {
+          const uint64_t kd = tc::sdesc_sw128(
+              tc::smem_u32(KQ + (kk >> 2) * (128 * 128) + (kk & 3) * 32), 16, 1024);
+          tc::mma_bf16_ss(tmG, kd, kd, idG, kk > 0);  // G = [K; Q] K^T
+        }
+        tc::mma_commit(&sh.bar_g);
+#pragma unroll
+        for (int kk = 0; kk < kD6D / 16; ++kk) {
+          const uint64_t kd = tc::sdesc_sw128(
+              tc::smem_u32(KQ + (kk >> 2) * (128 * 128) + (kk & 3) * 32), 16, 1024);
+          tc::mma_bf16_ts(tmW, tmS + kk * 8, kd, idW, kk > 0);  // W^T = S0^T [K; Q]^T
+        }
+        tc::mma_commit(&sh.bar_mma);
+      }
+      __syncwarp();
     }
     bad |= !tc::mbar_wait(&sh.bar_g, ph, &sh.abort_flag);
     tc::fence_after_sync();
 
-    // ---- tables from G (every exponential taken unconditionally, the masks
-    // applied as selects): warps 0-1 A^T (key rows), warps 2-3 M2 (query rows,
-    // stored over [K; Q] once the state products have read it) and then T's
-    // diagonal blocks
+    // ---- tables from G, 32 columns per group (every exponential taken
+    // unconditionally, the masks applied as selects): warps 0-1 and 4-5 A^T (key
+    // rows), warps 2-3 and 6-7 M2 (query rows, stored over [K; Q] once the state
+    // products have read it); then T's diagonal blocks on warps 6-7
     {
-      const int row = tid & 63;
-      if (tid < 64) {
+      const int row = tid & 63, c0 = 32 * grp;
+      uint32_t gr[32];
+      ck_ld32(tmG + lane_off + c0, gr);
+      if (col < 64) {
         const float gi = sh.gc2[row];
-#pragma unroll 1
-        for (int h = 0; h < 2; ++h) {
-          uint32_t gr[32];
-          float v[32];
-          ck_ld32(tmG + lane_off + 32 * h, gr);
+        float v[32];
 #pragma unroll
-          for (int k = 0; k < 32; ++k) {
-            const int t = 32 * h + k;
-            const float a = sh.bc[t] * tc::ex2(sh.gc2[t] - gi) * __uint_as_float(gr[k]);
-            v[k] = t > row ? a : 0.f;
-          }
-          ck_store32(AT, row, 32 * h, v);
+        for (int k = 0; k < 32; ++k) {
+          const int t = c0 + k;
+          const float a = sh.bc[t] * tc::ex2(sh.gc2[t] - gi) * __uint_as_float(gr[k]);
+          v[k] = t > row ? a : 0.f;
         }
-        tc::named_bar_arrive(5, 128);  // A^T to warps 2-3
+        ck_store32(AT, row, c0, v);
+        tc::named_bar_arrive(5, 192);  // A^T to warps 6-7
       } else {
         const bool live = row < B;
         const float gB = sh.gc2[B - 1];
-        uint32_t wv[32];  // the row's 64 values as bf16 pairs
+        uint32_t wv[16];  // the row's 32 values as bf16 pairs
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          uint32_t gr[32];
-          ck_ld32(tmG + lane_off + 32 * h, gr);
-#pragma unroll
-          for (int e = 0; e < 16; ++e) {
-            // the row factor exp(gamma_{B-1} - gamma_i), zero for i >= B
-            const int i = 32 * h + 2 * e;
-            const float m0 = tc::ex2(gB - sh.gc2[i]) * __uint_as_float(gr[2 * e]);
-            const float m1 = tc::ex2(gB - sh.gc2[i + 1]) * __uint_as_float(gr[2 * e + 1]);
-            wv[16 * h + e] =
-                ck_pack(live && i < B ? m0 : 0.f, live && i + 1 < B ? m1 : 0.f);
-          }
+        for (int e = 0; e < 16; ++e) {
+          // the row factor exp(gamma_{B-1} - gamma_i), zero for i >= B
+          const int i = c0 + 2 * e;
+          const float m0 = tc::ex2(gB - sh.gc2[i]) * __uint_as_float(gr[2 * e]);
+          const float m1 = tc::ex2(gB - sh.gc2[i + 1]) * __uint_as_float(gr[2 * e + 1]);
+          wv[e] = ck_pack(live && i < B ? m0 : 0.f, live && i + 1 < B ? m1 : 0.f);
+        }
+        if (grp == 1) {
+          tc::named_bar_sync(5, 192);
+          ck_diag_inverse(AT, Tf, 2 * (warp - 6) + (lane >> 4), lane & 15);
         }
         bad |= !tc::mbar_wait(&sh.bar_mma, ph_mma, &sh.abort_flag);  // [K; Q] read
 #pragma unroll
-        for (int u = 0; u < 8; ++u)
-          *reinterpret_cast<uint4*>(M2s + row * 128 + ((u ^ (row & 7)) << 4)) =
+        for (int u = 0; u < 4; ++u)
+          *reinterpret_cast<uint4*>(M2s + row * 128 + (((4 * grp + u) ^ (row & 7)) << 4)) =
               make_uint4(wv[4 * u], wv[4 * u + 1], wv[4 * u + 2], wv[4 * u + 3]);
         tc::fence_async_smem();  // M2 is the second MMA's operand
-        tc::named_bar_sync(5, 128);
-        ck_diag_inverse(AT, Tf, 2 * (warp - 2) + (lane >> 4), lane & 15);
       }
     }
 
-    // ---- X = diag(beta) (V - diag(Gam) K S0), all 64 tokens, into tensor
+    // ---- X = diag(beta) (V - diag(Gam) K S0), 32 tokens per group, into tensor
     // memory as bf16 high and low parts over S0^T (which the first MMAs have read)
     bad |= !tc::mbar_wait(&sh.bar_mma, ph_mma, &sh.abort_flag);
     ph_mma ^= 1u;
@@ -364,27 +364,24 @@ __global__ void __launch_bounds__(kD6Threads, 2)
     bad |= !tc::mbar_wait(&sh.bar_v, ph, &sh.abort_flag);
     if (tid == kIssuer) v_out = false;
     {
-      const uint8_t* vb = Vs + (tid >> 6) * (kCkC * 128) + (tid & 63) * 2;
-#pragma unroll 1
-      for (int h = 0; h < 2; ++h) {
-        const int t0 = 32 * h;
-        uint32_t w[32], hi[16], lo[16];
-        ck_ld32(tmW + lane_off + t0, w);
+      const uint8_t* vb = Vs + (col >> 6) * (kCkC * 128) + (col & 63) * 2;
+      const int t0 = 32 * grp;
+      uint32_t w[32], hi[16], lo[16];
+      ck_ld32(tmW + lane_off + t0, w);
 #pragma unroll
-        for (int e = 0; e < 16; ++e) {
-          float xv[2];
+      for (int e = 0; e < 16; ++e) {
+        float xv[2];
 #pragma unroll
-          for (int f = 0; f < 2; ++f) {
-            const int u = 2 * e + f, t = t0 + u;
-            const float vt = __uint_as_float(
-                (uint32_t)*reinterpret_cast<const unsigned short*>(vb + t * 128) << 16);
-            xv[f] = sh.bc[t] * (vt - sh.Gc[t] * __uint_as_float(w[u]));
-          }
-          ck_split(xv[0], xv[1], hi[e], lo[e]);
+        for (int f = 0; f < 2; ++f) {
+          const int u = 2 * e + f, t = t0 + u;
+          const float vt = __uint_as_float(
+              (uint32_t)*reinterpret_cast<const unsigned short*>(vb + t * 128) << 16);
+          xv[f] = sh.bc[t] * (vt - sh.Gc[t] * __uint_as_float(w[u]));
         }
-        tc::tmem_st16(tmS + lane_off + 16 * h, hi);
-        tc::tmem_st16(tmS + lane_off + 32 + 16 * h, lo);
+        ck_split(xv[0], xv[1], hi[e], lo[e]);
       }
+      tc::tmem_st16(tmS + lane_off + 16 * grp, hi);
+      tc::tmem_st16(tmS + lane_off + 32 + 16 * grp, lo);
       tc::tmem_st_wait();
     }
     tc::fence_before_sync();
@@ -396,54 +393,59 @@ __global__ void __launch_bounds__(kD6Threads, 2)
     }
 
     // ---- T = (I + A)^{-1} below its diagonal blocks: block column 0 on
-    // warps 0-1, 1 on warp 2, 2 (and the strip of 3) on warp 3
-    if (warp < 2)
-      ck_tcol<64>(AT, Tf, Tb, 0, 1, tid, 1);
+    // warps 0-3, 1 on warps 4-5, 2 (and the strip of 3) on warps 6-7
+    if (warp < 4)
+      ck_tcol<128>(AT, Tf, Tb, 0, 1, tid, 1);
     else
-      ck_tcol<32>(AT, Tf, Tb, warp - 1, warp == 2 ? 1 : 2, lane, warp);
+      ck_tcol<64>(AT, Tf, Tb, 1 + ((warp - 4) >> 1), warp < 6 ? 1 : 2, tid & 63, warp < 6 ? 2 : 3);
     if (__syncthreads_or(bad)) break;  // T as bf16 high / low parts; A^T and T read
-    if (tid == kIssuer) {
+    if (warp == kIssuer / 32) {
       if (it_next >= 0) {  // A^T and T read: the next item's second half
-        issue_s0(it_next, slot_next, 1);
         s0b_out = true;
         s0b_par = ph ^ 1u;
       }
-      const uint32_t tb = tc::smem_u32(Tb);
-#pragma unroll
-      for (int kk = 0; kk < kCkC / 16; ++kk) {
-        const uint64_t bh = tc::sdesc_sw128(tb + kk * 32, 16, 1024);
-        const uint64_t bl = tc::sdesc_sw128(tb + 8192 + kk * 32, 16, 1024);
-        tc::mma_bf16_ts(tmW, tmS + kk * 8, bh, id64, kk > 0);  // delta^T = X^T T^T
-        tc::mma_bf16_ts(tmW, tmS + kk * 8, bl, id64, 1);
-        tc::mma_bf16_ts(tmW, tmS + 32 + kk * 8, bh, id64, 1);
-      }
-      tc::mma_commit(&sh.bar_mma);
       mma_out = true;
+      if (tc::elect_one()) {
+        if (it_next >= 0) issue_s0(it_next, slot_next, 1);
+        const uint32_t tb = tc::smem_u32(Tb);
+#pragma unroll
+        for (int kk = 0; kk < kCkC / 16; ++kk) {
+          const uint64_t bh = tc::sdesc_sw128(tb + kk * 32, 16, 1024);
+          const uint64_t bl = tc::sdesc_sw128(tb + 8192 + kk * 32, 16, 1024);
+          tc::mma_bf16_ts(tmW, tmS + kk * 8, bh, id64, kk > 0);  // delta^T = X^T T^T
+          tc::mma_bf16_ts(tmW, tmS + kk * 8, bl, id64, 1);
+          tc::mma_bf16_ts(tmW, tmS + 32 + kk * 8, bh, id64, 1);
+        }
+        tc::mma_commit(&sh.bar_mma);
+      }
+      __syncwarp();
     }
     bad |= !tc::mbar_wait(&sh.bar_mma, ph_mma, &sh.abort_flag);
     ph_mma ^= 1u;
     tc::fence_after_sync();
     if (tid == kIssuer) mma_out = false;
     // delta^T as bf16 pairs over X^T's high part
-#pragma unroll 1
-    for (int h = 0; h < 2; ++h) {
+    {
       uint32_t d[32], w[16];
-      ck_ld32(tmW + lane_off + 32 * h, d);
+      ck_ld32(tmW + lane_off + 32 * grp, d);
 #pragma unroll
       for (int e = 0; e < 16; ++e) w[e] = ck_pack(__uint_as_float(d[2 * e]), __uint_as_float(d[2 * e + 1]));
-      tc::tmem_st16(tmS + lane_off + 16 * h, w);
+      tc::tmem_st16(tmS + lane_off + 16 * grp, w);
     }
     tc::tmem_st_wait();
     tc::fence_before_sync();
     if (__syncthreads_or(bad)) break;  // delta^T complete
-    if (tid == kIssuer) {
-      tc::fence_after_sync();
-#pragma unroll
-      for (int kk = 0; kk < kCkC / 16; ++kk)
-        tc::mma_bf16_ts(tmG, tmS + kk * 8, tc::sdesc_sw128(tc::smem_u32(M2s + kk * 32), 16, 1024),
-                        id64, kk > 0);  // O2^T = delta^T M2^T, over G
-      tc::mma_commit(&sh.bar_mma);
+    if (warp == kIssuer / 32) {
       mma_out = true;
+      tc::fence_after_sync();
+      if (tc::elect_one()) {
+#pragma unroll
+        for (int kk = 0; kk < kCkC / 16; ++kk)
+          tc::mma_bf16_ts(tmG, tmS + kk * 8, tc::sdesc_sw128(tc::smem_u32(M2s + kk * 32), 16, 1024),
+                          id64, kk > 0);  // O2^T = delta^T M2^T, over G
+        tc::mma_commit(&sh.bar_mma);
+      }
+      __syncwarp();
     }
     bad |= !tc::mbar_wait(&sh.bar_mma, ph_mma, &sh.abort_flag);
     ph_mma ^= 1u;
@@ -464,10 +466,9 @@ __global__ void __launch_bounds__(kD6Threads, 2)
       const float sG = p.scale * sh.Gc[B - 1];
       const bool odd = lane & 1;
       __nv_bfloat16* out = static_cast<__nv_bfloat16*>(p.out_blockend) +
-                           ((size_t)r * B * p.Hv + j) * kD6D + (tid & ~1);
-#pragma unroll 1
-      for (int h = 0; h < 2; ++h) {
-        const int t0 = 32 * h;
+                           ((size_t)r * B * p.Hv + j) * kD6D + (col & ~1);
+      {
+        const int t0 = 32 * grp;
         uint32_t o2[32], wq[32];
         tc::tmem_ld16(tmG + lane_off + t0, *reinterpret_cast<uint32_t(*)[16]>(&o2[0]));
         tc::tmem_ld16(tmG + lane_off + t0 + 16, *reinterpret_cast<uint32_t(*)[16]>(&o2[16]));

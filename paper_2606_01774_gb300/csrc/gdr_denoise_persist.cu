@@ -294,35 +294,39 @@ __global__ void __launch_bounds__(kDpThreads, 2)
     tc::tmem_st_wait();
     tc::fence_before_sync();
     if (__syncthreads_or(bad)) break;  // S0^T complete, the state buffer read
-    if (tid == kIssuer) {
+    if (warp == kIssuer / 32) {  // converged; one elected lane issues
       bad |= !tc::mbar_wait(&sh.bar_kq, ph, &sh.abort_flag);
       kq_out = false;
-      tc::fence_after_sync();
-      // the Gram first, committed on its own: A^T and M2 are built while the
-      // state products run
-#pragma unroll
-      for (int kk = 0; kk < kDpD / 16; ++kk) {
-        const uint8_t* kc = KQs + (kk >> 2) * (2 * BM * 128) + (kk & 3) * 32;
-        tc::mma_bf16_ss(tmG, tc::sdesc_sw128(tc::smem_u32(kc - kG0 * 128), 16, 1024),
-                        tc::sdesc_sw128(tc::smem_u32(kc), 16, 1024), idG, kk > 0);  // G = [K;Q] K^T
-      }
-      tc::mma_commit(&sh.bar_g);
-#pragma unroll
-      for (int kk = 0; kk < kDpD / 16; ++kk) {
-        const uint8_t* kc = KQs + (kk >> 2) * (2 * BM * 128) + (kk & 3) * 32;
-        tc::mma_bf16_ts(tmW, tmS + kk * 8, tc::sdesc_sw128(tc::smem_u32(kc), 16, 1024), idW,
-                        kk > 0);  // W^T = S0^T [K;Q]^T
-      }
-      tc::mma_commit(&sh.bar_mma);
       mma_out = true;
-      // the state buffer is free: the next item's state streams in during
-      // this item's products, solve and readout (issued after the MMAs, off
-      // their path)
+      __syncwarp();
+      tc::fence_after_sync();
+      if (tc::elect_one()) {
+        // the Gram first, committed on its own: A^T and M2 are built while the
+        // state products run
+#pragma unroll
+        for (int kk = 0; kk < kDpD / 16; ++kk) {
+          const uint8_t* kc = KQs + (kk >> 2) * (2 * BM * 128) + (kk & 3) * 32;
+          tc::mma_bf16_ss(tmG, tc::sdesc_sw128(tc::smem_u32(kc - kG0 * 128), 16, 1024),
+                          tc::sdesc_sw128(tc::smem_u32(kc), 16, 1024), idG, kk > 0);  // G = [K;Q] K^T
+        }
+        tc::mma_commit(&sh.bar_g);
+#pragma unroll
+        for (int kk = 0; kk < kDpD / 16; ++kk) {
+          const uint8_t* kc = KQs + (kk >> 2) * (2 * BM * 128) + (kk & 3) * 32;
+          tc::mma_bf16_ts(tmW, tmS + kk * 8, tc::sdesc_sw128(tc::smem_u32(kc), 16, 1024), idW,
+                          kk > 0);  // W^T = S0^T [K;Q]^T
+        }
+        tc::mma_commit(&sh.bar_mma);
+        // the state buffer is free: the next item's state streams in during
+        // this item's products, solve and readout (issued after the MMAs, off
+        // their path)
+        if (it_next >= 0) issue_s0(it_next, slot_next);
+      }
       if (it_next >= 0) {
-        issue_s0(it_next, slot_next);
         s0_out = true;
         s0_par = ph ^ 1u;
       }
+      __syncwarp();
     }
     bad |= !tc::mbar_wait(&sh.bar_v, ph, &sh.abort_flag);
     if (tid == kIssuer) v_out = false;
@@ -531,18 +535,21 @@ __global__ void __launch_bounds__(kDpThreads, 2)
     }
     tc::fence_before_sync();
     if (__syncthreads_or(bad)) break;  // N complete; A^T, M2 and T read
-    if (tid == kIssuer) {
-      tc::fence_after_sync();
-#pragma unroll
-      for (int kk = 0; kk < BM / 16; ++kk) {  // O2^T = X^T N^T, over G
-        const uint64_t nh = tc::sdesc_sw128(tc::smem_u32(Nbs + kk * 32), 16, 1024);
-        const uint64_t nl = tc::sdesc_sw128(tc::smem_u32(Nbs + BM * 128 + kk * 32), 16, 1024);
-        tc::mma_bf16_ts(tmG, tmS + kk * 8, nh, idO, kk > 0);
-        tc::mma_bf16_ts(tmG, tmS + kk * 8, nl, idO, 1);
-        tc::mma_bf16_ts(tmG, tmS + BM / 2 + kk * 8, nh, idO, 1);
-      }
-      tc::mma_commit(&sh.bar_mma);
+    if (warp == kIssuer / 32) {
       mma_out = true;
+      tc::fence_after_sync();
+      if (tc::elect_one()) {
+#pragma unroll
+        for (int kk = 0; kk < BM / 16; ++kk) {  // O2^T = X^T N^T, over G
+          const uint64_t nh = tc::sdesc_sw128(tc::smem_u32(Nbs + kk * 32), 16, 1024);
+          const uint64_t nl = tc::sdesc_sw128(tc::smem_u32(Nbs + BM * 128 + kk * 32), 16, 1024);
+          tc::mma_bf16_ts(tmG, tmS + kk * 8, nh, idO, kk > 0);
+          tc::mma_bf16_ts(tmG, tmS + kk * 8, nl, idO, 1);
+          tc::mma_bf16_ts(tmG, tmS + BM / 2 + kk * 8, nh, idO, 1);
+        }
+        tc::mma_commit(&sh.bar_mma);
+      }
+      __syncwarp();
     }
     bad |= !tc::mbar_wait(&sh.bar_mma, ph_mma, &sh.abort_flag);
     ph_mma ^= 1u;

@@ -59,17 +59,20 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
 // Waits for the phase with the given parity to complete.  Gives up after
 // `limit_ns` nanoseconds (or as soon as *abort becomes non-zero) and returns
 // false; every pipeline wait in this library goes through here, so no kernel
-// can spin forever.
+// can spin forever.  The timer is first read after 64 tries: a read of
+// %globaltimer takes longer than most waits last, and one before the first retry
+// was on the chain of every wait that was not over yet.
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity,
                                           const volatile int* abort,
                                           uint64_t limit_ns = 2000000000ull) {
-  if (mbar_try_wait(bar, parity)) return true;
-  const uint64_t t0 = globaltimer_ns();
+  uint64_t t0 = 0;
   for (uint32_t it = 1;; ++it) {
     if (mbar_try_wait(bar, parity)) return true;
     if ((it & 63u) == 0) {
       if (abort && *abort) return false;
-      if (globaltimer_ns() - t0 > limit_ns) return false;
+      const uint64_t now = globaltimer_ns();
+      if (t0 == 0) t0 = now;
+      if (now - t0 > limit_ns) return false;
     }
   }
 }
