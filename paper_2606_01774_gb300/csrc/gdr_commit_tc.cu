@@ -18,7 +18,8 @@
 //
 //   MMA 1  G   = K K^T             M=128 (rows t), N=Bp, K=128       bf16
 //   MMA 2  W^T = S0^T K^T          M=128 (c),      N=Bp, K=128       S0^T = hi + lo
-//   solve  (I + A) delta = X       fp32, thread c on column c, right-looking
+//   solve  (I + A) delta = X       fp32, thread c on column c, right-looking by
+//                                  blocks of 16 tokens
 //   MMA 3  D  += delta'^T K        M=128 (c),      N=128, K=16 ceil(n/16)   delta' = hi + lo
 //
 // with D = S^(n)^T accumulating on top of Gam_{n-1} S0^T and delta'_i =
@@ -29,7 +30,15 @@
 // what the committed state's fp32-grade accuracy needs.  The Gam_{n-1} S0
 // term is formed in fp32 from the loaded state itself.
 //
-// Persistent CTAs, two per SM (97 KiB of shared memory, 256 tensor-memory
+// Tokens past n take no part: the block loops below end at ceil(n / 16).  They
+// are loops also because the kernel is bound by its instruction stream (each
+// phase runs once per item and the warps' paths do not fit in the instruction
+// cache): the unrolled 64-token solve alone was 41 KB of code and 10.5k of an
+// item's 27k cycles, whatever n.  128 requests, blocks of 64, n = 1..64: 221 -> 169
+// us per call (n = 64 throughout: 223 either way); 64 requests, blocks of 32: n =
+// 1..32 67.9 -> 64.5, n = 32 68.0 -> 68.4.
+//
+// Persistent CTAs, two per SM (99 KiB of shared memory, 256 tensor-memory
 // columns each), 128 threads, each walking the (request, value head) items
 // blockIdx.x, blockIdx.x + gridDim.x, ...  The state (64 KiB) arrives by one
 // bulk copy, the keys and values by TMA (64-row key boxes with 128-byte
@@ -140,6 +149,8 @@ __global__ void __launch_bounds__(kCtThreads, 2)
     gdr_commit_tc_kernel(const __grid_constant__ CtMaps maps, GdrParams p) {
   using C = CtCfg<BM>;
   constexpr int kATs = C::kATs;
+  // block loops: unrolled where the whole block count is at most two
+  constexpr int kU = BM <= 32 ? BM / 16 : 1;
   extern __shared__ uint8_t smem_raw[];
   __shared__ CtShared sh;
   uint8_t* base = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -151,7 +162,6 @@ __global__ void __launch_bounds__(kCtThreads, 2)
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int total = p.R * p.Hv;
   const int B = p.B;
-  const int Bp = (B + 15) & ~15;
 
   int slot = 0, n = 0;
   int it = ct_next(p, blockIdx.x, total, slot, n);
@@ -228,11 +238,11 @@ __global__ void __launch_bounds__(kCtThreads, 2)
   int cs = cand_slot(cand), ca = cand_len(cand);
   uint32_t ph = 0;      // parity of the item's state and key/value loads
   uint32_t ph_mma = 0;  // parity of the next MMA completion (two per item)
-  const uint32_t idN = tc::idesc_bf16(128, Bp, false, false);
   const uint32_t idU = tc::idesc_bf16(128, 128, false, true);
 
 #pragma unroll 1
   while (true) {
+    const int nb = (n + 15) >> 4;  // blocks of 16 tokens that take part
     // the block's gates: gamma = inclusive prefix sum of the log-gates
     if (warp == 0) {
       float g0 = gq0, g1 = gq1;
@@ -295,30 +305,40 @@ __global__ void __launch_bounds__(kCtThreads, 2)
     tc::tmem_st_wait();
     tc::fence_before_sync();
     if (!ct_wait(&sh.bar_k, ph, sh, p.dev_status)) break;  // also orders the stores above
-    if (tid == 0) {
+    if (warp == 0) {  // converged; one elected lane issues
       k_out = false;
-      tc::fence_after_sync();
-#pragma unroll
-      for (int kk = 0; kk < kCtD / 16; ++kk) {
-        const uint8_t* kc = Ks + (kk >> 2) * (64 * 128) + (kk & 3) * 32;
-        const uint64_t kd = tc::sdesc_sw128(tc::smem_u32(kc), 16, 1024);
-        // A operand rows kG0.. are the keys; the rows before read the bytes
-        // ahead of the chunk (the state buffer, then the first chunk), which
-        // only reach lanes nobody reads
-        const uint64_t kg = tc::sdesc_sw128(tc::smem_u32(kc - kG0 * 128), 16, 1024);
-        tc::mma_bf16_ss(tmG, kg, kd, idN, kk > 0);                // G = K K^T
-        tc::mma_bf16_ts(tmW, tmS + kk * 8, kd, idN, kk > 0);      // W^T = S0hi^T K^T
-        tc::mma_bf16_ts(tmW, tmS + 64 + kk * 8, kd, idN, 1u);     //     + S0lo^T K^T
-      }
-      tc::mma_commit(&sh.bar_mma);
       mma_out = true;
+      tc::fence_after_sync();
+      if (tc::elect_one()) {
+        const uint32_t idN = tc::idesc_bf16(128, 16 * nb, false, false);
+#pragma unroll 1  // unrolled, the descriptors are hoisted and the solve spills
+        for (int kk = 0; kk < kCtD / 16; ++kk) {
+          const uint8_t* kc = Ks + (kk >> 2) * (64 * 128) + (kk & 3) * 32;
+          const uint64_t kd = tc::sdesc_sw128(tc::smem_u32(kc), 16, 1024);
+          // A operand rows kG0.. are the keys; the rows before read the bytes
+          // ahead of the chunk (the state buffer, then the first chunk), which
+          // only reach lanes nobody reads
+          const uint64_t kg = tc::sdesc_sw128(tc::smem_u32(kc - kG0 * 128), 16, 1024);
+          tc::mma_bf16_ss(tmG, kg, kd, idN, kk > 0);                // G = K K^T
+          tc::mma_bf16_ts(tmW, tmS + kk * 8, kd, idN, kk > 0);      // W^T = S0hi^T K^T
+          tc::mma_bf16_ts(tmW, tmS + 64 + kk * 8, kd, idN, 1u);     //     + S0lo^T K^T
+        }
+        tc::mma_commit(&sh.bar_mma);
+      }
+      __syncwarp();
     }
     // this thread's value column (rows past B arrive as zeros)
     uint32_t vraw[BM];
     {
       const uint8_t* vb = Rs + (tid >> 6) * (BM * 128) + (tid & 63) * 2;
 #pragma unroll
-      for (int t = 0; t < BM; ++t) vraw[t] = *reinterpret_cast<const unsigned short*>(vb + t * 128);
+      for (int t0 = 0; t0 < BM; t0 += 16) {
+        if (t0 < n) {
+#pragma unroll
+          for (int t = t0; t < t0 + 16; ++t)
+            vraw[t] = *reinterpret_cast<const unsigned short*>(vb + t * 128);
+        }
+      }
     }
     if (!ct_wait(&sh.bar_mma, ph_mma, sh, p.dev_status)) break;  // the values are read
     ph_mma ^= 1u;
@@ -337,30 +357,34 @@ __global__ void __launch_bounds__(kCtThreads, 2)
       }
     }
     // A^T from the Gram rows t < BM (the warps holding those lanes); rows of
-    // A at or past n are zero, so the solve below may run all BM steps
+    // A at or past n are zero, so the solve below may run whole blocks
     if (warp >= kG0 / 32) {
       const int t = tid - kG0;
-      uint32_t gr[BM];
+      const float bt = t >= 0 ? sh.beta[t] : 0.f, gt = t >= 0 ? sh.gam2[t] : 0.f;
+      constexpr int kC = 16;
+#pragma unroll kU
+      for (int b = 0; b < BM / 16; ++b) {
+        if (b >= nb) break;
+        const int c0 = 16 * b;
+        uint32_t gr[kC];
 #pragma unroll
-      for (int c0 = 0; c0 < BM; c0 += 16)
-        tc::tmem_ld16(tmG + lane_off + c0, *reinterpret_cast<uint32_t(*)[16]>(&gr[c0]));
-      tc::tmem_ld_wait();
-      if (t >= 0) {
-        // the log-gates go to registers first (16-byte loads) and every
-        // exponential is taken unconditionally, the mask applied as a
-        // select: a branch per element would serialise the chains
-        float g2r[BM];
+        for (int c = 0; c < kC; c += 16)
+          tc::tmem_ld16(tmG + lane_off + c0 + c, *reinterpret_cast<uint32_t(*)[16]>(&gr[c]));
+        tc::tmem_ld_wait();
+        if (t >= 0) {
+          // every exponential is taken unconditionally, the mask applied as a
+          // select: a branch per element would serialise the chains
 #pragma unroll
-        for (int i4 = 0; i4 < BM / 4; ++i4) {
-          const float4 q = *reinterpret_cast<const float4*>(&sh.gam2[4 * i4]);
-          g2r[4 * i4] = q.x, g2r[4 * i4 + 1] = q.y, g2r[4 * i4 + 2] = q.z, g2r[4 * i4 + 3] = q.w;
-        }
-        const float bt = sh.beta[t], gt = sh.gam2[t];
-        const bool live = t < n;
+          for (int i4 = 0; i4 < kC / 4; ++i4) {
+            const float4 q = *reinterpret_cast<const float4*>(&sh.gam2[c0 + 4 * i4]);
+            const float gi[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
-        for (int i = 0; i < BM; ++i) {
-          const float a = bt * tc::ex2(gt - g2r[i]) * __uint_as_float(gr[i]);
-          AT[i * kATs + t] = (live && i < t) ? a : 0.f;
+            for (int e = 0; e < 4; ++e) {
+              const int i = c0 + 4 * i4 + e;
+              const float a = bt * tc::ex2(gt - gi[e]) * __uint_as_float(gr[4 * i4 + e]);
+              AT[i * kATs + t] = (t < n && i < t) ? a : 0.f;
+            }
+          }
         }
       }
     }
@@ -368,8 +392,9 @@ __global__ void __launch_bounds__(kCtThreads, 2)
     float x[BM];
 #pragma unroll
     for (int c0 = 0; c0 < BM; c0 += 16) {
+      if (c0 >= n) break;  // uniform
       uint32_t w[16];
-      tc::tmem_ld16(tmW + lane_off + c0, w);  // columns past Bp: stale, used by no kept row
+      tc::tmem_ld16(tmW + lane_off + c0, w);
       tc::tmem_ld_wait();
 #pragma unroll
       for (int e4 = 0; e4 < 4; ++e4) {
@@ -392,63 +417,79 @@ __global__ void __launch_bounds__(kCtThreads, 2)
       s0_par = ph ^ 1u;
     }
 
-    // (I + A) delta = X, right-looking: once delta_t is final it leaves the
-    // remaining rows (A^T row t as 16-byte broadcast loads).  Rows t >= n
-    // only touch rows past n (A^T is zero there), which nothing keeps.
+    // (I + A) delta = X, right-looking: once a block's deltas are final they
+    // leave the later blocks (A^T rows as 16-byte broadcast loads), which move
+    // down in the registers, and go to tensor memory as delta'_t =
+    // exp(gamma_{n-1} - gamma_t) delta_t (t < n) in bf16 hi and lo parts.
+#pragma unroll kU
+    for (int b = 0; b < BM / 16; ++b) {
+      if (kU == 1 && b >= nb) break;  // uniform (two blocks: 69.6 us with the branch, 68.4 without)
+      const float* ab = AT + 16 * b * kATs + 16 * b;
 #pragma unroll
-    for (int t = 0; t < BM; ++t) {
-      const float dt = x[t];
-      const float* ar = AT + t * kATs;
+      for (int t = 0; t < 16; ++t) {
+        const float dt = x[t];
 #pragma unroll
-      for (int u4 = (t + 1) / 4; u4 < BM / 4; ++u4) {
-        const float4 a = *reinterpret_cast<const float4*>(ar + 4 * u4);
-        if (4 * u4 + 0 > t) x[4 * u4 + 0] = fmaf(-a.x, dt, x[4 * u4 + 0]);
-        if (4 * u4 + 1 > t) x[4 * u4 + 1] = fmaf(-a.y, dt, x[4 * u4 + 1]);
-        if (4 * u4 + 2 > t) x[4 * u4 + 2] = fmaf(-a.z, dt, x[4 * u4 + 2]);
-        if (4 * u4 + 3 > t) x[4 * u4 + 3] = fmaf(-a.w, dt, x[4 * u4 + 3]);
-      }
-    }
-    // delta'_t = exp(gamma_{n-1} - gamma_t) delta_t (t < n), as bf16 hi and lo parts
-    {
-      float dr[BM];
-#pragma unroll
-      for (int i4 = 0; i4 < BM / 4; ++i4) {
-        const float4 q = *reinterpret_cast<const float4*>(&sh.dsc[4 * i4]);
-        dr[4 * i4] = q.x, dr[4 * i4 + 1] = q.y, dr[4 * i4 + 2] = q.z, dr[4 * i4 + 3] = q.w;
-      }
-#pragma unroll
-      for (int c0 = 0; c0 < C::kDP; c0 += 16) {
-        uint32_t hi[16], lo[16];
-#pragma unroll
-        for (int e = 0; e < 16; ++e) {
-          const int t = 2 * (c0 + e);
-          float a = 0.f, b = 0.f;
-          if (t < BM) {
-            const float xa = x[t] * dr[t], xb = x[t + 1] * dr[t + 1];
-            a = t < n ? xa : 0.f;
-            b = t + 1 < n ? xb : 0.f;
-          }
-          split_pair(a, b, hi[e], lo[e]);
+        for (int u4 = (t + 1) / 4; u4 < 4; ++u4) {
+          const float4 a = *reinterpret_cast<const float4*>(ab + t * kATs + 4 * u4);
+          if (4 * u4 + 0 > t) x[4 * u4 + 0] = fmaf(-a.x, dt, x[4 * u4 + 0]);
+          if (4 * u4 + 1 > t) x[4 * u4 + 1] = fmaf(-a.y, dt, x[4 * u4 + 1]);
+          if (4 * u4 + 2 > t) x[4 * u4 + 2] = fmaf(-a.z, dt, x[4 * u4 + 2]);
+          if (4 * u4 + 3 > t) x[4 * u4 + 3] = fmaf(-a.w, dt, x[4 * u4 + 3]);
         }
-        tc::tmem_st16(tmW + lane_off + c0, hi);
-        tc::tmem_st16(tmW + lane_off + C::kDP + c0, lo);
       }
+      uint32_t hi[8], lo[8];
+#pragma unroll
+      for (int i4 = 0; i4 < 4; ++i4) {
+        const float4 q = *reinterpret_cast<const float4*>(&sh.dsc[16 * b + 4 * i4]);
+        const float dr[4] = {q.x, q.y, q.z, q.w};
+        float v[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const float xv = x[4 * i4 + e] * dr[e];
+          v[e] = 16 * b + 4 * i4 + e < n ? xv : 0.f;
+        }
+        split_pair(v[0], v[1], hi[2 * i4], lo[2 * i4]);
+        split_pair(v[2], v[3], hi[2 * i4 + 1], lo[2 * i4 + 1]);
+      }
+      tc::tmem_st8(tmW + lane_off + 8 * b, hi);
+      tc::tmem_st8(tmW + lane_off + C::kDP + 8 * b, lo);
+#pragma unroll
+      for (int k = 1; k < BM / 16; ++k) {
+        if (k < BM / 16 - (kU > 1 ? b : 0) && b + k < nb) {  // uniform
+#pragma unroll
+          for (int t = 0; t < 16; ++t) {
+            const float dt = x[t];
+#pragma unroll
+            for (int u4 = 0; u4 < 4; ++u4) {
+              const float4 a = *reinterpret_cast<const float4*>(ab + t * kATs + 16 * k + 4 * u4);
+              x[16 * k + 4 * u4 + 0] = fmaf(-a.x, dt, x[16 * k + 4 * u4 + 0]);
+              x[16 * k + 4 * u4 + 1] = fmaf(-a.y, dt, x[16 * k + 4 * u4 + 1]);
+              x[16 * k + 4 * u4 + 2] = fmaf(-a.z, dt, x[16 * k + 4 * u4 + 2]);
+              x[16 * k + 4 * u4 + 3] = fmaf(-a.w, dt, x[16 * k + 4 * u4 + 3]);
+            }
+          }
+        }
+      }
+#pragma unroll
+      for (int i = 0; i + 16 < BM; ++i) x[i] = x[i + 16];
     }
     tc::tmem_st_wait();
     tc::fence_before_sync();
     __syncthreads();  // also: A^T read, its region free for the next values
-    if (tid == 0) {
-      tc::fence_after_sync();
-      // D += delta'^T K: the keys [t][i] as an MN-major operand (i contiguous)
-      const int ksteps = (n + 15) >> 4;
-#pragma unroll 1
-      for (int kk = 0; kk < ksteps; ++kk) {
-        const uint64_t kb = tc::sdesc_sw128(tc::smem_u32(Ks + kk * 2048), 64 * 128, 1024);
-        tc::mma_bf16_ts(tmS, tmW + kk * 8, kb, idU, 1u);
-        tc::mma_bf16_ts(tmS, tmW + C::kDP + kk * 8, kb, idU, 1u);
-      }
-      tc::mma_commit(&sh.bar_mma);
+    if (warp == 0) {
       mma_out = true;
+      tc::fence_after_sync();
+      if (tc::elect_one()) {
+        // D += delta'^T K: the keys [t][i] as an MN-major operand (i contiguous)
+#pragma unroll 1
+        for (int kk = 0; kk < nb; ++kk) {
+          const uint64_t kb = tc::sdesc_sw128(tc::smem_u32(Ks + kk * 2048), 64 * 128, 1024);
+          tc::mma_bf16_ts(tmS, tmW + kk * 8, kb, idU, 1u);
+          tc::mma_bf16_ts(tmS, tmW + C::kDP + kk * 8, kb, idU, 1u);
+        }
+        tc::mma_commit(&sh.bar_mma);
+      }
+      __syncwarp();
     }
     if (!ct_wait(&sh.bar_mma, ph_mma, sh, p.dev_status)) break;
     ph_mma ^= 1u;
