@@ -393,11 +393,10 @@ __global__ void __launch_bounds__(kD6Threads, 2)
     }
 
     // ---- T = (I + A)^{-1} below its diagonal blocks: block column 0 on
-    // warps 0-3, 1 on warps 4-5, 2 (and the strip of 3) on warps 6-7
-    if (warp < 4)
-      ck_tcol<128>(AT, Tf, Tb, 0, 1, tid, 1);
-    else
-      ck_tcol<64>(AT, Tf, Tb, 1 + ((warp - 4) >> 1), warp < 6 ? 1 : 2, tid & 63, warp < 6 ? 2 : 3);
+    // warps 0-1, 1 on warps 2-3, 2 (and the strip of 3) on warps 4-5.  One copy of
+    // the column code; twice the warps on column 0 take a second (140.7 and 139.2 us
+    // per multistep_batch128 call).
+    if (warp < 6) ck_tcol<64>(AT, Tf, Tb, warp >> 1, warp < 4 ? 1 : 2, tid & 63, 1 + (warp >> 1));
     if (__syncthreads_or(bad)) break;  // T as bf16 high / low parts; A^T and T read
     if (warp == kIssuer / 32) {
       if (it_next >= 0) {  // A^T and T read: the next item's second half

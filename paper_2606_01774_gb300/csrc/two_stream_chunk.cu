@@ -84,9 +84,10 @@ struct alignas(16) CkShared {
   alignas(16) float gc2[kCkC];  // clean gamma_t log2(e), from the chunk start
   alignas(16) float Gc[kCkC];   // clean exp(gamma_t)
   alignas(16) float bc[kCkC];   // clean beta
-  alignas(16) float gn2[kCkC];  // noisy gamma~_t log2(e), from the block start
+  alignas(16) float ngn2[kCkC];  // noisy -gamma~_t log2(e), from the block start
   alignas(16) float Gn[kCkC];   // noisy exp(gamma~_t)
   alignas(16) float bn[kCkC];   // noisy beta~
+  alignas(16) float one[kCkC];  // ones
 };
 
 struct CkMaps {
@@ -119,6 +120,7 @@ __global__ void __launch_bounds__(kCkThreads, 1)
   const int n_chunks = p.L / kCkC;
   const int total = p.N * p.Hv * n_chunks;
 
+  if (tid < kCkC) sh.one[tid] = 1.f;
   if (tid == kIssuer) {
     sh.abort_flag = 0;
     tc::mbar_init(&sh.bar_s0, 1);
@@ -243,8 +245,8 @@ __global__ void __launch_bounds__(kCkThreads, 1)
         sh.bc[lane] = ba;
         sh.bc[lane + 32] = bb;
       } else {
-        sh.gn2[lane] = x0 * 1.4426950408889634f;
-        sh.gn2[lane + 32] = x1 * 1.4426950408889634f;
+        sh.ngn2[lane] = -x0 * 1.4426950408889634f;
+        sh.ngn2[lane + 32] = -x1 * 1.4426950408889634f;
         sh.Gn[lane] = expf(x0);
         sh.Gn[lane + 32] = expf(x1);
         sh.bn[lane] = ba;
@@ -278,14 +280,14 @@ __global__ void __launch_bounds__(kCkThreads, 1)
       if (tc::elect_one()) {
         // the Gram first, committed on its own: the tables are built from it
         // while the state products run
-#pragma unroll
+#pragma unroll 1
         for (int kk = 0; kk < kCkD / 16; ++kk) {
           const uint64_t kd = tc::sdesc_sw128(
               tc::smem_u32(KX + (kk >> 2) * (192 * 128) + (kk & 3) * 32), 16, 1024);
           tc::mma_bf16_ss(tmG, kd, kd, id192, kk > 0);  // G = [K; K~] [K; K~; Q~]^T
         }
         tc::mma_commit(&sh.bar_g);
-#pragma unroll
+#pragma unroll 1
         for (int kk = 0; kk < kCkD / 16; ++kk) {
           const uint64_t kd = tc::sdesc_sw128(
               tc::smem_u32(KX + (kk >> 2) * (192 * 128) + (kk & 3) * 32), 16, 1024);
@@ -311,100 +313,93 @@ __global__ void __launch_bounds__(kCkThreads, 1)
       const int row = col & 63;
       const bool krow = col < 64;
       const int m0 = row & ~(B - 1);  // the block start of this row's token
-      if (grp == 0) {
-        if (krow) {
-          // warps 0-1: A^T row i of the clean system
-          const float gi = sh.gc2[row];
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            uint32_t gr[32];
-            float v[32];
-            ck_ld32(tmG + lane_off + 32 * h, gr);
-#pragma unroll
-            for (int k = 0; k < 32; ++k) {
-              const int t = 32 * h + k;
-              const float a = sh.bc[t] * tc::ex2(sh.gc2[t] - gi) * __uint_as_float(gr[k]);
-              v[k] = t > row ? a : 0.f;
-            }
-            ck_store32(AT, row, 32 * h, v);
-          }
-          tc::named_bar_arrive(5, 128);  // A^T to warps 4-5
-        } else {
-          // warps 2-3: A~ row t
-          const float bt = sh.bn[row], gt = sh.gn2[row];
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            uint32_t gr[32];
-            float v[32];
-            ck_ld32(tmG + lane_off + 64 + 32 * h, gr);
-#pragma unroll
-            for (int k = 0; k < 32; ++k) {
-              const int i = 32 * h + k;
-              const float a = bt * tc::ex2(gt - sh.gn2[i]) * __uint_as_float(gr[k]);
-              v[k] = (i >= m0 && i < row) ? a : 0.f;
-            }
-            ck_store32(An, row, 32 * h, v);
-          }
-        }
-      } else {
-        if (krow) {
-          // warps 4-5: P row i, 128 columns (the noisy keys, then queries),
-          // P[i][y] = [i < mB] exp(gamma_{mB-1} - gamma_i) (k_i . y)
-          // the factor depends on the row and the block only: one per block
-          const float gi = sh.gc2[row];
+      if (grp == 1 && krow) {
+        // warps 4-5: P row i, 128 columns (the noisy keys, then queries),
+        // P[i][y] = [i < mB] exp(gamma_{mB-1} - gamma_i) (k_i . y)
+        // the factor depends on the row and the block only: one per block
+        const float gi = sh.gc2[row];
 #pragma unroll 1
-          for (int h = 0; h < 4; ++h) {  // columns 32 h .. of the 128: tokens 32 (h % 2) ..
-            const int tq = 32 * (h & 1);
-            float fm[32 / B];
+        for (int h = 0; h < 4; ++h) {  // columns 32 h .. of the 128: tokens 32 (h % 2) ..
+          const int tq = 32 * (h & 1);
+          float fm[32 / B];
 #pragma unroll
-            for (int m = 0; m < 32 / B; ++m) {
-              const int mb = tq + m * B;
-              const float a = tc::ex2(sh.gc2[mb > 0 ? mb - 1 : 0] - gi);
-              fm[m] = row < mb ? a : 0.f;
-            }
-            uint32_t gr[32];
-            ck_ld32(tmG + lane_off + 64 + 32 * h, gr);
-#pragma unroll
-            for (int u4 = 0; u4 < 4; ++u4) {  // 16-byte units of 8 columns
-              const int u = 4 * (h & 1) + u4;   // unit within the 64-column chunk
-              uint32_t w[4];
-#pragma unroll
-              for (int e = 0; e < 4; ++e) {
-                float pv[2];
-#pragma unroll
-                for (int f = 0; f < 2; ++f) {
-                  const int k = 8 * u4 + 2 * e + f;  // column within the 32: token tq + k
-                  pv[f] = fm[k / B] * __uint_as_float(gr[k]);
-                }
-                w[e] = ck_pack(pv[0], pv[1]);
-              }
-              // MN-major SW128: chunk h / 2, row i, 16-byte unit u ^ (i % 8)
-              *reinterpret_cast<uint4*>(Ps + (h >> 1) * (kCkC * 128) + row * 128 +
-                                        ((u ^ (row & 7)) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
-            }
+          for (int m = 0; m < 32 / B; ++m) {
+            const int mb = tq + m * B;
+            const float a = tc::ex2(sh.gc2[mb > 0 ? mb - 1 : 0] - gi);
+            fm[m] = row < mb ? a : 0.f;
           }
-          tc::fence_async_smem();  // P is the second MMA's operand
-          // the diagonal blocks of T once warps 0-1 have written A^T: blocks
-          // 2 (warp - 4) and 2 (warp - 4) + 1, a column of one per lane
-          tc::named_bar_sync(5, 128);
-          ck_diag_inverse(AT, Tf, 2 * (warp - 4) + (lane >> 4), lane & 15);
-        } else {
-          // warps 6-7: Aqk^T row i (noisy key i): exp(gamma~_end - gamma~_i) (q~_l . k~_i)
-          // for the queries l of its block
-          const float f = tc::ex2(sh.gn2[m0 + B - 1] - sh.gn2[row]);
+          uint32_t gr[32];
+          ck_ld32(tmG + lane_off + 64 + 32 * h, gr);
 #pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            uint32_t gr[32];
-            float v[32];
-            ck_ld32(tmG + lane_off + 128 + 32 * h, gr);
+          for (int u4 = 0; u4 < 4; ++u4) {  // 16-byte units of 8 columns
+            const int u = 4 * (h & 1) + u4;   // unit within the 64-column chunk
+            uint32_t w[4];
 #pragma unroll
-            for (int k = 0; k < 32; ++k) {
-              const int l = 32 * h + k;
-              v[k] = (l >= m0 && l < m0 + B) ? f * __uint_as_float(gr[k]) : 0.f;
+            for (int e = 0; e < 4; ++e) {
+              float pv[2];
+#pragma unroll
+              for (int f = 0; f < 2; ++f) {
+                const int k = 8 * u4 + 2 * e + f;  // column within the 32: token tq + k
+                pv[f] = fm[k / B] * __uint_as_float(gr[k]);
+              }
+              w[e] = ck_pack(pv[0], pv[1]);
             }
-            ck_store32(AqT, row, 32 * h, v);
+            // MN-major SW128: chunk h / 2, row i, 16-byte unit u ^ (i % 8)
+            *reinterpret_cast<uint4*>(Ps + (h >> 1) * (kCkC * 128) + row * 128 +
+                                      ((u ^ (row & 7)) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
           }
         }
+        tc::fence_async_smem();  // P is the second MMA's operand
+        // the diagonal blocks of T once warps 0-1 have written A^T: blocks
+        // 2 (warp - 4) and 2 (warp - 4) + 1, a column of one per lane
+        tc::named_bar_sync(5, 128);
+        ck_diag_inverse(AT, Tf, 2 * (warp - 4) + (lane >> 4), lane & 15);
+      } else {
+        // warps 0-1: A^T row i of the clean system; 2-3: A~ row t; 6-7: Aqk^T row i
+        // (noisy key i): exp(gamma~_end - gamma~_i) (q~_l . k~_i) for the queries l of
+        // its block.  One code path, element = rf cf[c] exp2(cg[c] + rg) G[row][c] for
+        // c in [lo, hi), since the kernel is bound by its instruction stream: the
+        // three copies, and their halves unrolled, took 75 us per two_stream_train_b4
+        // call where this takes 71.4.
+        float* tbl = AT;
+        const float *cf = sh.bc, *cg = sh.gc2;
+        float rf = 1.f, rg = -sh.gc2[row];
+        int gcol = 0, lo = row + 1, hi = kCkC;
+        if (grp == 1) {
+          tbl = AqT;
+          cf = cg = sh.one;
+          rf = tc::ex2(sh.ngn2[row] - sh.ngn2[m0 + B - 1]);
+          rg = -1.f;  // exp2(0)
+          gcol = 128, lo = m0, hi = m0 + B;
+        } else if (!krow) {
+          tbl = An;
+          cf = sh.one;
+          cg = sh.ngn2;
+          rf = sh.bn[row];
+          rg = -sh.ngn2[row];
+          gcol = 64, lo = m0, hi = row;
+        }
+#pragma unroll 1
+        for (int h = 0; h < 2; ++h) {
+          uint32_t gr[32];
+          float v[32];
+          ck_ld32(tmG + lane_off + gcol + 32 * h, gr);
+          const float4* cf4 = reinterpret_cast<const float4*>(cf + 32 * h);
+          const float4* cg4 = reinterpret_cast<const float4*>(cg + 32 * h);
+#pragma unroll
+          for (int k4 = 0; k4 < 8; ++k4) {
+            const float4 f4 = cf4[k4], g4 = cg4[k4];
+            const float fv[4] = {f4.x, f4.y, f4.z, f4.w}, gv[4] = {g4.x, g4.y, g4.z, g4.w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              const int c = 32 * h + 4 * k4 + e;
+              const float a = rf * fv[e] * tc::ex2(gv[e] + rg) * __uint_as_float(gr[4 * k4 + e]);
+              v[4 * k4 + e] = (c >= lo && c < hi) ? a : 0.f;
+            }
+          }
+          ck_store32(tbl, row, 32 * h, v);
+        }
+        if (grp == 0 && krow) tc::named_bar_arrive(5, 128);  // A^T to warps 4-5
       }
     }
     // ---- X = diag(beta) (V - diag(Gam) K S0), tokens 32 grp .. 32 grp + 31,
@@ -463,7 +458,7 @@ __global__ void __launch_bounds__(kCkThreads, 1)
       mma_out = true;
       if (tc::elect_one()) {
         const uint32_t tb = tc::smem_u32(Vc);
-#pragma unroll
+#pragma unroll 1
         for (int kk = 0; kk < kCkC / 16; ++kk) {
           const uint64_t bh = tc::sdesc_sw128(tb + kk * 32, 16, 1024);
           const uint64_t bl = tc::sdesc_sw128(tb + 8192 + kk * 32, 16, 1024);
@@ -499,7 +494,7 @@ __global__ void __launch_bounds__(kCkThreads, 1)
       mma_out = true;
       tc::fence_after_sync();
       if (tc::elect_one()) {
-#pragma unroll
+#pragma unroll 1
         for (int kk = 0; kk < kCkC / 16; ++kk)
           tc::mma_bf16_ts(tmG, tmS + kk * 8,
                           tc::sdesc_sw128(tc::smem_u32(Ps + kk * 2048), kCkC * 128, 1024), id128,
