@@ -1,5 +1,6 @@
 // State commit at the accepted length on tcgen05 tensor cores: bf16
-// activations, d_k = d_v = 128, B <= 64, no token-causal outputs.
+// activations, d_k = d_v = 128, B <= 64; for B = 9..32 also with the
+// token-causal outputs of the state-update pass.
 //
 // For one (request r, value head j) with q/k head h, accepted length n > 0 and
 // frozen state S0, the committed state is the chunkwise form of the block's
@@ -38,6 +39,23 @@
 // us per call (n = 64 throughout: 223 either way); 64 requests, blocks of 32: n =
 // 1..32 67.9 -> 64.5, n = 32 68.0 -> 68.4.
 //
+// With token-causal outputs (CAUSAL) every token takes part, and
+//
+//   M2[l][i] = exp(gamma_l - gamma_i) (q_l . k_i),   i <= l < B
+//   out[l]   = s (Gam_l S0^T q_l + sum_{i<=l} M2[l][i] delta_i)
+//
+// G takes the query rows and W^T the query columns as well, and a thread
+// accumulates its column's outputs as its deltas become final.  The register
+// recurrence that this replaces is exact fp32, so the fp32 operands enter as three
+// bf16 terms (24 bits) and the log-gates are summed in double precision and kept
+// as a multiple of 2^-10 and a remainder, whose differences are exact where they
+// matter: over 32 tokens the committed states are 1.7e-7 off 64 bits where the
+// recurrence's are 6.0e-7.  State update of 64 requests (32 heads): B = 32 208 ->
+// 118 us, B = 16 123 -> 81.  Blocks of 8 and fewer stay with the recurrence, which
+// is as fast there (84 and 78 us at B = 8) and closer (1.15e-7 against 1.28e-7:
+// the tensor core's accumulation rounds toward zero); B = 33..64 would need 320
+// tensor-memory columns of the 256 that two CTAs per SM leave each.
+//
 // Persistent CTAs, two per SM (99 KiB of shared memory, 256 tensor-memory
 // columns each), 128 threads, each walking the (request, value head) items
 // blockIdx.x, blockIdx.x + gridDim.x, ...  The state (64 KiB) arrives by one
@@ -65,9 +83,11 @@ namespace {
 constexpr int kCtThreads = 128;
 constexpr int kCtD = 128;  // d_k = d_v
 
-template <int BM>
+template <int BM, bool CAUSAL>
 struct CtCfg {
-  static constexpr int kK = 2 * 64 * 128;          // keys: 2 chunks of 64 rows x 128 B (SW128)
+  // keys: 2 chunks of 64 rows x 128 B (SW128); CAUSAL: keys, then queries, 2 x BM rows
+  static constexpr int kRows = CAUSAL ? 2 * BM : 64;
+  static constexpr int kK = 2 * kRows * 128;
   static constexpr int kS0 = kCtD * kCtD * 4;      // S0 fp32 [i][c]
   static constexpr int kATs = BM + 4;              // row stride of A^T (floats)
   static constexpr int kAT = BM * kATs * 4;        // A^T[i][t] = A[t][i]
@@ -76,20 +96,25 @@ struct CtCfg {
   static constexpr int kR = kAT > kV ? kAT : kV;
   // tensor-memory columns of each bf16 part of delta'^T (whole 16-column stores)
   static constexpr int kDP = BM / 2 < 16 ? 16 : BM / 2;
-  static constexpr int kSmem = kS0 + kK + kR;  // state, keys, values / A^T
+  static constexpr int kM2 = CAUSAL ? kAT : 0;     // M2^T[i][l] = M2[l][i]
+  static constexpr int kSmem = kS0 + kK + kR + kM2;
+  static constexpr int kTerms = CAUSAL ? 3 : 2;    // bf16 terms of an fp32 operand
 };
 
 struct CtMaps {
-  CUtensorMap k;  // keys   (128, Hk, B, R) box (64, 1, 64, 1), 128-byte swizzle
+  // keys and (CAUSAL) queries (128, Hk, B, R) box (64, 1, 64, 1), CAUSAL (64, 1, BM, 1),
+  // 128-byte swizzle
+  CUtensorMap k, q;
   CUtensorMap v;  // values (128, Hv, B, R) box (64, 1, BM, 1), no swizzle
 };
 
 struct alignas(16) CtShared {
-  uint64_t bar_s0, bar_k, bar_mma;
+  uint64_t bar_s0, bar_k, bar_mma, bar_g;
   uint32_t tmem_base;
   int abort_flag;
   // 16-byte aligned: read as float4 broadcasts
-  alignas(16) float gam2[64];  // gamma_t log2(e)
+  alignas(16) float gam2[64];  // gamma_t log2(e) (CAUSAL: its multiple of 2^-10)
+  alignas(16) float glo[32];   // CAUSAL: the remainder
   alignas(16) float Gam[64];   // exp(gamma_t)
   alignas(16) float beta[64];
   alignas(16) float dsc[64];   // exp(gamma_{n-1} - gamma_t) for t < n, else 0 (delta' factor)
@@ -107,8 +132,9 @@ __device__ __forceinline__ bool ct_wait(uint64_t* bar, uint32_t parity, CtShared
 }
 
 // The next item at or after `it` (stride gridDim.x) with a valid slot and
-// accepted length n > 0; items with a bad slot or length are flagged and
+// accepted length n > 0 (CAUSAL: n >= 0); items with a bad slot or length are flagged and
 // skipped.  Called by every thread with the same arguments.
+template <bool CAUSAL>
 __device__ __forceinline__ int ct_next(const GdrParams& p, int it, int total, int& slot, int& n) {
   for (; it < total; it += gridDim.x) {
     const int r = it / p.Hv;
@@ -122,7 +148,7 @@ __device__ __forceinline__ int ct_next(const GdrParams& p, int it, int total, in
       if (threadIdx.x == 0) flag(p.dev_status, FLARE_DEV_BAD_ACCEPT_LEN);
       continue;
     }
-    if (a == 0) continue;
+    if (a == 0 && !CAUSAL) continue;
     slot = s;
     n = a;
     return it;
@@ -134,20 +160,27 @@ __device__ __forceinline__ uint32_t bf2_bits(__nv_bfloat162 b) {
   return *reinterpret_cast<uint32_t*>(&b);
 }
 
-// x = hi + lo for the pair (a, b): hi = bf16(x), lo = bf16(x - hi)
-__device__ __forceinline__ void split_pair(float a, float b, uint32_t& hi, uint32_t& lo) {
-  const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
-  const float2 hf = __bfloat1622float2(h);
-  hi = bf2_bits(h);
-  lo = bf2_bits(__floats2bfloat162_rn(a - hf.x, b - hf.y));
+// The pair (a, b) in N bf16 terms, each the rounding of what the ones before left
+template <int N>
+__device__ __forceinline__ void split_terms(float a, float b, uint32_t (&w)[N]) {
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+    const float2 hf = __bfloat1622float2(h);
+    w[i] = bf2_bits(h);
+    a -= hf.x;
+    b -= hf.y;
+  }
 }
 
 }  // namespace
 
-template <int BM>
+template <int BM, bool CAUSAL>
 __global__ void __launch_bounds__(kCtThreads, 2)
     gdr_commit_tc_kernel(const __grid_constant__ CtMaps maps, GdrParams p) {
-  using C = CtCfg<BM>;
+  static_assert(!CAUSAL || BM <= 32, "tensor memory");
+  using C = CtCfg<BM, CAUSAL>;
+  constexpr int kT = C::kTerms;
   constexpr int kATs = C::kATs;
   // block loops: unrolled where the whole block count is at most two
   constexpr int kU = BM <= 32 ? BM / 16 : 1;
@@ -158,13 +191,14 @@ __global__ void __launch_bounds__(kCtThreads, 2)
   uint8_t* Ks = base + C::kS0;
   uint8_t* Rs = Ks + C::kK;  // the values, then A^T
   float* AT = reinterpret_cast<float*>(Rs);
+  float* M2T = reinterpret_cast<float*>(Rs + C::kR);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int total = p.R * p.Hv;
   const int B = p.B;
 
   int slot = 0, n = 0;
-  int it = ct_next(p, blockIdx.x, total, slot, n);
+  int it = ct_next<CAUSAL>(p, blockIdx.x, total, slot, n);
   if (it < 0) return;  // the same answer on every thread
 
   if (tid == 0) {
@@ -172,6 +206,7 @@ __global__ void __launch_bounds__(kCtThreads, 2)
     tc::mbar_init(&sh.bar_s0, 1);
     tc::mbar_init(&sh.bar_k, 1);
     tc::mbar_init(&sh.bar_mma, 1);
+    tc::mbar_init(&sh.bar_g, 1);
     tc::fence_mbar_init();
   }
   if (warp == 0) tc::tmem_alloc(&sh.tmem_base, 256);
@@ -179,13 +214,14 @@ __global__ void __launch_bounds__(kCtThreads, 2)
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t tmem = sh.tmem_base;
-  const uint32_t tmS = tmem;             // S0^T hi [0,64) and lo [64,128); then D
-  const uint32_t tmW = tmem + 128;       // W^T; then delta'^T hi [0,kDP) and lo [kDP,2kDP)
-  // G: row t on lane kG0 + t, the top BM lanes (warps 2-3), so that warp 0,
-  // which also scans the gates and issues the copies and MMAs, is not the
-  // one building A^T
-  constexpr int kG0 = 128 - BM;
-  const uint32_t tmG = tmem + 128 + BM;
+  const uint32_t tmS = tmem;            // S0^T's terms, 64 columns each; then D
+  const uint32_t tmW = tmem + 64 * kT;  // W^T; then delta'^T's terms, kDP columns each
+  // G: row t on lane kG0 + t, the top lanes (warps 2-3), so that warp 0, which
+  // also scans the gates and issues the copies and MMAs, is not the one building
+  // A^T.  CAUSAL: the query rows after the key rows, in W^T's columns (read before
+  // W^T is formed)
+  constexpr int kG0 = 128 - (CAUSAL ? 2 : 1) * BM;
+  const uint32_t tmG = CAUSAL ? tmW : tmem + 128 + BM;
   const uint32_t lane_off = (uint32_t)(warp * 32) << 16;
 
   auto state_of = [&](int item, int s) {
@@ -203,7 +239,11 @@ __global__ void __launch_bounds__(kCtThreads, 2)
     const int r = item / p.Hv, j = item % p.Hv, h = j / (p.Hv / p.Hk);
     tc::mbar_expect_tx(&sh.bar_k, C::kK + C::kV);
     tc::tma_load_4d(Ks, &maps.k, &sh.bar_k, 0, h, 0, r);
-    tc::tma_load_4d(Ks + 64 * 128, &maps.k, &sh.bar_k, 64, h, 0, r);
+    tc::tma_load_4d(Ks + C::kRows * 128, &maps.k, &sh.bar_k, 64, h, 0, r);
+    if constexpr (CAUSAL) {
+      tc::tma_load_4d(Ks + BM * 128, &maps.q, &sh.bar_k, 0, h, 0, r);
+      tc::tma_load_4d(Ks + (C::kRows + BM) * 128, &maps.q, &sh.bar_k, 64, h, 0, r);
+    }
     tc::tma_load_4d(Rs, &maps.v, &sh.bar_k, 0, j, 0, r);
     tc::tma_load_4d(Rs + BM * 128, &maps.v, &sh.bar_k, 64, j, 0, r);
   };
@@ -242,9 +282,26 @@ __global__ void __launch_bounds__(kCtThreads, 2)
 
 #pragma unroll 1
   while (true) {
-    const int nb = (n + 15) >> 4;  // blocks of 16 tokens that take part
+    const int m = CAUSAL ? B : n;   // tokens that take part
+    const int nb = (m + 15) >> 4;  // and their blocks of 16
     // the block's gates: gamma = inclusive prefix sum of the log-gates
-    if (warp == 0) {
+    if (CAUSAL && warp == 0) {
+      double g = (double)gq0;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const double a = __shfl_up_sync(0xffffffffu, g, o);
+        if (lane >= o) g += a;
+      }
+      const double g2 = g * 1.4426950408889634;
+      const double gn2 = __shfl_sync(0xffffffffu, g2, (n - 1) & 31);
+      const float hi = rintf((float)g2 * 1024.f) * (1.f / 1024.f);
+      sh.gam2[lane] = hi;
+      sh.glo[lane] = (float)(g2 - (double)hi);
+      sh.Gam[lane] = expf((float)g);
+      sh.beta[lane] = bq0;
+      sh.dsc[lane] = lane < n ? tc::ex2((float)(gn2 - g2)) : 0.f;
+    }
+    if (!CAUSAL && warp == 0) {
       float g0 = gq0, g1 = gq1;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
@@ -274,12 +331,12 @@ __global__ void __launch_bounds__(kCtThreads, 2)
     // first such item after it (bad ones flagged on the way)
     int it_next = -1, slot_next = 0, n_next = 0;
     if (cand < total) {
-      if (cs >= 0 && cs < p.nslots && ca > 0 && ca <= B) {
+      if (cs >= 0 && cs < p.nslots && ca >= (CAUSAL ? 0 : 1) && ca <= B) {
         it_next = cand;
         slot_next = cs;
         n_next = ca;
       } else {
-        it_next = ct_next(p, cand, total, slot_next, n_next);
+        it_next = ct_next<CAUSAL>(p, cand, total, slot_next, n_next);
       }
     }
     if (it_next >= 0) {
@@ -291,37 +348,71 @@ __global__ void __launch_bounds__(kCtThreads, 2)
 
     if (!ct_wait(&sh.bar_s0, ph, sh, p.dev_status)) break;
     if (tid == 0) s0_out = false;
-    // S0^T (column c = tid of S0) into tensor memory as bf16 hi and lo parts
+    if (CAUSAL && warp == 0) {  // the Gram first, while the state is split
+      const bool ok = __all_sync(0xffffffffu, tc::mbar_wait(&sh.bar_k, ph, &sh.abort_flag));
+      tc::fence_after_sync();
+      if (ok && tc::elect_one()) {
+        const uint32_t idG = tc::idesc_bf16(128, BM, false, false);
+#pragma unroll 1
+        for (int kk = 0; kk < kCtD / 16; ++kk) {
+          const uint8_t* kc = Ks + (kk >> 2) * (C::kRows * 128) + (kk & 3) * 32;
+          tc::mma_bf16_ss(tmG, tc::sdesc_sw128(tc::smem_u32(kc - kG0 * 128), 16, 1024),
+                          tc::sdesc_sw128(tc::smem_u32(kc), 16, 1024), idG, kk > 0);
+        }
+        tc::mma_commit(&sh.bar_g);
+      }
+      __syncwarp();
+    }
+    // S0^T (column c = tid of S0) into tensor memory as bf16 terms
 #pragma unroll 1
     for (int i0 = 0; i0 < kCtD; i0 += 32) {
-      uint32_t hi[16], lo[16];
+      uint32_t w[kT][16];
 #pragma unroll
-      for (int e = 0; e < 16; ++e)
-        split_pair(S0s[(i0 + 2 * e) * kCtD + tid], S0s[(i0 + 2 * e + 1) * kCtD + tid], hi[e],
-                   lo[e]);
-      tc::tmem_st16(tmS + lane_off + i0 / 2, hi);
-      tc::tmem_st16(tmS + lane_off + 64 + i0 / 2, lo);
+      for (int e = 0; e < 16; ++e) {
+        uint32_t s[kT];
+        split_terms<kT>(S0s[(i0 + 2 * e) * kCtD + tid], S0s[(i0 + 2 * e + 1) * kCtD + tid], s);
+#pragma unroll
+        for (int x = 0; x < kT; ++x) w[x][e] = s[x];
+      }
+#pragma unroll
+      for (int x = 0; x < kT; ++x) tc::tmem_st16(tmS + lane_off + 64 * x + i0 / 2, w[x]);
     }
     tc::tmem_st_wait();
     tc::fence_before_sync();
     if (!ct_wait(&sh.bar_k, ph, sh, p.dev_status)) break;  // also orders the stores above
+    uint32_t gc[CAUSAL ? BM : 1];  // CAUSAL: this lane's row of G
+    if constexpr (CAUSAL) {
+      if (!ct_wait(&sh.bar_g, ph, sh, p.dev_status)) break;
+      tc::fence_after_sync();
+      if (warp >= kG0 / 32) {
+#pragma unroll
+        for (int c = 0; c < BM; c += 16)
+          tc::tmem_ld16(tmG + lane_off + c, *reinterpret_cast<uint32_t(*)[16]>(&gc[c]));
+        tc::tmem_ld_wait();
+      }
+      tc::fence_before_sync();
+      __syncthreads();  // G read: W^T may take its columns
+    }
     if (warp == 0) {  // converged; one elected lane issues
       k_out = false;
       mma_out = true;
       tc::fence_after_sync();
       if (tc::elect_one()) {
-        const uint32_t idN = tc::idesc_bf16(128, 16 * nb, false, false);
+        const uint32_t idN = tc::idesc_bf16(128, CAUSAL ? 2 * BM : 16 * nb, false, false);
 #pragma unroll 1  // unrolled, the descriptors are hoisted and the solve spills
         for (int kk = 0; kk < kCtD / 16; ++kk) {
-          const uint8_t* kc = Ks + (kk >> 2) * (64 * 128) + (kk & 3) * 32;
+          const uint8_t* kc = Ks + (kk >> 2) * (C::kRows * 128) + (kk & 3) * 32;
           const uint64_t kd = tc::sdesc_sw128(tc::smem_u32(kc), 16, 1024);
-          // A operand rows kG0.. are the keys; the rows before read the bytes
-          // ahead of the chunk (the state buffer, then the first chunk), which
-          // only reach lanes nobody reads
-          const uint64_t kg = tc::sdesc_sw128(tc::smem_u32(kc - kG0 * 128), 16, 1024);
-          tc::mma_bf16_ss(tmG, kg, kd, idN, kk > 0);                // G = K K^T
-          tc::mma_bf16_ts(tmW, tmS + kk * 8, kd, idN, kk > 0);      // W^T = S0hi^T K^T
-          tc::mma_bf16_ts(tmW, tmS + 64 + kk * 8, kd, idN, 1u);     //     + S0lo^T K^T
+          if constexpr (!CAUSAL) {
+            // A operand rows kG0.. are the keys; the rows before read the bytes
+            // ahead of the chunk (the state buffer, then the first chunk), which
+            // only reach lanes nobody reads
+            const uint64_t kg = tc::sdesc_sw128(tc::smem_u32(kc - kG0 * 128), 16, 1024);
+            tc::mma_bf16_ss(tmG, kg, kd, idN, kk > 0);  // G = K K^T
+          }
+#pragma unroll
+          for (int x = 0; x < kT; ++x)  // W^T = S0^T [K; Q]^T, term by term
+            tc::mma_bf16_ts(tmW, tmS + 64 * x + kk * 8, kd, idN, kk > 0 || x > 0);
         }
         tc::mma_commit(&sh.bar_mma);
       }
@@ -333,10 +424,35 @@ __global__ void __launch_bounds__(kCtThreads, 2)
       const uint8_t* vb = Rs + (tid >> 6) * (BM * 128) + (tid & 63) * 2;
 #pragma unroll
       for (int t0 = 0; t0 < BM; t0 += 16) {
-        if (t0 < n) {
+        if (t0 < m) {
 #pragma unroll
           for (int t = t0; t < t0 + 16; ++t)
             vraw[t] = *reinterpret_cast<const unsigned short*>(vb + t * 128);
+        }
+      }
+    }
+    if constexpr (CAUSAL) {
+      __syncthreads();  // the values are read: A^T may take their place
+      // A^T from the key rows of G and M2^T from its query rows, while W^T is formed:
+      // one path, the row factor and the end of the mask apart
+      if (warp >= kG0 / 32) {
+        const int row = tid - kG0, u = row & (BM - 1);
+        const bool key = row < BM;
+        const float rf = key ? sh.beta[u] : 1.f;
+        const float gh = sh.gam2[u], gl = sh.glo[u];
+        const int end = u < B ? (key ? u : u + 1) : 0;
+        float* dst = (key ? AT : M2T) + u;
+#pragma unroll
+        for (int i4 = 0; i4 < BM / 4; ++i4) {
+          const float4 h4 = *reinterpret_cast<const float4*>(&sh.gam2[4 * i4]);
+          const float4 l4 = *reinterpret_cast<const float4*>(&sh.glo[4 * i4]);
+          const float hv[4] = {h4.x, h4.y, h4.z, h4.w}, lv[4] = {l4.x, l4.y, l4.z, l4.w};
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const int i = 4 * i4 + e;
+            const float a = rf * tc::ex2((gh - hv[e]) + (gl - lv[e])) * __uint_as_float(gc[i]);
+            dst[i * kATs] = i < end ? a : 0.f;
+          }
         }
       }
     }
@@ -346,7 +462,7 @@ __global__ void __launch_bounds__(kCtThreads, 2)
     tc::fence_after_sync();
 
     // the accumulator starts at Gam_{n-1} S0^T (fp32, from the loaded state)
-    {
+    if (!CAUSAL || n > 0) {
       const float Gn = sh.Gam[n - 1];
 #pragma unroll 2
       for (int i0 = 0; i0 < kCtD; i0 += 16) {
@@ -358,7 +474,7 @@ __global__ void __launch_bounds__(kCtThreads, 2)
     }
     // A^T from the Gram rows t < BM (the warps holding those lanes); rows of
     // A at or past n are zero, so the solve below may run whole blocks
-    if (warp >= kG0 / 32) {
+    if (!CAUSAL && warp >= kG0 / 32) {
       const int t = tid - kG0;
       const float bt = t >= 0 ? sh.beta[t] : 0.f, gt = t >= 0 ? sh.gam2[t] : 0.f;
       constexpr int kC = 16;
@@ -392,7 +508,7 @@ __global__ void __launch_bounds__(kCtThreads, 2)
     float x[BM];
 #pragma unroll
     for (int c0 = 0; c0 < BM; c0 += 16) {
-      if (c0 >= n) break;  // uniform
+      if (c0 >= m) break;  // uniform
       uint32_t w[16];
       tc::tmem_ld16(tmW + lane_off + c0, w);
       tc::tmem_ld_wait();
@@ -406,6 +522,18 @@ __global__ void __launch_bounds__(kCtThreads, 2)
           const int t = c0 + 4 * e4 + e;
           x[t] = bb[e] * (__uint_as_float(vraw[t] << 16) - gg[e] * __uint_as_float(w[4 * e4 + e]));
         }
+      }
+    }
+    // CAUSAL: the outputs start at Gam_l S0^T q_l
+    float o[CAUSAL ? BM : 1];
+    if constexpr (CAUSAL) {
+#pragma unroll
+      for (int c0 = 0; c0 < BM; c0 += 16) {
+        uint32_t w[16];
+        tc::tmem_ld16(tmW + lane_off + BM + c0, w);
+        tc::tmem_ld_wait();
+#pragma unroll
+        for (int e = 0; e < 16; ++e) o[c0 + e] = sh.Gam[c0 + e] * __uint_as_float(w[e]);
       }
     }
     tc::fence_before_sync();
@@ -437,7 +565,7 @@ __global__ void __launch_bounds__(kCtThreads, 2)
           if (4 * u4 + 3 > t) x[4 * u4 + 3] = fmaf(-a.w, dt, x[4 * u4 + 3]);
         }
       }
-      uint32_t hi[8], lo[8];
+      uint32_t dw[kT][8];
 #pragma unroll
       for (int i4 = 0; i4 < 4; ++i4) {
         const float4 q = *reinterpret_cast<const float4*>(&sh.dsc[16 * b + 4 * i4]);
@@ -448,11 +576,30 @@ __global__ void __launch_bounds__(kCtThreads, 2)
           const float xv = x[4 * i4 + e] * dr[e];
           v[e] = 16 * b + 4 * i4 + e < n ? xv : 0.f;
         }
-        split_pair(v[0], v[1], hi[2 * i4], lo[2 * i4]);
-        split_pair(v[2], v[3], hi[2 * i4 + 1], lo[2 * i4 + 1]);
+#pragma unroll
+        for (int f = 0; f < 2; ++f) {
+          uint32_t s[kT];
+          split_terms<kT>(v[2 * f], v[2 * f + 1], s);
+#pragma unroll
+          for (int y = 0; y < kT; ++y) dw[y][2 * i4 + f] = s[y];
+        }
       }
-      tc::tmem_st8(tmW + lane_off + 8 * b, hi);
-      tc::tmem_st8(tmW + lane_off + C::kDP + 8 * b, lo);
+#pragma unroll
+      for (int y = 0; y < kT; ++y) tc::tmem_st8(tmW + lane_off + C::kDP * y + 8 * b, dw[y]);
+      if constexpr (CAUSAL) {  // the block's deltas into the outputs at and after it
+#pragma unroll
+        for (int t = 0; t < 16; ++t) {
+          const float dt = x[t];
+#pragma unroll
+          for (int l4 = 4 * b; l4 < BM / 4; ++l4) {
+            const float4 a = *reinterpret_cast<const float4*>(M2T + (16 * b + t) * kATs + 4 * l4);
+            o[4 * l4 + 0] = fmaf(a.x, dt, o[4 * l4 + 0]);
+            o[4 * l4 + 1] = fmaf(a.y, dt, o[4 * l4 + 1]);
+            o[4 * l4 + 2] = fmaf(a.z, dt, o[4 * l4 + 2]);
+            o[4 * l4 + 3] = fmaf(a.w, dt, o[4 * l4 + 3]);
+          }
+        }
+      }
 #pragma unroll
       for (int k = 1; k < BM / 16; ++k) {
         if (k < BM / 16 - (kU > 1 ? b : 0) && b + k < nb) {  // uniform
@@ -482,14 +629,29 @@ __global__ void __launch_bounds__(kCtThreads, 2)
       if (tc::elect_one()) {
         // D += delta'^T K: the keys [t][i] as an MN-major operand (i contiguous)
 #pragma unroll 1
-        for (int kk = 0; kk < nb; ++kk) {
-          const uint64_t kb = tc::sdesc_sw128(tc::smem_u32(Ks + kk * 2048), 64 * 128, 1024);
-          tc::mma_bf16_ts(tmS, tmW + kk * 8, kb, idU, 1u);
-          tc::mma_bf16_ts(tmS, tmW + C::kDP + kk * 8, kb, idU, 1u);
+        for (int kk = 0; kk < (n + 15) >> 4; ++kk) {
+          const uint64_t kb = tc::sdesc_sw128(tc::smem_u32(Ks + kk * 2048), C::kRows * 128, 1024);
+#pragma unroll
+          for (int y = 0; y < kT; ++y) tc::mma_bf16_ts(tmS, tmW + C::kDP * y + kk * 8, kb, idU, 1u);
         }
         tc::mma_commit(&sh.bar_mma);
       }
       __syncwarp();
+    }
+    if constexpr (CAUSAL) {
+      // adjacent lanes swap one value so that each stores a bf16 pair of two columns
+      const bool odd = lane & 1;
+      __nv_bfloat16* out = static_cast<__nv_bfloat16*>(p.out_causal) +
+                           ((size_t)(it / p.Hv) * B * p.Hv + it % p.Hv) * kCtD + (tid & ~1);
+#pragma unroll
+      for (int l = 0; l < BM; l += 2) {
+        const float a = p.scale * o[l], b = p.scale * o[l + 1];
+        const float recv = __shfl_xor_sync(0xffffffffu, odd ? a : b, 1);
+        const int row = odd ? l + 1 : l;
+        const __nv_bfloat162 w = odd ? __floats2bfloat162_rn(recv, b) : __floats2bfloat162_rn(a, recv);
+        if (row < B)
+          *reinterpret_cast<__nv_bfloat162*>(out + (size_t)row * p.Hv * kCtD) = w;
+      }
     }
     if (!ct_wait(&sh.bar_mma, ph_mma, sh, p.dev_status)) break;
     ph_mma ^= 1u;
@@ -504,7 +666,7 @@ __global__ void __launch_bounds__(kCtThreads, 2)
       }
     }
     // the committed state: lane c holds S^(n)[i][c] over i
-    {
+    if (!CAUSAL || n > 0) {
       float* Sg = state_of(it, slot) + tid;
 #pragma unroll 1
       for (int i0 = 0; i0 < kCtD; i0 += 32) {
@@ -529,6 +691,7 @@ __global__ void __launch_bounds__(kCtThreads, 2)
     if (s0_out) tc::mbar_wait(&sh.bar_s0, s0_par, nullptr, 100000000ull);
     if (k_out) tc::mbar_wait(&sh.bar_k, k_par, nullptr, 100000000ull);
     if (mma_out) tc::mbar_wait(&sh.bar_mma, ph_mma, nullptr, 100000000ull);
+    if (CAUSAL) tc::mbar_wait(&sh.bar_g, ph, nullptr, 100000000ull);
   }
   tc::fence_before_sync();
   __syncthreads();
@@ -572,14 +735,15 @@ bool ct_act_map(CUtensorMap* m, const void* x, int H, int B, int R, int rows, bo
          CUDA_SUCCESS;
 }
 
-template <int BM>
+template <int BM, bool CAUSAL>
 cudaError_t launch_ct(const GdrParams& p, cudaStream_t stream) {
   CtMaps maps;
-  if (!ct_act_map(&maps.k, p.k, p.Hk, p.B, p.R, 64, true) ||
+  if (!ct_act_map(&maps.k, p.k, p.Hk, p.B, p.R, CAUSAL ? BM : 64, true) ||
+      (CAUSAL && !ct_act_map(&maps.q, p.q, p.Hk, p.B, p.R, BM, true)) ||
       !ct_act_map(&maps.v, p.v, p.Hv, p.B, p.R, BM, false))
     return cudaErrorInvalidValue;
-  const int smem = CtCfg<BM>::kSmem + 1024;
-  cudaError_t e = cudaFuncSetAttribute(gdr_commit_tc_kernel<BM>,
+  const int smem = CtCfg<BM, CAUSAL>::kSmem + 1024;
+  cudaError_t e = cudaFuncSetAttribute(gdr_commit_tc_kernel<BM, CAUSAL>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
   int dev = 0, sms = kNumSMs;
@@ -587,21 +751,23 @@ cudaError_t launch_ct(const GdrParams& p, cudaStream_t stream) {
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const long items = (long)p.R * p.Hv;
   const int grid = (int)(items < 2L * sms ? items : 2L * sms);
-  gdr_commit_tc_kernel<BM><<<grid, kCtThreads, smem, stream>>>(maps, p);
+  gdr_commit_tc_kernel<BM, CAUSAL><<<grid, kCtThreads, smem, stream>>>(maps, p);
   note_launches(1);
   return cudaGetLastError();
 }
 
 }  // namespace
 
-bool gdr_commit_tc_supported(int B, int dk, int dv) {
-  return B >= 1 && B <= 64 && dk == kCtD && dv == kCtD;
+bool gdr_commit_tc_supported(int B, int dk, int dv, bool causal) {
+  return B >= (causal ? 9 : 1) && B <= (causal ? 32 : 64) && dk == kCtD && dv == kCtD;
 }
 
 cudaError_t launch_gdr_commit_tc(const GdrParams& p, cudaStream_t stream) {
   if (p.R == 0) return cudaSuccess;
-  if (p.B <= 16) return launch_ct<16>(p, stream);
-  return p.B <= 32 ? launch_ct<32>(p, stream) : launch_ct<64>(p, stream);
+  if (p.out_causal)
+    return p.B <= 16 ? launch_ct<16, true>(p, stream) : launch_ct<32, true>(p, stream);
+  if (p.B <= 16) return launch_ct<16, false>(p, stream);
+  return p.B <= 32 ? launch_ct<32, false>(p, stream) : launch_ct<64, false>(p, stream);
 }
 
 }  // namespace flare

@@ -1,0 +1,56 @@
+"""The tensor-core commit with token-causal outputs (B <= 32, 128 x 128 states) at the
+edges of its 16-token blocks, for ragged accepted lengths with zeros among them, and
+its precision: the fp32 operands enter as three bf16 terms, so a committed state is
+as close to 64 bits as the fp32 recurrence's (each about 2^-24 per product, a
+few such per sum: below 1e-6)."""
+import numpy as np
+import pytest
+import torch
+
+from gpu_helpers import assert_out_close, gen, install_states, oracle_commit, rel_fro, run_commit
+from paper_2606_01774_gb300 import workloads
+
+pytestmark = pytest.mark.gpu
+LARGE = workloads.WORKLOADS["serving_batch64"]
+STATE_REL = 1e-6
+
+
+@pytest.mark.parametrize("block", [1, 2, 15, 16, 17, 31, 32])
+@pytest.mark.parametrize("heads", [(16, 32), (3, 3)])
+def test_causal_commit_matches_oracle(block, heads):
+    spec = LARGE.replace(num_requests=6, block_len=block, num_qk_heads=heads[0],
+                         num_v_heads=heads[1], seed=200 + block)
+    w = gen(spec)
+    install_states(w)
+    pool = w.state_pool.clone()
+    acc = torch.tensor([0, block, block // 2, 1, max(block - 1, 0), 0], dtype=torch.int32).cuda()
+    out = run_commit(w, pool, causal=True, accept_len=acc)
+    ref = oracle_commit(w, w.state_pool, causal=True, accept_len=acc)
+    assert_out_close(out, ref["causal"], "bf16", f"B = {block}")
+    slots = w.state_slot.long()
+    got = pool[slots].double().cpu().numpy()
+    for r in range(spec.num_requests):
+        if acc[r] == 0:  # untouched, bit for bit
+            assert torch.equal(pool[slots[r]].view(torch.int32), w.state_pool[slots[r]].view(torch.int32))
+        else:
+            assert rel_fro(got[r], ref["state"][r]) < STATE_REL, (r, rel_fro(got[r], ref["state"][r]))
+
+
+def test_causal_commit_with_more_items_than_ctas():
+    # 40 requests x 32 heads on 304 CTAs: every CTA walks several items, some of
+    # them without accepted tokens
+    spec = LARGE.replace(num_requests=40, block_len=27, seed=219)
+    w = gen(spec)
+    install_states(w, requests=[0, 13, 39])
+    pool = w.state_pool.clone()
+    acc = (torch.arange(40, dtype=torch.int32) * 7 % 28).cuda()
+    out = run_commit(w, pool, causal=True, accept_len=acc)
+    sample = [0, 4, 13, 39]  # accepted 0, 0, 7, 21
+    ref = oracle_commit(w, w.state_pool, requests=sample, causal=True, accept_len=acc)
+    assert_out_close(out[sample], ref["causal"], "bf16", "sampled requests")
+    got = pool[w.state_slot.long()[sample]].double().cpu().numpy()
+    for i in range(len(sample)):
+        assert rel_fro(got[i], ref["state"][i]) < STATE_REL
+    used = torch.zeros(pool.shape[0], dtype=torch.bool)
+    used[w.state_slot.long().cpu()] = True
+    assert np.isnan(pool[(~used).cuda()].cpu().numpy()).all()  # free slots untouched
