@@ -51,7 +51,7 @@
 // as a multiple of 2^-10 and a remainder, whose differences are exact where they
 // matter: over 32 tokens the committed states are 1.7e-7 off 64 bits where the
 // recurrence's are 6.0e-7.  State update of 64 requests (32 heads): B = 32 208 ->
-// 118 us, B = 16 123 -> 81.  Blocks of 8 and fewer stay with the recurrence, which
+// 113 us, B = 16 123 -> 80.  Blocks of 8 and fewer stay with the recurrence, which
 // is as fast there (84 and 78 us at B = 8) and closer (1.15e-7 against 1.28e-7:
 // the tensor core's accumulation rounds toward zero); B = 33..64 would need 320
 // tensor-memory columns of the 256 that two CTAs per SM leave each.
@@ -108,16 +108,20 @@ struct CtMaps {
   CUtensorMap v;  // values (128, Hv, B, R) box (64, 1, BM, 1), no swizzle
 };
 
+// The gate factors of an item's tokens, 16-byte aligned (read as float4 broadcasts)
+struct alignas(16) CtGates {
+  float gam2[64];  // gamma_t log2(e) (CAUSAL: its multiple of 2^-10)
+  float glo[32];   // CAUSAL: the remainder
+  float Gam[64];   // exp(gamma_t)
+  float beta[64];
+  float dsc[64];   // exp(gamma_{n-1} - gamma_t) for t < n, else 0 (delta' factor)
+};
+
 struct alignas(16) CtShared {
   uint64_t bar_s0, bar_k, bar_mma, bar_g;
   uint32_t tmem_base;
   int abort_flag;
-  // 16-byte aligned: read as float4 broadcasts
-  alignas(16) float gam2[64];  // gamma_t log2(e) (CAUSAL: its multiple of 2^-10)
-  alignas(16) float glo[32];   // CAUSAL: the remainder
-  alignas(16) float Gam[64];   // exp(gamma_t)
-  alignas(16) float beta[64];
-  alignas(16) float dsc[64];   // exp(gamma_{n-1} - gamma_t) for t < n, else 0 (delta' factor)
+  CtGates g[2];  // this item's and the next one's
 };
 
 __device__ __forceinline__ bool ct_wait(uint64_t* bar, uint32_t parity, CtShared& sh,
@@ -256,6 +260,51 @@ __global__ void __launch_bounds__(kCtThreads, 2)
     bq0 = lane < B ? p.beta[gb + (size_t)lane * p.Hv] : 0.f;
     bq1 = lane + 32 < B ? p.beta[gb + (size_t)(lane + 32) * p.Hv] : 0.f;
   };
+  // warp 0: the gate factors of the item whose gates it holds (gamma = inclusive
+  // prefix sum of the log-gates), while another item's products run
+  auto gate_factors = [&](CtGates& g, int n) {
+    if constexpr (CAUSAL) {
+      double s = (double)gq0;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const double a = __shfl_up_sync(0xffffffffu, s, o);
+        if (lane >= o) s += a;
+      }
+      const double g2 = s * 1.4426950408889634;
+      const double gn2 = __shfl_sync(0xffffffffu, g2, (n - 1) & 31);
+      const float hi = rintf((float)g2 * 1024.f) * (1.f / 1024.f);
+      g.gam2[lane] = hi;
+      g.glo[lane] = (float)(g2 - (double)hi);
+      g.Gam[lane] = expf((float)s);
+      g.beta[lane] = bq0;
+      g.dsc[lane] = lane < n ? tc::ex2((float)(gn2 - g2)) : 0.f;
+    } else {
+      float g0 = gq0, g1 = gq1;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const float a = __shfl_up_sync(0xffffffffu, g0, o);
+        const float b = __shfl_up_sync(0xffffffffu, g1, o);
+        if (lane >= o) {
+          g0 += a;
+          g1 += b;
+        }
+      }
+      g1 += __shfl_sync(0xffffffffu, g0, 31);
+      const float g20 = g0 * 1.4426950408889634f, g21 = g1 * 1.4426950408889634f;
+      // gamma_{n-1}: lane (n - 1) % 32 of the half holding it
+      const float gn0 = __shfl_sync(0xffffffffu, g20, (n - 1) & 31);
+      const float gn1 = __shfl_sync(0xffffffffu, g21, (n - 1) & 31);
+      const float gn2 = n > 32 ? gn1 : gn0;
+      g.gam2[lane] = g20;
+      g.gam2[lane + 32] = g21;
+      g.Gam[lane] = expf(g0);
+      g.Gam[lane + 32] = expf(g1);
+      g.beta[lane] = bq0;
+      g.beta[lane + 32] = bq1;
+      g.dsc[lane] = lane < n ? tc::ex2(gn2 - g20) : 0.f;
+      g.dsc[lane + 32] = lane + 32 < n ? tc::ex2(gn2 - g21) : 0.f;
+    }
+  };
   // slot and accepted length of the candidate after the next item, one item ahead
   auto cand_slot = [&](int c) { return c < total ? p.state_slot[c / p.Hv] : -1; };
   auto cand_len = [&](int c) {
@@ -273,7 +322,15 @@ __global__ void __launch_bounds__(kCtThreads, 2)
     issue_kv(it);
     s0_out = k_out = true;
   }
-  if (warp == 0) load_gates(it);
+  // where the wait for W^T has room for it, the next item's gate factors are formed
+  // there (256 requests of 16 heads, B = 16: 97.5 -> 94.6 us; CAUSAL, B = 32, 64
+  // requests: 118 -> 113); elsewhere while the state is waited for (CAUSAL, B = 16:
+  // 141.6 and 144 early)
+  constexpr bool kEarly = BM == 32 || (BM == 16 && !CAUSAL);
+  if (warp == 0) {
+    load_gates(it);
+    if (kEarly) gate_factors(sh.g[0], n);
+  }
   int cand = it + gridDim.x;
   int cs = cand_slot(cand), ca = cand_len(cand);
   uint32_t ph = 0;      // parity of the item's state and key/value loads
@@ -282,51 +339,10 @@ __global__ void __launch_bounds__(kCtThreads, 2)
 
 #pragma unroll 1
   while (true) {
+    const CtGates& gt = sh.g[kEarly ? ph : 0];
+    if (!kEarly && warp == 0) gate_factors(sh.g[0], n);
     const int m = CAUSAL ? B : n;   // tokens that take part
     const int nb = (m + 15) >> 4;  // and their blocks of 16
-    // the block's gates: gamma = inclusive prefix sum of the log-gates
-    if (CAUSAL && warp == 0) {
-      double g = (double)gq0;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const double a = __shfl_up_sync(0xffffffffu, g, o);
-        if (lane >= o) g += a;
-      }
-      const double g2 = g * 1.4426950408889634;
-      const double gn2 = __shfl_sync(0xffffffffu, g2, (n - 1) & 31);
-      const float hi = rintf((float)g2 * 1024.f) * (1.f / 1024.f);
-      sh.gam2[lane] = hi;
-      sh.glo[lane] = (float)(g2 - (double)hi);
-      sh.Gam[lane] = expf((float)g);
-      sh.beta[lane] = bq0;
-      sh.dsc[lane] = lane < n ? tc::ex2((float)(gn2 - g2)) : 0.f;
-    }
-    if (!CAUSAL && warp == 0) {
-      float g0 = gq0, g1 = gq1;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const float a = __shfl_up_sync(0xffffffffu, g0, o);
-        const float b = __shfl_up_sync(0xffffffffu, g1, o);
-        if (lane >= o) {
-          g0 += a;
-          g1 += b;
-        }
-      }
-      g1 += __shfl_sync(0xffffffffu, g0, 31);
-      const float g20 = g0 * 1.4426950408889634f, g21 = g1 * 1.4426950408889634f;
-      // gamma_{n-1}: lane (n - 1) % 32 of the half holding it
-      const float gn0 = __shfl_sync(0xffffffffu, g20, (n - 1) & 31);
-      const float gn1 = __shfl_sync(0xffffffffu, g21, (n - 1) & 31);
-      const float gn2 = n > 32 ? gn1 : gn0;
-      sh.gam2[lane] = g20;
-      sh.gam2[lane + 32] = g21;
-      sh.Gam[lane] = expf(g0);
-      sh.Gam[lane + 32] = expf(g1);
-      sh.beta[lane] = bq0;
-      sh.beta[lane + 32] = bq1;
-      sh.dsc[lane] = lane < n ? tc::ex2(gn2 - g20) : 0.f;
-      sh.dsc[lane + 32] = lane + 32 < n ? tc::ex2(gn2 - g21) : 0.f;
-    }
     // the next item: the candidate when it is valid and has n > 0, else the
     // first such item after it (bad ones flagged on the way)
     int it_next = -1, slot_next = 0, n_next = 0;
@@ -431,6 +447,7 @@ __global__ void __launch_bounds__(kCtThreads, 2)
         }
       }
     }
+    if (kEarly && warp == 0 && it_next >= 0) gate_factors(sh.g[ph ^ 1], n_next);
     if constexpr (CAUSAL) {
       __syncthreads();  // the values are read: A^T may take their place
       // A^T from the key rows of G and M2^T from its query rows, while W^T is formed:
@@ -438,14 +455,14 @@ __global__ void __launch_bounds__(kCtThreads, 2)
       if (warp >= kG0 / 32) {
         const int row = tid - kG0, u = row & (BM - 1);
         const bool key = row < BM;
-        const float rf = key ? sh.beta[u] : 1.f;
-        const float gh = sh.gam2[u], gl = sh.glo[u];
+        const float rf = key ? gt.beta[u] : 1.f;
+        const float gh = gt.gam2[u], gl = gt.glo[u];
         const int end = u < B ? (key ? u : u + 1) : 0;
         float* dst = (key ? AT : M2T) + u;
 #pragma unroll
         for (int i4 = 0; i4 < BM / 4; ++i4) {
-          const float4 h4 = *reinterpret_cast<const float4*>(&sh.gam2[4 * i4]);
-          const float4 l4 = *reinterpret_cast<const float4*>(&sh.glo[4 * i4]);
+          const float4 h4 = *reinterpret_cast<const float4*>(&gt.gam2[4 * i4]);
+          const float4 l4 = *reinterpret_cast<const float4*>(&gt.glo[4 * i4]);
           const float hv[4] = {h4.x, h4.y, h4.z, h4.w}, lv[4] = {l4.x, l4.y, l4.z, l4.w};
 #pragma unroll
           for (int e = 0; e < 4; ++e) {
@@ -463,7 +480,7 @@ __global__ void __launch_bounds__(kCtThreads, 2)
 
     // the accumulator starts at Gam_{n-1} S0^T (fp32, from the loaded state)
     if (!CAUSAL || n > 0) {
-      const float Gn = sh.Gam[n - 1];
+      const float Gn = gt.Gam[n - 1];
 #pragma unroll 2
       for (int i0 = 0; i0 < kCtD; i0 += 16) {
         uint32_t d[16];
@@ -476,7 +493,7 @@ __global__ void __launch_bounds__(kCtThreads, 2)
     // A at or past n are zero, so the solve below may run whole blocks
     if (!CAUSAL && warp >= kG0 / 32) {
       const int t = tid - kG0;
-      const float bt = t >= 0 ? sh.beta[t] : 0.f, gt = t >= 0 ? sh.gam2[t] : 0.f;
+      const float bt = t >= 0 ? gt.beta[t] : 0.f, gm = t >= 0 ? gt.gam2[t] : 0.f;
       constexpr int kC = 16;
 #pragma unroll kU
       for (int b = 0; b < BM / 16; ++b) {
@@ -492,12 +509,12 @@ __global__ void __launch_bounds__(kCtThreads, 2)
           // select: a branch per element would serialise the chains
 #pragma unroll
           for (int i4 = 0; i4 < kC / 4; ++i4) {
-            const float4 q = *reinterpret_cast<const float4*>(&sh.gam2[c0 + 4 * i4]);
+            const float4 q = *reinterpret_cast<const float4*>(&gt.gam2[c0 + 4 * i4]);
             const float gi[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
               const int i = c0 + 4 * i4 + e;
-              const float a = bt * tc::ex2(gt - gi[e]) * __uint_as_float(gr[4 * i4 + e]);
+              const float a = bt * tc::ex2(gm - gi[e]) * __uint_as_float(gr[4 * i4 + e]);
               AT[i * kATs + t] = (t < n && i < t) ? a : 0.f;
             }
           }
@@ -514,8 +531,8 @@ __global__ void __launch_bounds__(kCtThreads, 2)
       tc::tmem_ld_wait();
 #pragma unroll
       for (int e4 = 0; e4 < 4; ++e4) {
-        const float4 b4 = *reinterpret_cast<const float4*>(&sh.beta[c0 + 4 * e4]);
-        const float4 g4 = *reinterpret_cast<const float4*>(&sh.Gam[c0 + 4 * e4]);
+        const float4 b4 = *reinterpret_cast<const float4*>(&gt.beta[c0 + 4 * e4]);
+        const float4 g4 = *reinterpret_cast<const float4*>(&gt.Gam[c0 + 4 * e4]);
         const float bb[4] = {b4.x, b4.y, b4.z, b4.w}, gg[4] = {g4.x, g4.y, g4.z, g4.w};
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
@@ -523,6 +540,15 @@ __global__ void __launch_bounds__(kCtThreads, 2)
           x[t] = bb[e] * (__uint_as_float(vraw[t] << 16) - gg[e] * __uint_as_float(w[4 * e4 + e]));
         }
       }
+    }
+    // CAUSAL: keys at and past n to zero for the update (their deltas are zero there,
+    // but a rejected token's key may be infinite or NaN)
+    if constexpr (CAUSAL) {
+      const int n16 = (((n + 15) & ~15) - n) * 16;  // 16-byte pieces: 8 of each 64-column chunk
+      for (int e = tid; e < n16; e += kCtThreads)
+        *reinterpret_cast<uint4*>(Ks + ((e >> 3) & 1) * (C::kRows * 128) + (n + (e >> 4)) * 128 +
+                                  (e & 7) * 16) = make_uint4(0u, 0u, 0u, 0u);
+      tc::fence_async_smem();
     }
     // CAUSAL: the outputs start at Gam_l S0^T q_l
     float o[CAUSAL ? BM : 1];
@@ -533,7 +559,7 @@ __global__ void __launch_bounds__(kCtThreads, 2)
         tc::tmem_ld16(tmW + lane_off + BM + c0, w);
         tc::tmem_ld_wait();
 #pragma unroll
-        for (int e = 0; e < 16; ++e) o[c0 + e] = sh.Gam[c0 + e] * __uint_as_float(w[e]);
+        for (int e = 0; e < 16; ++e) o[c0 + e] = gt.Gam[c0 + e] * __uint_as_float(w[e]);
       }
     }
     tc::fence_before_sync();
@@ -568,7 +594,7 @@ __global__ void __launch_bounds__(kCtThreads, 2)
       uint32_t dw[kT][8];
 #pragma unroll
       for (int i4 = 0; i4 < 4; ++i4) {
-        const float4 q = *reinterpret_cast<const float4*>(&sh.dsc[16 * b + 4 * i4]);
+        const float4 q = *reinterpret_cast<const float4*>(&gt.dsc[16 * b + 4 * i4]);
         const float dr[4] = {q.x, q.y, q.z, q.w};
         float v[4];
 #pragma unroll
@@ -586,16 +612,18 @@ __global__ void __launch_bounds__(kCtThreads, 2)
       }
 #pragma unroll
       for (int y = 0; y < kT; ++y) tc::tmem_st8(tmW + lane_off + C::kDP * y + 8 * b, dw[y]);
-      if constexpr (CAUSAL) {  // the block's deltas into the outputs at and after it
+      if constexpr (CAUSAL) {
+        // the block's deltas into the outputs at and after their tokens (only those: an
+        // infinite or NaN delta must not reach an earlier output through 0 * NaN)
 #pragma unroll
         for (int t = 0; t < 16; ++t) {
           const float dt = x[t];
 #pragma unroll
-          for (int l4 = 4 * b; l4 < BM / 4; ++l4) {
+          for (int l4 = 4 * b + t / 4; l4 < BM / 4; ++l4) {
             const float4 a = *reinterpret_cast<const float4*>(M2T + (16 * b + t) * kATs + 4 * l4);
-            o[4 * l4 + 0] = fmaf(a.x, dt, o[4 * l4 + 0]);
-            o[4 * l4 + 1] = fmaf(a.y, dt, o[4 * l4 + 1]);
-            o[4 * l4 + 2] = fmaf(a.z, dt, o[4 * l4 + 2]);
+            if (4 * l4 + 0 >= 16 * b + t) o[4 * l4 + 0] = fmaf(a.x, dt, o[4 * l4 + 0]);
+            if (4 * l4 + 1 >= 16 * b + t) o[4 * l4 + 1] = fmaf(a.y, dt, o[4 * l4 + 1]);
+            if (4 * l4 + 2 >= 16 * b + t) o[4 * l4 + 2] = fmaf(a.z, dt, o[4 * l4 + 2]);
             o[4 * l4 + 3] = fmaf(a.w, dt, o[4 * l4 + 3]);
           }
         }

@@ -54,3 +54,24 @@ def test_causal_commit_with_more_items_than_ctas():
     used = torch.zeros(pool.shape[0], dtype=torch.bool)
     used[w.state_slot.long().cpu()] = True
     assert np.isnan(pool[(~used).cuda()].cpu().numpy()).all()  # free slots untouched
+
+
+@pytest.mark.parametrize("block,token", [(32, 20), (16, 3), (27, 16)])
+def test_infinite_and_nan_tokens_stay_after_their_place(block, token):
+    """A token whose key or value is infinite or NaN changes no output before it and no
+    state committed before it."""
+    spec = LARGE.replace(num_requests=4, block_len=block, seed=230 + block)
+    w = gen(spec)
+    install_states(w)
+    acc = torch.tensor([token, 0, token - 1, 1], dtype=torch.int32).cuda()
+    clean_pool, pool = w.state_pool.clone(), w.state_pool.clone()
+    clean = run_commit(w, clean_pool, causal=True, accept_len=acc)
+    w.commit.v[0, token, :, 5] = float("inf")
+    w.commit.v[1, token] = float("nan")
+    w.commit.k[2, token, :, 0] = float("nan")
+    w.commit.k[3, token] = float("inf")
+    out = run_commit(w, pool, causal=True, accept_len=acc)
+    assert torch.equal(out[:, :token], clean[:, :token])
+    slots = w.state_slot.long()
+    assert torch.equal(pool[slots], clean_pool[slots])
+    assert not torch.isfinite(out[:, token:].float()).all()
