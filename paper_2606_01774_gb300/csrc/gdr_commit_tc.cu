@@ -44,14 +44,15 @@
 //   M2[l][i] = exp(gamma_l - gamma_i) (q_l . k_i),   i <= l < B
 //   out[l]   = s (Gam_l S0^T q_l + sum_{i<=l} M2[l][i] delta_i)
 //
-// G takes the query rows and W^T the query columns as well, and a thread
-// accumulates its column's outputs as its deltas become final.  The register
+// G takes the query rows and W^T the query columns as well, and the sum is a
+// product of the deltas and M2 in two bf16 terms each (2^-16, below the outputs'
+// rounding).  The register
 // recurrence that this replaces is exact fp32, so the fp32 operands enter as three
 // bf16 terms (24 bits) and the log-gates are summed in double precision and kept
 // as a multiple of 2^-10 and a remainder, whose differences are exact where they
 // matter: over 32 tokens the committed states are 1.7e-7 off 64 bits where the
 // recurrence's are 6.0e-7.  State update of 64 requests (32 heads): B = 32 208 ->
-// 113 us, B = 16 123 -> 80.  Blocks of 8 and fewer stay with the recurrence, which
+// 107 us, B = 16 123 -> 80.  Blocks of 8 and fewer stay with the recurrence, which
 // is as fast there (84 and 78 us at B = 8) and closer (1.15e-7 against 1.28e-7:
 // the tensor core's accumulation rounds toward zero); B = 33..64 would need 320
 // tensor-memory columns of the 256 that two CTAs per SM leave each.
@@ -96,7 +97,7 @@ struct CtCfg {
   static constexpr int kR = kAT > kV ? kAT : kV;
   // tensor-memory columns of each bf16 part of delta'^T (whole 16-column stores)
   static constexpr int kDP = BM / 2 < 16 ? 16 : BM / 2;
-  static constexpr int kM2 = CAUSAL ? kAT : 0;     // M2^T[i][l] = M2[l][i]
+  static constexpr int kM2 = CAUSAL ? 2 * BM * 128 : 0;  // M2[l][i] bf16 hi, lo (K-major SW128)
   static constexpr int kSmem = kS0 + kK + kR + kM2;
   static constexpr int kTerms = CAUSAL ? 3 : 2;    // bf16 terms of an fp32 operand
 };
@@ -193,9 +194,9 @@ __global__ void __launch_bounds__(kCtThreads, 2)
   uint8_t* base = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   float* S0s = reinterpret_cast<float*>(base);
   uint8_t* Ks = base + C::kS0;
-  uint8_t* Rs = Ks + C::kK;  // the values, then A^T
+  uint8_t* M2s = Ks + C::kK;
+  uint8_t* Rs = M2s + C::kM2;  // the values, then A^T
   float* AT = reinterpret_cast<float*>(Rs);
-  float* M2T = reinterpret_cast<float*>(Rs + C::kR);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int total = p.R * p.Hv;
@@ -226,6 +227,9 @@ __global__ void __launch_bounds__(kCtThreads, 2)
   // W^T is formed)
   constexpr int kG0 = 128 - (CAUSAL ? 2 : 1) * BM;
   const uint32_t tmG = CAUSAL ? tmW : tmem + 128 + BM;
+  // CAUSAL, in the state's third term once W^T is formed: delta^T hi and lo (BM / 2
+  // columns each) and O2^T
+  const uint32_t tmX = tmS + 128, tmO = tmS + 160;
   const uint32_t lane_off = (uint32_t)(warp * 32) << 16;
 
   auto state_of = [&](int item, int s) {
@@ -324,7 +328,7 @@ __global__ void __launch_bounds__(kCtThreads, 2)
   }
   // where the wait for W^T has room for it, the next item's gate factors are formed
   // there (256 requests of 16 heads, B = 16: 97.5 -> 94.6 us; CAUSAL, B = 32, 64
-  // requests: 118 -> 113); elsewhere while the state is waited for (CAUSAL, B = 16:
+  // requests: 5 us of 118); elsewhere while the state is waited for (CAUSAL, B = 16:
   // 141.6 and 144 early)
   constexpr bool kEarly = BM == 32 || (BM == 16 && !CAUSAL);
   if (warp == 0) {
@@ -398,7 +402,7 @@ __global__ void __launch_bounds__(kCtThreads, 2)
     if (!ct_wait(&sh.bar_k, ph, sh, p.dev_status)) break;  // also orders the stores above
     uint32_t gc[CAUSAL ? BM : 1];  // CAUSAL: this lane's row of G
     if constexpr (CAUSAL) {
-      if (!ct_wait(&sh.bar_g, ph, sh, p.dev_status)) break;
+      if (!ct_wait(&sh.bar_g, 0, sh, p.dev_status)) break;  // two completions per item
       tc::fence_after_sync();
       if (warp >= kG0 / 32) {
 #pragma unroll
@@ -450,27 +454,42 @@ __global__ void __launch_bounds__(kCtThreads, 2)
     if (kEarly && warp == 0 && it_next >= 0) gate_factors(sh.g[ph ^ 1], n_next);
     if constexpr (CAUSAL) {
       __syncthreads();  // the values are read: A^T may take their place
-      // A^T from the key rows of G and M2^T from its query rows, while W^T is formed:
-      // one path, the row factor and the end of the mask apart
+      // A^T from the key rows of G and M2 from its query rows, while W^T is formed:
+      // one path, the row factor, the end of the mask and the destination apart
       if (warp >= kG0 / 32) {
         const int row = tid - kG0, u = row & (BM - 1);
         const bool key = row < BM;
         const float rf = key ? gt.beta[u] : 1.f;
         const float gh = gt.gam2[u], gl = gt.glo[u];
         const int end = u < B ? (key ? u : u + 1) : 0;
-        float* dst = (key ? AT : M2T) + u;
 #pragma unroll
-        for (int i4 = 0; i4 < BM / 4; ++i4) {
-          const float4 h4 = *reinterpret_cast<const float4*>(&gt.gam2[4 * i4]);
-          const float4 l4 = *reinterpret_cast<const float4*>(&gt.glo[4 * i4]);
-          const float hv[4] = {h4.x, h4.y, h4.z, h4.w}, lv[4] = {l4.x, l4.y, l4.z, l4.w};
+        for (int i8 = 0; i8 < BM / 8; ++i8) {
+          float v[8];
 #pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const int i = 4 * i4 + e;
-            const float a = rf * tc::ex2((gh - hv[e]) + (gl - lv[e])) * __uint_as_float(gc[i]);
-            dst[i * kATs] = i < end ? a : 0.f;
+          for (int h = 0; h < 2; ++h) {
+            const float4 h4 = *reinterpret_cast<const float4*>(&gt.gam2[8 * i8 + 4 * h]);
+            const float4 l4 = *reinterpret_cast<const float4*>(&gt.glo[8 * i8 + 4 * h]);
+            const float hv[4] = {h4.x, h4.y, h4.z, h4.w}, lv[4] = {l4.x, l4.y, l4.z, l4.w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              const int i = 8 * i8 + 4 * h + e;
+              const float a = rf * tc::ex2((gh - hv[e]) + (gl - lv[e])) * __uint_as_float(gc[i]);
+              v[4 * h + e] = i < end ? a : 0.f;
+            }
+          }
+          if (key) {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) AT[(8 * i8 + e) * kATs + u] = v[e];
+          } else {
+            uint32_t s[4][2];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) split_terms<2>(v[2 * e], v[2 * e + 1], s[e]);
+            uint8_t* dst = M2s + u * 128 + ((i8 ^ (u & 7)) << 4);
+            *reinterpret_cast<uint4*>(dst) = make_uint4(s[0][0], s[1][0], s[2][0], s[3][0]);
+            *reinterpret_cast<uint4*>(dst + BM * 128) = make_uint4(s[0][1], s[1][1], s[2][1], s[3][1]);
           }
         }
+        tc::fence_async_smem();  // M2 is an MMA operand
       }
     }
     if (!ct_wait(&sh.bar_mma, ph_mma, sh, p.dev_status)) break;  // the values are read
@@ -552,6 +571,7 @@ __global__ void __launch_bounds__(kCtThreads, 2)
     }
     // CAUSAL: the outputs start at Gam_l S0^T q_l
     float o[CAUSAL ? BM : 1];
+    int first_bad = BM;  // the first token whose delta is infinite or NaN in this column
     if constexpr (CAUSAL) {
 #pragma unroll
       for (int c0 = 0; c0 < BM; c0 += 16) {
@@ -613,20 +633,26 @@ __global__ void __launch_bounds__(kCtThreads, 2)
 #pragma unroll
       for (int y = 0; y < kT; ++y) tc::tmem_st8(tmW + lane_off + C::kDP * y + 8 * b, dw[y]);
       if constexpr (CAUSAL) {
-        // the block's deltas into the outputs at and after their tokens (only those: an
-        // infinite or NaN delta must not reach an earlier output through 0 * NaN)
+        // delta as the readout's operand: zero where infinite or NaN, which must not
+        // reach the outputs before its token through 0 * NaN
+        uint32_t xh[8], xl[8];
 #pragma unroll
-        for (int t = 0; t < 16; ++t) {
-          const float dt = x[t];
+        for (int e = 0; e < 8; ++e) {
+          float v[2];
 #pragma unroll
-          for (int l4 = 4 * b + t / 4; l4 < BM / 4; ++l4) {
-            const float4 a = *reinterpret_cast<const float4*>(M2T + (16 * b + t) * kATs + 4 * l4);
-            if (4 * l4 + 0 >= 16 * b + t) o[4 * l4 + 0] = fmaf(a.x, dt, o[4 * l4 + 0]);
-            if (4 * l4 + 1 >= 16 * b + t) o[4 * l4 + 1] = fmaf(a.y, dt, o[4 * l4 + 1]);
-            if (4 * l4 + 2 >= 16 * b + t) o[4 * l4 + 2] = fmaf(a.z, dt, o[4 * l4 + 2]);
-            o[4 * l4 + 3] = fmaf(a.w, dt, o[4 * l4 + 3]);
+          for (int f = 0; f < 2; ++f) {
+            const int t = 2 * e + f;
+            const bool fin = fabsf(x[t]) < INFINITY;
+            v[f] = fin ? x[t] : 0.f;
+            first_bad = min(first_bad, fin ? BM : 16 * b + t);
           }
+          uint32_t s[2];
+          split_terms<2>(v[0], v[1], s);
+          xh[e] = s[0];
+          xl[e] = s[1];
         }
+        tc::tmem_st8(tmX + lane_off + 8 * b, xh);
+        tc::tmem_st8(tmX + lane_off + BM / 2 + 8 * b, xl);
       }
 #pragma unroll
       for (int k = 1; k < BM / 16; ++k) {
@@ -655,6 +681,18 @@ __global__ void __launch_bounds__(kCtThreads, 2)
       mma_out = true;
       tc::fence_after_sync();
       if (tc::elect_one()) {
+        if constexpr (CAUSAL) {  // O2^T = delta^T M2^T
+          const uint32_t idO = tc::idesc_bf16(128, BM, false, false);
+#pragma unroll
+          for (int kk = 0; kk < BM / 16; ++kk) {
+            const uint64_t mh = tc::sdesc_sw128(tc::smem_u32(M2s + kk * 32), 16, 1024);
+            const uint64_t ml = tc::sdesc_sw128(tc::smem_u32(M2s + BM * 128 + kk * 32), 16, 1024);
+            tc::mma_bf16_ts(tmO, tmX + kk * 8, mh, idO, kk > 0);
+            tc::mma_bf16_ts(tmO, tmX + kk * 8, ml, idO, 1u);
+            tc::mma_bf16_ts(tmO, tmX + BM / 2 + kk * 8, mh, idO, 1u);
+          }
+          tc::mma_commit(&sh.bar_g);
+        }
         // D += delta'^T K: the keys [t][i] as an MN-major operand (i contiguous)
 #pragma unroll 1
         for (int kk = 0; kk < (n + 15) >> 4; ++kk) {
@@ -667,6 +705,20 @@ __global__ void __launch_bounds__(kCtThreads, 2)
       __syncwarp();
     }
     if constexpr (CAUSAL) {
+      if (!ct_wait(&sh.bar_g, 1, sh, p.dev_status)) break;
+      tc::fence_after_sync();
+#pragma unroll
+      for (int c0 = 0; c0 < BM; c0 += 16) {
+        uint32_t w[16];
+        tc::tmem_ld16(tmO + lane_off + c0, w);
+        tc::tmem_ld_wait();
+#pragma unroll
+        for (int e = 0; e < 16; ++e) o[c0 + e] += __uint_as_float(w[e]);
+      }
+      if (first_bad < BM) {
+#pragma unroll
+        for (int l = 0; l < BM; ++l) o[l] = l < first_bad ? o[l] : __uint_as_float(0x7fffffffu);
+      }
       // adjacent lanes swap one value so that each stores a bf16 pair of two columns
       const bool odd = lane & 1;
       __nv_bfloat16* out = static_cast<__nv_bfloat16*>(p.out_causal) +
@@ -719,7 +771,10 @@ __global__ void __launch_bounds__(kCtThreads, 2)
     if (s0_out) tc::mbar_wait(&sh.bar_s0, s0_par, nullptr, 100000000ull);
     if (k_out) tc::mbar_wait(&sh.bar_k, k_par, nullptr, 100000000ull);
     if (mma_out) tc::mbar_wait(&sh.bar_mma, ph_mma, nullptr, 100000000ull);
-    if (CAUSAL) tc::mbar_wait(&sh.bar_g, ph, nullptr, 100000000ull);
+    if (CAUSAL) {  // whichever of the item's two completions is under way
+      tc::mbar_wait(&sh.bar_g, 0, nullptr, 50000000ull);
+      tc::mbar_wait(&sh.bar_g, 1, nullptr, 50000000ull);
+    }
   }
   tc::fence_before_sync();
   __syncthreads();
