@@ -548,10 +548,6 @@ cudaError_t launch_lin_tc(const GdrParams& p, cudaStream_t stream) {
 
 }  // namespace
 
-bool gdr_denoise_tc_supported(int B, int dk, int dv) {
-  return B >= 1 && B <= kBmax && (dk == 64 || dk == 128) && (dv == 64 || dv == 128);
-}
-
 cudaError_t launch_gdr_denoise_tc(const GdrParams& p, cudaStream_t stream) {
   if (p.dk == 128 && p.dv == 128) return launch_lin_tc<128, 128>(p, stream);
   if (p.dk == 128 && p.dv == 64) return launch_lin_tc<128, 64>(p, stream);

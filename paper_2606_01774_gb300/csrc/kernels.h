@@ -71,7 +71,6 @@ struct SoftmaxPlan {
   size_t workspace_bytes;
 };
 
-bool gdr_denoise_tc_supported(int B, int dk, int dv);
 bool gdr_denoise_persist_supported(int B, int dk, int dv);
 cudaError_t launch_gdr_denoise_persist(const GdrParams& p, cudaStream_t stream);
 bool gdr_denoise_chunk64_supported(int B, int dk, int dv);
