@@ -325,8 +325,12 @@ flare_status flare_verify_linear_attn(const flare_linear_desc* d, int32_t max_ve
   p.max_verify = max_verify;
   p.verify_states = verify_states;
   p.dev_status = dev_status;
-  const cudaError_t e = launch_gdr_verify(p, d->act_dtype == FLARE_DT_BF16,
-                                          static_cast<cudaStream_t>(stream));
+  const bool bf16 = d->act_dtype == FLARE_DT_BF16;
+  // as for the commit with token-causal outputs
+  const cudaError_t e =
+      (bf16 && gdr_commit_tc_supported(p.B, p.dk, p.dv, true))
+          ? launch_gdr_commit_tc(p, static_cast<cudaStream_t>(stream))
+          : launch_gdr_verify(p, bf16, static_cast<cudaStream_t>(stream));
   return e == cudaSuccess ? FLARE_OK : FLARE_ERR_CUDA;
 }
 

@@ -32,6 +32,10 @@
 // token K is written to the pool, and the draft rows read the block-end state
 // once the loop is done.
 //
+// bf16 calls with 128 x 128 states leave this kernel for the tensor-core one: the
+// commit alone at any block length, with token-causal outputs and the verify round
+// at 9..32 tokens.
+//
 // And it is the denoise pass of fp32 activations: every token is stepped, no state
 // is written, and all rows read the block-end state.  That pass had a kernel with
 // the state in shared memory and four CTA barriers per token; its latency for one

@@ -1,6 +1,8 @@
 // State commit at the accepted length on tcgen05 tensor cores: bf16
 // activations, d_k = d_v = 128, B <= 64; for B = 9..32 also with the
-// token-causal outputs of the state-update pass.
+// token-causal outputs of the state-update pass, and the AR-Trust verify round
+// (decoding appendix, block layout [anchor, d_0 .. d_{K-1}, MASK ...]; serving
+// appendix, cache-and-scatter).
 //
 // For one (request r, value head j) with q/k head h, accepted length n > 0 and
 // frozen state S0, the committed state is the chunkwise form of the block's
@@ -36,7 +38,7 @@
 // phase runs once per item and the warps' paths do not fit in the instruction
 // cache): the unrolled 64-token solve alone was 41 KB of code and 10.5k of an
 // item's 27k cycles, whatever n.  128 requests, blocks of 64, n = 1..64: 221 -> 169
-// us per call (n = 64 throughout: 223 either way); 64 requests, blocks of 32: n =
+// us per call, 160 with the items ranked (n = 64 throughout: 223 either way); 64 requests, blocks of 32: n =
 // 1..32 67.9 -> 64.5, n = 32 68.0 -> 68.4.
 //
 // With token-causal outputs (CAUSAL) every token takes part, and
@@ -57,9 +59,19 @@
 // the tensor core's accumulation rounds toward zero); B = 33..64 would need 320
 // tensor-memory columns of the 256 that two CTAs per SM leave each.
 //
+// The verify round (VERIFY) is the causal form with other outputs: rows l <= K read
+// the state after their own token and rows past K the block-end state, so M2 is
+// causal or full by row; the pool takes S^(K+1), and the states after the anchor and
+// the first K-1 drafts are streamed out from fp32 registers, S <- exp(g_t) S + k_t
+// delta_t^T, 4 adjacent columns by 32 rows a thread (16-byte stores, a
+// quarter-warp on 128 contiguous bytes; a column per thread 283 us, this 277).  It
+// is bound by those state writes: 64 requests (32 heads, 31 tokens, up to 15 drafts) move 1.56 GB,
+// 230 us at the measured bandwidth; 307 us as a register recurrence, which stepped all 31 tokens.
+// One request 33 -> 25 us, 100 requests of the 16-head layer with 7 drafts 153 -> 143.
+//
 // Persistent CTAs, two per SM (99 KiB of shared memory, 256 tensor-memory
-// columns each), 128 threads, each walking the (request, value head) items
-// blockIdx.x, blockIdx.x + gridDim.x, ...  The state (64 KiB) arrives by one
+// columns each), 128 threads, each walking one (request, value head) item of
+// every round over the CTAs.  The state (64 KiB) arrives by one
 // bulk copy, the keys and values by TMA (64-row key boxes with 128-byte
 // swizzle, rows past B zero-filled); the next item's state is requested as
 // soon as this item's has been read out of shared memory (before its solve),
@@ -109,13 +121,17 @@ struct CtMaps {
   CUtensorMap v;  // values (128, Hv, B, R) box (64, 1, BM, 1), no swizzle
 };
 
+// Requests that a CTA ranks by length, where an item's cost follows it.
+constexpr int kCtOrder = 256;
+
 // The gate factors of an item's tokens, 16-byte aligned (read as float4 broadcasts)
 struct alignas(16) CtGates {
   float gam2[64];  // gamma_t log2(e) (CAUSAL: its multiple of 2^-10)
   float glo[32];   // CAUSAL: the remainder
   float Gam[64];   // exp(gamma_t)
   float beta[64];
-  float dsc[64];   // exp(gamma_{n-1} - gamma_t) for t < n, else 0 (delta' factor)
+  float dsc[64];   // exp(gamma_{n-1} - gamma_t) for t < n, else 0 (delta' factor);
+                   // VERIFY: exp(g_t)
 };
 
 struct alignas(16) CtShared {
@@ -123,6 +139,7 @@ struct alignas(16) CtShared {
   uint32_t tmem_base;
   int abort_flag;
   CtGates g[2];  // this item's and the next one's
+  uint16_t order[kCtOrder];  // requests, longest first
 };
 
 __device__ __forceinline__ bool ct_wait(uint64_t* bar, uint32_t parity, CtShared& sh,
@@ -136,29 +153,41 @@ __device__ __forceinline__ bool ct_wait(uint64_t* bar, uint32_t parity, CtShared
   return all;
 }
 
-// The next item at or after `it` (stride gridDim.x) with a valid slot and
-// accepted length n > 0 (CAUSAL: n >= 0); items with a bad slot or length are flagged and
-// skipped.  Called by every thread with the same arguments.
-template <bool CAUSAL>
-__device__ __forceinline__ int ct_next(const GdrParams& p, int it, int total, int& slot, int& n) {
-  for (; it < total; it += gridDim.x) {
+// The tokens of request r that decide what its items cost: the accepted length,
+// or the held drafts.
+template <int MODE>
+__device__ __forceinline__ int ct_len(const GdrParams& p, int r) {
+  return MODE == 2 ? p.verify_len[r] : p.accept_len ? p.accept_len[r] : p.B;
+}
+
+// A CTA's first position at or after k whose item has a valid slot and
+// accepted length n > 0 (CAUSAL: n >= 0; VERIFY: n = K + 1 for K held drafts), or -1;
+// items with a bad slot or length are flagged and skipped.  item_at(k) is the
+// item of position k, -1 past the last.  Called by every thread with the same
+// arguments.
+template <int MODE, typename F>
+__device__ __forceinline__ int ct_next(const GdrParams& p, F&& item_at, int k, int& it, int& slot,
+                                       int& n) {
+  for (;; ++k) {
+    it = item_at(k);
+    if (it < 0) return -1;
     const int r = it / p.Hv;
     const int s = p.state_slot[r];
     if (s < 0 || s >= p.nslots) {
       if (threadIdx.x == 0) flag(p.dev_status, FLARE_DEV_BAD_SLOT);
       continue;
     }
-    const int a = p.accept_len ? p.accept_len[r] : p.B;
-    if (a < 0 || a > p.B) {
-      if (threadIdx.x == 0) flag(p.dev_status, FLARE_DEV_BAD_ACCEPT_LEN);
+    const int a = ct_len<MODE>(p, r);
+    if (a < 0 || a > (MODE == 2 ? min(p.max_verify, p.B - 1) : p.B)) {
+      if (threadIdx.x == 0)
+        flag(p.dev_status, MODE == 2 ? FLARE_DEV_BAD_VERIFY_LEN : FLARE_DEV_BAD_ACCEPT_LEN);
       continue;
     }
-    if (a == 0 && !CAUSAL) continue;
+    if (a == 0 && MODE == 0) continue;
     slot = s;
-    n = a;
-    return it;
+    n = MODE == 2 ? a + 1 : a;
+    return k;
   }
-  return -1;
 }
 
 __device__ __forceinline__ uint32_t bf2_bits(__nv_bfloat162 b) {
@@ -180,9 +209,11 @@ __device__ __forceinline__ void split_terms(float a, float b, uint32_t (&w)[N]) 
 
 }  // namespace
 
-template <int BM, bool CAUSAL>
+// MODE 0: commit; 1: commit with token-causal outputs; 2: AR-Trust verify round.
+template <int BM, int MODE>
 __global__ void __launch_bounds__(kCtThreads, 2)
     gdr_commit_tc_kernel(const __grid_constant__ CtMaps maps, GdrParams p) {
+  constexpr bool CAUSAL = MODE != 0, VERIFY = MODE == 2;
   static_assert(!CAUSAL || BM <= 32, "tensor memory");
   using C = CtCfg<BM, CAUSAL>;
   constexpr int kT = C::kTerms;
@@ -202,9 +233,46 @@ __global__ void __launch_bounds__(kCtThreads, 2)
   const int total = p.R * p.Hv;
   const int B = p.B;
 
-  int slot = 0, n = 0;
-  int it = ct_next<CAUSAL>(p, blockIdx.x, total, slot, n);
-  if (it < 0) return;  // the same answer on every thread
+  // The items of a CTA, one of each round over the CTAs.  Where an item's cost follows
+  // its request's length (blocks of 64, whose loops end with the accepted tokens,
+  // and the verify round, which writes a state per held draft) and the lengths differ,
+  // the requests are taken longest first, so that a round's items are alike: in the
+  // order given, 64 requests with 0..15 drafts leave a CTA up to a third more states
+  // than the mean (verify round and commit 292 us, ranked 277; commit of 128
+  // requests, n = 1..64, 170 and 160; every other round backwards 164).
+  constexpr bool kRanked = BM == 64 || VERIFY;
+  bool ranked = kRanked && p.R > 1 && p.R <= kCtOrder && total > (int)gridDim.x;
+  if (ranked) {
+    int* keys = reinterpret_cast<int*>(S0s);  // before the first state is requested
+    const int len0 = ct_len<MODE>(p, 0);
+    bool differ = false;
+    for (int r = tid; r < kCtOrder; r += kCtThreads) {
+      const int len = r < p.R ? ct_len<MODE>(p, r) : len0;
+      differ |= len != len0;
+      keys[r] = r < p.R ? (min(max(len, 0), 64) << 8) | (kCtOrder - 1 - r) : -1;
+    }
+    ranked = __syncthreads_or(differ);
+    for (int r = tid; ranked && r < p.R; r += kCtThreads) {
+      const int key = keys[r];
+      int rank = 0;
+      for (int i = 0; i < p.R; i += 4) {
+        const int4 q = *reinterpret_cast<const int4*>(keys + i);
+        rank += (q.x > key) + (q.y > key) + (q.z > key) + (q.w > key);
+      }
+      sh.order[rank] = (uint16_t)r;
+    }
+    tc::fence_async_smem();
+    __syncthreads();
+  }
+  auto item_at = [&](int k) -> int {
+    const int i = k * (int)gridDim.x + (int)blockIdx.x;
+    if (i >= total) return -1;
+    return ranked ? sh.order[i / p.Hv] * p.Hv + i % p.Hv : i;
+  };
+
+  int slot = 0, n = 0, it = 0;
+  int pos = ct_next<MODE>(p, item_at, 0, it, slot, n);
+  if (pos < 0) return;  // the same answer on every thread
 
   if (tid == 0) {
     sh.abort_flag = 0;
@@ -281,7 +349,7 @@ __global__ void __launch_bounds__(kCtThreads, 2)
       g.glo[lane] = (float)(g2 - (double)hi);
       g.Gam[lane] = expf((float)s);
       g.beta[lane] = bq0;
-      g.dsc[lane] = lane < n ? tc::ex2((float)(gn2 - g2)) : 0.f;
+      g.dsc[lane] = VERIFY ? expf(gq0) : lane < n ? tc::ex2((float)(gn2 - g2)) : 0.f;
     } else {
       float g0 = gq0, g1 = gq1;
 #pragma unroll
@@ -310,10 +378,8 @@ __global__ void __launch_bounds__(kCtThreads, 2)
     }
   };
   // slot and accepted length of the candidate after the next item, one item ahead
-  auto cand_slot = [&](int c) { return c < total ? p.state_slot[c / p.Hv] : -1; };
-  auto cand_len = [&](int c) {
-    return c < total ? (p.accept_len ? p.accept_len[c / p.Hv] : B) : 0;
-  };
+  auto cand_slot = [&](int c) { return c >= 0 ? p.state_slot[c / p.Hv] : -1; };
+  auto cand_len = [&](int c) { return c >= 0 ? ct_len<MODE>(p, c / p.Hv) : 0; };
 
   // thread 0's record of what is in flight (and the parity its barrier
   // phase completes with), for a clean exit after a timeout
@@ -335,7 +401,7 @@ __global__ void __launch_bounds__(kCtThreads, 2)
     load_gates(it);
     if (kEarly) gate_factors(sh.g[0], n);
   }
-  int cand = it + gridDim.x;
+  int cand = item_at(pos + 1);
   int cs = cand_slot(cand), ca = cand_len(cand);
   uint32_t ph = 0;      // parity of the item's state and key/value loads
   uint32_t ph_mma = 0;  // parity of the next MMA completion (two per item)
@@ -350,18 +416,20 @@ __global__ void __launch_bounds__(kCtThreads, 2)
     // the next item: the candidate when it is valid and has n > 0, else the
     // first such item after it (bad ones flagged on the way)
     int it_next = -1, slot_next = 0, n_next = 0;
-    if (cand < total) {
-      if (cs >= 0 && cs < p.nslots && ca >= (CAUSAL ? 0 : 1) && ca <= B) {
+    if (cand >= 0) {
+      ++pos;
+      if (cs >= 0 && cs < p.nslots && ca >= (CAUSAL ? 0 : 1) &&
+          ca <= (VERIFY ? min(p.max_verify, B - 1) : B)) {
         it_next = cand;
         slot_next = cs;
-        n_next = ca;
+        n_next = VERIFY ? ca + 1 : ca;
       } else {
-        it_next = ct_next<CAUSAL>(p, cand, total, slot_next, n_next);
+        pos = ct_next<MODE>(p, item_at, pos, it_next, slot_next, n_next);
       }
     }
     if (it_next >= 0) {
       if (warp == 0) load_gates(it_next);
-      cand = it_next + gridDim.x;
+      cand = item_at(pos + 1);
       cs = cand_slot(cand);
       ca = cand_len(cand);
     }
@@ -460,8 +528,10 @@ __global__ void __launch_bounds__(kCtThreads, 2)
         const int row = tid - kG0, u = row & (BM - 1);
         const bool key = row < BM;
         const float rf = key ? gt.beta[u] : 1.f;
-        const float gh = gt.gam2[u], gl = gt.glo[u];
-        const int end = u < B ? (key ? u : u + 1) : 0;
+        // the gate a row reads to: its own token's, a draft row's the block's last
+        const int ug = VERIFY && !key && u >= n ? B - 1 : u;
+        const float gh = gt.gam2[ug], gl = gt.glo[ug];
+        const int end = u < B ? (key ? u : ug + 1) : 0;
 #pragma unroll
         for (int i8 = 0; i8 < BM / 8; ++i8) {
           float v[8];
@@ -498,7 +568,7 @@ __global__ void __launch_bounds__(kCtThreads, 2)
     tc::fence_after_sync();
 
     // the accumulator starts at Gam_{n-1} S0^T (fp32, from the loaded state)
-    if (!CAUSAL || n > 0) {
+    if (!VERIFY && (!CAUSAL || n > 0)) {
       const float Gn = gt.Gam[n - 1];
 #pragma unroll 2
       for (int i0 = 0; i0 < kCtD; i0 += 16) {
@@ -562,7 +632,7 @@ __global__ void __launch_bounds__(kCtThreads, 2)
     }
     // CAUSAL: keys at and past n to zero for the update (their deltas are zero there,
     // but a rejected token's key may be infinite or NaN)
-    if constexpr (CAUSAL) {
+    if constexpr (CAUSAL && !VERIFY) {
       const int n16 = (((n + 15) & ~15) - n) * 16;  // 16-byte pieces: 8 of each 64-column chunk
       for (int e = tid; e < n16; e += kCtThreads)
         *reinterpret_cast<uint4*>(Ks + ((e >> 3) & 1) * (C::kRows * 128) + (n + (e >> 4)) * 128 +
@@ -579,13 +649,14 @@ __global__ void __launch_bounds__(kCtThreads, 2)
         tc::tmem_ld16(tmW + lane_off + BM + c0, w);
         tc::tmem_ld_wait();
 #pragma unroll
-        for (int e = 0; e < 16; ++e) o[c0 + e] = gt.Gam[c0 + e] * __uint_as_float(w[e]);
+        for (int e = 0; e < 16; ++e)
+          o[c0 + e] = gt.Gam[VERIFY && c0 + e >= n ? B - 1 : c0 + e] * __uint_as_float(w[e]);
       }
     }
     tc::fence_before_sync();
     __syncthreads();  // A^T published; the state buffer, W^T and G read
     // the next item's state streams in while this one is solved and stored
-    if (tid == 0 && it_next >= 0) {
+    if (!VERIFY && tid == 0 && it_next >= 0) {
       issue_s0(it_next, slot_next);
       s0_out = true;
       s0_par = ph ^ 1u;
@@ -611,27 +682,34 @@ __global__ void __launch_bounds__(kCtThreads, 2)
           if (4 * u4 + 3 > t) x[4 * u4 + 3] = fmaf(-a.w, dt, x[4 * u4 + 3]);
         }
       }
-      uint32_t dw[kT][8];
+      if constexpr (VERIFY) {  // delta_t itself, for the states' recurrence
+        uint32_t w[16];
 #pragma unroll
-      for (int i4 = 0; i4 < 4; ++i4) {
-        const float4 q = *reinterpret_cast<const float4*>(&gt.dsc[16 * b + 4 * i4]);
-        const float dr[4] = {q.x, q.y, q.z, q.w};
-        float v[4];
+        for (int e = 0; e < 16; ++e) w[e] = __float_as_uint(x[e]);
+        tc::tmem_st16(tmW + lane_off + 16 * b, w);
+      } else {
+        uint32_t dw[kT][8];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const float xv = x[4 * i4 + e] * dr[e];
-          v[e] = 16 * b + 4 * i4 + e < n ? xv : 0.f;
+        for (int i4 = 0; i4 < 4; ++i4) {
+          const float4 q = *reinterpret_cast<const float4*>(&gt.dsc[16 * b + 4 * i4]);
+          const float dr[4] = {q.x, q.y, q.z, q.w};
+          float v[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const float xv = x[4 * i4 + e] * dr[e];
+            v[e] = 16 * b + 4 * i4 + e < n ? xv : 0.f;
+          }
+#pragma unroll
+          for (int f = 0; f < 2; ++f) {
+            uint32_t s[kT];
+            split_terms<kT>(v[2 * f], v[2 * f + 1], s);
+#pragma unroll
+            for (int y = 0; y < kT; ++y) dw[y][2 * i4 + f] = s[y];
+          }
         }
 #pragma unroll
-        for (int f = 0; f < 2; ++f) {
-          uint32_t s[kT];
-          split_terms<kT>(v[2 * f], v[2 * f + 1], s);
-#pragma unroll
-          for (int y = 0; y < kT; ++y) dw[y][2 * i4 + f] = s[y];
-        }
+        for (int y = 0; y < kT; ++y) tc::tmem_st8(tmW + lane_off + C::kDP * y + 8 * b, dw[y]);
       }
-#pragma unroll
-      for (int y = 0; y < kT; ++y) tc::tmem_st8(tmW + lane_off + C::kDP * y + 8 * b, dw[y]);
       if constexpr (CAUSAL) {
         // delta as the readout's operand: zero where infinite or NaN, which must not
         // reach the outputs before its token through 0 * NaN
@@ -694,13 +772,15 @@ __global__ void __launch_bounds__(kCtThreads, 2)
           tc::mma_commit(&sh.bar_g);
         }
         // D += delta'^T K: the keys [t][i] as an MN-major operand (i contiguous)
+        if constexpr (!VERIFY) {
 #pragma unroll 1
         for (int kk = 0; kk < (n + 15) >> 4; ++kk) {
           const uint64_t kb = tc::sdesc_sw128(tc::smem_u32(Ks + kk * 2048), C::kRows * 128, 1024);
 #pragma unroll
           for (int y = 0; y < kT; ++y) tc::mma_bf16_ts(tmS, tmW + C::kDP * y + kk * 8, kb, idU, 1u);
         }
-        tc::mma_commit(&sh.bar_mma);
+          tc::mma_commit(&sh.bar_mma);
+        }
       }
       __syncwarp();
     }
@@ -717,7 +797,8 @@ __global__ void __launch_bounds__(kCtThreads, 2)
       }
       if (first_bad < BM) {
 #pragma unroll
-        for (int l = 0; l < BM; ++l) o[l] = l < first_bad ? o[l] : __uint_as_float(0x7fffffffu);
+        for (int l = 0; l < BM; ++l)
+          o[l] = l < first_bad && (!VERIFY || l < n) ? o[l] : __uint_as_float(0x7fffffffu);
       }
       // adjacent lanes swap one value so that each stores a bf16 pair of two columns
       const bool odd = lane & 1;
@@ -733,29 +814,98 @@ __global__ void __launch_bounds__(kCtThreads, 2)
           *reinterpret_cast<__nv_bfloat162*>(out + (size_t)row * p.Hv * kCtD) = w;
       }
     }
-    if (!ct_wait(&sh.bar_mma, ph_mma, sh, p.dev_status)) break;
-    ph_mma ^= 1u;
-    tc::fence_after_sync();
-    if (tid == 0) {
-      mma_out = false;
-      if (it_next >= 0) {  // the update, the last reader of these keys, is done
+    if constexpr (VERIFY) {
+      // the states S^(t) = S after tokens 0..t, t < K, streamed out, and S^(K) into the
+      // pool: S <- exp(g_t) S + k_t delta_t in fp32 from the state itself, a thread on
+      // rows 32 warp .. and four adjacent columns, so that a warp's store is a whole
+      // row.  The deltas go there through shared memory (M2 and A^T are read).
+      float* Ds = reinterpret_cast<float*>(M2s);  // delta_t[c]
+      static_assert(C::kM2 + C::kR >= BM * kCtD * 4, "room for the deltas");
+#pragma unroll
+      for (int c0 = 0; c0 < BM; c0 += 16) {
+        uint32_t w[16];
+        tc::tmem_ld16(tmW + lane_off + c0, w);
+        tc::tmem_ld_wait();
+#pragma unroll
+        for (int e = 0; e < 16; ++e) Ds[(c0 + e) * kCtD + tid] = __uint_as_float(w[e]);
+      }
+      uint64_t s[32][2];  // rows 32 warp + i, columns 4 lane .. as two pairs
+#pragma unroll
+      for (int i = 0; i < 32; ++i) {
+        const ulonglong2 v =
+            *reinterpret_cast<const ulonglong2*>(S0s + (32 * warp + i) * kCtD + 4 * lane);
+        s[i][0] = v.x;
+        s[i][1] = v.y;
+      }
+      __syncthreads();  // the deltas are there, the state buffer is read
+      if (tid == 0) {
+        mma_out = false;
+        if (it_next >= 0) {
+          tc::fence_async_smem();
+          issue_s0(it_next, slot_next);
+          s0_out = true;
+          s0_par = ph ^ 1u;
+        }
+      }
+      const int r = it / p.Hv, j = it % p.Hv;
+#pragma unroll 1
+      for (int t = 0; t < n; ++t) {
+        const ulonglong2 d = *reinterpret_cast<const ulonglong2*>(Ds + t * kCtD + 4 * lane);
+        const uint64_t a2 = f2_dup(gt.dsc[t]);
+        float* dst = (t + 1 < n ? p.verify_states + (((size_t)r * p.max_verify + t) * p.Hv + j) *
+                                                        kCtD * kCtD
+                                : state_of(it, slot)) + 32 * warp * kCtD + 4 * lane;
+        const uint8_t* kr = Ks + (warp >> 1) * (C::kRows * 128) + t * 128;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {  // 16-byte units of the key's row: 8 state rows each
+          const uint4 k = *reinterpret_cast<const uint4*>(
+              kr + (((4 * (warp & 1) + u) ^ (t & 7)) << 4));
+          const uint32_t kw[4] = {k.x, k.y, k.z, k.w};
+#pragma unroll
+          for (int e = 0; e < 8; ++e) {
+            const uint64_t k2 = f2_dup(__uint_as_float(
+                (e & 1) ? kw[e >> 1] & 0xffff0000u : kw[e >> 1] << 16));
+            uint64_t(&v)[2] = s[8 * u + e];
+            v[0] = f2_fma(k2, d.x, f2_mul(a2, v[0]));
+            v[1] = f2_fma(k2, d.y, f2_mul(a2, v[1]));
+            __stcs(reinterpret_cast<ulonglong2*>(dst + (8 * u + e) * kCtD),
+                   make_ulonglong2(v[0], v[1]));
+          }
+        }
+      }
+      tc::fence_before_sync();
+      __syncthreads();  // the deltas and the keys, the last of this item's inputs, are read
+      if (tid == 0 && it_next >= 0) {
         tc::fence_async_smem();
         issue_kv(it_next);
         k_out = true;
         k_par = ph ^ 1u;
       }
-    }
-    // the committed state: lane c holds S^(n)[i][c] over i
-    if (!CAUSAL || n > 0) {
-      float* Sg = state_of(it, slot) + tid;
+    } else {
+      if (!ct_wait(&sh.bar_mma, ph_mma, sh, p.dev_status)) break;
+      ph_mma ^= 1u;
+      tc::fence_after_sync();
+      if (tid == 0) {
+        mma_out = false;
+        if (it_next >= 0) {  // the update, the last reader of these keys, is done
+          tc::fence_async_smem();
+          issue_kv(it_next);
+          k_out = true;
+          k_par = ph ^ 1u;
+        }
+      }
+      // the committed state: lane c holds S^(n)[i][c] over i
+      if (!CAUSAL || n > 0) {
+        float* Sg = state_of(it, slot) + tid;
 #pragma unroll 1
-      for (int i0 = 0; i0 < kCtD; i0 += 32) {
-        uint32_t d[32];
-        tc::tmem_ld16(tmS + lane_off + i0, *reinterpret_cast<uint32_t(*)[16]>(&d[0]));
-        tc::tmem_ld16(tmS + lane_off + i0 + 16, *reinterpret_cast<uint32_t(*)[16]>(&d[16]));
-        tc::tmem_ld_wait();
+        for (int i0 = 0; i0 < kCtD; i0 += 32) {
+          uint32_t d[32];
+          tc::tmem_ld16(tmS + lane_off + i0, *reinterpret_cast<uint32_t(*)[16]>(&d[0]));
+          tc::tmem_ld16(tmS + lane_off + i0 + 16, *reinterpret_cast<uint32_t(*)[16]>(&d[16]));
+          tc::tmem_ld_wait();
 #pragma unroll
-        for (int e = 0; e < 32; ++e) Sg[(size_t)(i0 + e) * kCtD] = __uint_as_float(d[e]);
+          for (int e = 0; e < 32; ++e) Sg[(size_t)(i0 + e) * kCtD] = __uint_as_float(d[e]);
+        }
       }
     }
     if (it_next < 0) break;
@@ -818,15 +968,16 @@ bool ct_act_map(CUtensorMap* m, const void* x, int H, int B, int R, int rows, bo
          CUDA_SUCCESS;
 }
 
-template <int BM, bool CAUSAL>
+template <int BM, int MODE>
 cudaError_t launch_ct(const GdrParams& p, cudaStream_t stream) {
+  constexpr bool CAUSAL = MODE != 0;
   CtMaps maps;
   if (!ct_act_map(&maps.k, p.k, p.Hk, p.B, p.R, CAUSAL ? BM : 64, true) ||
       (CAUSAL && !ct_act_map(&maps.q, p.q, p.Hk, p.B, p.R, BM, true)) ||
       !ct_act_map(&maps.v, p.v, p.Hv, p.B, p.R, BM, false))
     return cudaErrorInvalidValue;
   const int smem = CtCfg<BM, CAUSAL>::kSmem + 1024;
-  cudaError_t e = cudaFuncSetAttribute(gdr_commit_tc_kernel<BM, CAUSAL>,
+  cudaError_t e = cudaFuncSetAttribute(gdr_commit_tc_kernel<BM, MODE>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
   int dev = 0, sms = kNumSMs;
@@ -834,7 +985,7 @@ cudaError_t launch_ct(const GdrParams& p, cudaStream_t stream) {
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const long items = (long)p.R * p.Hv;
   const int grid = (int)(items < 2L * sms ? items : 2L * sms);
-  gdr_commit_tc_kernel<BM, CAUSAL><<<grid, kCtThreads, smem, stream>>>(maps, p);
+  gdr_commit_tc_kernel<BM, MODE><<<grid, kCtThreads, smem, stream>>>(maps, p);
   note_launches(1);
   return cudaGetLastError();
 }
@@ -847,10 +998,10 @@ bool gdr_commit_tc_supported(int B, int dk, int dv, bool causal) {
 
 cudaError_t launch_gdr_commit_tc(const GdrParams& p, cudaStream_t stream) {
   if (p.R == 0) return cudaSuccess;
-  if (p.out_causal)
-    return p.B <= 16 ? launch_ct<16, true>(p, stream) : launch_ct<32, true>(p, stream);
-  if (p.B <= 16) return launch_ct<16, false>(p, stream);
-  return p.B <= 32 ? launch_ct<32, false>(p, stream) : launch_ct<64, false>(p, stream);
+  if (p.verify_len) return p.B <= 16 ? launch_ct<16, 2>(p, stream) : launch_ct<32, 2>(p, stream);
+  if (p.out_causal) return p.B <= 16 ? launch_ct<16, 1>(p, stream) : launch_ct<32, 1>(p, stream);
+  if (p.B <= 16) return launch_ct<16, 0>(p, stream);
+  return p.B <= 32 ? launch_ct<32, 0>(p, stream) : launch_ct<64, 0>(p, stream);
 }
 
 }  // namespace flare

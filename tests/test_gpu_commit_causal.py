@@ -75,3 +75,70 @@ def test_infinite_and_nan_tokens_stay_after_their_place(block, token):
     slots = w.state_slot.long()
     assert torch.equal(pool[slots], clean_pool[slots])
     assert not torch.isfinite(out[:, token:].float()).all()
+
+
+@pytest.mark.parametrize("block", [9, 16, 17, 31, 32])
+def test_verify_round_on_tensor_cores(block):
+    """The same kernel's verify mode: no held draft, one, and as many as the block
+    takes; the cached and live states to 1e-6, slots of skipped requests untouched."""
+    from gpu_helpers import oracle_verify, run_verify_linear
+    from paper_2606_01774_gb300 import flare
+
+    most = block - 1
+    spec = LARGE.replace(num_requests=6, block_len=block, verify_horizon=2, seed=240 + block)
+    w = gen(spec)
+    install_states(w)
+    held = torch.tensor([0, 1, most, block // 2, most + 1, 5], dtype=torch.int32).cuda()
+    before = w.state_pool.clone()
+    out, rec = run_verify_linear(w, most, verify_len=held, expect_bits=flare.FLARE_DEV_BAD_VERIFY_LEN)
+    good = [0, 1, 2, 3, 5]
+    ref = oracle_verify(w, before, most, good, held)
+    assert_out_close(out[good], ref["out"], "bf16", f"L = {block}")
+    slots = w.state_slot.long()
+    for i, r in enumerate(good):
+        assert rel_fro(w.state_pool[slots[r]].double().cpu().numpy(), ref["state"][i]) < STATE_REL
+        for t in range(int(held[r])):
+            assert rel_fro(rec[r, t].double().cpu().numpy(), ref["records"][i][t]) < STATE_REL
+        assert torch.isnan(rec[r, int(held[r]):]).all()  # not written
+    assert torch.equal(w.state_pool[slots[4]], before[slots[4]]) and torch.isnan(rec[4]).all()
+
+
+@pytest.mark.parametrize("requests", [10, 255, 256, 257])
+@pytest.mark.parametrize("verify", [False, True])
+def test_ranked_items_give_what_the_order_given_does(requests, verify):
+    """More items than CTAs and ragged lengths: the requests are taken longest first
+    (up to 256 of them).  An item's arithmetic does not depend on its turn, so every
+    state is bit for bit what it is for its requests two at a time (fewer items than
+    CTAs: the order given), and a bad length is flagged and skipped in either."""
+    from gpu_helpers import run_verify_linear
+    from paper_2606_01774_gb300 import flare
+
+    heads, block = (16, 32) if requests == 10 else (2, 2), 9 if verify else 64
+    spec = LARGE.replace(num_requests=requests, block_len=block, num_qk_heads=heads[0],
+                         num_v_heads=heads[1], state_prefix_tokens=8, seed=260)
+    w = workloads.generate(spec, "cuda", softmax=False)
+    install_states(w, [0])
+    top = block - 1 if verify else block
+    length = torch.randint(0, top + 1, (requests,), generator=torch.Generator().manual_seed(1),
+                           dtype=torch.int32).cuda()
+    if verify:
+        length[3] = top + 1
+
+    def run(req):
+        part = lambda b: workloads.LinearBlock(*(t[req].contiguous() for t in
+                                                 (b.q, b.k, b.v, b.log_decay, b.beta)))
+        x = workloads.Workload(spec.replace(num_requests=len(req)), None, w.state_pool.clone(),
+                               w.state_slot[req].contiguous(), [part(w.denoise[0])], part(w.commit))
+        n = length[req].contiguous()
+        if verify:
+            res = run_verify_linear(x, top, verify_len=n, expect_bits=flare.FLARE_DEV_BAD_VERIFY_LEN
+                                    if (n > top).any() else 0)
+        else:
+            res = ()
+            run_commit(x, x.state_pool, accept_len=n)
+        return (x.state_pool[x.state_slot.long()], *res)
+
+    whole = run(list(range(requests)))
+    for req in ([0, 1], [2, 4], [requests - 2, requests - 1]):
+        for a, b in zip(whole, run(req)):
+            assert torch.equal(a[req].view(torch.int16), b.view(torch.int16))
