@@ -1,7 +1,7 @@
 // State commit at the accepted length on tcgen05 tensor cores: bf16
-// activations, d_k = d_v = 128, B <= 64; for B = 9..32 also with the
-// token-causal outputs of the state-update pass, and the AR-Trust verify round
-// (decoding appendix, block layout [anchor, d_0 .. d_{K-1}, MASK ...]; serving
+// activations, d_k = d_v = 128, B <= 64; for B = 9..64 also with the
+// token-causal outputs of the state-update pass, and for B = 9..32 the AR-Trust
+// verify round (decoding appendix, block layout [anchor, d_0 .. d_{K-1}, MASK ...]; serving
 // appendix, cache-and-scatter).
 //
 // For one (request r, value head j) with q/k head h, accepted length n > 0 and
@@ -48,16 +48,28 @@
 //
 // G takes the query rows and W^T the query columns as well, and the sum is a
 // product of the deltas and M2 in two bf16 terms each (2^-16, below the outputs'
-// rounding).  The register
-// recurrence that this replaces is exact fp32, so the fp32 operands enter as three
-// bf16 terms (24 bits) and the log-gates are summed in double precision and kept
+// rounding).  The register recurrence that this replaces is exact fp32, so what
+// decides the state's precision is as close: the fp32 operands enter as three
+// bf16 terms (24 bits); the log-gates are summed in double precision and kept
 // as a multiple of 2^-10 and a remainder, whose differences are exact where they
-// matter: over 32 tokens the committed states are 1.7e-7 off 64 bits where the
-// recurrence's are 6.0e-7.  State update of 64 requests (32 heads): B = 32 208 ->
-// 107 us, B = 16 123 -> 80.  Blocks of 8 and fewer stay with the recurrence, which
-// is as fast there (84 and 78 us at B = 8) and closer (1.15e-7 against 1.28e-7:
-// the tensor core's accumulation rounds toward zero); B = 33..64 would need 320
-// tensor-memory columns of the 256 that two CTAs per SM leave each.
+// matter; the solve sums Gam_t S0^T k_t + sum_i A_ti delta_i, which is small beside
+// v_t, before it takes it from v_t once; and the update adds its small terms first,
+// as the tensor core rounds every step toward zero.  The committed states are 7.5e-8
+// off 64 bits at B = 9..32 (1.25e-7 without the solve's order, 1.7e-7 without the
+// update's as well), where the recurrence's are 1.4e-7 to 6.4e-7.  State update of 64
+// requests (32 heads) with its append, B = 32: 208 -> 97 us.  Blocks of 8 and
+// fewer stay with the recurrence: 82 and 77 us at B = 8 for 64 requests, 14.4 and
+// 16.5 for one; 71 and 77 at B = 4.
+//
+// Blocks of 33..64 with outputs (LONG) run as two halves of 32 tokens, the second
+// from the state after the first, which each thread leaves, its column, where the
+// first one's state was: in one piece they would need 320 tensor-memory columns, of
+// the 256 that two CTAs per SM leave each.  Where fewer than 32 tokens are accepted
+// the first half sums twice, to the accepted length for the pool and over all 32 for
+// the second half.  As the recurrence is closer for these blocks (7.1e-8: it walks
+// the gates one by one where they fall below 2^-40), the last token of a sum, its
+// largest term, adds in fp32 (6.7e-8; without 7.6e-8 and 330 us).  State update of
+// 128 requests, B = 64: 738 -> 351 us; of 64, B = 33, the worst case, 217 -> 175.
 //
 // The verify round (VERIFY) is the causal form with other outputs: rows l <= K read
 // the state after their own token and rows past K the block-end state, so M2 is
@@ -96,7 +108,7 @@ namespace {
 constexpr int kCtThreads = 128;
 constexpr int kCtD = 128;  // d_k = d_v
 
-template <int BM, bool CAUSAL>
+template <int BM, bool CAUSAL, bool LONG = false>
 struct CtCfg {
   // keys: 2 chunks of 64 rows x 128 B (SW128); CAUSAL: keys, then queries, 2 x BM rows
   static constexpr int kRows = CAUSAL ? 2 * BM : 64;
@@ -110,7 +122,9 @@ struct CtCfg {
   // tensor-memory columns of each bf16 part of delta'^T (whole 16-column stores)
   static constexpr int kDP = BM / 2 < 16 ? 16 : BM / 2;
   static constexpr int kM2 = CAUSAL ? 2 * BM * 128 : 0;  // M2[l][i] bf16 hi, lo (K-major SW128)
-  static constexpr int kSmem = kS0 + kK + kR + kM2;
+  // LONG: the 16 keys around the accepted length, and (fp32) the last one of each sum
+  static constexpr int kKz = LONG ? 2 * 16 * 128 + 2 * kCtD * 4 : 0;
+  static constexpr int kSmem = kS0 + kK + kR + kM2 + kKz;
   static constexpr int kTerms = CAUSAL ? 3 : 2;    // bf16 terms of an fp32 operand
 };
 
@@ -209,13 +223,14 @@ __device__ __forceinline__ void split_terms(float a, float b, uint32_t (&w)[N]) 
 
 }  // namespace
 
-// MODE 0: commit; 1: commit with token-causal outputs; 2: AR-Trust verify round.
+// MODE 0: commit; 1: commit with token-causal outputs; 2: AR-Trust verify round;
+// 3: as 1 for B = 33..64, in two halves.
 template <int BM, int MODE>
 __global__ void __launch_bounds__(kCtThreads, 2)
     gdr_commit_tc_kernel(const __grid_constant__ CtMaps maps, GdrParams p) {
-  constexpr bool CAUSAL = MODE != 0, VERIFY = MODE == 2;
+  constexpr bool CAUSAL = MODE != 0, VERIFY = MODE == 2, LONG = MODE == 3;
   static_assert(!CAUSAL || BM <= 32, "tensor memory");
-  using C = CtCfg<BM, CAUSAL>;
+  using C = CtCfg<BM, CAUSAL, LONG>;
   constexpr int kT = C::kTerms;
   constexpr int kATs = C::kATs;
   // block loops: unrolled where the whole block count is at most two
@@ -226,6 +241,8 @@ __global__ void __launch_bounds__(kCtThreads, 2)
   float* S0s = reinterpret_cast<float*>(base);
   uint8_t* Ks = base + C::kS0;
   uint8_t* M2s = Ks + C::kK;
+  uint8_t* Kz = M2s + C::kM2 + C::kR;
+  float* Kt = reinterpret_cast<float*>(Kz + 2 * 16 * 128);
   uint8_t* Rs = M2s + C::kM2;  // the values, then A^T
   float* AT = reinterpret_cast<float*>(Rs);
 
@@ -270,8 +287,8 @@ __global__ void __launch_bounds__(kCtThreads, 2)
     return ranked ? sh.order[i / p.Hv] * p.Hv + i % p.Hv : i;
   };
 
-  int slot = 0, n = 0, it = 0;
-  int pos = ct_next<MODE>(p, item_at, 0, it, slot, n);
+  int slot = 0, n_item = 0, it = 0;
+  int pos = ct_next<MODE>(p, item_at, 0, it, slot, n_item);
   if (pos < 0) return;  // the same answer on every thread
 
   if (tid == 0) {
@@ -311,26 +328,31 @@ __global__ void __launch_bounds__(kCtThreads, 2)
       tc::bulk_load(S0s + q * (kCtD * kCtD / 4), src + q * (kCtD * kCtD / 4), C::kS0 / 4,
                     &sh.bar_s0);
   };
-  auto issue_kv = [&](int item) {
+  // LONG: half h of an item is tokens 32 h .. of its block
+  auto half_len = [&](int h) { return LONG ? min(B - 32 * h, 32) : B; };
+  auto half_n = [&](int n, int h) { return LONG ? min(max(n - 32 * h, 0), half_len(h)) : n; };
+  auto issue_kv = [&](int item, int half) {
+    const int t0 = 32 * half;
     const int r = item / p.Hv, j = item % p.Hv, h = j / (p.Hv / p.Hk);
     tc::mbar_expect_tx(&sh.bar_k, C::kK + C::kV);
-    tc::tma_load_4d(Ks, &maps.k, &sh.bar_k, 0, h, 0, r);
-    tc::tma_load_4d(Ks + C::kRows * 128, &maps.k, &sh.bar_k, 64, h, 0, r);
+    tc::tma_load_4d(Ks, &maps.k, &sh.bar_k, 0, h, t0, r);
+    tc::tma_load_4d(Ks + C::kRows * 128, &maps.k, &sh.bar_k, 64, h, t0, r);
     if constexpr (CAUSAL) {
-      tc::tma_load_4d(Ks + BM * 128, &maps.q, &sh.bar_k, 0, h, 0, r);
-      tc::tma_load_4d(Ks + (C::kRows + BM) * 128, &maps.q, &sh.bar_k, 64, h, 0, r);
+      tc::tma_load_4d(Ks + BM * 128, &maps.q, &sh.bar_k, 0, h, t0, r);
+      tc::tma_load_4d(Ks + (C::kRows + BM) * 128, &maps.q, &sh.bar_k, 64, h, t0, r);
     }
-    tc::tma_load_4d(Rs, &maps.v, &sh.bar_k, 0, j, 0, r);
-    tc::tma_load_4d(Rs + BM * 128, &maps.v, &sh.bar_k, 64, j, 0, r);
+    tc::tma_load_4d(Rs, &maps.v, &sh.bar_k, 0, j, t0, r);
+    tc::tma_load_4d(Rs + BM * 128, &maps.v, &sh.bar_k, 64, j, t0, r);
   };
   // warp 0 holds the gates of the item it will process next, loaded one item ahead
   float gq0 = 0.f, gq1 = 0.f, bq0 = 0.f, bq1 = 0.f;
-  auto load_gates = [&](int item) {
-    const size_t gb = (size_t)(item / p.Hv) * B * p.Hv + item % p.Hv;
-    gq0 = lane < B ? p.log_decay[gb + (size_t)lane * p.Hv] : 0.f;
-    gq1 = lane + 32 < B ? p.log_decay[gb + (size_t)(lane + 32) * p.Hv] : 0.f;
-    bq0 = lane < B ? p.beta[gb + (size_t)lane * p.Hv] : 0.f;
-    bq1 = lane + 32 < B ? p.beta[gb + (size_t)(lane + 32) * p.Hv] : 0.f;
+  auto load_gates = [&](int item, int half) {
+    const size_t gb = ((size_t)(item / p.Hv) * B + 32 * half) * p.Hv + item % p.Hv;
+    const int m = half_len(half);
+    gq0 = lane < m ? p.log_decay[gb + (size_t)lane * p.Hv] : 0.f;
+    gq1 = lane + 32 < m ? p.log_decay[gb + (size_t)(lane + 32) * p.Hv] : 0.f;
+    bq0 = lane < m ? p.beta[gb + (size_t)lane * p.Hv] : 0.f;
+    bq1 = lane + 32 < m ? p.beta[gb + (size_t)(lane + 32) * p.Hv] : 0.f;
   };
   // warp 0: the gate factors of the item whose gates it holds (gamma = inclusive
   // prefix sum of the log-gates), while another item's products run
@@ -389,7 +411,7 @@ __global__ void __launch_bounds__(kCtThreads, 2)
     tc::prefetch_tmap(&maps.k);
     tc::prefetch_tmap(&maps.v);
     issue_s0(it, slot);
-    issue_kv(it);
+    issue_kv(it, 0);
     s0_out = k_out = true;
   }
   // where the wait for W^T has room for it, the next item's gate factors are formed
@@ -398,25 +420,63 @@ __global__ void __launch_bounds__(kCtThreads, 2)
   // 141.6 and 144 early)
   constexpr bool kEarly = BM == 32 || (BM == 16 && !CAUSAL);
   if (warp == 0) {
-    load_gates(it);
-    if (kEarly) gate_factors(sh.g[0], n);
+    load_gates(it, 0);
+    if (kEarly) gate_factors(sh.g[0], half_n(n_item, 0));
   }
   int cand = item_at(pos + 1);
   int cs = cand_slot(cand), ca = cand_len(cand);
-  uint32_t ph = 0;      // parity of the item's state and key/value loads
+  // LONG: the last token of a sum, its largest term, in fp32 after the others
+  auto add_last = [&](uint32_t(&d)[32], const float* k, float delta) {
+#pragma unroll
+    for (int e4 = 0; e4 < 8; ++e4) {
+      const float4 a = *reinterpret_cast<const float4*>(k + 4 * e4);
+      const float ka[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        d[4 * e4 + e] = __float_as_uint(fmaf(delta, ka[e], __uint_as_float(d[4 * e4 + e])));
+    }
+  };
+  int half = 0;
+  uint32_t ph = 0;      // parity of the key/value loads (and, one per item, the state's)
+  uint32_t ph_s0 = 0;   // LONG: parity of the item's state load
   uint32_t ph_mma = 0;  // parity of the next MMA completion (two per item)
   const uint32_t idU = tc::idesc_bf16(128, 128, false, true);
+  // D += delta'^T K over the first n tokens (the keys [t][i] as an MN-major operand, i
+  // contiguous).  CAUSAL: the small terms first, and in each the older tokens, as every
+  // step rounds the accumulator toward zero and so should find it small.
+  auto update = [&](int n) {
+#pragma unroll 1
+    for (int y = CAUSAL ? kT - 1 : 0; CAUSAL ? y >= 0 : y < 1; CAUSAL ? --y : ++y) {
+#pragma unroll 1
+      for (int kk = 0; kk < (n + 15) >> 4; ++kk) {
+        const uint64_t kb =
+            LONG && n < 16 * (kk + 1)
+                ? tc::sdesc_sw128(tc::smem_u32(Kz), 2048, 1024)
+                : tc::sdesc_sw128(tc::smem_u32(Ks + kk * 2048), C::kRows * 128, 1024);
+#pragma unroll
+        for (int z = 0; z < (CAUSAL ? 1 : kT); ++z)
+          tc::mma_bf16_ts(tmS, tmW + C::kDP * (y + z) + kk * 8, kb, idU, 1u);
+      }
+    }
+  };
 
 #pragma unroll 1
   while (true) {
     const CtGates& gt = sh.g[kEarly ? ph : 0];
+    const int Bh = half_len(half), n = half_n(n_item, half);
+    const int out0 = LONG ? 32 * half : 0;  // the first output row
     if (!kEarly && warp == 0) gate_factors(sh.g[0], n);
-    const int m = CAUSAL ? B : n;   // tokens that take part
+    const int m = CAUSAL ? Bh : n;  // tokens that take part
     const int nb = (m + 15) >> 4;  // and their blocks of 16
     // the next item: the candidate when it is valid and has n > 0, else the
     // first such item after it (bad ones flagged on the way)
     int it_next = -1, slot_next = 0, n_next = 0;
-    if (cand >= 0) {
+    const int half_next = LONG ? half ^ 1 : 0;
+    if (half_next) {
+      it_next = it;
+      slot_next = slot;
+      n_next = n_item;
+    } else if (cand >= 0) {
       ++pos;
       if (cs >= 0 && cs < p.nslots && ca >= (CAUSAL ? 0 : 1) &&
           ca <= (VERIFY ? min(p.max_verify, B - 1) : B)) {
@@ -428,14 +488,22 @@ __global__ void __launch_bounds__(kCtThreads, 2)
       }
     }
     if (it_next >= 0) {
-      if (warp == 0) load_gates(it_next);
-      cand = item_at(pos + 1);
-      cs = cand_slot(cand);
-      ca = cand_len(cand);
+      if (warp == 0) load_gates(it_next, half_next);
+      if (!half_next) {
+        cand = item_at(pos + 1);
+        cs = cand_slot(cand);
+        ca = cand_len(cand);
+      }
     }
 
-    if (!ct_wait(&sh.bar_s0, ph, sh, p.dev_status)) break;
-    if (tid == 0) s0_out = false;
+    // the second half's state is in place: each thread left its column there
+    if (!half) {
+      if (!ct_wait(&sh.bar_s0, LONG ? ph_s0 : ph, sh, p.dev_status)) break;
+      ph_s0 ^= 1u;
+      if (tid == 0) s0_out = false;
+    } else {
+      __syncthreads();  // the half's gate factors
+    }
     if (CAUSAL && warp == 0) {  // the Gram first, while the state is split
       const bool ok = __all_sync(0xffffffffu, tc::mbar_wait(&sh.bar_k, ph, &sh.abort_flag));
       tc::fence_after_sync();
@@ -507,19 +575,26 @@ __global__ void __launch_bounds__(kCtThreads, 2)
       __syncwarp();
     }
     // this thread's value column (rows past B arrive as zeros)
-    uint32_t vraw[BM];
+    // CAUSAL: in pairs of tokens
+    uint32_t vraw[CAUSAL ? BM / 2 : BM];
     {
       const uint8_t* vb = Rs + (tid >> 6) * (BM * 128) + (tid & 63) * 2;
 #pragma unroll
       for (int t0 = 0; t0 < BM; t0 += 16) {
         if (t0 < m) {
 #pragma unroll
-          for (int t = t0; t < t0 + 16; ++t)
-            vraw[t] = *reinterpret_cast<const unsigned short*>(vb + t * 128);
+          for (int t = t0; t < t0 + 16; ++t) {
+            const uint32_t v = *reinterpret_cast<const unsigned short*>(vb + t * 128);
+            if (!CAUSAL)
+              vraw[t] = v;
+            else
+              vraw[t / 2] = (t & 1) ? vraw[t / 2] | v << 16 : v;
+          }
         }
       }
     }
-    if (kEarly && warp == 0 && it_next >= 0) gate_factors(sh.g[ph ^ 1], n_next);
+    if (kEarly && warp == 0 && it_next >= 0)
+      gate_factors(sh.g[ph ^ 1], half_n(n_next, half_next));
     if constexpr (CAUSAL) {
       __syncthreads();  // the values are read: A^T may take their place
       // A^T from the key rows of G and M2 from its query rows, while W^T is formed:
@@ -527,11 +602,10 @@ __global__ void __launch_bounds__(kCtThreads, 2)
       if (warp >= kG0 / 32) {
         const int row = tid - kG0, u = row & (BM - 1);
         const bool key = row < BM;
-        const float rf = key ? gt.beta[u] : 1.f;
         // the gate a row reads to: its own token's, a draft row's the block's last
         const int ug = VERIFY && !key && u >= n ? B - 1 : u;
         const float gh = gt.gam2[ug], gl = gt.glo[ug];
-        const int end = u < B ? (key ? u : ug + 1) : 0;
+        const int end = u < Bh ? (key ? u : ug + 1) : 0;
 #pragma unroll
         for (int i8 = 0; i8 < BM / 8; ++i8) {
           float v[8];
@@ -543,7 +617,7 @@ __global__ void __launch_bounds__(kCtThreads, 2)
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
               const int i = 8 * i8 + 4 * h + e;
-              const float a = rf * tc::ex2((gh - hv[e]) + (gl - lv[e])) * __uint_as_float(gc[i]);
+              const float a = tc::ex2((gh - hv[e]) + (gl - lv[e])) * __uint_as_float(gc[i]);
               v[4 * h + e] = i < end ? a : 0.f;
             }
           }
@@ -610,7 +684,8 @@ __global__ void __launch_bounds__(kCtThreads, 2)
         }
       }
     }
-    // X = diag(beta) (V - diag(Gam) W) for this thread's column
+    // X = diag(beta) (V - diag(Gam) W) for this thread's column; CAUSAL: diag(Gam) W, to
+    // which the solve adds, so that a delta is rounded at its own size once
     float x[BM];
 #pragma unroll
     for (int c0 = 0; c0 < BM; c0 += 16) {
@@ -626,13 +701,34 @@ __global__ void __launch_bounds__(kCtThreads, 2)
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
           const int t = c0 + 4 * e4 + e;
-          x[t] = bb[e] * (__uint_as_float(vraw[t] << 16) - gg[e] * __uint_as_float(w[4 * e4 + e]));
+          if constexpr (CAUSAL)
+            x[t] = gg[e] * __uint_as_float(w[4 * e4 + e]);
+          else
+            x[t] = bb[e] * (__uint_as_float(vraw[t] << 16) - gg[e] * __uint_as_float(w[4 * e4 + e]));
         }
       }
     }
     // CAUSAL: keys at and past n to zero for the update (their deltas are zero there,
     // but a rejected token's key may be infinite or NaN)
-    if constexpr (CAUSAL && !VERIFY) {
+    if constexpr (LONG) {  // the first half's advance to its end needs them all: a copy
+      const int b0 = n & ~15;
+      for (int e = tid; (n & 15) && e < 256; e += kCtThreads) {
+        const int row = e >> 4, c = (e >> 3) & 1;
+        const int at = row * 128 + (e & 7) * 16;
+        *reinterpret_cast<uint4*>(Kz + c * 2048 + at) =
+            b0 + row < n ? *reinterpret_cast<const uint4*>(Ks + c * (C::kRows * 128) + b0 * 128 + at)
+                         : make_uint4(0u, 0u, 0u, 0u);
+      }
+      tc::fence_async_smem();
+#pragma unroll
+      for (int x = 0; x < 2; ++x) {
+        const int t = x ? 31 : max(n - 1, 0);
+        const uint8_t* kr = Ks + (tid >> 6) * (C::kRows * 128) + t * 128 +
+                            ((((tid >> 3) & 7) ^ (t & 7)) << 4) + (tid & 7) * 2;
+        Kt[x * kCtD + tid] =
+            __uint_as_float((uint32_t)*reinterpret_cast<const unsigned short*>(kr) << 16);
+      }
+    } else if constexpr (CAUSAL && !VERIFY) {
       const int n16 = (((n + 15) & ~15) - n) * 16;  // 16-byte pieces: 8 of each 64-column chunk
       for (int e = tid; e < n16; e += kCtThreads)
         *reinterpret_cast<uint4*>(Ks + ((e >> 3) & 1) * (C::kRows * 128) + (n + (e >> 4)) * 128 +
@@ -656,23 +752,31 @@ __global__ void __launch_bounds__(kCtThreads, 2)
     tc::fence_before_sync();
     __syncthreads();  // A^T published; the state buffer, W^T and G read
     // the next item's state streams in while this one is solved and stored
-    if (!VERIFY && tid == 0 && it_next >= 0) {
+    if (!VERIFY && !half_next && tid == 0 && it_next >= 0) {
+      if (LONG) tc::fence_async_smem();
       issue_s0(it_next, slot_next);
       s0_out = true;
-      s0_par = ph ^ 1u;
+      s0_par = LONG ? ph_s0 : ph ^ 1u;
     }
 
     // (I + A) delta = X, right-looking: once a block's deltas are final they
     // leave the later blocks (A^T rows as 16-byte broadcast loads), which move
     // down in the registers, and go to tensor memory as delta'_t =
     // exp(gamma_{n-1} - gamma_t) delta_t (t < n) in bf16 hi and lo parts.
+    float dl[LONG ? BM : 1];  // LONG: the deltas
+    float d_last = 0.f;       // and the last accepted token's, which adds in fp32
 #pragma unroll kU
     for (int b = 0; b < BM / 16; ++b) {
       if (kU == 1 && b >= nb) break;  // uniform (two blocks: 69.6 us with the branch, 68.4 without)
       const float* ab = AT + 16 * b * kATs + 16 * b;
 #pragma unroll
       for (int t = 0; t < 16; ++t) {
-        const float dt = x[t];
+        if constexpr (CAUSAL) {  // delta_t = beta_t (v_t - the sum)
+          const uint32_t v2 = vraw[8 * b + t / 2];
+          x[t] = gt.beta[16 * b + t] *
+                 (__uint_as_float((t & 1) ? v2 & 0xffff0000u : v2 << 16) - x[t]);
+        }
+        const float dt = CAUSAL ? -x[t] : x[t];
 #pragma unroll
         for (int u4 = (t + 1) / 4; u4 < 4; ++u4) {
           const float4 a = *reinterpret_cast<const float4*>(ab + t * kATs + 4 * u4);
@@ -680,6 +784,13 @@ __global__ void __launch_bounds__(kCtThreads, 2)
           if (4 * u4 + 1 > t) x[4 * u4 + 1] = fmaf(-a.y, dt, x[4 * u4 + 1]);
           if (4 * u4 + 2 > t) x[4 * u4 + 2] = fmaf(-a.z, dt, x[4 * u4 + 2]);
           if (4 * u4 + 3 > t) x[4 * u4 + 3] = fmaf(-a.w, dt, x[4 * u4 + 3]);
+        }
+      }
+      if constexpr (LONG) {
+#pragma unroll
+        for (int e = 0; e < 16; ++e) {
+          dl[16 * b + e] = x[e];
+          d_last = 16 * b + e == n - 1 ? x[e] : d_last;
         }
       }
       if constexpr (VERIFY) {  // delta_t itself, for the states' recurrence
@@ -697,7 +808,7 @@ __global__ void __launch_bounds__(kCtThreads, 2)
 #pragma unroll
           for (int e = 0; e < 4; ++e) {
             const float xv = x[4 * i4 + e] * dr[e];
-            v[e] = 16 * b + 4 * i4 + e < n ? xv : 0.f;
+            v[e] = 16 * b + 4 * i4 + e < (LONG ? n - 1 : n) ? xv : 0.f;
           }
 #pragma unroll
           for (int f = 0; f < 2; ++f) {
@@ -737,7 +848,7 @@ __global__ void __launch_bounds__(kCtThreads, 2)
         if (k < BM / 16 - (kU > 1 ? b : 0) && b + k < nb) {  // uniform
 #pragma unroll
           for (int t = 0; t < 16; ++t) {
-            const float dt = x[t];
+            const float dt = CAUSAL ? -x[t] : x[t];
 #pragma unroll
             for (int u4 = 0; u4 < 4; ++u4) {
               const float4 a = *reinterpret_cast<const float4*>(ab + t * kATs + 16 * k + 4 * u4);
@@ -773,12 +884,7 @@ __global__ void __launch_bounds__(kCtThreads, 2)
         }
         // D += delta'^T K: the keys [t][i] as an MN-major operand (i contiguous)
         if constexpr (!VERIFY) {
-#pragma unroll 1
-        for (int kk = 0; kk < (n + 15) >> 4; ++kk) {
-          const uint64_t kb = tc::sdesc_sw128(tc::smem_u32(Ks + kk * 2048), C::kRows * 128, 1024);
-#pragma unroll
-          for (int y = 0; y < kT; ++y) tc::mma_bf16_ts(tmS, tmW + C::kDP * y + kk * 8, kb, idU, 1u);
-        }
+          update(n);
           tc::mma_commit(&sh.bar_mma);
         }
       }
@@ -803,14 +909,14 @@ __global__ void __launch_bounds__(kCtThreads, 2)
       // adjacent lanes swap one value so that each stores a bf16 pair of two columns
       const bool odd = lane & 1;
       __nv_bfloat16* out = static_cast<__nv_bfloat16*>(p.out_causal) +
-                           ((size_t)(it / p.Hv) * B * p.Hv + it % p.Hv) * kCtD + (tid & ~1);
+                           (((size_t)(it / p.Hv) * B + out0) * p.Hv + it % p.Hv) * kCtD + (tid & ~1);
 #pragma unroll
       for (int l = 0; l < BM; l += 2) {
         const float a = p.scale * o[l], b = p.scale * o[l + 1];
         const float recv = __shfl_xor_sync(0xffffffffu, odd ? a : b, 1);
         const int row = odd ? l + 1 : l;
         const __nv_bfloat162 w = odd ? __floats2bfloat162_rn(recv, b) : __floats2bfloat162_rn(a, recv);
-        if (row < B)
+        if (row < Bh)
           *reinterpret_cast<__nv_bfloat162*>(out + (size_t)row * p.Hv * kCtD) = w;
       }
     }
@@ -877,7 +983,7 @@ __global__ void __launch_bounds__(kCtThreads, 2)
       __syncthreads();  // the deltas and the keys, the last of this item's inputs, are read
       if (tid == 0 && it_next >= 0) {
         tc::fence_async_smem();
-        issue_kv(it_next);
+        issue_kv(it_next, 0);
         k_out = true;
         k_par = ph ^ 1u;
       }
@@ -887,15 +993,16 @@ __global__ void __launch_bounds__(kCtThreads, 2)
       tc::fence_after_sync();
       if (tid == 0) {
         mma_out = false;
-        if (it_next >= 0) {  // the update, the last reader of these keys, is done
+        // the update, the last reader of these keys, is done
+        if (it_next >= 0 && !(half_next && n < 32)) {
           tc::fence_async_smem();
-          issue_kv(it_next);
+          issue_kv(it_next, half_next);
           k_out = true;
           k_par = ph ^ 1u;
         }
       }
       // the committed state: lane c holds S^(n)[i][c] over i
-      if (!CAUSAL || n > 0) {
+      if (!CAUSAL || (n > 0 && !(half_next && n_item > 32))) {
         float* Sg = state_of(it, slot) + tid;
 #pragma unroll 1
         for (int i0 = 0; i0 < kCtD; i0 += 32) {
@@ -903,15 +1010,85 @@ __global__ void __launch_bounds__(kCtThreads, 2)
           tc::tmem_ld16(tmS + lane_off + i0, *reinterpret_cast<uint32_t(*)[16]>(&d[0]));
           tc::tmem_ld16(tmS + lane_off + i0 + 16, *reinterpret_cast<uint32_t(*)[16]>(&d[16]));
           tc::tmem_ld_wait();
+          if constexpr (LONG) add_last(d, Kt + i0, d_last);
 #pragma unroll
           for (int e = 0; e < 32; ++e) Sg[(size_t)(i0 + e) * kCtD] = __uint_as_float(d[e]);
         }
       }
     }
+    if constexpr (LONG) {
+      // the second half starts from the state after 32 tokens, whatever is accepted:
+      // where that is not the sum just taken, a second one, over all 32
+      if (half_next) {
+        if (n < 32) {
+          const float G31 = gt.Gam[31], e31 = gt.gam2[31], l31 = gt.glo[31];
+#pragma unroll 2
+          for (int i0 = 0; i0 < kCtD; i0 += 16) {
+            uint32_t d[16];
+#pragma unroll
+            for (int e = 0; e < 16; ++e) d[e] = __float_as_uint(G31 * S0s[(i0 + e) * kCtD + tid]);
+            tc::tmem_st16(tmS + lane_off + i0, d);
+          }
+#pragma unroll
+          for (int b = 0; b < 2; ++b) {
+            uint32_t dw[kT][8];
+#pragma unroll
+            for (int f = 0; f < 8; ++f) {
+              float v[2];
+#pragma unroll
+              for (int e = 0; e < 2; ++e) {
+                const int i = 16 * b + 2 * f + e;
+                v[e] = i < 31 ? dl[i] * tc::ex2((e31 - gt.gam2[i]) + (l31 - gt.glo[i])) : 0.f;
+              }
+              uint32_t s[kT];
+              split_terms<kT>(v[0], v[1], s);
+#pragma unroll
+              for (int y = 0; y < kT; ++y) dw[y][f] = s[y];
+            }
+#pragma unroll
+            for (int y = 0; y < kT; ++y) tc::tmem_st8(tmW + lane_off + C::kDP * y + 8 * b, dw[y]);
+          }
+          tc::tmem_st_wait();
+          tc::fence_before_sync();
+          __syncthreads();
+          if (warp == 0) {
+            mma_out = true;
+            tc::fence_after_sync();
+            if (tc::elect_one()) {
+              update(32);
+              tc::mma_commit(&sh.bar_mma);
+            }
+            __syncwarp();
+          }
+          if (!ct_wait(&sh.bar_mma, ph_mma, sh, p.dev_status)) break;
+          ph_mma ^= 1u;
+          tc::fence_after_sync();
+          if (tid == 0) {
+            mma_out = false;
+            tc::fence_async_smem();
+            issue_kv(it, 1);
+            k_out = true;
+            k_par = ph ^ 1u;
+          }
+        }
+#pragma unroll 1
+        for (int i0 = 0; i0 < kCtD; i0 += 32) {
+          uint32_t d[32];
+          tc::tmem_ld16(tmS + lane_off + i0, *reinterpret_cast<uint32_t(*)[16]>(&d[0]));
+          tc::tmem_ld16(tmS + lane_off + i0 + 16, *reinterpret_cast<uint32_t(*)[16]>(&d[16]));
+          tc::tmem_ld_wait();
+          add_last(d, Kt + (n < 32 ? kCtD : 0) + i0, dl[31]);
+#pragma unroll
+          for (int e = 0; e < 32; ++e) S0s[(i0 + e) * kCtD + tid] = __uint_as_float(d[e]);
+        }
+        tc::fence_async_smem();  // the next item's state is copied over it
+      }
+      half = half_next;
+    }
     if (it_next < 0) break;
     it = it_next;
     slot = slot_next;
-    n = n_next;
+    n_item = n_next;
     ph ^= 1u;
   }
 
@@ -976,7 +1153,7 @@ cudaError_t launch_ct(const GdrParams& p, cudaStream_t stream) {
       (CAUSAL && !ct_act_map(&maps.q, p.q, p.Hk, p.B, p.R, BM, true)) ||
       !ct_act_map(&maps.v, p.v, p.Hv, p.B, p.R, BM, false))
     return cudaErrorInvalidValue;
-  const int smem = CtCfg<BM, CAUSAL>::kSmem + 1024;
+  const int smem = CtCfg<BM, CAUSAL, MODE == 3>::kSmem + 1024;
   cudaError_t e = cudaFuncSetAttribute(gdr_commit_tc_kernel<BM, MODE>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
@@ -993,12 +1170,17 @@ cudaError_t launch_ct(const GdrParams& p, cudaStream_t stream) {
 }  // namespace
 
 bool gdr_commit_tc_supported(int B, int dk, int dv, bool causal) {
-  return B >= (causal ? 9 : 1) && B <= (causal ? 32 : 64) && dk == kCtD && dv == kCtD;
+  return B >= (causal ? 9 : 1) && B <= 64 && dk == kCtD && dv == kCtD;
+}
+
+bool gdr_verify_tc_supported(int B, int dk, int dv) {
+  return B >= 9 && B <= 32 && dk == kCtD && dv == kCtD;
 }
 
 cudaError_t launch_gdr_commit_tc(const GdrParams& p, cudaStream_t stream) {
   if (p.R == 0) return cudaSuccess;
   if (p.verify_len) return p.B <= 16 ? launch_ct<16, 2>(p, stream) : launch_ct<32, 2>(p, stream);
+  if (p.out_causal && p.B > 32) return launch_ct<32, 3>(p, stream);
   if (p.out_causal) return p.B <= 16 ? launch_ct<16, 1>(p, stream) : launch_ct<32, 1>(p, stream);
   if (p.B <= 16) return launch_ct<16, 0>(p, stream);
   return p.B <= 32 ? launch_ct<32, 0>(p, stream) : launch_ct<64, 0>(p, stream);

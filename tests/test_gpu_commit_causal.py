@@ -1,4 +1,4 @@
-"""The tensor-core commit with token-causal outputs (B <= 32, 128 x 128 states) at the
+"""The tensor-core commit with token-causal outputs (128 x 128 states) at the
 edges of its 16-token blocks, for ragged accepted lengths with zeros among them, and
 its precision: the fp32 operands enter as three bf16 terms, so a committed state is
 as close to 64 bits as the fp32 recurrence's (each about 2^-24 per product, a
@@ -36,16 +36,41 @@ def test_causal_commit_matches_oracle(block, heads):
             assert rel_fro(got[r], ref["state"][r]) < STATE_REL, (r, rel_fro(got[r], ref["state"][r]))
 
 
-def test_causal_commit_with_more_items_than_ctas():
+@pytest.mark.parametrize("block", [33, 47, 48, 49, 63, 64])
+def test_blocks_in_two_halves(block):
+    """Blocks of 33..64 run as two halves of 32 tokens: lengths accepted in the first half
+    (its end and the edges of its 16-token parts), at the seam and in the second."""
+    n = sorted({0, 1, 15, 16, 17, 31, 32, 33, 40, min(48, block), block - 1, block})
+    n = [x for x in n if x <= block]
+    spec = LARGE.replace(num_requests=len(n), block_len=block, num_qk_heads=3, num_v_heads=3,
+                         seed=220 + block)
+    w = gen(spec)
+    install_states(w)
+    pool = w.state_pool.clone()
+    acc = torch.tensor(n, dtype=torch.int32).cuda()
+    out = run_commit(w, pool, causal=True, accept_len=acc)
+    ref = oracle_commit(w, w.state_pool, causal=True, accept_len=acc)
+    assert_out_close(out, ref["causal"], "bf16", f"B = {block}")
+    slots = w.state_slot.long()
+    got = pool[slots].double().cpu().numpy()
+    for r in range(len(n)):
+        if n[r] == 0:
+            assert torch.equal(pool[slots[r]], w.state_pool[slots[r]])
+        else:
+            assert rel_fro(got[r], ref["state"][r]) < STATE_REL, (n[r], rel_fro(got[r], ref["state"][r]))
+
+
+@pytest.mark.parametrize("block", [27, 64])
+def test_causal_commit_with_more_items_than_ctas(block):
     # 40 requests x 32 heads on 304 CTAs: every CTA walks several items, some of
     # them without accepted tokens
-    spec = LARGE.replace(num_requests=40, block_len=27, seed=219)
+    spec = LARGE.replace(num_requests=40, block_len=block, seed=219)
     w = gen(spec)
     install_states(w, requests=[0, 13, 39])
     pool = w.state_pool.clone()
-    acc = (torch.arange(40, dtype=torch.int32) * 7 % 28).cuda()
+    acc = (torch.arange(40, dtype=torch.int32) * 7 % (block + 1)).cuda()
     out = run_commit(w, pool, causal=True, accept_len=acc)
-    sample = [0, 4, 13, 39]  # accepted 0, 0, 7, 21
+    sample = [0, 4, 13, 39]
     ref = oracle_commit(w, w.state_pool, requests=sample, causal=True, accept_len=acc)
     assert_out_close(out[sample], ref["causal"], "bf16", "sampled requests")
     got = pool[w.state_slot.long()[sample]].double().cpu().numpy()
@@ -56,7 +81,7 @@ def test_causal_commit_with_more_items_than_ctas():
     assert np.isnan(pool[(~used).cuda()].cpu().numpy()).all()  # free slots untouched
 
 
-@pytest.mark.parametrize("block,token", [(32, 20), (16, 3), (27, 16)])
+@pytest.mark.parametrize("block,token", [(32, 20), (16, 3), (27, 16), (64, 20), (64, 32), (45, 40)])
 def test_infinite_and_nan_tokens_stay_after_their_place(block, token):
     """A token whose key or value is infinite or NaN changes no output before it and no
     state committed before it."""
