@@ -162,8 +162,16 @@ def kernel_of_call(spec):
             "softmax": "softmax_tc_kernel",
             "commit": "gdr_commit_tc_kernel" if tc_state else "gdr_commit_kernel",
             "shortconv": "short_conv_kernel", "shortconv_commit": "short_conv_kernel"}
-VERIFY_KERNEL_OF = {"linear": "gdr_commit_kernel", "softmax": "softmax_tc_kernel",
+VERIFY_KERNEL_OF = {"linear": "gdr_commit_tc_kernel", "softmax": "softmax_tc_kernel",
                     "commit": "verify_commit_kernel"}
+
+
+def traffic_kernel_of(spec, call, kernel):
+    """The kernel whose traffic summary goes with `call`: bf16 softmax calls with more
+    than 128 query rows per kv head and D >= 128 run the two-SM form of the softmax."""
+    rows = spec.num_q_heads // spec.num_kv_heads * spec.block_len
+    pair = spec.act_dtype == "bf16" and rows > 128 and spec.head_dim >= 128
+    return "softmax_pair_kernel" if call == "softmax" and pair else kernel
 
 
 def profiled_traffic(kernel, workload):
@@ -779,7 +787,8 @@ def summarise(fr, per, timed_s, clk):
         peak_source = f"{peaks['source']} (hbm_gbs)"
     roof["frac"] = roof["achieved"] / roof["peak"]
     kernel_of = VERIFY_KERNEL_OF if fr.verify else kernel_of_call(s)
-    roof["traffic"] = profiled_traffic(kernel_of[dom], s.name) if dom in kernel_of else None
+    roof["traffic"] = profiled_traffic(traffic_kernel_of(s, dom, kernel_of[dom]), s.name) \
+        if dom in kernel_of else None
     roof["kernel"] = kd["kernel"]
     roof["peak_source"] = peak_source
     roof["algorithmic_per_launch"] = kd["flops"] if roof["bound"] == "tensor" else kd["bytes"]

@@ -334,9 +334,10 @@ flare_status flare_short_conv(const flare_conv_desc* desc, const void* x, void* 
  * advanced over the clean tokens of the chunk's earlier blocks (f_blk), on
  * chip; no block-boundary state is written.  The clean outputs are the clean
  * chunkwise pass's and are not formed here.  Value head j reads q/k head
- * j / (Hv / Hk).  Arithmetic: bf16 activations run the state's products and
- * updates as tf32 tensor-core products with fp32 accumulation (the state
- * itself stays fp32); fp32 activations run exact fp32.
+ * j / (Hv / Hk).  Arithmetic: bf16 activations run the products with
+ * the state, rounded to bf16, and the block's dot products as bf16 tensor-core
+ * products and the clean deltas as split-bf16 ones, all with fp32 accumulation;
+ * fp32 activations run exact fp32.
  *   chunk_states  [N, Hv, L/C, dk, dv]   fp32
  *   k, v          [N, L, Hk, dk], [N, L, Hv, dv]   clean, act_dtype
  *   log_decay, beta [N, L, Hv]           clean, fp32
@@ -357,8 +358,8 @@ flare_status flare_two_stream_fwd(const flare_two_stream_desc* desc, const float
 
 /*
  * Bytes of device workspace flare_block_softmax_attn needs for `desc`
- * (the longest-first order of the work units and the partial outputs of split
- * prefixes).  May be 0.  Host-only, no GPU work.
+ * (the partial outputs of split prefixes and, above 512 requests whose prefixes
+ * are not split, the longest-first order).  May be 0.  Host-only, no GPU work.
  */
 flare_status flare_softmax_workspace_size(const flare_softmax_desc* desc, size_t* bytes);
 
@@ -430,8 +431,8 @@ flare_status flare_append_kv(const flare_softmax_desc* desc, const void* k_blk, 
  * requests are in flight (they synchronize the device and can fail under
  * memory pressure), or a plugin host that passes only the request's own
  * tensors.  Same arguments, layouts, outputs and status bits as
- * flare_block_softmax_attn, minus the workspace: the workspace (work order and split partials) lives in a
- * file-scope device array of FLARE_NOALLOC_SCRATCH_BYTES that the library
+ * flare_block_softmax_attn, minus the workspace, which lives in a file-scope
+ * device array of FLARE_NOALLOC_SCRATCH_BYTES that the library
  * holds on every GPU that loads it, until the process exits.
  *  - This call allocates nothing (no cudaMalloc, cudaFree or allocating
  *    library routine).

@@ -121,9 +121,9 @@ SoftmaxPlan plan_softmax(int R, int B, int Hq, int Hkv, int D, int page_size, in
   if (bf16 && softmax_pair_supported(B, Hq, Hkv, D, page_size)) {
     // two-SM kernel, for every shape with a second row tile to share the keys
     // with (at M <= 128 the second CTA would have no rows): 256 query rows per
-    // pair of CTAs, one pair per two SMs.  One SM per row tile takes 1.023 ms
-    // where this takes 0.763 (128 requests, B = 64, G = 8) and 0.150 against
-    // 0.128 (64 requests, B = 32, G = 8).  Splits as below, over 128-key tiles.
+    // pair of CTAs, one pair per two SMs.  One SM per row tile takes 1.03 ms
+    // where this takes 0.76 (128 requests, B = 64, G = 8) and 0.150 against
+    // 0.118 (64 requests, B = 32, G = 8).  Splits as below, over 128-key tiles.
     pl.kernel = 2;
     pl.rows_per_cta = 128;
     pl.n_split = tc_splits((long)R * Hkv * ((M + 255) / 256), num_sms / 2, (prefix_max + 127) / 128,

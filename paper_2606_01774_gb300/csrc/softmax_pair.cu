@@ -13,10 +13,10 @@
 // two streams through its shared memory and the rings' bytes in flight set the
 // tile rate, not the tensor pipe; the pair halves both per product.
 //
-// Measured (GB300, start against this kernel): 128 requests, blocks of 64,
-// prefixes of 1024..16384, D = 256: 1.023 -> 0.763 ms per call back to back
-// (1.54 PFLOP/s, at the power cap; 0.65 ms, 1.81 PFLOP/s, in short bursts);
-// 64 requests, blocks of 32, prefixes of 512..8192: 0.150 -> 0.128 ms.  Bound
+// Measured (GB300, one SM per row tile against this kernel): 128 requests, blocks of
+// 64, prefixes of 1024..16384, D = 256: 1.03 -> 0.76 ms per call back to back
+// (1.5 PFLOP/s, at the power cap; 0.65 ms, 1.81 PFLOP/s, in short bursts);
+// 64 requests, blocks of 32, prefixes of 512..8192: 0.150 -> 0.118 ms.  Bound
 // by the tensor pipe (1.26 us per 128-key tile of a pair, 0.99 us at the clock's
 // peak rate) and, for the smaller call, by HBM.
 
