@@ -25,6 +25,7 @@ constexpr int kMaxBlock = 64;  // tokens of a block; at least one thread each
 __global__ void __launch_bounds__(kAppendThreads)
     append_kv_kernel(SoftmaxParams p, const int32_t* append_len, void* k_pool, void* v_pool,
                      int row_shift) {  // log2 of the 16-byte chunks of a (token, head) row
+  stream_order();
   __shared__ int pages[kMaxBlock];
   const int r = blockIdx.x, tid = threadIdx.x;
   const int P = p.prefix_len[r];
@@ -81,8 +82,9 @@ cudaError_t launch_append_kv(const SoftmaxParams& p, const int32_t* append_len, 
   while ((16 << row_shift) < p.D * elem_bytes) ++row_shift;
   const size_t block = ((size_t)p.B * p.Hkv) << row_shift;
   const size_t slices = (block + kAppendThreads * kChunks - 1) / (kAppendThreads * kChunks);
-  append_kv_kernel<<<dim3((unsigned)p.R, (unsigned)(slices < 65535 ? slices : 65535)),
-                     kAppendThreads, 0, stream>>>(p, append_len, k_pool, v_pool, row_shift);
+  const dim3 grid((unsigned)p.R, (unsigned)(slices < 65535 ? slices : 65535));
+  launch_kernel(append_kv_kernel, grid, kAppendThreads, 0, stream, p, append_len, k_pool, v_pool,
+                row_shift);
   note_launches(1);
   return cudaGetLastError();
 }

@@ -92,6 +92,7 @@ __device__ __forceinline__ void stage_rows(float* dst, const T* src, size_t stri
 // 3: denoise pass (block-end readout, the pool is only read).
 template <typename T, int DK, int DV, int MODE>
 __global__ void __launch_bounds__(2 * DV, 2) gdr_commit_kernel(GdrParams p) {
+  stream_order();
   constexpr bool CAUSAL = MODE != 0;  // queries staged, readouts written
   constexpr bool VERIFY = MODE == 2;
   constexpr bool DENOISE = MODE == 3;
@@ -351,7 +352,7 @@ cudaError_t launch_commit_t(const GdrParams& p, cudaStream_t stream) {
                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem_for(kCBmax));
   if (e != cudaSuccess) return e;
-  gdr_commit_kernel<T, DK, DV, MODE><<<p.R * p.Hv, 2 * DV, smem_for(p.B), stream>>>(p);
+  launch_kernel(gdr_commit_kernel<T, DK, DV, MODE>, p.R * p.Hv, 2 * DV, smem_for(p.B), stream, p);
   note_launches(1);
   return cudaGetLastError();
 }

@@ -228,6 +228,7 @@ __device__ __forceinline__ void split_terms(float a, float b, uint32_t (&w)[N]) 
 template <int BM, int MODE>
 __global__ void __launch_bounds__(kCtThreads, 2)
     gdr_commit_tc_kernel(const __grid_constant__ CtMaps maps, GdrParams p) {
+  stream_order();
   constexpr bool CAUSAL = MODE != 0, VERIFY = MODE == 2, LONG = MODE == 3;
   static_assert(!CAUSAL || BM <= 32, "tensor memory");
   using C = CtCfg<BM, CAUSAL, LONG>;
@@ -1162,7 +1163,7 @@ cudaError_t launch_ct(const GdrParams& p, cudaStream_t stream) {
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const long items = (long)p.R * p.Hv;
   const int grid = (int)(items < 2L * sms ? items : 2L * sms);
-  gdr_commit_tc_kernel<BM, MODE><<<grid, kCtThreads, smem, stream>>>(maps, p);
+  launch_kernel(gdr_commit_tc_kernel<BM, MODE>, grid, kCtThreads, smem, stream, maps, p);
   note_launches(1);
   return cudaGetLastError();
 }

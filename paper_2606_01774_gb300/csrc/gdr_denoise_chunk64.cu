@@ -111,6 +111,7 @@ __device__ __forceinline__ int d6_next(const GdrParams& p, int it, int total, in
 
 __global__ void __launch_bounds__(kD6Threads, 2)
     gdr_denoise_chunk64_kernel(const __grid_constant__ D6Maps maps, GdrParams p) {
+  stream_order();
   using C = D6Cfg;
   constexpr int kIssuer = 32;  // warp 1 issues every copy and MMA
   // no static shared memory, so that the dynamic window starts 1024-byte
@@ -570,7 +571,7 @@ cudaError_t launch_gdr_denoise_chunk64(const GdrParams& p, cudaStream_t stream) 
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const long items = (long)p.R * p.Hv;
   const int grid = (int)(items < 2L * sms ? items : 2L * sms);
-  gdr_denoise_chunk64_kernel<<<grid, kD6Threads, smem, stream>>>(maps, p);
+  launch_kernel(gdr_denoise_chunk64_kernel, grid, kD6Threads, smem, stream, maps, p);
   note_launches(1);
   return cudaGetLastError();
 }

@@ -146,6 +146,7 @@ __device__ __forceinline__ void dp_diag_inverse(const float* AT, float* Tf, int 
 template <int BM>
 __global__ void __launch_bounds__(kDpThreads, 2)
     gdr_denoise_persist_kernel(const __grid_constant__ DpMaps maps, GdrParams p) {
+  stream_order();
   using C = DpCfg<BM>;
   constexpr int kATs = C::kATs;
   constexpr int kG0 = C::kG0;
@@ -660,7 +661,7 @@ cudaError_t launch_dp(const GdrParams& p, cudaStream_t stream) {
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const long items = (long)p.R * p.Hv;
   const int grid = (int)(items < 2L * sms ? items : 2L * sms);
-  gdr_denoise_persist_kernel<BM><<<grid, kDpThreads, smem, stream>>>(maps, p);
+  launch_kernel(gdr_denoise_persist_kernel<BM>, grid, kDpThreads, smem, stream, maps, p);
   note_launches(1);
   return cudaGetLastError();
 }

@@ -134,6 +134,7 @@ __device__ __forceinline__ void store16_sw128(uint8_t* tile, int row, int c0, co
 template <int DK, int DV, int BM>
 __global__ void __launch_bounds__(kLinThreads, LinCfg<DK, DV, BM>::kMinBlocks)
     gdr_denoise_tc_kernel(const __grid_constant__ LinMaps maps, GdrParams p) {
+  stream_order();
   using C = LinCfg<DK, DV, BM>;
   constexpr int kATs = C::kATs;
   extern __shared__ uint8_t smem_raw[];
@@ -534,7 +535,7 @@ cudaError_t launch_lin_tc_bm(const GdrParams& p, cudaStream_t stream) {
   cudaError_t e = cudaFuncSetAttribute(gdr_denoise_tc_kernel<DK, DV, BM>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  gdr_denoise_tc_kernel<DK, DV, BM><<<p.R * p.Hv, kLinThreads, smem, stream>>>(maps, p);
+  launch_kernel(gdr_denoise_tc_kernel<DK, DV, BM>, p.R * p.Hv, kLinThreads, smem, stream, maps, p);
   note_launches(1);
   return cudaGetLastError();
 }

@@ -134,6 +134,7 @@ __device__ __forceinline__ int conv_check(const ConvParams& p, int r) {
 template <typename T, int W>
 __global__ void __launch_bounds__(kConvThreads + 32, ConvCols<T>::kCtasPerSM)
     short_conv_kernel(const __grid_constant__ ConvMaps maps, ConvParams p) {
+  stream_order();
   constexpr int E = sizeof(T);
   constexpr int kColBytes = ConvCols<T>::kColBytes;
   constexpr int kSlabBytes = ConvCols<T>::kSlabBytes;
@@ -397,7 +398,8 @@ cudaError_t launch_conv_w(const ConvParams& p, int grid, cudaStream_t stream) {
   if (p.C % (512 / (int)sizeof(T)) == 0 && rows_total < (1l << 31))
     maps.use = sc_map<T>(&maps.x_halo, p.x, p.C, rows_total, kChunkRows + W - 1) &&
                sc_map<T>(&maps.x_first, p.x, p.C, rows_total, kChunkRows);
-  short_conv_kernel<T, W><<<grid, kConvThreads + 32, ConvCols<T>::kSmem, stream>>>(maps, p);
+  launch_kernel(short_conv_kernel<T, W>, grid, kConvThreads + 32, ConvCols<T>::kSmem, stream, maps,
+                p);
   note_launches(1);
   return cudaGetLastError();
 }

@@ -309,6 +309,7 @@ __device__ __forceinline__ bool softmax_row(uint32_t sbuf, int lim, float scale_
 template <int D>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
     softmax_pair_kernel(const __grid_constant__ PairMaps maps, SoftmaxParams p) {
+  stream_order();
   using C = PairCfg<D>;
   extern __shared__ uint8_t smem_raw[];
   __shared__ PairShared sh;
@@ -848,7 +849,8 @@ cudaError_t launch_pair_d(const SoftmaxParams& p, const SoftmaxPlan& plan, cudaS
   if (plan.num_ctas <= 0) return cudaErrorInvalidValue;
   if (p.order) err = launch_softmax_order(p, stream);
   if (err != cudaSuccess) return err;
-  softmax_pair_kernel<D><<<(unsigned)plan.num_ctas, kPairThreads, smem, stream>>>(maps, p);
+  launch_kernel(softmax_pair_kernel<D>, (unsigned)plan.num_ctas, kPairThreads, smem, stream, maps,
+                p);
   note_launches(1);
   err = cudaGetLastError();
   return err == cudaSuccess && p.n_split > 1 ? launch_softmax_merge(p, stream) : err;

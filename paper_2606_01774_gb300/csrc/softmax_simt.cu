@@ -43,6 +43,7 @@ __device__ __forceinline__ void widen(const uint4& v, float* f) {
 // one request of 2 heads, D = 64, 40 keys took 22 us.)
 template <typename T, int D>
 __global__ void __launch_bounds__(kThreads) softmax_simt_kernel(SoftmaxParams p) {
+  stream_order();
   constexpr int kVec = 16 / sizeof(T);         // elements of a 16-byte load
   constexpr int kLoads = kTile * (D / kVec) / kThreads;  // per thread and array
   constexpr int kKs = D + 4;                   // key row stride: 16-byte reads of 8 rows tile the banks
@@ -227,6 +228,7 @@ __global__ void __launch_bounds__(kThreads) softmax_simt_kernel(SoftmaxParams p)
 // lse = log sum_s exp(lse_s), out = sum_s exp(lse_s - lse) out_s.
 template <typename T>
 __global__ void __launch_bounds__(256) softmax_combine_kernel(SoftmaxParams p) {
+  stream_order();
   const int item = blockIdx.x, m = blockIdx.y;
   const int r = item / p.Hkv, kvh = item % p.Hkv;
   const int M = p.B * p.G;
@@ -284,7 +286,7 @@ cudaError_t launch_simt_d(const SoftmaxParams& p, const SoftmaxPlan& plan, cudaS
   if (e != cudaSuccess) return e;
   const int M = p.B * p.G;
   dim3 grid(plan.n_split, p.R * p.Hkv, (M + kRows - 1) / kRows);
-  softmax_simt_kernel<T, D><<<grid, kThreads, smem, stream>>>(p);
+  launch_kernel(softmax_simt_kernel<T, D>, grid, kThreads, smem, stream, p);
   note_launches(1);
   e = cudaGetLastError();
   if (e != cudaSuccess || plan.n_split == 1) return e;
@@ -305,9 +307,9 @@ cudaError_t launch_simt(const SoftmaxParams& p, const SoftmaxPlan& plan, cudaStr
 cudaError_t launch_softmax_combine(const SoftmaxParams& p, bool bf16, cudaStream_t stream) {
   const dim3 grid(p.R * p.Hkv, p.B * p.G);
   if (bf16)
-    softmax_combine_kernel<__nv_bfloat16><<<grid, 256, 0, stream>>>(p);
+    launch_kernel(softmax_combine_kernel<__nv_bfloat16>, grid, 256, 0, stream, p);
   else
-    softmax_combine_kernel<float><<<grid, 256, 0, stream>>>(p);
+    launch_kernel(softmax_combine_kernel<float>, grid, 256, 0, stream, p);
   note_launches(1);
   return cudaGetLastError();
 }

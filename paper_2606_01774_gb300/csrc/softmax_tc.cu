@@ -203,6 +203,7 @@ constexpr int kOrderThreads = 1024;
 constexpr int kOrderKeys = 4 * kOrderThreads;
 
 __global__ void __launch_bounds__(kOrderThreads) softmax_order_kernel(SoftmaxParams p) {
+  stream_order();
   __shared__ int start[kOrderKeys];
   __shared__ int wsum[kOrderThreads / 32];
   __shared__ int n_valid;
@@ -275,6 +276,7 @@ constexpr int kMergeWarps = 8;
 
 template <int D>
 __global__ void __launch_bounds__(32 * kMergeWarps) softmax_merge_kernel(SoftmaxParams p) {
+  stream_order();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int M = p.B * p.G;
   const long long row = (long long)blockIdx.x * kMergeWarps + warp;
@@ -327,6 +329,7 @@ __global__ void __launch_bounds__(32 * kMergeWarps) softmax_merge_kernel(Softmax
 template <int D>
 __global__ void __launch_bounds__(kThreadsTC, 1)
     softmax_tc_kernel(const __grid_constant__ TcMaps maps, SoftmaxParams p) {
+  stream_order();
   using C = TcCfg<D>;
   constexpr int kSB = C::kSBuf;
   extern __shared__ uint8_t smem_raw[];
@@ -885,7 +888,7 @@ bool encode_map(CUtensorMap* m, const void* ptr, int rank, const uint64_t* dims,
 
 cudaError_t launch_softmax_order(const SoftmaxParams& p, cudaStream_t stream) {
   if (!p.order || !p.n_valid) return cudaErrorInvalidValue;
-  softmax_order_kernel<<<1, kOrderThreads, 0, stream>>>(p);
+  launch_kernel(softmax_order_kernel, 1, kOrderThreads, 0, stream, p);
   note_launches(1);
   return cudaGetLastError();
 }
@@ -894,9 +897,9 @@ cudaError_t launch_softmax_merge(const SoftmaxParams& p, cudaStream_t stream) {
   const long long rows = (long long)p.R * p.Hkv * p.B * p.G;
   const unsigned grid = (unsigned)((rows + kMergeWarps - 1) / kMergeWarps);
   switch (p.D) {
-    case 64: softmax_merge_kernel<64><<<grid, 32 * kMergeWarps, 0, stream>>>(p); break;
-    case 128: softmax_merge_kernel<128><<<grid, 32 * kMergeWarps, 0, stream>>>(p); break;
-    default: softmax_merge_kernel<256><<<grid, 32 * kMergeWarps, 0, stream>>>(p); break;
+    case 64: launch_kernel(softmax_merge_kernel<64>, grid, 32 * kMergeWarps, 0, stream, p); break;
+    case 128: launch_kernel(softmax_merge_kernel<128>, grid, 32 * kMergeWarps, 0, stream, p); break;
+    default: launch_kernel(softmax_merge_kernel<256>, grid, 32 * kMergeWarps, 0, stream, p); break;
   }
   note_launches(1);
   return cudaGetLastError();
@@ -940,7 +943,7 @@ cudaError_t launch_tc_d(const SoftmaxParams& p, const SoftmaxPlan& plan, cudaStr
   if (plan.num_ctas <= 0) return cudaErrorInvalidValue;
   if (p.order) err = launch_softmax_order(p, stream);
   if (err != cudaSuccess) return err;
-  softmax_tc_kernel<D><<<(unsigned)plan.num_ctas, kThreadsTC, smem, stream>>>(maps, p);
+  launch_kernel(softmax_tc_kernel<D>, (unsigned)plan.num_ctas, kThreadsTC, smem, stream, maps, p);
   note_launches(1);
   err = cudaGetLastError();
   return err == cudaSuccess && p.n_split > 1 ? launch_softmax_merge(p, stream) : err;

@@ -88,6 +88,7 @@ __device__ __forceinline__ void ts_stage(T* dst, const T* src, size_t stride) {
 template <typename T, int DK, int DV, int B>
 __global__ void __launch_bounds__(2 * DV, (B <= 4 && sizeof(T) == 2) ? 2 : 1)
     two_stream_fwd_kernel(TwoStreamParams p) {
+  stream_order();
   constexpr int kThreads = 2 * DV;
   constexpr int kR = DK / 8;  // state rows per thread
   static_assert(kR % 16 == 0, "a thread's state rows are read 16 at a time");
@@ -319,7 +320,7 @@ cudaError_t launch_ts_t(const TwoStreamParams& p, cudaStream_t stream) {
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   const unsigned grid = (unsigned)((size_t)p.N * p.Hv * (p.L / kTsChunk));
-  two_stream_fwd_kernel<T, DK, DV, B><<<grid, 2 * DV, smem, stream>>>(p);
+  launch_kernel(two_stream_fwd_kernel<T, DK, DV, B>, grid, 2 * DV, smem, stream, p);
   note_launches(1);
   return cudaGetLastError();
 }

@@ -100,6 +100,7 @@ struct CkMaps {
 template <int B>
 __global__ void __launch_bounds__(kCkThreads, 1)
     two_stream_chunk_kernel(const __grid_constant__ CkMaps maps, TwoStreamParams p) {
+  stream_order();
   using C = CkCfg;
   constexpr int kIssuer = 32;  // warp 1 issues every copy and MMA
   extern __shared__ uint8_t smem_raw[];
@@ -705,7 +706,7 @@ cudaError_t launch_ck(const TwoStreamParams& p, cudaStream_t stream) {
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const long items = (long)p.N * p.Hv * (p.L / kCkC);
   const int grid = (int)(items < sms ? items : sms);
-  two_stream_chunk_kernel<B><<<grid, kCkThreads, smem, stream>>>(maps, p);
+  launch_kernel(two_stream_chunk_kernel<B>, grid, kCkThreads, smem, stream, maps, p);
   note_launches(1);
   return cudaGetLastError();
 }

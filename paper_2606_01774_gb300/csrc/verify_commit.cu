@@ -19,6 +19,7 @@ constexpr int kVecPerTile = kCopyThreads * kVecPerThread;       // 64 KiB per CT
 }  // namespace
 
 __global__ void __launch_bounds__(kCopyThreads) verify_commit_kernel(VerifyCommitParams p) {
+  stream_order();
   const int tile = blockIdx.x, r = blockIdx.y, l = blockIdx.z;
   const int slot = p.state_slot[r], K = p.verify_len[r], a = p.accept[r];
   const bool first = tile == 0 && l == 0 && threadIdx.x == 0;
@@ -53,8 +54,8 @@ cudaError_t launch_verify_commit(const VerifyCommitParams& p, cudaStream_t strea
   if (p.R == 0 || p.n_layers == 0) return cudaSuccess;
   const size_t n_vec = p.state_elems / 4;
   const unsigned tiles = (unsigned)((n_vec + kVecPerTile - 1) / kVecPerTile);
-  verify_commit_kernel<<<dim3(tiles, (unsigned)p.R, (unsigned)p.n_layers), kCopyThreads, 0,
-                         stream>>>(p);
+  launch_kernel(verify_commit_kernel, dim3(tiles, (unsigned)p.R, (unsigned)p.n_layers),
+                kCopyThreads, 0, stream, p);
   note_launches(1);
   return cudaGetLastError();
 }
