@@ -13,7 +13,9 @@ namespace flare {
 // the stream (launch_kernel) and begins with this: its CTAs are set up as the kernel
 // ahead drains, and touch no memory before all of that kernel's work is done and
 // visible.  Every thread comes here, so that a grid that has ended implies the grids
-// before it.  Between two calls this takes out most of the launch gap, a fixed
+// before it, and before any tensor-memory allocation: a kernel ahead that lets its
+// dependents start early could otherwise need the columns that its dependents hold.
+// Between two calls this takes out most of the launch gap, a fixed
 // cost of about 2 us: one request's step (four launches) 45.3 -> 37.8 us, ShortConv
 // of 64 requests 19.3 -> 17.1, linear 45.3 -> 43.0, state update 97.3 -> 93.5, verify
 // round 279 -> 272.  An early trigger (griddepcontrol.launch_dependents at the

@@ -57,7 +57,7 @@
 // as the tensor core rounds every step toward zero.  The committed states are 7.5e-8
 // off 64 bits at B = 9..32 (1.25e-7 without the solve's order, 1.7e-7 without the
 // update's as well), where the recurrence's are 1.4e-7 to 6.4e-7.  State update of 64
-// requests (32 heads) with its append, B = 32: 208 -> 97 us.  Blocks of 8 and
+// requests (32 heads) with its append, B = 32: 208 -> 93 us.  Blocks of 8 and
 // fewer stay with the recurrence: 82 and 77 us at B = 8 for 64 requests, 14.4 and
 // 16.5 for one; 71 and 77 at B = 4.
 //
@@ -67,9 +67,10 @@
 // the 256 that two CTAs per SM leave each.  Where fewer than 32 tokens are accepted
 // the first half sums twice, to the accepted length for the pool and over all 32 for
 // the second half.  As the recurrence is closer for these blocks (7.1e-8: it walks
-// the gates one by one where they fall below 2^-40), the last token of a sum, its
-// largest term, adds in fp32 (6.7e-8; without 7.6e-8 and 330 us).  State update of
-// 128 requests, B = 64: 738 -> 351 us; of 64, B = 33, the worst case, 217 -> 175.
+// the gates one by one where they fall below 2^-40), the last token of a committed
+// sum, its largest term, adds in fp32 (6.7e-8, without 7.6e-8; in the first half's
+// sum over all 32 too it takes 16 us more and is no closer).  State update of 128
+// requests, B = 64: 738 -> 331 us; of 64, B = 33, the worst case, 217 -> 163.
 //
 // The verify round (VERIFY) is the causal form with other outputs: rows l <= K read
 // the state after their own token and rows past K the block-end state, so M2 is
@@ -122,8 +123,8 @@ struct CtCfg {
   // tensor-memory columns of each bf16 part of delta'^T (whole 16-column stores)
   static constexpr int kDP = BM / 2 < 16 ? 16 : BM / 2;
   static constexpr int kM2 = CAUSAL ? 2 * BM * 128 : 0;  // M2[l][i] bf16 hi, lo (K-major SW128)
-  // LONG: the 16 keys around the accepted length, and (fp32) the last one of each sum
-  static constexpr int kKz = LONG ? 2 * 16 * 128 + 2 * kCtD * 4 : 0;
+  // LONG: the 16 keys around the accepted length, and (fp32) the last of them
+  static constexpr int kKz = LONG ? 2 * 16 * 128 + kCtD * 4 : 0;
   static constexpr int kSmem = kS0 + kK + kR + kM2 + kKz;
   static constexpr int kTerms = CAUSAL ? 3 : 2;    // bf16 terms of an fp32 operand
 };
@@ -426,11 +427,11 @@ __global__ void __launch_bounds__(kCtThreads, 2)
   }
   int cand = item_at(pos + 1);
   int cs = cand_slot(cand), ca = cand_len(cand);
-  // LONG: the last token of a sum, its largest term, in fp32 after the others
-  auto add_last = [&](uint32_t(&d)[32], const float* k, float delta) {
+  // LONG: the last token of a committed sum, its largest term, in fp32 after the others
+  auto add_last = [&](uint32_t(&d)[32], int i0, float delta) {
 #pragma unroll
     for (int e4 = 0; e4 < 8; ++e4) {
-      const float4 a = *reinterpret_cast<const float4*>(k + 4 * e4);
+      const float4 a = *reinterpret_cast<const float4*>(Kt + i0 + 4 * e4);
       const float ka[4] = {a.x, a.y, a.z, a.w};
 #pragma unroll
       for (int e = 0; e < 4; ++e)
@@ -721,14 +722,10 @@ __global__ void __launch_bounds__(kCtThreads, 2)
                          : make_uint4(0u, 0u, 0u, 0u);
       }
       tc::fence_async_smem();
-#pragma unroll
-      for (int x = 0; x < 2; ++x) {
-        const int t = x ? 31 : max(n - 1, 0);
-        const uint8_t* kr = Ks + (tid >> 6) * (C::kRows * 128) + t * 128 +
-                            ((((tid >> 3) & 7) ^ (t & 7)) << 4) + (tid & 7) * 2;
-        Kt[x * kCtD + tid] =
-            __uint_as_float((uint32_t)*reinterpret_cast<const unsigned short*>(kr) << 16);
-      }
+      const int last = max(n - 1, 0);
+      const uint8_t* kr = Ks + (tid >> 6) * (C::kRows * 128) + last * 128 +
+                          ((((tid >> 3) & 7) ^ (last & 7)) << 4) + (tid & 7) * 2;
+      Kt[tid] = __uint_as_float((uint32_t)*reinterpret_cast<const unsigned short*>(kr) << 16);
     } else if constexpr (CAUSAL && !VERIFY) {
       const int n16 = (((n + 15) & ~15) - n) * 16;  // 16-byte pieces: 8 of each 64-column chunk
       for (int e = tid; e < n16; e += kCtThreads)
@@ -765,7 +762,9 @@ __global__ void __launch_bounds__(kCtThreads, 2)
     // down in the registers, and go to tensor memory as delta'_t =
     // exp(gamma_{n-1} - gamma_t) delta_t (t < n) in bf16 hi and lo parts.
     float dl[LONG ? BM : 1];  // LONG: the deltas
-    float d_last = 0.f;       // and the last accepted token's, which adds in fp32
+    // and the last accepted token's, which adds in fp32 where the sum is committed
+    float d_last = 0.f;
+    const int n_mma = LONG && !(half_next && n_item > 32) ? n - 1 : n;
 #pragma unroll kU
     for (int b = 0; b < BM / 16; ++b) {
       if (kU == 1 && b >= nb) break;  // uniform (two blocks: 69.6 us with the branch, 68.4 without)
@@ -809,7 +808,7 @@ __global__ void __launch_bounds__(kCtThreads, 2)
 #pragma unroll
           for (int e = 0; e < 4; ++e) {
             const float xv = x[4 * i4 + e] * dr[e];
-            v[e] = 16 * b + 4 * i4 + e < (LONG ? n - 1 : n) ? xv : 0.f;
+            v[e] = 16 * b + 4 * i4 + e < n_mma ? xv : 0.f;
           }
 #pragma unroll
           for (int f = 0; f < 2; ++f) {
@@ -1011,7 +1010,7 @@ __global__ void __launch_bounds__(kCtThreads, 2)
           tc::tmem_ld16(tmS + lane_off + i0, *reinterpret_cast<uint32_t(*)[16]>(&d[0]));
           tc::tmem_ld16(tmS + lane_off + i0 + 16, *reinterpret_cast<uint32_t(*)[16]>(&d[16]));
           tc::tmem_ld_wait();
-          if constexpr (LONG) add_last(d, Kt + i0, d_last);
+          if constexpr (LONG) add_last(d, i0, d_last);
 #pragma unroll
           for (int e = 0; e < 32; ++e) Sg[(size_t)(i0 + e) * kCtD] = __uint_as_float(d[e]);
         }
@@ -1039,7 +1038,7 @@ __global__ void __launch_bounds__(kCtThreads, 2)
 #pragma unroll
               for (int e = 0; e < 2; ++e) {
                 const int i = 16 * b + 2 * f + e;
-                v[e] = i < 31 ? dl[i] * tc::ex2((e31 - gt.gam2[i]) + (l31 - gt.glo[i])) : 0.f;
+                v[e] = dl[i] * tc::ex2((e31 - gt.gam2[i]) + (l31 - gt.glo[i]));
               }
               uint32_t s[kT];
               split_terms<kT>(v[0], v[1], s);
@@ -1078,7 +1077,7 @@ __global__ void __launch_bounds__(kCtThreads, 2)
           tc::tmem_ld16(tmS + lane_off + i0, *reinterpret_cast<uint32_t(*)[16]>(&d[0]));
           tc::tmem_ld16(tmS + lane_off + i0 + 16, *reinterpret_cast<uint32_t(*)[16]>(&d[16]));
           tc::tmem_ld_wait();
-          add_last(d, Kt + (n < 32 ? kCtD : 0) + i0, dl[31]);
+          if (n_item == 32) add_last(d, i0, d_last);
 #pragma unroll
           for (int e = 0; e < 32; ++e) S0s[(i0 + e) * kCtD + tid] = __uint_as_float(d[e]);
         }
