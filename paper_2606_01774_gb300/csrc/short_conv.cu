@@ -134,7 +134,6 @@ __device__ __forceinline__ int conv_check(const ConvParams& p, int r) {
 template <typename T, int W>
 __global__ void __launch_bounds__(kConvThreads + 32, ConvCols<T>::kCtasPerSM)
     short_conv_kernel(const __grid_constant__ ConvMaps maps, ConvParams p) {
-  stream_order();
   constexpr int E = sizeof(T);
   constexpr int kColBytes = ConvCols<T>::kColBytes;
   constexpr int kSlabBytes = ConvCols<T>::kSlabBytes;
@@ -166,16 +165,18 @@ __global__ void __launch_bounds__(kConvThreads + 32, ConvCols<T>::kCtasPerSM)
     n_issued = 0;
     tc::fence_mbar_init();
   }
+  if (tid == kConvThreads && maps.use) {
+    tc::prefetch_tmap(&maps.x_halo);
+    tc::prefetch_tmap(&maps.x_first);
+  }
+  // set up before the wait (one request 5.2 -> 4.9 us, 64 17.35 -> 17.22)
+  stream_order();
   __syncthreads();
 
   if (tid >= kConvThreads) {
     // producer warp: lane 0 stages every item of this CTA with the request's
     // slot, accepted length and validity
     if (tid == kConvThreads) {
-      if (maps.use) {
-        tc::prefetch_tmap(&maps.x_halo);
-        tc::prefetch_tmap(&maps.x_first);
-      }
       int k = 0;
       for (int idx = blockIdx.x; idx < n_items; idx += gridDim.x, ++k) {
         const int st = k % kStages;
